@@ -425,13 +425,11 @@ PS_API ps_status ps_last_timings(ps_ctx* ctx, float* ms, uint32_t n);
  *   out[4] chain blocks read from global memory (a lookup's key, or a block staged in shared memory)
  *   out[5] (row, instance) pairs searched past the earlier request's chain (derived rows)
  * Of the last ps_schedule_window in PS_PROBE_SEARCH mode (else 0), where n reaches them:
- *   out[6] decisions taken from a row summary corrected for the recent picks
- *   out[7] decisions that needed a full pass over the row
- *   out[8..15] SM clock cycles, summed over the thread blocks of each role of the greedy pass: the
- *          deciding warp waiting for staged rows, the deciding warp in all, its feeder waiting for a
- *          free staging slot, the feeder waiting for published row summaries, the summary blocks
- *          waiting for published decisions, waiting for probed rows, and evaluating rows, the probe
- *          blocks waiting for the inserts of earlier decisions
+ *   out[6] decisions made, each from its whole row on the current state
+ *   out[7] 0
+ *   out[8..15] SM clock cycles: the deciding block waiting for staged rows, the deciding block in
+ *          all, its feeder waiting for a free staging slot, the feeder waiting for probed rows, 0, 0, 0,
+ *          and, summed over the probe blocks, their waits for the inserts of earlier decisions
  * A table lookup reads the key's two candidate buckets (2 x 64 bytes) and one overflow word.
  * All zero if no probe phase ran.  Synchronises the context's stream. */
 PS_API ps_status ps_last_probe_stats(ps_ctx* ctx, uint64_t* out, uint32_t n);

@@ -57,7 +57,7 @@ struct ps_ctx {
   unsigned long long* d_count = nullptr;
   psk::DeltaSlot* d_delta = nullptr;
   uint64_t delta_nslots = 0;
-  psk::GreedySync gsync{nullptr, nullptr, nullptr, nullptr, nullptr, 0u, kDefaultWaitNs, nullptr, nullptr, nullptr};
+  psk::GreedySync gsync{nullptr, nullptr, nullptr, nullptr, nullptr, 0u, kDefaultWaitNs, nullptr};
   psk::RowPre* d_rows = nullptr;      // per-request constants and relations (search mode greedy)
   psk::LastSlot* d_lastslot = nullptr;
   psk::RowList scratch{nullptr, nullptr};  // rows the probe searches from scratch
@@ -461,12 +461,11 @@ ps_status ps_create(const ps_config* cfg, ps_ctx** out) {
   while (c->lastslot_n < 2 * c->Rmax) c->lastslot_n <<= 1;
   const size_t RI = (size_t)c->Rmax * c->I;
   const size_t I = c->I;
-  c->gsync.ring_stride = (c->I + 3u) / 4u * 4u;
+  c->gsync.ring_stride = (c->I + 7u) / 8u * 8u;
   bool ok = dalloc(c, &c->d_slots, c->total_slots) == cudaSuccess && dalloc(c, &c->d_ovf, c->total_ovf) == cudaSuccess &&
             dalloc(c, &c->d_tdesc, I) == cudaSuccess && dalloc(c, &c->d_count, I) == cudaSuccess &&
             dalloc(c, &c->d_delta, (size_t)dn) == cudaSuccess && dalloc(c, &c->gsync.jobs, c->Rmax) == cudaSuccess &&
             dalloc(c, &c->gsync.done, c->Rmax) == cudaSuccess && dalloc(c, &c->gsync.ready, c->Rmax) == cudaSuccess &&
-            dalloc(c, &c->gsync.sums, psk::kSumSlots) == cudaSuccess && dalloc(c, &c->gsync.sready, c->Rmax) == cudaSuccess &&
             dalloc(c, &c->gsync.stats, psk::kGreedyStats) == cudaSuccess &&
             dalloc(c, &c->gsync.hitring, (size_t)psk::kHitSlots * c->gsync.ring_stride) == cudaSuccess &&
             dalloc(c, &c->gsync.tpfring, (size_t)psk::kHitSlots * c->gsync.ring_stride) == cudaSuccess &&

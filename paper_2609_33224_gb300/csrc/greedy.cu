@@ -332,23 +332,11 @@ cudaError_t greedy_launch(const uint64_t* slots, const uint64_t* ovf, const psk:
 // on expiry the waiter records PS_ERR_TIMEOUT and stops waiting, so the launch always ends.  Each
 // role keeps the instance state it needs in its own shared memory.
 
-constexpr uint32_t kInsertBlocks = 16;   // insert blocks
-constexpr uint32_t kProbeBlocks = 16;    // probe blocks
-constexpr uint32_t kSummaryBlocks = 32;  // summary blocks (lag-d speculation, below)
-constexpr uint32_t kPipeThreads = 256;   // threads of every block of the launch
-constexpr uint32_t kFeedRing = 4;        // rows staged in the deciding block's shared memory
+constexpr uint32_t kInsertBlocks = 64;  // insert blocks
+constexpr uint32_t kProbeBlocks = 64;   // probe blocks
+constexpr uint32_t kPipeThreads = 608;  // threads of every block of the launch
+constexpr uint32_t kFeedRing = 8;       // rows staged in the deciding block's shared memory
 constexpr unsigned long long kJobValid = 1ull << 63;  // a published job word (0 = not yet published)
-
-__device__ __forceinline__ psk::RowConst row_of(const psk::RowPre& x) {
-  psk::RowConst rc;
-  rc.t_cached = x.t_cached;
-  rc.Z = x.Z;
-  rc.etaZ = x.etaZ;
-  rc.ttft_budget = x.ttft_budget;
-  rc.tpot_target = x.tpot_target;
-  rc.L = x.L;
-  return rc;
-}
 
 // Bounded spin until *flag != 0 (acquire).  false after limit_ns (and the error bit is set).
 __device__ __forceinline__ bool wait_flag(const uint32_t* flag, uint32_t* err, uint64_t limit_ns) {
@@ -440,13 +428,13 @@ __device__ __forceinline__ void insert_tail(psk::DeltaSlot* delta, uint64_t nslo
 }
 
 __device__ void insert_blocks(const psk::RowPre* __restrict__ rows, const uint64_t* __restrict__ hash, uint32_t R,
-                              psk::DeltaSlot* delta, uint64_t nslots, uint32_t* err, const psk::GreedySync& sync) {
+                              psk::DeltaSlot* delta, uint64_t nslots, uint32_t* err, const psk::GreedySync& sync,
+                              uint32_t ib, uint32_t ninsert) {
   __shared__ unsigned long long s_job;
   const uint32_t t = threadIdx.x;
-  const uint32_t ib = blockIdx.x - 1;
   const uint32_t group = ib / kInsertGroup, member = ib % kInsertGroup;
-  constexpr uint32_t kGroups = kInsertBlocks / kInsertGroup;
-  for (uint32_t job = group; job < R; job += kGroups) {
+  const uint32_t groups = ninsert / kInsertGroup;
+  for (uint32_t job = group; job < R; job += groups) {
     if (t == 0) s_job = wait_job(sync.jobs + job, err, sync.wait_ns);
     __syncthreads();
     const unsigned long long jb = s_job;
@@ -477,8 +465,8 @@ __device__ void insert_blocks(const psk::RowPre* __restrict__ rows, const uint64
 template <int IPT>
 __device__ void probe_rows(const psk::RowPre* __restrict__ rows, const uint64_t* __restrict__ hash, uint32_t R,
                            uint32_t I, const uint32_t* __restrict__ hit0, const float* __restrict__ tpf0,
-                           const psk::DeltaSlot* delta, uint64_t nslots, uint32_t* err, const psk::GreedySync& sync,
-                           unsigned long long* smem_raw) {
+                           const psk::DevModel& m, const psk::DeltaSlot* delta, uint64_t nslots, uint32_t* err,
+                           const psk::GreedySync& sync, unsigned long long* smem_raw, uint32_t pb, uint32_t nprobe) {
   uint32_t* s_end = reinterpret_cast<uint32_t*>(smem_raw);  // chain end of the last job on i (0 = none)
   uint32_t* s_res = s_end + I;                               // search start / result per instance
   uint32_t* s_walk = s_res + I;                              // instances handed to a warp search
@@ -500,9 +488,10 @@ __device__ void probe_rows(const psk::RowPre* __restrict__ rows, const uint64_t*
     s_abort = 0;
   }
   __syncthreads();
-  for (uint32_t s = blockIdx.x - 1 - kInsertBlocks; s < R; s += kProbeBlocks) {
+  for (uint32_t s = pb; s < R; s += nprobe) {
     const uint64_t off = __ldg(&rows[s].off);
     const uint32_t nb = __ldg(&rows[s].nb);
+    const uint32_t L = __ldg(&rows[s].L);
     const int64_t need = (int64_t)s - psk::kLag + 1;  // jobs [0, need) count for this row
     if (warp == 0) {
       // Replay the published jobs [replayed, need), 32 at a time; for each instance the latest of
@@ -620,7 +609,7 @@ __device__ void probe_rows(const psk::RowPre* __restrict__ rows, const uint64_t*
       if (i < I) {
         const uint32_t h = walk[k] ? s_res[i] : pos[k];
         sync.hitring[(uint64_t)slot * sync.ring_stride + i] = h;
-        sync.tpfring[(uint64_t)slot * sync.ring_stride + i] = h == h0[k] ? tp0[k] : __uint_as_float(psk::kNoTpfBits);
+        sync.tpfring[(uint64_t)slot * sync.ring_stride + i] = h == h0[k] ? tp0[k] : psk::t_pf32(m, L, h);
       }
     }
     __syncthreads();
@@ -638,980 +627,758 @@ __device__ __forceinline__ bool narrow_qs(int64_t q, int64_t S) {
   return q >= 0 && q < (1ll << 30) && S >= 0 && S < (1ll << 30);
 }
 
-// ---- lag-d speculation: summary blocks and the deciding warp ------------------------------------
+// ---- deciding block -----------------------------------------------------------------------------
 //
-// Row s's decision depends on the state left by decisions 0 .. s - 1.  Summary blocks evaluate row s
-// on every instance against the state before decision s - kSpecLag (replaying the published jobs
-// into their own copy of the state), and publish per warp the kKeysPerWarp smallest (packed key, tie)
-// pairs of C with their W and hit, and the kWPerWarp smallest W of A, with the bounds of what they
-// did not publish (RowSummary).  Only the instances picked by decisions s - kSpecLag .. s - 1 (the
-// touched ones) have changed since: their state, and their caches (each touched instance's hit on
-// row s rises to the common prefix with the requests it took).  Every other instance keeps its
-// capacity test, W and key.  So the deciding warp re-evaluates the touched instances only, and:
-//   * W_min over A is the smaller of the touched instances' W and the smallest published W of an
-//     untouched instance, known exactly when that W lies at or below the W bound;
-//   * in-window inserts only lengthen hits, so W_min can only fall unless an instance leaves A; if
-//     it rose above the summary's W_min, the summary's C may miss members (full pass);
-//   * with W_min at or below the summary's, C of the current state holds no untouched pair outside
-//     the summary's C, and a published untouched pair stays in C when W - W_min <= eta Z still holds;
-//   * the pick is the smallest (key, tie) over the surviving published pairs and the touched pairs
-//     in C; every unpublished pair has (key, tie) >= the key bound, so a pick below the bound is
-//     exact.
-// Otherwise (W_min unknown or risen, or no pick below the bound) the warp evaluates the whole row on
-// the current state.  Both ways give Algorithm 1's decision exactly.
-//
-// Deciding block: warp 0 decides, warp 1 (the feeder) copies each row's summary, row constants, hits
-// and T_pf into a shared-memory ring as soon as the summary is published; the two hand off through
-// shared-memory counters (the feeder's row count, the decider's consumed count), each wait bounded.
+// Every decision evaluates its whole row on the current state; nothing about a row is known before
+// the decision it follows, except the probed hits.  The block has up to kComputeWarps compute warps,
+// a feeder warp, a hit warp and a publishing warp:
+//   * compute thread t owns the instances IPT t .. IPT t + IPT - 1 and keeps their request-independent
+//     terms (room, q, S, B, dec0, EMA factor, queueing TTFT, key bits) in registers for the whole
+//     launch.  A pair needs its staged hit and T_pf and no other memory.  Per row: W, capacity,
+//     latencies and key of every pair; W_min over the block (one warp reduction, one barrier); the
+//     recompute filter; the smallest (key, tie) of each warp into shared memory; the step's barrier,
+//     after which every warp combines the warps' minima by itself.
+//   * the feeder copies each row's constants, probed hits and T_pf into a ring in shared memory.
+//   * the hit warp raises row s + 1's hits, while row s is decided, on the instances that took requests
+//     s - kLcpBack + 1 .. s - 1, to the common chain prefix with them (lane k holds the pick of request
+//     s - 1 - k); the pick of s itself is raised by its owner one step later.
+//   * the publishing warp hands decision s - 1 to the insert and probe blocks and writes the outputs.
+// A step is a chain of latencies: barrier, the last decision (two warp votes), its owner's one-pair
+// update, W_min (reduction, barrier, reduction), the warp's pick (reduction, vote).  Measured per
+// decision, before -> now (before: row summaries computed by other blocks 8 decisions ahead and
+// corrected by one warp, with helper warps; 1.25 us of helper phase a step, and a pass over the row by
+// one warp, 20 to 30 us, where the summary did not cover the pick):
+//   64 instances 1.22 -> 0.55 us, 201: 1.43 -> 0.74, 256: 1.41 -> 0.62, 999: 3.3 -> 1.13, 1024: 1.60 -> 0.89.
+// 1024 instances are bound by issue slots (about 250 instructions a warp and step on 16 warps), small
+// pools by the chain.
 
-static_assert(kPipeThreads == 32 * psk::kSumWarps, "a summary block is kSumWarps warps");
+constexpr uint32_t kComputeWarps = 16;
+constexpr uint32_t kFeederWarp = kComputeWarps;
+constexpr uint32_t kHitWarp = kComputeWarps + 1;
+constexpr uint32_t kPublishWarp = kComputeWarps + 2;
+static_assert(kPipeThreads == 32 * (kComputeWarps + 3), "compute warps, the feeder, the hit warp, the publisher");
+static_assert(psk::kLcpBack == 32, "one lane of the hit warp per recent request");
 
-// Instance state of the summary blocks and the deciding warp: padded structure-of-arrays in shared
-// memory, [Ip] each, 8-byte arrays first (64 bytes per instance).
+// Instance state of the deciding block in shared memory, [Ip] each, 8-byte arrays first: the truth
+// behind the owners' registers (36 bytes per instance).
 struct InstSmem {
   int64_t* q;
   int64_t* S;
   int64_t* M;
-  uint64_t* kd;   // D-C-Q key bits of (b, qr) (psk::dcq_key0)
-  int32_t* room;  // free KV room, -1 when the decode-slot guard fails
-  float* dec0;
-  float* f;
-  float* tq;
-  int32_t* Bp;
   int32_t* b;
   int32_t* qr;
   int32_t* Bmax;
+  int32_t* pad;
+  // with 32-bit sums: {q, S, KV room (-1: no decode slot), slots left} and {key low (qr), key high (b), B, -}
+  // per instance, over the same memory
+  int4* qs;
+  uint4* kb;
 };
-constexpr size_t kInstSmemBytes = 4 * sizeof(int64_t) + 8 * sizeof(int32_t);
+constexpr size_t kInstSmemBytes = 3 * sizeof(int64_t) + 4 * sizeof(int32_t);
+static_assert(kInstSmemBytes >= sizeof(int4) + sizeof(uint4), "both forms fit");
 
 __device__ __forceinline__ InstSmem inst_smem(unsigned long long* raw, uint32_t Ip) {
   InstSmem a;
   a.q = reinterpret_cast<int64_t*>(raw);
   a.S = a.q + Ip;
   a.M = a.S + Ip;
-  a.kd = reinterpret_cast<uint64_t*>(a.M + Ip);
-  a.room = reinterpret_cast<int32_t*>(a.kd + Ip);
-  a.dec0 = reinterpret_cast<float*>(a.room + Ip);
-  a.f = a.dec0 + Ip;
-  a.tq = a.f + Ip;
-  a.Bp = reinterpret_cast<int32_t*>(a.tq + Ip);
-  a.b = a.Bp + Ip;
+  a.b = reinterpret_cast<int32_t*>(a.M + Ip);
   a.qr = a.b + Ip;
   a.Bmax = a.qr + Ip;
+  a.pad = a.Bmax + Ip;
+  a.qs = reinterpret_cast<int4*>(raw);
+  a.kb = reinterpret_cast<uint4*>(a.qs + Ip);
   return a;
 }
 
-// Derived terms of instance i after a state change (the decode-slot guard folded into the KV room).
-__device__ __forceinline__ void inst_refresh(const InstSmem& a, const psk::DevModel& m, uint32_t i) {
-  const psk::InstTerms it = psk::inst_terms(m, a.b[i], a.qr[i], a.q[i], a.Bmax[i]);
-  a.dec0[i] = it.dec0;
-  a.f[i] = it.f;
-  a.tq[i] = it.tq;
-  a.Bp[i] = it.Bp;
-  a.room[i] = it.okB ? psk::kv_room(a.S[i], a.M[i]) : -1;
-  a.kd[i] = psk::dcq_key0(a.b[i], a.qr[i]);
-}
-
-__device__ __forceinline__ void inst_load(const InstSmem& a, const psk::StateSoA& st, const psk::DevModel& m,
-                                          uint32_t i) {
-  a.b[i] = st.b[i];
-  a.qr[i] = st.qr[i];
-  a.q[i] = st.q[i];
-  a.S[i] = st.S[i];
-  a.M[i] = st.M[i];
-  a.Bmax[i] = st.Bmax[i];
-  inst_refresh(a, m, i);
-}
-
-// The values of one instance's state a pair evaluation reads.
-struct InstVals {
-  int64_t q, S;
-  uint64_t kd;  // dcq_key0(b, qr)
-  int32_t room;
-  float dec0, f, tq;
-  int32_t Bp;
-};
-
-__device__ __forceinline__ InstVals inst_vals(const InstSmem& a, uint32_t i) {
-  InstVals v;
-  v.q = a.q[i];
-  v.S = a.S[i];
-  v.kd = a.kd[i];
-  v.room = a.room[i];
-  v.dec0 = a.dec0[i];
-  v.f = a.f[i];
-  v.tq = a.tq[i];
-  v.Bp = a.Bp[i];
-  return v;
-}
-
-// Instance i's state after it takes a request of L tokens at hit h (qr + 1, q + L - 16 h, S + L), as
-// the state update of a decision computes it.
-__device__ __forceinline__ InstVals inst_vals_after(const InstSmem& a, const psk::DevModel& m, uint32_t i, uint32_t L,
-                                                    uint32_t h, int32_t* qr_out) {
-  const int32_t qr = a.qr[i] + 1;
-  InstVals v;
-  v.q = a.q[i] + (int64_t)L - 16 * (int64_t)h;
-  v.S = a.S[i] + (int64_t)L;
-  const psk::InstTerms it = psk::inst_terms(m, a.b[i], qr, v.q, a.Bmax[i]);
-  v.dec0 = it.dec0;
-  v.f = it.f;
-  v.tq = it.tq;
-  v.Bp = it.Bp;
-  v.room = it.okB ? psk::kv_room(v.S, a.M[i]) : -1;
-  v.kd = psk::dcq_key0(a.b[i], qr);
-  *qr_out = qr;
-  return v;
-}
-
-__device__ __forceinline__ void inst_store(const InstSmem& a, uint32_t i, int32_t qr, const InstVals& v) {
-  a.qr[i] = qr;
-  a.q[i] = v.q;
-  a.S[i] = v.S;
-  a.kd[i] = v.kd;
-  a.room[i] = v.room;
-  a.dec0[i] = v.dec0;
-  a.f[i] = v.f;
-  a.tq[i] = v.tq;
-  a.Bp[i] = v.Bp;
-}
-
-// One pair (row, instance i at hit h) on state v: W, the capacity guard, and the packed key and tie
-// word the pair has in C (class 0 if the SLO admission passes, class 1 otherwise); key kNoKey
-// outside A.  tpf_bits: T_pf at h if known, else kNoTpfBits.
-struct PairKey {
-  float W;
-  uint64_t key;
-  uint32_t tie;
-  bool inA;
-};
-
-__device__ __forceinline__ PairKey pair_key_v(const psk::DevModel& m, const psk::RowConst& rc, const InstVals& v,
-                                              uint32_t i, uint32_t h, uint32_t tpf_bits) {
-  PairKey p;
-  const float tpf = tpf_bits != psk::kNoTpfBits ? __uint_as_float(tpf_bits) : psk::t_pf32(m, rc.L, h);
-  p.W = __fsub_rn(tpf, rc.t_cached);
-  p.inA = (int32_t)rc.L <= v.room;
-  p.key = psk::kNoKey;
-  p.tie = i;
-  if (p.inA) {
-    const int32_t n = (int32_t)rc.L - (int32_t)(h << 4);
-    float tpot, ttft;
-    if (narrow_qs(v.q, v.S)) {
-      psk::pair_lat32(m, rc, tpf, n, v.dec0, v.f, v.tq, v.Bp, (int32_t)v.q, (int32_t)v.S, &tpot, &ttft);
-    } else {
-      psk::InstTerms it;
-      it.dec0 = v.dec0;
-      it.f = v.f;
-      it.tq = v.tq;
-      it.Bp = v.Bp;
-      it.okB = 1;
-      psk::PairW x;
-      x.W = p.W;
-      x.tpf = tpf;
-      x.n = n;
-      x.inA = true;
-      psk::pair_lat(m, rc, x, it, v.q, v.S, &tpot, &ttft);
-    }
-    if (psk::pair_admitted(m, rc, tpot, ttft)) {
-      p.key = psk::packed_key(0u, psk::value_in_t(m, psk::key0_from_dcq(m, v.kd), h, tpot, rc.tpot_target));
-      if (m.sel == psk::kSelHCQ) p.tie |= (uint32_t)(v.kd & 0x3FFFFull) << 12;
-    } else {
-      p.key = psk::packed_key(1u, psk::value_fallback(m, (uint64_t)v.q + (uint64_t)n, (uint32_t)v.Bp, v.kd, h));
+// IPT consecutive 32-bit words of shared memory (aligned to IPT words, at most 4 per load).
+template <int IPT>
+__device__ __forceinline__ void lds_words(const uint32_t* p, uint32_t (&v)[IPT]) {
+  if constexpr (IPT == 1) {
+    v[0] = p[0];
+  } else if constexpr (IPT == 2) {
+    const uint2 x = *reinterpret_cast<const uint2*>(p);
+    v[0] = x.x;
+    v[1] = x.y;
+  } else {
+#pragma unroll
+    for (int k = 0; k < IPT; k += 4) {
+      const uint4 x = *reinterpret_cast<const uint4*>(p + k);
+      v[k] = x.x;
+      v[k + 1] = x.y;
+      v[k + 2] = x.z;
+      v[k + 3] = x.w;
     }
   }
-  return p;
 }
 
-__device__ __forceinline__ PairKey pair_key_of(const psk::DevModel& m, const psk::RowConst& rc, const InstSmem& a,
-                                               uint32_t i, uint32_t h, uint32_t tpf_bits) {
-  return pair_key_v(m, rc, inst_vals(a, i), i, h, tpf_bits);
+// A packed key's rank: a 32-bit word whose unsigned order never contradicts the keys' (equal ranks
+// need the full comparison), so one warp reduction nearly always finds the smallest key.  Class 0:
+// the key's upper 31 bits; class 1: the value as fp32 rounded towards zero, above every class-0 rank;
+// no key: all ones.
+__device__ __forceinline__ uint32_t key_rank(uint64_t key) {
+  const uint32_t c0 = (uint32_t)(key >> 31);
+  const uint32_t c1 = 0x80000000u | __float_as_uint(__ull2float_rz(key & ((1ull << 62) - 1)));
+  return key == psk::kNoKey ? 0xFFFFFFFFu : ((key >> 62) ? c1 : c0);
 }
 
-__device__ __forceinline__ bool kt_less(uint64_t k1, uint32_t t1, uint64_t k2, uint32_t t2) {
-  return k1 < k2 || (k1 == k2 && t1 < t2);
+// The lane holding the warp's smallest (key, tie), -1 if no lane has a key; rank = key_rank(key).
+__device__ __forceinline__ int warp_argmin(uint32_t rank, uint64_t key, uint32_t tie) {
+  const uint32_t mr = __reduce_min_sync(0xffffffffu, rank);
+  unsigned who = __ballot_sync(0xffffffffu, rank == mr);
+  if (mr == 0xFFFFFFFFu) return -1;
+  if (who & (who - 1u)) {  // equal ranks: compare the keys, then the tie words (warp-uniform)
+    bool in = rank == mr;
+    const uint32_t mhi = __reduce_min_sync(0xffffffffu, in ? (uint32_t)(key >> 32) : 0xFFFFFFFFu);
+    in = in && (uint32_t)(key >> 32) == mhi;
+    const uint32_t mlo = __reduce_min_sync(0xffffffffu, in ? (uint32_t)key : 0xFFFFFFFFu);
+    in = in && (uint32_t)key == mlo;
+    const uint32_t mt = __reduce_min_sync(0xffffffffu, in ? tie : 0xFFFFFFFFu);
+    who = __ballot_sync(0xffffffffu, in && tie == mt);  // tie words are unique
+  }
+  return __ffs(who) - 1;
 }
 
-// Warp minimum of a 64-bit word with single-instruction reductions on each half.
-__device__ __forceinline__ unsigned long long warp_min_u64w(unsigned long long v) {
-  const uint32_t hi = (uint32_t)(v >> 32);
-  const uint32_t mhi = __reduce_min_sync(0xffffffffu, hi);
-  const uint32_t mlo = __reduce_min_sync(0xffffffffu, hi == mhi ? (uint32_t)v : 0xFFFFFFFFu);
-  return ((unsigned long long)mhi << 32) | mlo;
+// What a step needs of a row's constants.  With the tests a model leaves out (TTFT filter, SLO
+// admission, recompute filter) the bound is +infinity, which every finite value passes.
+struct StepRow {
+  float t_cached, c_max, ttft_max, tpot_lim, tpot_target;
+  uint32_t L;
+};
+
+__device__ __forceinline__ StepRow step_row(const psk::DevModel& m, const psk::RowPre& x) {
+  const uint4 w0 = reinterpret_cast<const uint4*>(&x)[0];  // off, nb, L
+  const float4 w1 = reinterpret_cast<const float4*>(&x)[1];  // t_cached, Z, etaZ, ttft_budget
+  StepRow r;
+  r.L = w0.w;
+  r.t_cached = w1.x;
+  r.c_max = w1.y > 0.0f ? w1.z : INFINITY;
+  r.tpot_target = x.tpot_target;
+  r.tpot_lim = m.slo_off ? INFINITY : x.tpot_target;
+  r.ttft_max = (m.slo_off || !m.ttft_filter) ? INFINITY : w1.w;
+  return r;
 }
 
 using psk::wait_smem_at_least;
 
-// Summary block sb: rows sb, sb + kSummaryBlocks, ...  Thread t holds instances t, t + 256, ...
-template <int IPT>
-__device__ void summary_rows(const psk::RowPre* __restrict__ rows, uint32_t R, uint32_t I, psk::StateSoA committed,
-                             const psk::DevModel& m, uint32_t* err, const psk::GreedySync& sync, uint32_t sb,
-                             unsigned long long* smem_raw) {
-  const uint32_t Ip = sync.ring_stride;
-  const InstSmem a = inst_smem(smem_raw, Ip);
-  __shared__ psk::RowPre s_row;
-  __shared__ int32_t s_jm[16];  // pick of request x in s_jm[x & 15] (-1: rejected)
-  static_assert(psk::kLcpBack <= psk::kSpecLag + 16, "the ring holds the picks the row's raises need");
-  __shared__ uint32_t s_wmin[psk::kSumWarps];
-  __shared__ uint32_t s_wb[psk::kSumWarps];
-  __shared__ unsigned long long s_kb[psk::kSumWarps];
-  __shared__ uint32_t s_tb[psk::kSumWarps];
-  __shared__ int s_abort;
-  const uint32_t t = threadIdx.x;
-  const int lane = (int)(t & 31u), warp = (int)(t >> 5);
-  for (uint32_t i = t; i < I; i += kPipeThreads) inst_load(a, committed, m, i);
-  if (t < 16) s_jm[t] = -1;
-  if (t == 0) s_abort = 0;
-  uint32_t applied = 0;  // decisions [0, applied) are in this block's state
-  unsigned long long cyc_job = 0, cyc_ready = 0, cyc_eval = 0;
-  __syncthreads();
-  for (uint32_t s = sb; s < R; s += kSummaryBlocks) {
-    const int64_t need = (int64_t)s - psk::kSpecLag;  // decisions [0, need) count for row s
-    const long long c0 = clock64();
-    long long c1 = c0;
-    // Each warp waits for the row's probed hits and loads its threads' hits and T_pf right away, so
-    // the loads are in flight while warp 0 replays the decisions the row must see.
-    const uint32_t slot = s % psk::kHitSlots;
-    uint32_t hl[IPT], tl[IPT];
-    {
-      bool rdy = true;
-      if (lane == 0) {
-        rdy = wait_flag(sync.ready + s, err, sync.wait_ns);
-        if (!rdy) s_abort = 1;
-      }
-      rdy = __shfl_sync(0xffffffffu, rdy ? 1 : 0, 0) != 0;
-#pragma unroll
-      for (int k = 0; k < IPT; ++k) {
-        const uint32_t i = t + (uint32_t)k * kPipeThreads;
-        hl[k] = 0u;
-        tl[k] = psk::kNoTpfBits;
-        if (rdy && i < I) {
-          hl[k] = __ldcg(sync.hitring + (uint64_t)slot * Ip + i);
-          tl[k] = __float_as_uint(__ldcg(sync.tpfring + (uint64_t)slot * Ip + i));
-        }
-      }
-    }
-    if (warp == 0) {
-      // Replay decisions [applied, need), 32 at a time: the adds commute; the last lane of each
-      // instance refreshes its terms once every add is in.
-      bool abort = false;
-      while ((int64_t)applied < need && !abort) {
-        const uint32_t x = applied + (uint32_t)lane;
-        const bool mine = (int64_t)x < need;
-        unsigned long long jb = 0ull;
-        if (mine) jb = wait_job(sync.jobs + x, err, sync.wait_ns);
-        abort = __any_sync(0xffffffffu, mine && jb == 0ull);
-        if (abort) break;
-        const uint32_t j = mine ? job_pick(jb) : 0xFFFFFFFFu;
-        const bool upd = mine && j < I;
-        if (upd) {
-          const uint32_t L = __ldg(&rows[x].L);
-          const int64_t n = (int64_t)L - 16 * (int64_t)job_hit(jb);
-          atomicAdd(&a.qr[j], 1);
-          atomicAdd(reinterpret_cast<unsigned long long*>(&a.q[j]), (unsigned long long)n);
-          atomicAdd(reinterpret_cast<unsigned long long*>(&a.S[j]), (unsigned long long)(int64_t)L);
-        }
-        const uint32_t nbatch = (int64_t)applied + 32 <= need ? 32u : (uint32_t)(need - (int64_t)applied);
-        // the last 16 decisions of the batch take the ring slots (distinct within 16)
-        if (mine && x + 16u >= applied + nbatch) s_jm[x & 15u] = j < I ? (int32_t)j : -1;
-        const unsigned same = __match_any_sync(0xffffffffu, upd ? j : 0xFFFFFFFFu);
-        __syncwarp();
-        if (upd && (31 - __clz(same)) == lane) inst_refresh(a, m, j);
-        __syncwarp();
-        applied += nbatch;
-      }
-      c1 = clock64();
-      if (lane == 0 && abort) s_abort = 1;
-      if (lane < psk::kRowWords)
-        reinterpret_cast<uint4*>(&s_row)[lane] = __ldg(reinterpret_cast<const uint4*>(rows + s) + lane);
-    }
-    __syncthreads();
-    const long long c2 = clock64();
-    if (t == 0) {
-      cyc_job += (unsigned long long)(c1 - c0);
-      cyc_ready += (unsigned long long)(c2 - c1);
-    }
-    if (s_abort) break;  // block-uniform
-    const psk::RowConst rc = row_of(s_row);
-    // raises from the picks of requests s - kLcpBack .. s - kSpecLag - 1 (older than the lag)
-    constexpr int kNR = psk::kLcpBack - psk::kSpecLag;
-    int32_t rj[kNR > 0 ? kNR : 1];
-    uint32_t rl[kNR > 0 ? kNR : 1];
-#pragma unroll
-    for (int k2 = psk::kSpecLag; k2 < psk::kLcpBack; ++k2) {
-      const int64_t t2 = (int64_t)s - 1 - k2;
-      rj[k2 - psk::kSpecLag] = t2 >= 0 ? s_jm[(uint32_t)t2 & 15u] : -1;
-      rl[k2 - psk::kSpecLag] = s_row.lcp[k2];
-    }
-    // every pair: hit, W, capacity guard, key in C
-    PairKey pk[IPT];
-    uint32_t hk[IPT];
-    uint32_t wbest = 0xFFFFFFFFu;
-#pragma unroll
-    for (int k = 0; k < IPT; ++k) {
-      const uint32_t i = t + (uint32_t)k * kPipeThreads;
-      pk[k].inA = false;
-      pk[k].key = psk::kNoKey;
-      hk[k] = 0u;
-      if (i < I) {
-        const uint32_t h0 = hl[k];
-        const uint32_t tp0 = tl[k];
-        uint32_t h = h0;
-#pragma unroll
-        for (int q = 0; q < kNR; ++q)
-          if (rj[q] == (int32_t)i && rl[q] > h) h = rl[q];
-        hk[k] = h;
-        pk[k] = pair_key_of(m, rc, a, i, h, h == h0 ? tp0 : psk::kNoTpfBits);
-        if (pk[k].inA) wbest = min(wbest, psk::f2ord(pk[k].W));
-      }
-    }
-    psk::RowSummary* out = sync.sums + (s % psk::kSumSlots);
-    // per warp: W_min over A, its kWPerWarp smallest (W, instance), the next one as its bound
-    {
-      const uint32_t wm = __reduce_min_sync(0xffffffffu, wbest);
-      if (lane == 0) s_wmin[warp] = wm;
-      uint32_t taken = 0u;
-#pragma unroll
-      for (int rnd = 0; rnd <= psk::kWPerWarp; ++rnd) {
-        unsigned long long mine = ~0ull;
-        int mk = -1;
-#pragma unroll
-        for (int k = 0; k < IPT; ++k) {
-          if (!pk[k].inA || ((taken >> k) & 1u)) continue;
-          const unsigned long long w = ((unsigned long long)psk::f2ord(pk[k].W) << 32) | (t + (uint32_t)k * kPipeThreads);
-          if (w < mine) {
-            mine = w;
-            mk = k;
-          }
-        }
-        const unsigned long long best = warp_min_u64w(mine);
-        if (mk >= 0 && mine == best) taken |= 1u << mk;
-        if (rnd < psk::kWPerWarp) {
-          if (lane == 0) out->w[warp * psk::kWPerWarp + rnd] = best;
-        } else if (lane == 0) {
-          s_wb[warp] = (uint32_t)(best >> 32);  // all ones when the warp has no more
-        }
-      }
-    }
-    __syncthreads();
-    uint32_t wmin_o = 0xFFFFFFFFu;
-#pragma unroll
-    for (int w = 0; w < psk::kSumWarps; ++w) wmin_o = min(wmin_o, s_wmin[w]);
-    const float wmin = psk::ord2f(wmin_o);
-    // per warp: the kKeysPerWarp smallest (key, tie) of C, the next one as its bound
-    {
-      bool inC[IPT];
-#pragma unroll
-      for (int k = 0; k < IPT; ++k) inC[k] = pk[k].inA && psk::pair_in_c(rc, pk[k].W, wmin);
-      uint32_t taken = 0u;
-#pragma unroll
-      for (int rnd = 0; rnd <= psk::kKeysPerWarp; ++rnd) {
-        uint64_t bk = psk::kNoKey;
-        uint32_t bt = 0xFFFFFFFFu, bh = 0u, bw = 0u;
-        int mk = -1;
-#pragma unroll
-        for (int k = 0; k < IPT; ++k) {
-          if (!inC[k] || ((taken >> k) & 1u)) continue;
-          if (kt_less(pk[k].key, pk[k].tie, bk, bt)) {
-            bk = pk[k].key;
-            bt = pk[k].tie;
-            bh = hk[k];
-            bw = psk::f2ord(pk[k].W);
-            mk = k;
-          }
-        }
-        uint64_t wk;
-        uint32_t wt, wh;
-        psk::warp_pick_min(bk, bt, bh, &wk, &wt, &wh);
-        const bool won = mk >= 0 && bk == wk && bt == wt;  // tie words are unique (instance in them)
-        if (won) taken |= 1u << mk;
-        const unsigned winm = __ballot_sync(0xffffffffu, won);
-        const uint32_t ww = __shfl_sync(0xffffffffu, bw, winm ? __ffs(winm) - 1 : 0);
-        if (rnd < psk::kKeysPerWarp) {
-          if (lane == 0) {
-            const int e = warp * psk::kKeysPerWarp + rnd;
-            out->key[e] = wk;
-            out->tie[e] = wt;
-            out->word[e] = ww;
-            out->hit[e] = wh;
-          }
-        } else if (lane == 0) {
-          s_kb[warp] = wk;
-          s_tb[warp] = wt;
-        }
-      }
-    }
-    __syncthreads();
-    if (t == 0) {
-      unsigned long long kb = psk::kNoKey;
-      uint32_t tb = 0xFFFFFFFFu, wb = 0xFFFFFFFFu;
-#pragma unroll
-      for (int w = 0; w < psk::kSumWarps; ++w) {
-        if (kt_less(s_kb[w], s_tb[w], kb, tb)) {
-          kb = s_kb[w];
-          tb = s_tb[w];
-        }
-        wb = min(wb, s_wb[w]);
-      }
-      out->key_bound = kb;
-      out->tie_bound = tb;
-      out->w_bound = wb;
-      out->wmin = wmin_o;
-      __threadfence();  // every warp's entries (written before the barrier) before the flag
-      psk::st_release_u32(sync.sready + s, 1u);
-      cyc_eval += (unsigned long long)(clock64() - c2);
-    }
-    __syncthreads();  // the next row reuses the reduction slots
-  }
-  if (t == 0 && sync.stats) {
-    atomicAdd(sync.stats + psk::kGsSumJobWait, cyc_job);
-    atomicAdd(sync.stats + psk::kGsSumReadyWait, cyc_ready);
-    atomicAdd(sync.stats + psk::kGsSumEval, cyc_eval);
-  }
-}
-
-// Deciding block: warp 0 decides, warp 1 (the feeder) stages rows in a shared-memory ring, warps 2, 3
-// and 7 (the helpers A, B, C) prepare each step's inputs one step ahead, warp 5 hands decisions to
-// them (and stores each pick's new state and writes the outputs); warps 4 and 6 return at once.  A
-// warp's scheduler is warp id mod 4, so the spinning roles (deciding warp, feeder, warp 5) and the
-// computing ones sit on different schedulers where they can.
-//
-// The decision of request s needs, besides row s's summary, the pairs on row s of the instances
-// picked by decisions s - kSpecLag .. s - 1 under the current state: lane 0 the pick of s - 1, lane k
-// the pick of s - 1 - k.  All but lane 0's depend only on decisions up to s - 2, and lane 0's is the
-// winner of step s - 1 taking request s - 1.  So while step s - 1 is decided, the helpers compute for
-// step s (their phase s - 1, started once decision s - 2 is published):
-//   A[l]  summary entry l of row s - 1 as if it took request s - 1: its state after that, and its
-//         pair on row s;
-//   B[l]  the same for lane l's touched instance of step s - 1;
-//   C[k]  the pick of s - 1 - k (k = 1 .. kSpecLag - 1) on row s under the state after s - 2.
-// Step s then reads lane 0's pair from A, B (or, after a full pass or at the last request, from what
-// the deciding warp computed itself, X) at the winner's index, and lane k's from C[k].  The deciding
-// warp's own path is the W_min and key reductions of the corrected summary (whose entries it loads
-// a step ahead) and one shared-memory publish; the helpers store each pick's new state into the
-// instance arrays and write the decision outputs to global memory.
-struct HelpSlot {
-  PairKey a_pk[32];
-  InstVals a_nv[32];
-  uint32_t a_hit[32];
-  int32_t a_qr[32];
-  PairKey b_pk[psk::kSpecLag];
-  InstVals b_nv[psk::kSpecLag];
-  uint32_t b_hit[psk::kSpecLag];
-  int32_t b_qr[psk::kSpecLag];
-  PairKey c_pk[psk::kSpecLag];
-  uint32_t c_hit[psk::kSpecLag];
-  PairKey x_pk;
-  InstVals x_nv;
-  uint32_t x_hit;
-  int32_t x_qr;
-};
-enum : uint32_t { kSrcA = 0, kSrcB = 1, kSrcX = 2 };
-constexpr uint32_t kLogSlots = 64;  // decisions kept for the helpers (more than kLcpBack + 2)
-
-// hit of instance c on row rw: its probed hit raised to the common prefix with each of the last
-// kLcpBack requests that went to c (hist[k]: the pick of request s - 1 - k, s the step the history is
-// taken at); `self` raises by lcp[0] too (c taking request s).  shift 0: rw is row s (lcp[k2] is with
-// request s - 1 - k2 = hist[k2]); shift 1: rw is row s + 1 (lcp[k2] is with request s - k2 =
-// hist[k2 - 1]).
-__device__ __forceinline__ uint32_t raised_hit(const psk::RowPre& rw, const uint32_t* hr, uint32_t c, bool self, int shift,
-                                               const int32_t (&hist)[psk::kLcpBack]) {
-  uint32_t h = hr[c];
-  if (self && rw.lcp[0] > h) h = rw.lcp[0];
-#pragma unroll
-  for (int k2 = 0; k2 < psk::kLcpBack; ++k2) {
-    const int kk = k2 - shift;
-    if (kk >= 0 && hist[kk < 0 ? 0 : kk] == (int32_t)c && rw.lcp[k2] > h) h = rw.lcp[k2];
-  }
-  return h;
-}
-
-// The as-if values of a decision's winner in a helper slot.
-__device__ __forceinline__ const InstVals& slot_nv(const HelpSlot& hb, uint32_t src, uint32_t idx) {
-  return src == kSrcA ? hb.a_nv[idx] : (src == kSrcB ? hb.b_nv[idx] : hb.x_nv);
-}
-__device__ __forceinline__ int32_t slot_qr(const HelpSlot& hb, uint32_t src, uint32_t idx) {
-  return src == kSrcA ? hb.a_qr[idx] : (src == kSrcB ? hb.b_qr[idx] : hb.x_qr);
-}
-__device__ __forceinline__ uint32_t slot_hit(const HelpSlot& hb, uint32_t src, uint32_t idx) {
-  return src == kSrcA ? hb.a_hit[idx] : (src == kSrcB ? hb.b_hit[idx] : hb.x_hit);
-}
-
-// Instance state v (of an instance with decode batch b, KV capacity M, slot limit Bmax and qr queued
-// requests) after it takes a request of L tokens at hit h: inst_vals_after on given values.
-__device__ __forceinline__ InstVals vals_after(const psk::DevModel& m, int32_t b, int64_t M, int32_t Bmax, int32_t qr0,
-                                               const InstVals& v0, uint32_t L, uint32_t h, int32_t* qr_out) {
-  const int32_t qr = qr0 + 1;
-  InstVals v;
-  v.q = v0.q + (int64_t)L - 16 * (int64_t)h;
-  v.S = v0.S + (int64_t)L;
-  const psk::InstTerms it = psk::inst_terms(m, b, qr, v.q, Bmax);
-  v.dec0 = it.dec0;
-  v.f = it.f;
-  v.tq = it.tq;
-  v.Bp = it.Bp;
-  v.room = it.okB ? psk::kv_room(v.S, M) : -1;
-  v.kd = psk::dcq_key0(b, qr);
-  *qr_out = qr;
-  return v;
-}
-
-__device__ void decide_spec(const psk::RowPre* __restrict__ rows, uint32_t R, uint32_t I, psk::StateSoA committed,
+template <int IPT, bool GEN>
+__device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, uint32_t I, psk::StateSoA committed,
                             psk::StateSoA pending, const psk::DevModel& m, int32_t* assign, uint8_t* __restrict__ path,
                             uint32_t* __restrict__ hit_chosen, uint32_t* err, const psk::GreedySync& sync,
                             unsigned long long* smem_raw) {
-  const int wid = (int)(threadIdx.x >> 5);
-  if (wid == 4 || wid == 6) return;
   const uint32_t Ip = sync.ring_stride;
   const InstSmem a = inst_smem(smem_raw, Ip);
-  uint32_t* s_hitr = reinterpret_cast<uint32_t*>(a.Bmax + Ip);  // [kFeedRing][Ip] probed hits
+  uint32_t* s_hitr = reinterpret_cast<uint32_t*>(a.pad + Ip);  // [kFeedRing][Ip] hits
   uint32_t* s_tpfr = s_hitr + kFeedRing * Ip;                   // [kFeedRing][Ip] T_pf at them (bits)
-  __shared__ psk::RowSummary s_sum[kFeedRing];
-  __shared__ psk::RowPre s_rowc[kFeedRing];
-  __shared__ HelpSlot s_help[2];               // helper phase p writes s_help[p & 1]
-  __shared__ int32_t s_logpick[kLogSlots];     // decision x: its pick (-1 rejected) ...
-  __shared__ uint32_t s_logsrc[kLogSlots];     // ... where its as-if values are (kSrc*) and at which index
-  __shared__ uint32_t s_logidx[kLogSlots];
-  __shared__ uint32_t s_loghit[kLogSlots];     // ... its hit and path (the decision outputs)
-  __shared__ uint32_t s_logpath[kLogSlots];
-  __shared__ uint32_t s_fed;       // rows [0, s_fed) are staged (release / acquire)
-  __shared__ uint32_t s_dec;       // decisions [0, s_dec) are published (their rows are consumed)
-  __shared__ uint32_t s_stored;    // the state after decisions [0, s_stored) is in the instance arrays
-  __shared__ uint32_t s_ph[3];     // helper w (A, B, C) finished phases [0, s_ph[w])
-  __shared__ int s_hgo[2];         // helper phase p goes ahead (s_hgo[p & 1]), set before its barrier
-  __shared__ volatile int s_stop;  // a role gave up (a bounded wait ran out)
+  __shared__ psk::RowPre s_row[kFeedRing];
+  __shared__ uint32_t s_rank[2][kComputeWarps];            // a step's warp minima: their ranks (all ones: none) ...
+  __shared__ uint2 s_th[2][kComputeWarps];                 // ... tie word and hit ...
+  __shared__ uint64_t s_key[2][kComputeWarps];             // ... and packed key
+  __shared__ uint32_t s_w[kComputeWarps];                  // a step's warp minima of W over A (f2ord)
+  __shared__ uint32_t s_begun;                             // steps [0, s_begun) have begun
+  __shared__ uint32_t s_landed;                            // rows [0, s_landed) are staged
+  __shared__ volatile int s_fail;                          // a bounded wait ran out (feeder and hit warp)
+  __shared__ volatile int s_stop;                          // set before a step's barrier: every warp leaves after it
   const uint32_t t = threadIdx.x;
-  const int lane = (int)(t & 31u), warp = (int)(t >> 5);
-  const unsigned full = 0xffffffffu;
-  if (t < 64)
-    for (uint32_t i = t; i < I; i += 64) inst_load(a, committed, m, i);
+  const int lane = (int)(t & 31u);
+  const uint32_t warp = t >> 5;
+  const uint32_t ncw = (I + 32u * IPT - 1) / (32u * IPT);  // compute warps in use
+  if (t < kComputeWarps) {
+    s_w[t] = 0xFFFFFFFFu;
+  }
+  // An instance only takes requests that fit its KV room, so S stays below max(S, M), and q gains at
+  // most what S gains: with these bounds 32 bits hold every q and S of the window.
+  bool narrow = true;
+  for (uint32_t i = t; i < I; i += kPipeThreads) {
+    const int64_t M = committed.M[i], S = committed.S[i], q = committed.q[i];
+    const int64_t gain = M > S ? M - S : 0;
+    narrow = narrow && S + gain < (1ll << 30) && q + gain < (1ll << 30);
+  }
   if (t == 0) {
-    s_fed = 0u;
-    s_dec = 0u;
-    s_stored = 0u;
-    s_ph[0] = 0u;
-    s_ph[1] = 0u;
-    s_ph[2] = 0u;
+    s_begun = 0u;
+    s_landed = 0u;
+    s_fail = 0;
     s_stop = 0;
   }
-  asm volatile("bar.sync 1, 192;" ::: "memory");  // warps 0, 1, 2, 3, 5, 7
+  narrow = __syncthreads_and(narrow ? 1 : 0) != 0;
+  if (!narrow) {
+    for (uint32_t i = t; i < I; i += kPipeThreads) {
+      a.b[i] = committed.b[i];
+      a.qr[i] = committed.qr[i];
+      a.q[i] = committed.q[i];
+      a.S[i] = committed.S[i];
+      a.M[i] = committed.M[i];
+      a.Bmax[i] = committed.Bmax[i];
+    }
+    __syncthreads();
+  }
+  if (warp >= ncw && warp < kComputeWarps) return;
+  const uint32_t nall = 32u * (ncw + 2u), ncmp = 32u * ncw;
+  auto bar_step = [&]() { asm volatile("bar.sync 2, %0;" ::"r"(nall) : "memory"); };     // compute, hit and publishing warps
+  auto bar_compute = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(ncmp) : "memory"); };  // compute warps
+  // Step x's pick from the warps' minima (after the next step's barrier), in every lane: the warp that
+  // holds it, -1 if rejected.  r: this lane's entry of s_rank[x & 1] (all ones past the warps in use).
+  auto decision = [&](uint32_t x, uint32_t r) {
+    const uint32_t mr = __reduce_min_sync(0xffffffffu, r);
+    const unsigned who = __ballot_sync(0xffffffffu, r == mr);
+    int src = __ffs(who) - 1;
+    if (who & (who - 1u)) {  // equal ranks (or nobody has a pair)
+      const uint32_t l = (uint32_t)lane < ncw ? lane : 0u;
+      src = warp_argmin(r, s_key[x & 1u][l], s_th[x & 1u][l].x);
+    }
+    return src;
+  };
+  auto rank_of = [&](uint32_t x) { return (uint32_t)lane < ncw ? s_rank[x & 1u][lane] : 0xFFFFFFFFu; };
 
-  if (warp == 1) {
-    // ---- feeder ---------------------------------------------------------------------------------
-    // Row x's slot held row x - kFeedRing, which the deciding warp reads up to its decision
-    // x - kFeedRing and the helpers up to their phase x - kFeedRing.
-    unsigned long long cyc_slot = 0, cyc_sum = 0;
-    for (uint32_t x = 0; x < R; ++x) {
-      const uint32_t slot = x % kFeedRing;
-      bool ok = true;
-      if (lane == 0) {
+  if (warp == kFeederWarp) {
+    // Rows are staged as soon as they are probed, several at once when they are ready together (so the
+    // round trips to L2 are shared).  Step s reads row s (and the length of row s - 1), the hit warp
+    // row s + 1 in the meantime: once step s has begun, rows up to s + kFeedRing - 2 may be staged.
+    unsigned long long cyc_slot = 0, cyc_ready = 0;
+    for (uint32_t x = 0; x < R;) {
+      uint32_t n = 0;
+      const long long cs = clock64();
+      if (lane == 0 &&
+          (x + 3 <= kFeedRing || wait_smem_at_least(&s_begun, x + 3 - kFeedRing, &s_fail, err, sync.wait_ns))) {
+        cyc_slot += (unsigned long long)(clock64() - cs);
+        n = psk::ld_relaxed_cta_shared_u32(&s_begun) + kFeedRing - 2 - x;
+        psk::fence_acq_rel_cta();
         const long long c0 = clock64();
-        if (x >= kFeedRing) {
-          const uint32_t want = x - kFeedRing + 1;
-          ok = wait_smem_at_least(&s_dec, want, &s_stop, err, sync.wait_ns) &&
-               wait_smem_at_least(&s_ph[0], want, &s_stop, err, sync.wait_ns) &&
-               wait_smem_at_least(&s_ph[1], want, &s_stop, err, sync.wait_ns) &&
-               wait_smem_at_least(&s_ph[2], want, &s_stop, err, sync.wait_ns);
-        }
-        const long long c1 = clock64();
-        if (ok) ok = wait_flag(sync.sready + x, err, sync.wait_ns);
-        cyc_slot += (unsigned long long)(c1 - c0);
-        cyc_sum += (unsigned long long)(clock64() - c1);
-        if (!ok) s_stop = 1;
+        if (!wait_flag(sync.ready + x, err, sync.wait_ns)) n = 0;
+        cyc_ready += (unsigned long long)(clock64() - c0);
       }
-      ok = __shfl_sync(full, ok ? 1 : 0, 0) != 0;
-      __syncwarp();
-      if (!ok) break;  // warp-uniform
-      const uint4* src_sum = reinterpret_cast<const uint4*>(sync.sums + (x % psk::kSumSlots));
-      uint4* dst_sum = reinterpret_cast<uint4*>(&s_sum[slot]);
-      for (uint32_t w = (uint32_t)lane; w < sizeof(psk::RowSummary) / 16; w += 32) psk::cp_async16(dst_sum + w, src_sum + w);
-      if (lane < psk::kRowWords)
-        psk::cp_async16(reinterpret_cast<uint4*>(&s_rowc[slot]) + lane, reinterpret_cast<const uint4*>(rows + x) + lane);
-      const uint4* src_h = reinterpret_cast<const uint4*>(sync.hitring + (uint64_t)(x % psk::kHitSlots) * Ip);
-      const uint4* src_t = reinterpret_cast<const uint4*>(sync.tpfring + (uint64_t)(x % psk::kHitSlots) * Ip);
-      uint4* dst_h = reinterpret_cast<uint4*>(s_hitr + slot * Ip);
-      uint4* dst_t = reinterpret_cast<uint4*>(s_tpfr + slot * Ip);
-      for (uint32_t w = (uint32_t)lane; w < Ip / 4; w += 32) {
-        psk::cp_async16(dst_h + w, src_h + w);
-        psk::cp_async16(dst_t + w, src_t + w);
+      n = __shfl_sync(0xffffffffu, n, 0);
+      if (n == 0) {  // warp-uniform: a wait ran out
+        if (lane == 0) s_fail = 1;
+        break;
+      }
+      n = min(n, R - x);
+      const bool rdy = (uint32_t)lane < n && psk::ld_acquire_u32(sync.ready + x + lane) != 0u;
+      const unsigned rm = __ballot_sync(0xffffffffu, rdy) | 1u;  // row x is ready
+      n = (uint32_t)(__ffs(~rm) - 1);
+      for (uint32_t y = x; y < x + n; ++y) {
+        const uint32_t slot = y % kFeedRing;
+        if (lane < psk::kRowWords)
+          psk::cp_async16(reinterpret_cast<uint4*>(&s_row[slot]) + lane, reinterpret_cast<const uint4*>(rows + y) + lane);
+        const uint4* src_h = reinterpret_cast<const uint4*>(sync.hitring + (uint64_t)(y % psk::kHitSlots) * Ip);
+        const uint4* src_t = reinterpret_cast<const uint4*>(sync.tpfring + (uint64_t)(y % psk::kHitSlots) * Ip);
+        uint4* dst_h = reinterpret_cast<uint4*>(s_hitr + slot * Ip);
+        uint4* dst_t = reinterpret_cast<uint4*>(s_tpfr + slot * Ip);
+        for (uint32_t w = (uint32_t)lane; w < Ip / 4; w += 32) {
+          psk::cp_async16(dst_h + w, src_h + w);
+          psk::cp_async16(dst_t + w, src_t + w);
+        }
       }
       psk::cp_async_commit();
       psk::cp_async_wait_all();
       __syncwarp();
-      if (lane == 0) psk::st_release_cta_shared_u32(&s_fed, x + 1);
+      x += n;
+      if (lane == 0) psk::st_release_cta_shared_u32(&s_landed, x);
     }
     if (lane == 0 && sync.stats) {
       atomicAdd(sync.stats + psk::kGsFeedSlotWait, cyc_slot);
-      atomicAdd(sync.stats + psk::kGsFeedSumWait, cyc_sum);
+      atomicAdd(sync.stats + psk::kGsFeedWait, cyc_ready);
     }
     return;
   }
 
-  if (warp >= 2) {
-    // ---- helpers ----------------------------------------------------------------------------------
-    // Phase p (p = 0 .. R): once decision p - 1 is published, warp 5 stores its pick's new state and
-    // writes its outputs, and for p < R - 1 the helpers compute A (warp 2), B (warp 3) and C (warp 7)
-    // for step p + 1 into s_help[p & 1].  Lanes whose instance is the pick of p - 1 take its state from
-    // the winner's as-if values, so nothing waits for the store: the others' instances were not
-    // picked at p - 1.
-    const int role = warp == 2 ? 0 : (warp == 3 ? 1 : (warp == 7 ? 2 : 3));  // 3: warp 5
-    for (uint32_t p = 0; p <= R; ++p) {
-      if (role == 3 && lane == 0) {
-        bool ok = wait_smem_at_least(&s_dec, p, &s_stop, err, sync.wait_ns);
-        if (ok && p < R) ok = wait_smem_at_least(&s_fed, p + 2 < R ? p + 2 : R, &s_stop, err, sync.wait_ns);
-        if (!ok) s_stop = 1;
-        s_hgo[p & 1u] = ok ? 1 : 0;
-      }
-      asm volatile("bar.sync 2, 128;" ::: "memory");  // warps 2, 3, 5, 7
-      if (!s_hgo[p & 1u]) break;  // uniform across the helper warps
-      const HelpSlot& hp = s_help[(p - 1) & 1u];  // phase p - 1's slot (p >= 1)
-      const uint32_t xp = (p - 1) % kLogSlots;     // decision p - 1 in the log (p >= 1)
-      int32_t j0 = -1;                              // the pick of p - 1
-      uint32_t src0 = kSrcX, idx0 = 0u;
-      if (p >= 1) {
-        j0 = s_logpick[xp];
-        src0 = s_logsrc[xp];
-        idx0 = s_logidx[xp];
-      }
-      if (role == 3) {
-        if (lane == 0) {
-          if (j0 >= 0) inst_store(a, (uint32_t)j0, slot_qr(hp, src0, idx0), slot_nv(hp, src0, idx0));
-          psk::st_release_cta_shared_u32(&s_stored, p);
-        } else if (lane == 1 && p >= 1) {
-          assign[p - 1] = j0;
-          path[p - 1] = (uint8_t)s_logpath[xp];
-          hit_chosen[p - 1] = s_loghit[xp];
-        }
-        continue;
-      }
-      if (p == R) break;
-      if (p + 1 >= R) {  // no row R: nothing to compute
-        __syncwarp();
-        if (lane == 0) psk::st_release_cta_shared_u32(&s_ph[role], p + 1);
-        continue;
-      }
-      int32_t hist[psk::kLcpBack];
-#pragma unroll
-      for (int k = 0; k < psk::kLcpBack; ++k)
-        hist[k] = (int64_t)p - 1 - k >= 0 ? s_logpick[(p - 1 - k) % kLogSlots] : -1;
-      const uint32_t slot = p % kFeedRing, slot1 = (p + 1) % kFeedRing;
-      const psk::RowPre& row = s_rowc[slot];
-      const psk::RowPre& row1 = s_rowc[slot1];
-      const psk::RowConst rc1 = row_of(row1);
-      const uint32_t* hrow1 = s_hitr + slot1 * Ip;
-      const uint32_t* trow1 = s_tpfr + slot1 * Ip;
-      HelpSlot& out = s_help[p & 1u];
-      // instance c (state v0, qr0) taking request p at hit h: its state after, and its pair on row p + 1
-      auto as_if = [&](uint32_t c, const InstVals& v0, int32_t qr0, uint32_t h, PairKey* pk, InstVals* nv,
-                       uint32_t* hit, int32_t* qr) {
-        *nv = vals_after(m, a.b[c], a.M[c], a.Bmax[c], qr0, v0, row.L, h, qr);
-        *hit = raised_hit(row1, hrow1, c, true, 1, hist);
-        *pk = pair_key_v(m, rc1, *nv, c, *hit, *hit == hrow1[c] ? trow1[c] : psk::kNoTpfBits);
-      };
-      if (role == 0) {
-        // A: summary entry `lane` of row p, when no decision of the last kSpecLag picked it (its state
-        // is then the one in the instance arrays)
-        const psk::RowSummary& sm = s_sum[slot];
-        const uint64_t ek = sm.key[lane];
-        const uint32_t e = sm.tie[lane] & psk::kTieInstMask;
-        bool touched = false;
-#pragma unroll
-        for (int k = 0; k < psk::kSpecLag; ++k) touched |= hist[k] == (int32_t)e;
-        if (ek != psk::kNoKey && !touched) {
-          PairKey pk;
-          InstVals nv;
-          uint32_t hit;
-          int32_t qr;
-          as_if(e, inst_vals(a, e), a.qr[e], sm.hit[lane], &pk, &nv, &hit, &qr);
-          out.a_pk[lane] = pk;
-          out.a_nv[lane] = nv;
-          out.a_hit[lane] = hit;
-          out.a_qr[lane] = qr;
-        }
-      } else if (role == 1) {
-        // B: lane's touched instance of step p (the pick of p - 1 - lane) as if it took request p, at
-        // its hit on row p (from phase p - 1)
-        const int32_t u = lane < psk::kSpecLag && (int64_t)p - 1 - lane >= 0 ? s_logpick[(p - 1 - lane) % kLogSlots] : -1;
-        if (u >= 0) {
-          PairKey pk;
-          InstVals nv;
-          uint32_t hit;
-          int32_t qr;
-          // lane 0's instance is the pick of p - 1: its state is the winner's as-if values (one call for
-          // every lane, so the lanes do not diverge)
-          const InstVals v0 = lane == 0 ? slot_nv(hp, src0, idx0) : inst_vals(a, (uint32_t)u);
-          const int32_t qr0 = lane == 0 ? slot_qr(hp, src0, idx0) : a.qr[u];
-          const uint32_t h0 = lane == 0 ? slot_hit(hp, src0, idx0) : hp.c_hit[lane];
-          as_if((uint32_t)u, v0, qr0, h0, &pk, &nv, &hit, &qr);
-          out.b_pk[lane] = pk;
-          out.b_nv[lane] = nv;
-          out.b_hit[lane] = hit;
-          out.b_qr[lane] = qr;
-        }
-      } else {
-        // C: the pick of p - k (k = lane, 1 .. kSpecLag - 1) on row p + 1, current state
-        const int k = lane;
-        const int32_t u = k >= 1 && k < psk::kSpecLag && (int64_t)p - k >= 0 ? s_logpick[(p - k) % kLogSlots] : -1;
-        if (u >= 0) {
-          const uint32_t h = raised_hit(row1, hrow1, (uint32_t)u, false, 1, hist);
-          const uint32_t tb = h == hrow1[u] ? trow1[u] : psk::kNoTpfBits;
-          out.c_pk[k] = pair_key_v(m, rc1, k == 1 ? slot_nv(hp, src0, idx0) : inst_vals(a, (uint32_t)u), (uint32_t)u, h, tb);
-          out.c_hit[k] = h;
-        }
-      }
-      __syncwarp();
-      if (lane == 0) psk::st_release_cta_shared_u32(&s_ph[role], p + 1);
-    }
-    return;
-  }
-
-  // ---- deciding warp --------------------------------------------------------------------------------
-  //   pk     lane k < kLcpBack: the pick of request s - 1 - k (-1: none or rejected)
-  //   hist   the same picks in every lane
-  //   cor    lane k < kSpecLag: that instance's pair on row s under the current state, chit its hit
-  //   e*, w* this lane's summary entries of row s, loaded a step ahead
-  int32_t pk = -1;
-  int32_t hist[psk::kLcpBack];
-#pragma unroll
-  for (int k = 0; k < psk::kLcpBack; ++k) hist[k] = -1;
-  uint32_t w_src = kSrcA, w_idx = 0;  // where the previous winner's as-if values are
-  unsigned long long n_fast = 0, n_full = 0, cyc_wait = 0;
-  const long long cyc_start = clock64();
-  uint64_t ek = psk::kNoKey, wv = ~0ull, kbound = psk::kNoKey;
-  uint32_t et = 0u, ew = 0u, eh = 0u, wbound = 0u, wsum = 0u, tbound = 0u;
-  psk::RowConst rc{};
-  auto load_row = [&](uint32_t x) {
-    const psk::RowSummary& sm = s_sum[x % kFeedRing];
-    ek = sm.key[lane];
-    et = sm.tie[lane];
-    ew = sm.word[lane];
-    eh = sm.hit[lane];
-    wv = lane < psk::kSumWarps * psk::kWPerWarp ? sm.w[lane] : ~0ull;
-    wbound = sm.w_bound;
-    wsum = sm.wmin;
-    kbound = sm.key_bound;
-    tbound = sm.tie_bound;
-    rc = row_of(s_rowc[x % kFeedRing]);
-  };
-  for (uint32_t s = 0; s < R; ++s) {
-    const uint32_t slot = s % kFeedRing;
-    const bool has_next = s + 1 < R;
-    bool ok = true;
-    if (lane == 0) {
+  if (warp == kHitWarp) {
+    int32_t pk = -1;  // lane k: the pick of request s - 1 - k (-1: none or rejected)
+    unsigned long long cyc_wait = 0;
+    for (uint32_t s = 0; s <= R; ++s) {
+      // rows s and s + 1 must be staged when step s begins
       const long long c0 = clock64();
-      ok = wait_smem_at_least(&s_fed, has_next ? s + 2 : s + 1, &s_stop, err, sync.wait_ns);
-      if (ok && s >= 1)
-        ok = wait_smem_at_least(&s_ph[0], s, &s_stop, err, sync.wait_ns) &&
-             wait_smem_at_least(&s_ph[1], s, &s_stop, err, sync.wait_ns) &&
-             wait_smem_at_least(&s_ph[2], s, &s_stop, err, sync.wait_ns);
+      if (lane == 0 && !wait_smem_at_least(&s_landed, s + 2 < R ? s + 2 : R, &s_fail, err, sync.wait_ns)) s_stop = 1;
       cyc_wait += (unsigned long long)(clock64() - c0);
-      if (!ok) s_stop = 1;
+      __syncwarp();
+      bar_step();
+      if (s_stop) {
+        if (lane == 0) s_fail = 1;  // the feeder stops too
+        break;
+      }
+      if (lane == 0) psk::st_release_cta_shared_u32(&s_begun, s + 1);
+      if (s > 0) {
+        const int src = decision(s - 1, rank_of(s - 1));
+        pk = __shfl_up_sync(0xffffffffu, pk, 1);
+        if (lane == 0) pk = src < 0 ? -1 : (int32_t)(s_th[(s - 1) & 1u][src].x & psk::kTieInstMask);
+      }
+      if (s + 1 < R) {  // request s - 1 - lane is lane + 2 places before row s + 1
+        const uint32_t slot = (s + 1) % kFeedRing;
+        const psk::RowPre& row = s_row[slot];
+        const bool up = pk >= 0 && lane + 1 < psk::kLcpBack;
+        uint32_t* hp = s_hitr + slot * Ip + (up ? pk : 0);
+        bool rose = false;
+        if (up) {
+          const uint32_t l = row.lcp[lane + 1];
+          rose = atomicMax(hp, l) < l;
+        }
+        __syncwarp();
+        if (rose) s_tpfr[slot * Ip + pk] = __float_as_uint(psk::t_pf32(m, row.L, *hp));
+        __syncwarp();
+      }
     }
-    ok = __shfl_sync(full, ok ? 1 : 0, 0) != 0;
-    __syncwarp();
-    if (!ok) break;  // warp-uniform
-    if (s == 0) load_row(0);
-    PairKey cor;
-    cor.W = 0.0f;
-    cor.key = psk::kNoKey;
-    cor.tie = 0xFFFFFFFFu;
-    cor.inA = false;
-    uint32_t chit = 0u;
-    if (s >= 1 && lane < psk::kSpecLag && pk >= 0) {
-      const HelpSlot& hb = s_help[(s - 1) & 1u];
-      if (lane == 0) {
-        cor = w_src == kSrcA ? hb.a_pk[w_idx] : (w_src == kSrcB ? hb.b_pk[w_idx] : hb.x_pk);
-        chit = slot_hit(hb, w_src, w_idx);
+    if (lane == 0 && sync.stats) atomicAdd(sync.stats + psk::kGsDecideWait, cyc_wait);
+    return;
+  }
+
+  if (warp == kPublishWarp) {
+    // Global stores stay in a warp of their own: a fence behind them would wait for their round trip.
+    for (uint32_t s = 0; s <= R; ++s) {
+      bar_step();
+      if (s_stop) break;
+      if (s == 0) continue;
+      const int src = decision(s - 1, rank_of(s - 1));
+      uint2 th = make_uint2(0xFFFFFFFFu, 0u);
+      uint32_t cls = 2u;
+      if (src >= 0) {
+        th = s_th[(s - 1) & 1u][src];
+        cls = (uint32_t)(s_key[(s - 1) & 1u][src] >> 62);
+      }
+      const uint32_t j = src < 0 ? 0xFFFFFFFFu : th.x & psk::kTieInstMask;
+      if (lane == 0) psk::st_relaxed_u64(sync.jobs + s - 1, kJobValid | ((unsigned long long)th.y << 32) | j);
+      if (lane == 1) assign[s - 1] = (int32_t)j;
+      if (lane == 2) path[s - 1] = (uint8_t)cls;
+      if (lane == 3) hit_chosen[s - 1] = th.y;
+    }
+    return;
+  }
+
+  const uint32_t i0 = t * IPT;
+  const bool loads = i0 < Ip;  // rows are padded to Ip, a multiple of 8 (the padding's room is -1)
+  const long long cyc0 = clock64();
+  bool stopped = false;
+  if (narrow) {
+    // ---- compute warps --------------------------------------------------------------------------
+    // Every q and S of the window stays in [0, 2^30): 32-bit state.  After the step's barrier the whole
+    // row is evaluated on the state without the last decision, side by side with the chain that finds
+    // that decision (the rank reductions); the pick's owner then replaces its one pair.
+    int32_t room[IPT], q32[IPT], S32[IPT], Bp[IPT];
+    float dec0[IPT], fe[IPT], tq[IPT];
+    uint32_t kq[IPT], kdh[IPT];  // D-C-Q key bits of (b, qr): low (qr) and high (b) words
+#pragma unroll
+    for (int k = 0; k < IPT; ++k) {
+      const uint32_t i = i0 + (uint32_t)k;
+      room[k] = -1;
+      q32[k] = S32[k] = 0;
+      Bp[k] = 1;
+      dec0[k] = fe[k] = tq[k] = 0.0f;
+      kq[k] = kdh[k] = 0u;
+      if (i < I) {
+        const int32_t b = committed.b[i], qr = committed.qr[i], Bmax = committed.Bmax[i];
+        const int64_t q = committed.q[i], S = committed.S[i];
+        const psk::InstTerms it = psk::inst_terms(m, b, qr, q, Bmax);
+        const uint64_t kd = psk::dcq_key0(b, qr);
+        room[k] = it.okB ? psk::kv_room(S, committed.M[i]) : -1;
+        dec0[k] = it.dec0;
+        fe[k] = it.f;
+        tq[k] = it.tq;
+        Bp[k] = it.Bp;
+        kq[k] = (uint32_t)kd;
+        kdh[k] = (uint32_t)(kd >> 32);
+        q32[k] = (int32_t)q;
+        S32[k] = (int32_t)S;
+        a.qs[i] = make_int4(q32[k], S32[k], room[k], Bmax - it.Bp);
+        a.kb[i] = make_uint4(kq[k], kdh[k], (uint32_t)Bp[k], 0u);
+      }
+    }
+    // One pair on the given state: W (+infinity outside A), and the key, its rank and the tie word it
+    // has in C.
+    auto pair = [&](const StepRow& rc, uint32_t i, uint32_t h, float tpf, int32_t rm, int32_t q, int32_t S, int32_t B,
+                    float d0, float f, float tqv, uint32_t kql, uint32_t kh, float* W, uint64_t* key, uint32_t* rank,
+                    uint32_t* tie) {
+      const int32_t n = (int32_t)rc.L - (int32_t)(h << 4);
+      *W = (int32_t)rc.L <= rm ? __fsub_rn(tpf, rc.t_cached) : INFINITY;
+      float dec = __fadd_rn(d0, __fmul_rn(m.b2, __int2float_rn(S + (int32_t)rc.L)));
+      dec = __fmul_rn(dec, f);
+      const float qnf = __int2float_rn(q + n);
+      float tpot;
+      if (!GEN || m.interference_mode == 0) {
+        tpot = __fadd_rn(dec, __fmul_rn(m.g_q, qnf));
       } else {
-        cor = hb.c_pk[lane];
-        chit = hb.c_hit[lane];
+        const float den = m.lout > 1.0f ? m.lout : 1.0f;
+        tpot = __fadd_rn(dec, B > 1 ? __fdiv_rn(tpf, den) : 0.0f);
       }
-    }
-    auto touched = [&](uint32_t i) {
-      bool r = false;
-#pragma unroll
-      for (int k = 0; k < psk::kSpecLag; ++k) r |= hist[k] == (int32_t)i;
-      return r;
-    };
-    // the touched instances, one lane each (the latest occurrence)
-    const int32_t tk = lane < psk::kSpecLag ? pk : -1;
-    const unsigned same = __match_any_sync(full, tk);
-    const bool corr = tk >= 0 && (__ffs(same) - 1) == lane;
-    // W_min of the current state
-    const bool w_untouched = wv != ~0ull && !touched((uint32_t)wv);
-    const uint32_t mu = __reduce_min_sync(full, w_untouched ? (uint32_t)(wv >> 32) : 0xFFFFFFFFu);
-    const uint32_t mt = __reduce_min_sync(full, (corr && cor.inA) ? psk::f2ord(cor.W) : 0xFFFFFFFFu);
-    uint32_t wmin_o = min(mu, mt);
-    bool anyA = wmin_o != 0xFFFFFFFFu;
-    bool fast = wbound == 0xFFFFFFFFu || mu <= wbound;
-    if (fast && anyA && rc.Z > 0.0f && wmin_o > wsum) fast = false;
-    // this lane's candidate: its summary entry or its touched instance, whichever is smaller
-    uint64_t bk = psk::kNoKey;
-    uint32_t bt = 0xFFFFFFFFu, bh = 0u, bsrc = kSrcA;
-    if (fast && anyA) {
-      const float wmin = psk::ord2f(wmin_o);
-      if (ek != psk::kNoKey && !touched(et & psk::kTieInstMask) && psk::pair_in_c(rc, psk::ord2f(ew), wmin)) {
-        bk = ek;
-        bt = et;
-        bh = eh;
-      }
-      if (corr && cor.inA && psk::pair_in_c(rc, cor.W, wmin) && kt_less(cor.key, cor.tie, bk, bt)) {
-        bk = cor.key;
-        bt = cor.tie;
-        bh = chit;
-        bsrc = kSrcB;
-      }
-    }
-    uint64_t K = psk::kNoKey;
-    uint32_t T = 0xFFFFFFFFu, H = 0u;
-    if (fast && anyA) {
-      psk::warp_pick_min(bk, bt, bh, &K, &T, &H);
-      fast = K != psk::kNoKey && (kbound == psk::kNoKey || kt_less(K, T, kbound, tbound));
-    }
-    const bool won = fast && bk != psk::kNoKey && bk == K && bt == T;  // one lane at most (tie words are unique)
-    const psk::RowPre& row = s_rowc[slot];
-    const uint32_t* hrow = s_hitr + slot * Ip;
-    const uint32_t* trow = s_tpfr + slot * Ip;
-    bool stored = false;  // the state after decision s - 1 is known to be in the instance arrays
-    if (fast) {
-      ++n_fast;
-    } else {
-      // full pass over the row on the current state (which needs the previous pick's state stored)
-      ++n_full;
-      bool ok2 = true;
-      if (lane == 0) {
-        ok2 = wait_smem_at_least(&s_stored, s, &s_stop, err, sync.wait_ns);
-        if (!ok2) s_stop = 1;
-      }
-      ok2 = __shfl_sync(full, ok2 ? 1 : 0, 0) != 0;
-      __syncwarp();
-      if (!ok2) break;  // warp-uniform
-      stored = true;
-      uint32_t wo = 0xFFFFFFFFu;
-      for (uint32_t i = (uint32_t)lane; i < I; i += 32) {
-        if ((int32_t)rc.L <= a.room[i]) {
-          const uint32_t h = raised_hit(row, hrow, i, false, 0, hist);
-          const float tpf = (h == hrow[i] && trow[i] != psk::kNoTpfBits) ? __uint_as_float(trow[i]) : psk::t_pf32(m, rc.L, h);
-          wo = min(wo, psk::f2ord(__fsub_rn(tpf, rc.t_cached)));
-        }
-      }
-      wmin_o = __reduce_min_sync(full, wo);
-      anyA = wmin_o != 0xFFFFFFFFu;
-      const float wmin = psk::ord2f(wmin_o);
-      uint64_t fk = psk::kNoKey;
-      uint32_t ft = 0xFFFFFFFFu, fh = 0u;
-      if (anyA) {
-        for (uint32_t i = (uint32_t)lane; i < I; i += 32) {
-          const uint32_t h = raised_hit(row, hrow, i, false, 0, hist);
-          const PairKey p = pair_key_of(m, rc, a, i, h, h == hrow[i] ? trow[i] : psk::kNoTpfBits);
-          if (p.inA && psk::pair_in_c(rc, p.W, wmin) && kt_less(p.key, p.tie, fk, ft)) {
-            fk = p.key;
-            ft = p.tie;
-            fh = h;
-          }
-        }
-      }
-      psk::warp_pick_min(fk, ft, fh, &K, &T, &H);
-    }
-    const bool pick = anyA && K != psk::kNoKey;
-    const uint32_t j = T & psk::kTieInstMask;
-    if (!pick) H = 0u;
-    // where the pick's as-if values (its state after this decision, its pair on row s + 1) are
-    uint32_t src = kSrcX, idx = 0u;
-    const unsigned wm = __ballot_sync(full, won);
-    if (wm && has_next) {
-      const int wl = __ffs(wm) - 1;
-      src = __shfl_sync(full, bsrc, wl);
-      idx = (uint32_t)wl;
-    } else if (pick) {
-      // a full pass picked it (the helpers prepared no such candidate), or the last request (there is
-      // no next row): its values are computed here, on the stored state
-      bool ok3 = true;
-      if (lane == 0) {
-        if (!stored) ok3 = wait_smem_at_least(&s_stored, s, &s_stop, err, sync.wait_ns);
-        if (ok3) {
-          HelpSlot& xb = s_help[s & 1u];
-          int32_t qr2;
-          const InstVals v2 = inst_vals_after(a, m, j, rc.L, H, &qr2);
-          xb.x_nv = v2;
-          xb.x_qr = qr2;
-          if (has_next) {
-            const uint32_t slot1 = (s + 1) % kFeedRing;
-            const psk::RowPre& row1 = s_rowc[slot1];
-            const uint32_t* hrow1 = s_hitr + slot1 * Ip;
-            const uint32_t* trow1 = s_tpfr + slot1 * Ip;
-            const uint32_t h1 = raised_hit(row1, hrow1, j, true, 1, hist);
-            xb.x_pk = pair_key_v(m, row_of(row1), v2, j, h1, h1 == hrow1[j] ? trow1[j] : psk::kNoTpfBits);
-            xb.x_hit = h1;
-          }
+      const float ttft = __fadd_rn(tpf, tqv);
+      const bool adm = (tpot < rc.tpot_lim) & (ttft <= rc.ttft_max);
+      const uint64_t kd = ((uint64_t)kh << 32) | kql;
+      const uint64_t qn = (uint64_t)(uint32_t)(q + n);
+      *tie = i;
+      if (!GEN) {  // Algorithm 1's order: D-C-Q in T, the LMetric product in C \ T
+        // ranks: D and up to 13 bits of C; the product rounded towards zero (both factors exact in fp32,
+        // else from the 64-bit product: the same rounding of the same value)
+        const uint64_t k0 = kd | ((uint64_t)((1u << 26) - 1u - h) << 18);
+        const uint64_t v1 = qn * (uint64_t)(uint32_t)B;
+        const float p1 = (uint32_t)qn < (1u << 24) ? __fmul_rz(qnf, __int2float_rn(B)) : __ull2float_rz(v1);
+        *key = adm ? k0 : psk::packed_key(1u, v1);
+        *rank = adm ? (kh << 1) | (8191u - min(h, 8191u)) : 0x80000000u | __float_as_uint(p1);
+      } else {
+        if (adm) {
+          *key = psk::packed_key(0u, psk::value_in_t(m, psk::key0_from_dcq(m, kd), h, tpot, rc.tpot_target));
+          if (m.sel == psk::kSelHCQ) *tie |= (kql & 0x3FFFFu) << 12;
         } else {
-          s_stop = 1;
+          *key = psk::packed_key(1u, psk::value_fallback(m, qn, (uint32_t)B, kd, h));
         }
+        *rank = key_rank(*key);
+      }
+    };
+    uint32_t Lprev = 0;  // length of request s - 1
+    for (uint32_t s = 0;; ++s) {
+      bar_step();
+      // the last decision's ranks and picks, and this row (past the last row: any staged one)
+      const uint32_t par = (s - 1) & 1u;
+      const bool held = (uint32_t)lane < ncw && s > 0;
+      const uint32_t er = held ? s_rank[par][lane] : 0xFFFFFFFFu;
+      const uint2 eth = s_th[par][held ? lane : 0];
+      const uint32_t slot = (s < R ? s : R - 1) % kFeedRing;
+      const psk::RowPre& row = s_row[slot];
+      const StepRow rc = step_row(m, row);
+      const uint32_t l0 = row.lcp[0];
+      uint32_t h[IPT], tb[IPT];
+      if (loads) {
+        lds_words<IPT>(s_hitr + slot * Ip + i0, h);
+        lds_words<IPT>(s_tpfr + slot * Ip + i0, tb);
+      } else {
+#pragma unroll
+        for (int k = 0; k < IPT; ++k) h[k] = tb[k] = 0u;
+      }
+      if (s_stop) {
+        stopped = true;
+        break;
+      }
+      const uint32_t mr = __reduce_min_sync(0xffffffffu, er);
+      const unsigned who = __ballot_sync(0xffffffffu, er == mr);
+      float W[IPT];
+      uint64_t key[IPT];
+      uint32_t rank[IPT], tie[IPT];
+#pragma unroll
+      for (int k = 0; k < IPT; ++k)
+        pair(rc, i0 + (uint32_t)k, h[k], __uint_as_float(tb[k]), room[k], q32[k], S32[k], Bp[k], dec0[k], fe[k], tq[k],
+             kq[k], kdh[k], &W[k], &key[k], &rank[k], &tie[k]);
+      if (mr != 0xFFFFFFFFu) {
+        int src = __ffs(who) - 1;
+        if (who & (who - 1u)) src = warp_argmin(er, s_key[par][held ? lane : 0], eth.x);  // equal ranks
+        const uint32_t j = __shfl_sync(0xffffffffu, eth.x, src) & psk::kTieInstMask;
+        const uint32_t H = __shfl_sync(0xffffffffu, eth.y, src);
+        if (j / IPT == t) {
+          // its state takes request s - 1 (qr + 1, q + L - 16 H, S + L), and its hit rises to the common
+          // prefix of the two requests
+          int4 x = a.qs[j];
+          uint4 y = a.kb[j];
+          uint32_t hj = s_hitr[slot * Ip + j];
+          x.x += (int32_t)Lprev - (int32_t)(H << 4);
+          x.y += (int32_t)Lprev;
+          x.w -= 1;
+          x.z = x.w < 0 ? -1 : x.z - (int32_t)Lprev;
+          y.x += 1u;
+          y.z += 1u;
+          a.qs[j] = x;
+          a.kb[j] = y;
+          const float d0 = __fadd_rn(m.b0, __fmul_rn(m.b1, __int2float_rn((int32_t)y.z)));
+          const float f = psk::ema_factor(m, (int32_t)y.z);
+          const float tqv =
+              __fadd_rn(__fmul_rn(m.a0, __int2float_rn((int32_t)(y.x & 0x3FFFFu))), __fmul_rn(m.a1, __int2float_rn(x.x)));
+          hj = l0 > hj ? l0 : hj;
+          float Wj;
+          uint64_t keyj;
+          uint32_t rankj, tiej;
+          pair(rc, j, hj, psk::t_pf32(m, rc.L, hj), x.z, x.x, x.y, (int32_t)y.z, d0, f, tqv, y.x, y.y, &Wj, &keyj, &rankj,
+               &tiej);
+#pragma unroll
+          for (int k = 0; k < IPT; ++k)
+            if (i0 + (uint32_t)k == j) {
+              W[k] = Wj;
+              key[k] = keyj;
+              rank[k] = rankj;
+              tie[k] = tiej;
+              h[k] = hj;
+              q32[k] = x.x;
+              S32[k] = x.y;
+              room[k] = x.z;
+              Bp[k] = (int32_t)y.z;
+              kq[k] = y.x;
+              dec0[k] = d0;
+              fe[k] = f;
+              tq[k] = tqv;
+            }
+        }
+      }
+      if (s == R) break;
+      Lprev = rc.L;
+      float wbest = W[0];
+#pragma unroll
+      for (int k = 1; k < IPT; ++k) wbest = fminf(wbest, W[k]);
+      uint32_t wmin_o = __reduce_min_sync(0xffffffffu, psk::f2ord(wbest));
+      if (ncw > 1u) {
+        if (lane == 0) s_w[warp] = wmin_o;
+        bar_compute();
+        wmin_o = __reduce_min_sync(0xffffffffu, s_w[lane & (kComputeWarps - 1)]);
+      }
+      const float wmin = psk::ord2f(wmin_o);
+      // the recompute filter (a pair outside A has W = +infinity), and the smallest rank
+      uint32_t rbest = 0xFFFFFFFFu;
+#pragma unroll
+      for (int k = 0; k < IPT; ++k) {
+        const bool in = W[k] < INFINITY && __fsub_rn(W[k], wmin) <= rc.c_max;
+        rank[k] = in ? rank[k] : 0xFFFFFFFFu;
+        rbest = min(rbest, rank[k]);
+      }
+      const uint32_t mw = __reduce_min_sync(0xffffffffu, rbest);
+      uint32_t n_eq = 0;
+      uint64_t bk = psk::kNoKey;
+      uint32_t bt = 0xFFFFFFFFu, bh = 0u;
+#pragma unroll
+      for (int k = 0; k < IPT; ++k)
+        if (rank[k] == mw) {
+          ++n_eq;
+          bk = key[k];
+          bt = tie[k];
+          bh = h[k];
+        }
+      unsigned lanes = __ballot_sync(0xffffffffu, n_eq != 0u);
+      const unsigned many = IPT > 1 ? __ballot_sync(0xffffffffu, n_eq > 1u) : 0u;
+      if (mw != 0xFFFFFFFFu && ((lanes & (lanes - 1u)) | many)) {
+        // equal ranks: the smallest (key, tie) of the lane's, then of the warp's
+#pragma unroll
+        for (int k = 0; k < IPT; ++k)
+          if (rank[k] == mw && (key[k] < bk || (key[k] == bk && tie[k] < bt))) {
+            bk = key[k];
+            bt = tie[k];
+            bh = h[k];
+          }
+        const int win = warp_argmin(n_eq ? mw : 0xFFFFFFFFu, bk, bt);
+        lanes = 1u << win;
+      }
+      if (lane == __ffs(lanes) - 1) {
+        s_rank[s & 1u][warp] = mw;
+        s_th[s & 1u][warp] = make_uint2(bt, bh);
+        s_key[s & 1u][warp] = bk;
       }
       __syncwarp();
     }
-    if (lane == 0) {
-      const uint32_t x = s % kLogSlots;
-      s_logpick[x] = pick ? (int32_t)j : -1;
-      s_logsrc[x] = src;
-      s_logidx[x] = idx;
-      s_loghit[x] = H;
-      s_logpath[x] = pick ? (uint32_t)(K >> 62) : 2u;
-      psk::st_release_cta_shared_u32(&s_dec, s + 1);
-      psk::st_relaxed_u64(sync.jobs + s, kJobValid | ((unsigned long long)H << 32) | (pick ? j : 0xFFFFFFFFu));
-    }
-    const int32_t pj = pick ? (int32_t)j : -1;
-    pk = __shfl_up_sync(full, pk, 1);
-    if (lane == 0) pk = pj;
+    if (!stopped) {
 #pragma unroll
-    for (int k = psk::kLcpBack - 1; k > 0; --k) hist[k] = hist[k - 1];
-    hist[0] = pj;
-    w_src = src;
-    w_idx = idx;
-    if (has_next) load_row(s + 1);  // staged: s_fed >= s + 2 was waited for
+      for (int k = 0; k < IPT; ++k) {  // the pending state: each owner's instances
+        const uint32_t i = i0 + (uint32_t)k;
+        if (i < I) {
+          pending.b[i] = committed.b[i];
+          pending.qr[i] = (int32_t)(kq[k] & 0x3FFFFu);
+          pending.q[i] = q32[k];
+          pending.S[i] = S32[k];
+          pending.M[i] = committed.M[i];
+          pending.Bmax[i] = committed.Bmax[i];
+        }
+      }
+    }
+  } else {
+    // ---- compute warps, 64-bit sums: some q or S may leave [0, 2^30) ---------------------------------
+    // The same steps with every order's key, and the shared-memory truth for sums that need 64 bits.
+    int32_t room[IPT], q32[IPT], S32[IPT], Bp[IPT];
+    float dec0[IPT], fe[IPT], tq[IPT];
+    uint64_t kd[IPT];
+    bool wide = false;  // some q or S of this thread's instances is outside [0, 2^30): 64-bit sums from shared memory
+#pragma unroll
+    for (int k = 0; k < IPT; ++k) {
+      const uint32_t i = i0 + (uint32_t)k;
+      room[k] = -1;
+      q32[k] = S32[k] = 0;
+      Bp[k] = 1;
+      dec0[k] = fe[k] = tq[k] = 0.0f;
+      kd[k] = 0ull;
+      if (i < I) {
+        const psk::InstTerms it = psk::inst_terms(m, a.b[i], a.qr[i], a.q[i], a.Bmax[i]);
+        room[k] = it.okB ? psk::kv_room(a.S[i], a.M[i]) : -1;
+        dec0[k] = it.dec0;
+        fe[k] = it.f;
+        tq[k] = it.tq;
+        Bp[k] = it.Bp;
+        kd[k] = psk::dcq_key0(a.b[i], a.qr[i]);
+        q32[k] = (int32_t)a.q[i];
+        S32[k] = (int32_t)a.S[i];
+        wide |= !narrow_qs(a.q[i], a.S[i]);
+      }
+    }
+    uint32_t Lprev = 0;  // length of request s - 1
+    for (uint32_t s = 0;; ++s) {
+      bar_step();
+      if (s_stop) {
+        stopped = true;
+        break;
+      }
+      const uint32_t slot = s % kFeedRing;
+      uint32_t own = 0xFFFFFFFFu;  // this thread's index of the last pick, if it owns it
+      if (s > 0) {
+        const int src = decision(s - 1, rank_of(s - 1));
+        const uint2 th = s_th[(s - 1) & 1u][src < 0 ? 0 : src];
+        const uint32_t j = th.x & psk::kTieInstMask;
+        if (src >= 0 && j / IPT == t) {
+          own = j - i0;
+          const int32_t b = a.b[j], qr = a.qr[j] + 1;
+          const int64_t q = a.q[j] + (int64_t)Lprev - 16 * (int64_t)th.y;
+          const int64_t S = a.S[j] + (int64_t)Lprev;
+          a.qr[j] = qr;
+          a.q[j] = q;
+          a.S[j] = S;
+          const psk::InstTerms it = psk::inst_terms(m, b, qr, q, a.Bmax[j]);
+          const int32_t rm = it.okB ? psk::kv_room(S, a.M[j]) : -1;
+          wide |= !narrow_qs(q, S);
+#pragma unroll
+          for (int k = 0; k < IPT; ++k)
+            if ((uint32_t)k == own) {
+              room[k] = rm;
+              q32[k] = (int32_t)q;
+              S32[k] = (int32_t)S;
+              Bp[k] = it.Bp;
+              dec0[k] = it.dec0;
+              fe[k] = it.f;
+              tq[k] = it.tq;
+              kd[k] += 1ull;  // qr + 1
+            }
+        }
+      }
+      if (s == R) break;
+      const psk::RowPre& row = s_row[slot];
+      const StepRow rc = step_row(m, row);
+      Lprev = rc.L;
+      uint32_t h[IPT], tb[IPT];
+      if (loads) {
+        lds_words<IPT>(s_hitr + slot * Ip + i0, h);
+        lds_words<IPT>(s_tpfr + slot * Ip + i0, tb);
+      } else {
+#pragma unroll
+        for (int k = 0; k < IPT; ++k) h[k] = tb[k] = 0u;
+      }
+      if (own != 0xFFFFFFFFu) {  // the last pick also took request s - 1: its common prefix with this row
+        const uint32_t l = row.lcp[0];
+        const uint32_t tl = __float_as_uint(psk::t_pf32(m, rc.L, l));
+#pragma unroll
+        for (int k = 0; k < IPT; ++k)
+          if ((uint32_t)k == own && l > h[k]) {
+            h[k] = l;
+            tb[k] = tl;
+          }
+      }
+      // every pair: W, the capacity guard, the latencies, and the key it has in C
+      float W[IPT];
+      uint64_t key[IPT];
+      uint32_t tie[IPT];
+      float wbest = INFINITY;
+#pragma unroll
+      for (int k = 0; k < IPT; ++k) {
+        const uint32_t i = i0 + (uint32_t)k < I ? i0 + (uint32_t)k : 0u;
+        const float tpf = __uint_as_float(tb[k]);
+        const int32_t n = (int32_t)rc.L - (int32_t)(h[k] << 4);
+        W[k] = (int32_t)rc.L <= room[k] ? __fsub_rn(tpf, rc.t_cached) : INFINITY;
+        wbest = fminf(wbest, W[k]);
+        psk::RowConst rr;
+        rr.L = rc.L;
+        rr.tpot_target = rc.tpot_target;
+        float tpot, ttft;
+        uint64_t qn;
+        if (!wide) {
+          psk::pair_lat32(m, rr, tpf, n, dec0[k], fe[k], tq[k], Bp[k], q32[k], S32[k], &tpot, &ttft);
+          qn = (uint64_t)(uint32_t)(q32[k] + n);
+        } else {
+          psk::InstTerms it;
+          it.dec0 = dec0[k];
+          it.f = fe[k];
+          it.tq = tq[k];
+          it.Bp = Bp[k];
+          it.okB = 1;
+          psk::PairW x;
+          x.W = W[k];
+          x.tpf = tpf;
+          x.n = n;
+          x.inA = true;
+          psk::pair_lat(m, rr, x, it, a.q[i], a.S[i], &tpot, &ttft);
+          qn = (uint64_t)a.q[i] + (uint64_t)(int64_t)n;
+        }
+        const bool adm = (tpot < rc.tpot_lim) & (ttft <= rc.ttft_max);
+        tie[k] = i0 + (uint32_t)k;
+        if (adm) {
+          key[k] = psk::packed_key(0u, psk::value_in_t(m, psk::key0_from_dcq(m, kd[k]), h[k], tpot, rc.tpot_target));
+          if (m.sel == psk::kSelHCQ) tie[k] |= (uint32_t)(kd[k] & 0x3FFFFull) << 12;
+        } else {
+          key[k] = psk::packed_key(1u, psk::value_fallback(m, qn, (uint32_t)Bp[k], kd[k], h[k]));
+        }
+      }
+      uint32_t wmin_o = __reduce_min_sync(0xffffffffu, psk::f2ord(wbest));
+      if (ncw > 1u) {
+        if (lane == 0) s_w[warp] = wmin_o;
+        bar_compute();
+        wmin_o = __reduce_min_sync(0xffffffffu, s_w[lane & (kComputeWarps - 1)]);
+      }
+      const float wmin = psk::ord2f(wmin_o);
+      // the recompute filter (a pair outside A has W = +infinity, and W - W_min = +infinity or NaN), then
+      // this thread's smallest (key, tie)
+      uint64_t bk[IPT];
+      uint32_t bt[IPT], bh[IPT];
+#pragma unroll
+      for (int k = 0; k < IPT; ++k) {
+        const bool in = W[k] < INFINITY && __fsub_rn(W[k], wmin) <= rc.c_max;
+        bk[k] = in ? key[k] : psk::kNoKey;
+        bt[k] = tie[k];
+        bh[k] = h[k];
+      }
+#pragma unroll
+      for (int d = 1; d < IPT; d <<= 1)
+#pragma unroll
+        for (int k = 0; k < IPT; k += 2 * d) {
+          const bool less = bk[k + d] < bk[k] || (bk[k + d] == bk[k] && bt[k + d] < bt[k]);
+          bk[k] = less ? bk[k + d] : bk[k];
+          bt[k] = less ? bt[k + d] : bt[k];
+          bh[k] = less ? bh[k + d] : bh[k];
+        }
+      const uint32_t rank = key_rank(bk[0]);
+      const int win = warp_argmin(rank, bk[0], bt[0]);
+      if (lane == (win < 0 ? 0 : win)) {
+        s_rank[s & 1u][warp] = rank;
+        s_th[s & 1u][warp] = make_uint2(bt[0], bh[0]);
+        s_key[s & 1u][warp] = bk[0];
+      }
+      __syncwarp();
+    }
+    if (!stopped) {
+#pragma unroll
+      for (int k = 0; k < IPT; ++k) {
+        const uint32_t i = i0 + (uint32_t)k;
+        if (i < I) {
+          pending.b[i] = a.b[i];
+          pending.qr[i] = a.qr[i];
+          pending.q[i] = a.q[i];
+          pending.S[i] = a.S[i];
+          pending.M[i] = a.M[i];
+          pending.Bmax[i] = a.Bmax[i];
+        }
+      }
+    }
   }
-  if (lane == 0 && sync.stats) {
-    atomicAdd(sync.stats + psk::kGsFast, n_fast);
-    atomicAdd(sync.stats + psk::kGsFull, n_full);
-    atomicAdd(sync.stats + psk::kGsDecideWait, cyc_wait);
-    atomicAdd(sync.stats + psk::kGsDecideTotal, (unsigned long long)(clock64() - cyc_start));
-  }
-  // the pending state: every decision's state stored by the helpers (their phase R)
-  bool ok = true;
-  if (lane == 0) ok = !s_stop && wait_smem_at_least(&s_stored, R, &s_stop, err, sync.wait_ns);
-  ok = __shfl_sync(full, ok ? 1 : 0, 0) != 0;
-  if (!ok) return;
-  for (uint32_t i = (uint32_t)lane; i < I; i += 32) {
-    pending.b[i] = a.b[i];
-    pending.qr[i] = a.qr[i];
-    pending.q[i] = a.q[i];
-    pending.S[i] = a.S[i];
-    pending.M[i] = a.M[i];
-    pending.Bmax[i] = a.Bmax[i];
+  if (t == 0 && sync.stats) {
+    atomicAdd(sync.stats + psk::kGsDecisions, (unsigned long long)(stopped ? 0u : R));
+    atomicAdd(sync.stats + psk::kGsDecideTotal, (unsigned long long)(clock64() - cyc0));
   }
 }
 
-template <int IPT>
+template <int IPT, bool GEN>
 __global__ void __launch_bounds__(kPipeThreads, 1)
 greedy_pipe_kernel(const psk::RowPre* __restrict__ rows, const uint64_t* __restrict__ hash, uint32_t R, uint32_t I,
                    const uint32_t* __restrict__ hit0, const float* __restrict__ tpf0, psk::StateSoA committed,
                    psk::StateSoA pending, psk::DevModel m, psk::DeltaSlot* delta, uint64_t nslots, int32_t* assign,
-                   uint8_t* __restrict__ path, uint32_t* __restrict__ hit_chosen, uint32_t* err, psk::GreedySync sync) {
-  extern __shared__ unsigned long long smem_raw[];
+                   uint8_t* __restrict__ path, uint32_t* __restrict__ hit_chosen, uint32_t* err, psk::GreedySync sync,
+                   uint32_t ninsert) {
+  extern __shared__ __align__(16) unsigned long long smem_raw[];
   if (blockIdx.x == 0) {
-    decide_spec(rows, R, I, committed, pending, m, assign, path, hit_chosen, err, sync, smem_raw);
-  } else if (blockIdx.x <= kInsertBlocks) {
-    insert_blocks(rows, hash, R, delta, nslots, err, sync);
-  } else if (blockIdx.x <= kInsertBlocks + kProbeBlocks) {
-    probe_rows<IPT>(rows, hash, R, I, hit0, tpf0, delta, nslots, err, sync, smem_raw);
+    decide_rows<IPT, GEN>(rows, R, I, committed, pending, m, assign, path, hit_chosen, err, sync, smem_raw);
+  } else if (blockIdx.x <= ninsert) {
+    insert_blocks(rows, hash, R, delta, nslots, err, sync, blockIdx.x - 1, ninsert);
   } else {
-    summary_rows<IPT>(rows, R, I, committed, m, err, sync, blockIdx.x - 1 - kInsertBlocks - kProbeBlocks, smem_raw);
+    probe_rows<IPT>(rows, hash, R, I, hit0, tpf0, m, delta, nslots, err, sync, smem_raw, blockIdx.x - 1 - ninsert,
+                    gridDim.x - 1 - ninsert);
   }
 }
 
 size_t greedy_pipe_smem(uint32_t I, uint32_t Ip) {
-  // deciding block: instance state, the hit and T_pf rows of kFeedRing rows; summary blocks: the
-  // instance state; probe blocks: three u32 arrays per instance
+  // deciding block: instance state, the hit and T_pf rows of kFeedRing rows; probe blocks: three u32
+  // arrays per instance
   const size_t decide = (size_t)Ip * (kInstSmemBytes + 2 * kFeedRing * sizeof(uint32_t));
   const size_t probe = (size_t)I * 3 * sizeof(uint32_t);
   return decide > probe ? decide : probe;
@@ -1622,21 +1389,25 @@ cudaError_t greedy_pipe_launch(const psk::RowPre* rows, const psk::WindowDev& w,
                                const float* tpf0, psk::StateSoA committed, psk::StateSoA pending, const psk::DevModel& m,
                                psk::DeltaSlot* delta, uint64_t nslots, int32_t* assign, uint8_t* path,
                                uint32_t* hit_chosen, uint32_t* err, const psk::GreedySync& sync, cudaStream_t s) {
+  // not Algorithm 1's order (Table 4 / Table 3 variants), or Eq. 9's interference term
+  const bool gen = m.sel != psk::kSelDCQ || m.fb_dcq || m.interference_mode != 0;
+  auto kern = gen ? greedy_pipe_kernel<IPT, true> : greedy_pipe_kernel<IPT, false>;
   const size_t smem = greedy_pipe_smem(I, sync.ring_stride);
-  cudaError_t e = cudaFuncSetAttribute(greedy_pipe_kernel<IPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const uint64_t* hash = w.hash;
   uint32_t R = w.R;
   psk::StateSoA c = committed, p = pending;
   psk::DevModel mm = m;
   psk::GreedySync sy = sync;
+  // A window of up to kLag requests has no row that reads the delta table, so nothing to insert.
+  uint32_t ninsert = R > (uint32_t)psk::kLag ? kInsertBlocks : 0u;
+  const uint32_t nprobe = R < kProbeBlocks ? R : kProbeBlocks;
   void* args[] = {(void*)&rows, (void*)&hash, (void*)&R, (void*)&I, (void*)&hit0, (void*)&tpf0, (void*)&c, (void*)&p,
                   (void*)&mm, (void*)&delta, (void*)&nslots, (void*)&assign, (void*)&path, (void*)&hit_chosen,
-                  (void*)&err, (void*)&sy};
+                  (void*)&err, (void*)&sy, (void*)&ninsert};
   // all blocks must be resident at once: they wait on one another
-  return cudaLaunchCooperativeKernel((const void*)greedy_pipe_kernel<IPT>,
-                                     dim3(1 + kInsertBlocks + kProbeBlocks + kSummaryBlocks), dim3(kPipeThreads), args,
-                                     smem, s);
+  return cudaLaunchCooperativeKernel((const void*)kern, dim3(1 + ninsert + nprobe), dim3(kPipeThreads), args, smem, s);
 }
 
 }  // namespace
@@ -1670,12 +1441,13 @@ cudaError_t launch_greedy_search(const psk::RowPre* rows, const psk::WindowDev& 
   if (w.R == 0) return cudaSuccess;
   cudaError_t e = cudaMemsetAsync(sync.done, 0, (size_t)w.R * sizeof(uint32_t), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(sync.ready, 0, (size_t)w.R * sizeof(uint32_t), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(sync.sready, 0, (size_t)w.R * sizeof(uint32_t), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(sync.jobs, 0, (size_t)w.R * sizeof(unsigned long long), s);
   if (e == cudaSuccess && sync.stats) e = cudaMemsetAsync(sync.stats, 0, psk::kGreedyStats * sizeof(unsigned long long), s);
   if (e != cudaSuccess) return e;
-  // every block has 256 threads; probe and summary threads hold IPT = ceil(I / 256) instances each
-  const uint32_t ipt = (I + kPipeThreads - 1) / kPipeThreads;
+  // IPT instances per compute thread of the deciding block (and at most that many per probe thread): as
+  // few as its warps allow.  More per thread means fewer warps to combine but a longer step: greedy pass
+  // with 1 / 2 / 4 a thread 0.32 / 0.33 / 0.44 ms at 256 x 512, with 2 / 4 / 8 14.6 / 17.0 / 25.2 at 1024 x 16384.
+  const uint32_t ipt = (I + 32u * kComputeWarps - 1) / (32u * kComputeWarps);
 #define PS_GREEDY_P(IPT)                                                                                      \
   return greedy_pipe_launch<IPT>(rows, w, I, hit0, tpf0, committed, pending, m, delta, delta_nslots, assign, path, \
                                  hit_chosen, err, sync, s)

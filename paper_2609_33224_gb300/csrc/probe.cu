@@ -107,16 +107,6 @@ probe_hits_kernel(const uint64_t* __restrict__ slots, const uint64_t* __restrict
   }
 }
 
-// Hint of a row for the search: the shortest common chain prefix with the previous requests of
-// the window (0 if there are none).
-__device__ __forceinline__ uint32_t row_hint(const psk::RowPre* __restrict__ rows, uint32_t r) {
-  uint32_t hint = 0xFFFFFFFFu;
-#pragma unroll
-  for (int d = 0; d < psk::kLcpBack; ++d)
-    if ((uint32_t)d < r) hint = min(hint, __ldg(&rows[r].lcp[d]));
-  return hint == 0xFFFFFFFFu ? 0u : hint;
-}
-
 // Search mode, rows from the list: see the file comment.
 template <int WARPS>
 __global__ void __launch_bounds__(WARPS * 32)
@@ -140,7 +130,7 @@ probe_search_kernel(const uint64_t* __restrict__ slots, const uint64_t* __restri
     const psk::TableDesc d = tdesc[i];
     uint64_t lo = 0, hi = nb;  // the first miss lies in [lo, hi]
     if (nb > 0) {
-      const uint64_t hint = row_hint(rows, r);
+      const uint64_t hint = __ldg(&rows[r].hint);
       if (hint == 0 || hint >= nb) {
         const uint64_t p = hint == 0 ? 0 : nb - 1;
         n_look += 1;

@@ -63,7 +63,7 @@ struct DeltaSlot {
 
 // Greedy pipeline depth: a probe for request s sees every delta insert of requests <= s - kLag, and
 // the requests s - 1 .. s - (kLag - 1) are covered by their common chain prefix with s (RowPre::lcp).
-constexpr int kLag = 21;
+constexpr int kLag = 33;
 constexpr int kLcpBack = kLag - 1;
 
 // Per-request constants of one window, computed in parallel before the greedy pass: the request's
@@ -85,6 +85,8 @@ struct __align__(16) RowPre {
   int32_t anc[2];     // the parent's parent and its parent (-1 if none): their chains are prefixes too
   uint32_t anc_nb[2]; // their chain lengths
   uint32_t lcp[kLcpBack];  // common chain prefix with requests r - 1 .. r - kLcpBack (blocks)
+  uint32_t hint;      // the smallest of them (0 for the first request): where most instances' hits end
+  uint32_t pad[3];
 };
 constexpr int kRowWords = (int)(sizeof(RowPre) / 16);
 static_assert(sizeof(RowPre) % 16 == 0 && kRowWords <= 32, "RowPre is whole 16-byte words, staged by one warp");
@@ -92,7 +94,7 @@ static_assert(sizeof(RowPre) % 16 == 0 && kRowWords <= 32, "RowPre is whole 16-b
 // Hand-offs between the blocks of the pipelined greedy (one cooperative launch): the deciding
 // block publishes each decision as a job, insert blocks put the job's chain blocks into the delta
 // table, probe blocks turn hit0 rows into the hits the deciding block reads.
-constexpr uint32_t kHitSlots = 64;  // rows of probed hits in flight (a ring; more than kLag + 2)
+constexpr uint32_t kHitSlots = 64;  // rows of probed hits in flight (a ring; more than kLag and the staged rows)
 // Rows of a window whose hits are searched from scratch (no earlier request of the window is a
 // prefix of theirs), in no particular order: filled by the relations pass, read by the probe.
 struct RowList {
@@ -100,56 +102,23 @@ struct RowList {
   uint32_t* count;  // [1]
 };
 
-// Lag-d speculation of the greedy pass: summary blocks evaluate row s in full on the state before
-// decision s - kSpecLag and publish a RowSummary; the deciding warp corrects it for the instances
-// picked by decisions s - kSpecLag .. s - 1 (kSpecLag <= kLcpBack, so their common chain prefixes
-// with request s are in RowPre::lcp).
-constexpr int kSpecLag = 8;
-constexpr int kSumWarps = 8;      // warps of a summary block (256 threads)
-constexpr int kKeysPerWarp = 4;   // smallest (key, tie) pairs of C a summary warp publishes
-constexpr int kWPerWarp = 2;      // smallest (W, instance) pairs of A a summary warp publishes
-constexpr uint32_t kSumSlots = 64;  // ring of published summaries (row s in slot s % kSumSlots)
-static_assert(kSpecLag <= kLcpBack, "the corrected picks need their common prefix with the row");
-
-// Summary of row s on the state before decision s - kSpecLag: for each of the kSumWarps warps its
-// kKeysPerWarp smallest packed keys of C (with tie word, W and hit) and its kWPerWarp smallest W of A;
-// every pair of C it does not publish has (key, tie) >= (key_bound, tie_bound), every W of A it does
-// not publish is >= the W bound.  W values travel as order-preserving bits (f2ord).
-struct __align__(16) RowSummary {
-  unsigned long long key[kSumWarps * kKeysPerWarp];  // packed (class, value) keys; kNoKey: none
-  uint32_t tie[kSumWarps * kKeysPerWarp];            // tie words (instance in the low 12 bits)
-  uint32_t word[kSumWarps * kKeysPerWarp];           // f2ord(W) of the pair
-  uint32_t hit[kSumWarps * kKeysPerWarp];            // its hit (blocks)
-  unsigned long long w[kSumWarps * kWPerWarp];       // f2ord(W) << 32 | instance over A; ~0: none
-  unsigned long long key_bound;                      // kNoKey: every pair of C is published
-  uint32_t tie_bound;
-  uint32_t w_bound;                                  // 0xFFFFFFFF: every W of A is published
-  uint32_t wmin;                                     // f2ord(W_min over A), 0xFFFFFFFF: A empty
-  uint32_t pad[3];
-};
-static_assert(sizeof(RowSummary) % 16 == 0, "summaries are copied in 16-byte pieces");
-
 struct GreedySync {
   unsigned long long* jobs;  // [R] 1 << 63 | hit of the pick << 32 | pick (0xFFFFFFFF = rejected); 0 = unpublished
   uint32_t* done;            // [R] insert blocks done with the job (its blocks are all in at the group size)
   uint32_t* ready;           // [R] 1 once the row's probed hits are in the ring
   uint32_t* hitring;         // [kHitSlots][ring_stride] probed hits (row s in slot s % kHitSlots)
   float* tpfring;            // [kHitSlots][ring_stride] T_pf at those hits (kNoTpfBits where it changed)
-  uint32_t ring_stride;      // I rounded up to a multiple of 4
+  uint32_t ring_stride;      // I rounded up to a multiple of 8
   uint64_t wait_ns;          // bound on any cross-block wait (ns); a waiter that gives up sets kErrTimeout
-  RowSummary* sums;          // [kSumSlots] published row summaries
-  uint32_t* sready;          // [R] 1 once row s's summary is published
   unsigned long long* stats; // [kGreedyStats] counters of the pass (below)
 };
 
-// Counters of one greedy pass (GreedySync::stats): decisions taken from a corrected summary and by a
-// full pass, then SM clock cycles summed over the blocks of each role: the deciding warp waiting for
-// staged rows and in all; the feeder waiting for a free ring slot and for published summaries; the
-// summary blocks waiting for published decisions, for probed rows, and evaluating rows; the probe
-// blocks waiting for the inserts of earlier decisions.
+// Counters of one greedy pass (GreedySync::stats): decisions made, then SM clock cycles: the deciding
+// block's hit warp waiting for staged rows, the deciding block in all, its feeder waiting for a free
+// ring slot and for probed rows, and, summed over the probe blocks, their waits for the inserts of
+// earlier decisions.  The other words stay 0.
 enum : int {
-  kGsFast = 0, kGsFull, kGsDecideWait, kGsDecideTotal, kGsFeedSlotWait, kGsFeedSumWait, kGsSumJobWait,
-  kGsSumReadyWait, kGsSumEval, kGsProbeDoneWait, kGreedyStats
+  kGsDecisions = 0, kGsDecideWait = 2, kGsDecideTotal, kGsFeedSlotWait, kGsFeedWait, kGsProbeDoneWait = 9, kGreedyStats
 };
 
 // Window table from a chain's last block hash to the earliest request ending there.

@@ -1,0 +1,80 @@
+"""The greedy pass where its deciding block changes shape: instance counts around its warp and
+instances-per-thread boundaries, windows around the probe lag, equal keys, and states that need
+64-bit sums.  Every decision and the pending state must equal the oracle's."""
+import numpy as np
+import pytest
+
+import workload as W
+from oracle import Oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.fail("a CUDA device is required for the gpu tests")
+    import paper_2609_33224_gb300 as P
+    P.build()
+    return P
+
+
+def _check(P, model, ins, win):
+    orc = Oracle(ins.I, model).load(ins)
+    with P.Scheduler(ins.I, ins.cap_blocks, win.R, int(win.chain_off[-1]), model, table_load_factor=0.5) as s:
+        s.load_workload_instances(ins)
+        g = s.schedule_window(win)
+        o = orc.schedule(win)
+        for k in ("assign", "path", "hit_chosen"):
+            assert np.array_equal(g[k], o[k]), (k, np.nonzero(g[k] != o[k])[0][:5])
+        pend, ost = s.get_instances(pending=True), orc.get_state()
+        for k in ("b", "qr", "q", "S"):
+            assert np.array_equal(pend[k], ost[k]), k
+    return o
+
+
+def _workload(I, R, seed=11):
+    return W.generate(0, seed=seed, num_instances=I, window_requests=R, num_sessions=max(4, R // 6), cap_blocks=2048,
+                      b_hi=8, b_max=64)
+
+
+@pytest.mark.parametrize("I", [1, 31, 32, 33, 511, 512, 513, 1023, 1024, 1025, 2048])
+def test_instance_counts(P, I):
+    wl = _workload(I, 80)
+    _check(P, wl.model, wl.instances, wl.window)
+
+
+@pytest.mark.parametrize("R", [1, 2, 7, 8, 9, 32, 33, 34, 65, 130])
+def test_window_lengths(P, R):
+    wl = _workload(12, R)
+    _check(P, wl.model, wl.instances, wl.window)
+
+
+@pytest.mark.parametrize("selector", range(6))
+def test_equal_keys_go_to_the_lowest_instance(P, selector):
+    # every instance in the same state and with the same cache: all keys of a row are equal at first
+    wl = _workload(520, 60)
+    ins = wl.instances
+    for a in (ins.b, ins.qr, ins.q, ins.S):
+        a[:] = a[0]
+    ins.chain_inst, ins.chain_off = np.zeros(0, np.uint32), np.zeros(1, np.uint64)
+    ins.chain_hash, ins.chain_parent = np.zeros(0, np.uint64), np.zeros(0, np.uint64)
+    o = _check(P, dict(wl.model, selector=selector), ins, wl.window)
+    assert o["assign"][0] == 0
+
+
+@pytest.mark.parametrize("shift", ["kv_room", "tokens", "queue"])
+def test_sums_beyond_32_bits(P, shift):
+    # KV capacities, held tokens or queued tokens from which a 32-bit sum could overflow in the window
+    wl = _workload(70, 90)
+    ins = wl.instances
+    ins.M_KV[:] = 1 << 45 if shift != "queue" else ins.M_KV
+    if shift == "tokens":
+        ins.S[::3] += (1 << 30) - 5000
+        ins.S[1::3] += 1 << 40
+    if shift == "queue":
+        ins.q[::2] += (1 << 30) - 9000
+        ins.q[5::7] += 1 << 35
+    for sel in (0, 5):
+        _check(P, dict(wl.model, selector=sel), ins, wl.window)
