@@ -411,7 +411,7 @@ __device__ __forceinline__ void insert_tail(psk::DeltaSlot* delta, uint64_t nslo
     for (int q = 0; q < kInsertBatch; ++q) {
       old[q] = ~0ull;
       if (key[q] != psk::kEmpty && key[q] != psk::kTomb) {
-        slot[q] = psk::delta_home(key[q], nslots);
+        slot[q] = psk::delta_home(key[q], j, nslots);
         old[q] = atomicCAS(&delta[slot[q]].hash, psk::kEmpty, (unsigned long long)key[q]);
       }
     }
