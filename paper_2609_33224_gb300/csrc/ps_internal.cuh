@@ -9,8 +9,8 @@
 //                 memory round trip.  If both buckets are full the key goes to the first non-full
 //                 bucket after b1 (wrapping) and b1 plus every full bucket passed get their bit set
 //                 in the instance's overflow bitmap; at load factor 0.9 about 0.6% of keys take that
-//                 path.  Slot value 0 = empty.  Each table has a single writer (one warp per
-//                 instance), so placement needs no atomics and a key is never stored twice.
+//                 path.  Slot value 0 = empty.  Writers claim slots by compare-and-swap, each new key by
+//                 one thread, so a key is never stored twice.
 //   delta table   window-scoped set of (instance, block) pairs cached by the window's own earlier
 //                 decisions: one 16-byte slot {hash, instance + 1} per pair, linear probing from the
 //                 pair's home slot, sized at twice the window's block bound so it can never fill.
@@ -290,69 +290,6 @@ struct ReqStore {
   uint32_t* d_out;    // [I*M]
   uint32_t* d_rem;    // [I*M] remaining output tokens
 };
-
-// Warp-cooperative insert of one key by the instance's only writer warp (all 32 lanes call it with
-// the same arguments).  Lanes 0-7 read bucket b1, lanes 8-15 bucket b2; the key goes to the emptier
-// one.  With LRU metadata (meta.last_use != nullptr) a new block records (last_use, 0 children,
-// its parent's slot) and its cached parent gains a child; an existing block only has its last_use
-// raised.  parent_slot, if not ~0, is the parent's known slot (saves a lookup).  Returns the key's
-// slot, or ~0 if the table is full; *inserted tells whether the key is new.
-__device__ __forceinline__ uint64_t warp_insert(uint64_t* slots, uint64_t* ovf, const TableDesc d, uint64_t key,
-                                                bool* inserted, LruMeta meta = LruMeta{nullptr, nullptr, nullptr},
-                                                uint64_t parent = 0, uint32_t last_use = 0,
-                                                uint64_t parent_slot = ~0ull) {
-  const int lane = threadIdx.x & 31;
-  *inserted = false;
-  const uint64_t found = main_find(slots, ovf, d, key);
-  if (found != ~0ull) {
-    if (meta.last_use && lane == 0 && meta.last_use[found] < last_use) meta.last_use[found] = last_use;
-    __syncwarp();
-    return found;
-  }
-  const uint32_t b1 = fastrange32(key, d.nbkt);
-  const uint32_t b2 = fastrange32(remix(key), d.nbkt);
-  uint64_t idx = ~0ull;
-  if (lane < 8) idx = d.base + (uint64_t)b1 * kBucketSlots + lane;
-  else if (lane < 16) idx = d.base + (uint64_t)b2 * kBucketSlots + (lane - 8);
-  const uint64_t v = idx != ~0ull ? __ldcg(reinterpret_cast<const unsigned long long*>(slots + idx)) : ~0ull;
-  const unsigned empty = __ballot_sync(0xffffffffu, idx != ~0ull && v == kEmpty);
-  const unsigned e1 = empty & 0xFFu, e2 = empty & 0xFF00u;
-  int target = -1;
-  if (e1 || e2) {
-    // emptier bucket (more empty slots), b1 on ties
-    target = (__popc(e1) >= __popc(e2)) ? __ffs(e1) - 1 : __ffs(e2) - 1;
-  } else {
-    // both full: first non-full bucket after b1; mark b1 and every full bucket passed
-    uint32_t b = b1;
-    for (uint32_t step = 0; step < d.nbkt && target < 0; ++step) {
-      if (lane == 0) atomicOr(reinterpret_cast<unsigned long long*>(ovf + d.ovf + (b >> 6)), 1ull << (b & 63));
-      b = (b + 1 == d.nbkt) ? 0u : b + 1;
-      const uint64_t q = d.base + (uint64_t)b * kBucketSlots + (lane & 7);
-      const uint64_t w = lane < 8 ? __ldcg(reinterpret_cast<const unsigned long long*>(slots + q)) : ~0ull;
-      const unsigned em = __ballot_sync(0xffffffffu, lane < 8 && w == kEmpty);
-      if (em) {
-        target = __ffs(em) - 1;
-        idx = q;
-      }
-    }
-    if (target < 0) return ~0ull;
-  }
-  const uint64_t slot = __shfl_sync(0xffffffffu, idx, target);
-  uint64_t ps = kNoParent;
-  if (meta.last_use && parent != kEmpty) ps = parent_slot != ~0ull ? parent_slot : main_find(slots, ovf, d, parent);
-  if (lane == target) {
-    slots[slot] = key;
-    if (meta.last_use) {
-      meta.last_use[slot] = last_use;
-      meta.children[slot] = 0;
-      meta.parent[slot] = ps;
-    }
-  }
-  if (ps != kNoParent && lane == 0) meta.children[ps] += 1;
-  __syncwarp();
-  *inserted = true;
-  return slot;
-}
 
 // Insert of one key by one thread while other threads insert other keys into the same table (each
 // key by one thread only; a key cached before the batch is found and left in place): both
