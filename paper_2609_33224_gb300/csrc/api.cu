@@ -102,10 +102,9 @@ struct ps_ctx {
   // streaming: per-block LRU metadata, request store, capacities on the device, eviction buffers
   bool lru = false;
   psk::LruMeta meta{nullptr, nullptr, nullptr};
-  void* d_leafbuf = nullptr;
+  pskl::EvictScratch evict{};
+  uint32_t max_use = 0;  // largest last_use stamp given so far
   unsigned long long* d_cprefix = nullptr;  // [2 (Rmax + 1)] commit item prefixes
-  uint32_t* d_nleaf = nullptr;
-  uint32_t* d_more = nullptr;
   uint64_t max_instance_slots = 0;
   psk::ReqStore rq{};
   uint64_t* d_cap = nullptr;
@@ -494,9 +493,15 @@ ps_status ps_create(const ps_config* cfg, ps_ctx** out) {
     for (uint32_t i = 0; i < I; ++i)
       c->max_instance_slots = std::max<uint64_t>(c->max_instance_slots, (uint64_t)td[i].nbkt * psk::kBucketSlots);
     unsigned char* lb = nullptr;
-    ok = dalloc(c, &lb, pskl::evict_leafbuf_bytes(c->I)) == cudaSuccess && dalloc(c, &c->d_nleaf, I) == cudaSuccess &&
-         dalloc(c, &c->d_more, 1) == cudaSuccess;
-    c->d_leafbuf = lb;
+    unsigned char* plan = nullptr;
+    pskl::EvictScratch& ev = c->evict;
+    ok = dalloc(c, &lb, pskl::evict_leafbuf_bytes(c->I)) == cudaSuccess && dalloc(c, &ev.nleaf, I) == cudaSuccess &&
+         dalloc(c, &ev.more, 1) == cudaSuccess && dalloc(c, &plan, pskl::evict_plan_bytes(c->I)) == cudaSuccess &&
+         dalloc(c, &ev.hist, pskl::evict_hist_words(c->I)) == cudaSuccess &&
+         dalloc(c, &ev.cand, pskl::evict_cand_words(c->I)) == cudaSuccess && dalloc(c, &ev.list, I + 1) == cudaSuccess &&
+         dalloc(c, &ev.slow, I) == cudaSuccess;
+    ev.leafbuf = lb;
+    ev.plan = plan;
   }
   if (ok && c->lru)
     ok = dalloc(c, &c->meta.last_use, c->total_slots) == cudaSuccess &&
@@ -542,6 +547,7 @@ ps_status ps_create(const ps_config* cfg, ps_ctx** out) {
   if (c->lru)
     set = set && cudaMemsetAsync(c->meta.last_use, 0, c->total_slots * 4, c->stream) == cudaSuccess &&
           cudaMemsetAsync(c->meta.children, 0, c->total_slots * 4, c->stream) == cudaSuccess &&
+          cudaMemsetAsync(c->evict.hist, 0, pskl::evict_hist_words(c->I) * 4, c->stream) == cudaSuccess &&
           cudaMemsetAsync(c->meta.parent, 0xFF, c->total_slots * 8, c->stream) == cudaSuccess;  // kNoParent
   if (c->rq.M)
     set = set && cudaMemsetAsync(c->rq.q_head, 0, I * 4, c->stream) == cudaSuccess &&
@@ -711,6 +717,7 @@ ps_status ps_insert_chains(ps_ctx* c, uint64_t nchains, const uint32_t* inst, co
   } else {
     PS_TRY_CUDA(c, cudaMemcpy(&total, off + nchains, 8, cudaMemcpyDeviceToHost));
   }
+  c->max_use = std::max(c->max_use, last_use);
   cudaError_t e = pskl::launch_insert_chains(c->d_slots, c->d_ovf, c->d_tdesc, c->I, c->d_count, nchains, d_inst, d_off,
                                              d_hash, d_parent, total, c->meta, last_use, c->d_err, c->num_sms,
                                              c->stream);
@@ -886,6 +893,7 @@ ps_status ps_commit_window(ps_ctx* c, uint32_t last_use) {
   if (c->rq.M && c->pend_win.R && !c->pend_out)
     return fail(c, PS_ERR_INVALID, "request tracking needs the window's out_tokens");
   DeviceGuard g(c->device);
+  c->max_use = std::max(c->max_use, last_use);
   record(c, kEvCommit0);
   PS_TRY_CUDA(c, pskl::launch_commit(c->d_slots, c->d_ovf, c->d_tdesc, c->I, c->d_count, c->pend_win, c->d_assign,
                                      c->d_hchosen, c->meta, last_use, c->rq, c->pend_out, c->d_cprefix, c->d_err,
@@ -963,8 +971,8 @@ ps_status ps_advance_window(ps_ctx* c, const ps_advance_params* p) {
   PS_TRY_CUDA(c, pskl::launch_advance(c->st, c->I, c->rq, c->model, p->window_ms, p->prefill_tokens, c->d_err,
                                       c->stream));
   if (p->evict)
-    PS_TRY_CUDA(c, pskl::launch_evict(c->d_slots, c->d_tdesc, c->I, c->d_count, c->d_cap, c->meta, c->d_leafbuf,
-                                      c->d_nleaf, c->d_more, c->h_more, c->max_instance_slots, c->d_err, c->stream));
+    PS_TRY_CUDA(c, pskl::launch_evict(c->d_slots, c->d_tdesc, c->I, c->d_count, c->d_cap, c->meta, c->evict, c->h_more,
+                                      c->max_instance_slots, c->max_use, c->d_err, c->num_sms, c->stream));
   return finish(c);
 }
 

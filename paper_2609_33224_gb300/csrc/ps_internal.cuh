@@ -981,12 +981,28 @@ cudaError_t launch_commit(uint64_t* slots, uint64_t* ovf, const psk::TableDesc* 
                           uint32_t* err, int num_sms, cudaStream_t s);
 cudaError_t launch_advance(psk::StateSoA st, uint32_t I, const psk::ReqStore& rq, const psk::DevModel& m,
                            float window_ms, uint64_t prefill_tokens, uint32_t* err, cudaStream_t s);
+// Device scratch of the eviction: leafbuf holds evict_leafbuf_bytes(I) bytes, plan evict_plan_bytes(I),
+// hist evict_hist_words(I) words (zero between calls), cand evict_cand_words(I); nleaf, slow [I],
+// list [I + 1], more [1].
+struct EvictScratch {
+  void* leafbuf;
+  uint32_t* nleaf;
+  uint32_t* more;
+  void* plan;
+  uint32_t* hist;
+  uint32_t* cand;
+  uint32_t* list;
+  uint32_t* slow;
+};
 // Leaf-first LRU eviction of every instance over capacity (rounds until none is; synchronises the
-// stream between rounds).  leafbuf holds evict_leafbuf_bytes(I) bytes; nleaf [I], more [1] device
-// words; more_host one pinned word; max_instance_slots the largest table (slots) of an instance.
+// stream between rounds).  more_host one pinned word; max_instance_slots the largest table (slots) of
+// an instance; max_use the largest last_use stamp any block may have.
 cudaError_t launch_evict(uint64_t* slots, const psk::TableDesc* tdesc, uint32_t I, unsigned long long* count,
-                         const uint64_t* cap, psk::LruMeta meta, void* leafbuf, uint32_t* nleaf, uint32_t* more,
-                         uint32_t* more_host, uint64_t max_instance_slots, uint32_t* err, cudaStream_t s);
+                         const uint64_t* cap, psk::LruMeta meta, const EvictScratch& sc, uint32_t* more_host,
+                         uint64_t max_instance_slots, uint32_t max_use, uint32_t* err, int num_sms, cudaStream_t s);
+size_t evict_plan_bytes(uint32_t I);
+size_t evict_hist_words(uint32_t I);
+size_t evict_cand_words(uint32_t I);
 size_t evict_leafbuf_bytes(uint32_t I);
 cudaError_t launch_check_parents(const uint64_t* slots, const uint64_t* ovf, const psk::TableDesc* tdesc, uint32_t I,
                                  uint64_t nchains, const uint32_t* inst, const uint64_t* parent,

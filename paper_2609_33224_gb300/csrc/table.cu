@@ -536,7 +536,467 @@ __global__ void advance_kernel(psk::StateSoA st, uint32_t I, psk::ReqStore rq, p
   }
 }
 
-// Leaf-first LRU eviction of the instances over capacity, in rounds of two kernels:
+// A leaf candidate with its parent's slot (kLeafNoParent for none), so that evicting it needs no
+// dependent load before the parent's metadata can be read.  Five 32-bit words (the hash split).
+struct Leaf {
+  uint32_t last_use;
+  uint32_t slot;
+  uint32_t hash_lo, hash_hi;
+  uint32_t parent;
+};
+static_assert(sizeof(Leaf) == 20, "a leaf is five 32-bit words");
+constexpr uint32_t kLeafNoParent = 0xFFFFFFFFu;
+
+__device__ __forceinline__ uint32_t parent32(uint64_t p) {
+  return (p == psk::kNoParent || p == psk::kLinkPending) ? kLeafNoParent : (uint32_t)p;
+}
+
+// Leaf-first LRU eviction of the instances over capacity.
+//
+// Evicting the smallest leaf by (last_use, hash) again and again removes blocks in increasing order of
+// their subtree maximum of (last_use, hash), deeper first where two share it.  Where stamps never
+// increase down a chain (a commit stamps a request's whole chain, a bulk insert every block it touches)
+// a block's subtree maximum has its own last_use.  So with T the last_use value at which the blocks
+// counted from the oldest reach the excess E, the evicted blocks are exactly: every block older than T,
+// and of the blocks stamped T the k missing ones with the smallest subtree maximum of the hash over
+// blocks stamped T.  Four kernels find and evict them, every step parallel:
+//   list      the instances over capacity;
+//   hist      per instance a histogram of last_use over its slots (and its number of leaves), in one
+//             pass for stamps below 2048 and one more per further 11 bits; choose picks T and k;
+//   gather    the slots stamped below T and those stamped T (up to kClassMax each; at most kClassMax
+//             evictions a round);
+//   order     one thread block per instance checks that the stamps do not increase downwards among
+//             these blocks and that none of them has a newer child; finds the subtree maxima of the
+//             class T by doubling over the parent links in shared memory (a block pushes its maximum
+//             to its ancestor 2^r links up in round r); selects the k smallest; evicts.
+// An instance that fails the check, or has more blocks stamped T than shared memory holds, is evicted
+// one block at a time by the kernels after these.  Bound by the two scans of the tables (16 bytes a
+// slot).  1024 instances x 200K blocks, about 240 over capacity by up to 7.9K blocks: a streaming
+// window of 500 requests takes 2.08 ms; with one thread ordering each instance's evictions (1.2 us
+// each, 10 ms of the window) it took 11.8 ms.
+constexpr uint32_t kClassMax = 16384;   // blocks of one last_use value ordered in shared memory
+constexpr uint32_t kHistBits = 11;
+constexpr uint32_t kHistBins = 1u << kHistBits;
+constexpr uint32_t kOrderThreads = 1024;
+constexpr uint32_t kOrderPer = kClassMax / kOrderThreads;  // blocks per thread
+constexpr uint32_t kScanThreads = 512;
+constexpr uint64_t kScanChunk = 65536;  // slots a block scans before it merges its histogram
+constexpr uint32_t kNoJump = 0xFFFFu;
+static_assert(kClassMax < kNoJump, "16-bit block indices");
+constexpr uint32_t kMoreFast = 1u, kMoreSlow = 2u;  // bits of the "another round" word
+
+// Per over-capacity instance: the last_use range still open, what was counted below it, and the choice.
+struct EvictPlan {
+  uint32_t lo, hi;       // T lies in [lo, hi]
+  uint32_t below;        // blocks stamped below lo
+  uint32_t todo;         // evictions of this round
+  uint32_t k;            // of them, blocks stamped T (T = lo once chosen)
+  uint32_t n_old, n_cls; // gathered blocks
+  uint32_t leaves;
+};
+
+__global__ void __launch_bounds__(1024)
+evict_list_kernel(uint32_t I, const unsigned long long* __restrict__ count, const uint64_t* __restrict__ cap,
+                  const uint32_t* __restrict__ slow, uint32_t max_use, EvictPlan* plan, uint32_t* list, uint32_t* nlist) {
+  __shared__ uint32_t s_n;
+  if (threadIdx.x == 0) s_n = 0u;
+  __syncthreads();
+  for (uint32_t i = threadIdx.x; i < I; i += blockDim.x) {
+    const unsigned long long c = count[i];
+    if (c <= cap[i] || slow[i]) continue;
+    const unsigned long long E = c - cap[i];
+    EvictPlan p{};
+    p.hi = max_use;
+    p.todo = E < kClassMax ? (uint32_t)E : kClassMax;
+    plan[i] = p;
+    list[atomicAdd(&s_n, 1u)] = i;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) *nlist = s_n;
+}
+
+// Bin width of an open range as a shift.
+__device__ __forceinline__ uint32_t hist_shift(uint32_t lo, uint32_t hi) {
+  const uint32_t span = hi - lo;
+  return span < kHistBins ? 0u : 32u - (uint32_t)__clz(span) - kHistBits;
+}
+
+__global__ void __launch_bounds__(kScanThreads)
+evict_hist_kernel(const uint64_t* __restrict__ slots, const psk::TableDesc* __restrict__ tdesc, psk::LruMeta meta,
+                  EvictPlan* plan, const uint32_t* __restrict__ list, const uint32_t* __restrict__ nlist,
+                  uint64_t chunks, uint32_t* __restrict__ hist, bool first) {
+  __shared__ uint32_t s_bin[kHistBins];
+  __shared__ uint32_t s_leaves;
+  const uint64_t items = (uint64_t)*nlist * chunks;
+  for (uint64_t item = blockIdx.x; item < items; item += gridDim.x) {
+    const uint32_t i = list[item / chunks];
+    const psk::TableDesc d = tdesc[i];
+    const uint64_t n = (uint64_t)d.nbkt * psk::kBucketSlots, x0 = (item % chunks) * kScanChunk;
+    if (x0 >= n) continue;  // block-uniform
+    const uint64_t x1 = x0 + kScanChunk < n ? x0 + kScanChunk : n;
+    const uint32_t lo = plan[i].lo, hi = plan[i].hi, sh = hist_shift(lo, hi);
+    for (uint32_t b = threadIdx.x; b < kHistBins; b += kScanThreads) s_bin[b] = 0u;
+    if (threadIdx.x == 0) s_leaves = 0u;
+    __syncthreads();
+    uint32_t leaves = 0;
+    // two slots a thread (tables are whole 8-slot buckets)
+    for (uint64_t x = x0 + 2u * threadIdx.x; x < x1; x += 2u * kScanThreads) {
+      const ulonglong2 key = __ldcs(reinterpret_cast<const ulonglong2*>(slots + d.base + x));
+      const uint2 lu = __ldcs(reinterpret_cast<const uint2*>(meta.last_use + d.base + x));
+      if (key.x != psk::kEmpty && lu.x >= lo && lu.x <= hi) atomicAdd(&s_bin[(lu.x - lo) >> sh], 1u);
+      if (key.y != psk::kEmpty && lu.y >= lo && lu.y <= hi) atomicAdd(&s_bin[(lu.y - lo) >> sh], 1u);
+      if (first) {
+        const uint2 ch = __ldcs(reinterpret_cast<const uint2*>(meta.children + d.base + x));
+        leaves += (key.x != psk::kEmpty && ch.x == 0u) + (key.y != psk::kEmpty && ch.y == 0u);
+      }
+    }
+    if (first) {
+      leaves = __reduce_add_sync(0xffffffffu, leaves);
+      if ((threadIdx.x & 31u) == 0u && leaves) atomicAdd(&s_leaves, leaves);
+    }
+    __syncthreads();
+    for (uint32_t b = threadIdx.x; b < kHistBins; b += kScanThreads)
+      if (s_bin[b]) atomicAdd(&hist[(uint64_t)i * kHistBins + b], s_bin[b]);
+    if (first && threadIdx.x == 0) atomicAdd(&plan[i].leaves, s_leaves);
+    __syncthreads();
+  }
+}
+
+// Narrows the open range to the bin in which the count reaches the round's evictions; with one value
+// a bin that value is T.  Clears the histogram for the next pass.
+__global__ void __launch_bounds__(256)
+evict_choose_kernel(EvictPlan* plan, const uint32_t* __restrict__ list, const uint32_t* __restrict__ nlist,
+                    uint32_t* __restrict__ hist) {
+  constexpr uint32_t kPer = kHistBins / 256;
+  __shared__ uint32_t s_sum[256];
+  const uint32_t t = threadIdx.x;
+  for (uint32_t x = blockIdx.x; x < *nlist; x += gridDim.x) {
+    const uint32_t i = list[x];
+    const EvictPlan p = plan[i];
+    const uint32_t sh = hist_shift(p.lo, p.hi);
+    uint32_t v[kPer], sum = 0;
+#pragma unroll
+    for (uint32_t u = 0; u < kPer; ++u) {
+      uint32_t* b = &hist[(uint64_t)i * kHistBins + t * kPer + u];
+      v[u] = *b;
+      *b = 0u;
+      sum += v[u];
+    }
+    s_sum[t] = sum;
+    __syncthreads();
+    for (uint32_t dd = 1; dd < 256; dd <<= 1) {
+      const uint32_t y = t >= dd ? s_sum[t - dd] : 0u;
+      __syncthreads();
+      s_sum[t] += y;
+      __syncthreads();
+    }
+    uint32_t acc = p.below + s_sum[t] - sum;  // blocks stamped below this thread's bins
+#pragma unroll
+    for (uint32_t u = 0; u < kPer; ++u) {
+      if (acc < p.todo && acc + v[u] >= p.todo) {  // one thread, one bin
+        const uint32_t lo = p.lo + ((t * kPer + u) << sh);
+        const uint32_t w = (1u << sh) - 1u;
+        plan[i].lo = lo;
+        plan[i].hi = p.hi - lo < w ? p.hi : lo + w;
+        plan[i].below = acc;
+        plan[i].k = p.todo - acc;
+      }
+      acc += v[u];
+    }
+    __syncthreads();
+  }
+}
+
+// Gathers the slots stamped below T (first half of the instance's candidate buffer) and T (second half).
+__global__ void __launch_bounds__(kScanThreads)
+evict_gather_kernel(const uint64_t* __restrict__ slots, const psk::TableDesc* __restrict__ tdesc, psk::LruMeta meta,
+                    EvictPlan* plan, const uint32_t* __restrict__ list, const uint32_t* __restrict__ nlist,
+                    uint64_t chunks, uint32_t* __restrict__ cand) {
+  const uint64_t items = (uint64_t)*nlist * chunks;
+  const uint32_t lane = threadIdx.x & 31u;
+  for (uint64_t item = blockIdx.x; item < items; item += gridDim.x) {
+    const uint32_t i = list[item / chunks];
+    const psk::TableDesc d = tdesc[i];
+    const uint64_t n = (uint64_t)d.nbkt * psk::kBucketSlots, x0 = (item % chunks) * kScanChunk;
+    const uint64_t x1 = x0 + kScanChunk < n ? x0 + kScanChunk : n;
+    const uint32_t T = plan[i].lo;
+    uint32_t* out = cand + (uint64_t)i * 2u * kClassMax;
+    for (uint64_t xb = x0; xb < x1; xb += 4u * kScanThreads) {  // (tables are whole 8-slot buckets)
+      const uint64_t x = xb + 4u * threadIdx.x;
+      uint4 lu = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
+      const bool in = x < x1;
+      if (in) lu = __ldcs(reinterpret_cast<const uint4*>(meta.last_use + d.base + x));
+      const uint32_t l[4] = {lu.x, lu.y, lu.z, lu.w};
+      uint32_t oldm = 0u, clsm = 0u;
+      if (in && (l[0] <= T || l[1] <= T || l[2] <= T || l[3] <= T)) {
+        const ulonglong2 a = __ldcs(reinterpret_cast<const ulonglong2*>(slots + d.base + x));
+        const ulonglong2 b = __ldcs(reinterpret_cast<const ulonglong2*>(slots + d.base + x + 2));
+        const uint64_t key[4] = {a.x, a.y, b.x, b.y};
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (key[u] != psk::kEmpty) {
+            oldm |= (l[u] < T ? 1u : 0u) << u;
+            clsm |= (l[u] == T ? 1u : 0u) << u;
+          }
+      }
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        const uint32_t mask = half ? clsm : oldm;
+        const uint32_t mine = __popc(mask);
+        if (!__any_sync(0xffffffffu, mine != 0u)) continue;
+        uint32_t sum = mine;
+#pragma unroll
+        for (int dd = 1; dd < 32; dd <<= 1) {
+          const uint32_t y = __shfl_up_sync(0xffffffffu, sum, dd);
+          if (lane >= (uint32_t)dd) sum += y;
+        }
+        uint32_t at = 0;
+        if (lane == 31u) at = atomicAdd(half ? &plan[i].n_cls : &plan[i].n_old, sum);
+        at = __shfl_sync(0xffffffffu, at, 31) + sum - mine;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if ((mask >> u) & 1u) {
+            if (at < kClassMax) out[half * kClassMax + at] = (uint32_t)(d.base + x) + u;
+            ++at;
+          }
+      }
+    }
+  }
+}
+
+struct OrderSmem {
+  unsigned long long M[kClassMax];  // subtree maximum of the hash over the class
+  uint16_t jump[kClassMax];         // ancestor 2^r links up (kNoJump: past the class)
+  uint16_t dep[kClassMax];          // links to the topmost ancestor in the class, plus one
+  uint32_t hist[256];
+  unsigned long long sel;           // radix selection: the chosen bytes so far
+  uint32_t rank;                    // and the rank among the values that share them
+  uint32_t dep_max;
+};
+
+__global__ void __launch_bounds__(kOrderThreads)
+evict_order_kernel(uint64_t* slots, unsigned long long* count, const uint64_t* __restrict__ cap, psk::LruMeta meta,
+                   const EvictPlan* __restrict__ plan, const uint32_t* __restrict__ list,
+                   const uint32_t* __restrict__ nlist, const uint32_t* __restrict__ cand, uint32_t* slow, uint32_t* more,
+                   uint32_t max_leaves, uint32_t* err) {
+  extern __shared__ __align__(16) unsigned char order_raw[];
+  OrderSmem& s = *reinterpret_cast<OrderSmem*>(order_raw);
+  __shared__ unsigned long long s_children, s_inside;
+  const uint32_t t = threadIdx.x;
+  for (uint32_t item = blockIdx.x; item < *nlist; item += gridDim.x) {
+    const uint32_t i = list[item];
+    const EvictPlan p = plan[i];
+    const uint32_t T = p.lo, n = p.n_cls, n_old = p.n_old;
+    if (p.leaves > max_leaves) {  // (the limit of the one-at-a-time kernels, kept for every instance)
+      if (t == 0) atomicOr(err, psk::kErrLeavesFull);
+      continue;
+    }
+    if (n > kClassMax || n_old > kClassMax) {
+      if (t == 0) {
+        slow[i] = 1u;
+        atomicOr(more, kMoreSlow);
+      }
+      continue;
+    }
+    const uint32_t* old_slots = cand + (uint64_t)i * 2u * kClassMax;
+    const uint32_t* cls_slots = old_slots + kClassMax;
+    // check: every child of these blocks is one of them, and no child is newer than its parent
+    uint32_t slot[kOrderPer], par[kOrderPer];  // this thread's class blocks: slot, parent's slot if in the class
+    unsigned long long children = 0, inside = 0;
+    bool bad = false;
+#pragma unroll
+    for (uint32_t u = 0; u < kOrderPer; ++u) {
+      const uint32_t x = t + u * kOrderThreads;
+      slot[u] = par[u] = kLeafNoParent;
+      if (x < n) {
+        slot[u] = cls_slots[x];
+        children += meta.children[slot[u]];
+        const uint32_t ps = parent32(meta.parent[slot[u]]);
+        if (ps != kLeafNoParent) {
+          const uint32_t lp = meta.last_use[ps];
+          if (lp <= T) ++inside;
+          if (lp < T) bad = true;
+          if (lp == T) par[u] = ps;
+        }
+      }
+    }
+    for (uint32_t x = t; x < n_old; x += kOrderThreads) {
+      const uint32_t sl = old_slots[x];
+      children += meta.children[sl];
+      const uint32_t ps = parent32(meta.parent[sl]);
+      if (ps != kLeafNoParent) {
+        const uint32_t lp = meta.last_use[ps];
+        if (lp <= T) ++inside;
+        if (lp < meta.last_use[sl]) bad = true;
+      }
+    }
+    if (t == 0) {
+      s_children = 0ull;
+      s_inside = 0ull;
+    }
+    __syncthreads();
+    if (children) atomicAdd(&s_children, children);
+    if (inside) atomicAdd(&s_inside, inside);
+    bad = __syncthreads_or(bad ? 1 : 0) != 0;
+    if (bad || s_children != s_inside) {  // block-uniform
+      if (t == 0) {
+        slow[i] = 1u;
+        atomicOr(more, kMoreSlow);
+      }
+      __syncthreads();
+      continue;
+    }
+    uint32_t gone = 0u;  // bit u: this thread's class block u is evicted
+    if (p.k >= n) {
+      gone = (1u << kOrderPer) - 1u;
+    } else {
+      // A class block's index stands in for its (known) stamp while its children look it up.
+#pragma unroll
+      for (uint32_t u = 0; u < kOrderPer; ++u) {
+        const uint32_t x = t + u * kOrderThreads;
+        if (x < n) {
+          meta.last_use[slot[u]] = x;
+          s.M[x] = slots[slot[u]];
+          s.dep[x] = 1;
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (uint32_t u = 0; u < kOrderPer; ++u) {
+        const uint32_t x = t + u * kOrderThreads;
+        if (x < n) s.jump[x] = (uint16_t)(par[u] != kLeafNoParent ? __ldcg(meta.last_use + par[u]) : kNoJump);
+      }
+      __syncthreads();
+      for (;;) {  // at most 14 rounds: a path holds at most kClassMax blocks
+        uint32_t nj[kOrderPer];
+        uint32_t nd[kOrderPer];
+        bool any = false;
+#pragma unroll
+        for (uint32_t u = 0; u < kOrderPer; ++u) {
+          const uint32_t x = t + u * kOrderThreads;
+          nj[u] = kNoJump;
+          nd[u] = 0u;
+          if (x < n && s.jump[x] != kNoJump) {
+            const uint32_t j = s.jump[x];
+            any = true;
+            atomicMax(&s.M[j], s.M[x]);
+            nj[u] = s.jump[j];
+            nd[u] = s.dep[j];
+          }
+        }
+        if (!__syncthreads_or(any ? 1 : 0)) break;
+#pragma unroll
+        for (uint32_t u = 0; u < kOrderPer; ++u) {
+          const uint32_t x = t + u * kOrderThreads;
+          if (x < n && s.jump[x] != kNoJump) {
+            s.jump[x] = (uint16_t)nj[u];
+            s.dep[x] = (uint16_t)(s.dep[x] + nd[u]);
+          }
+        }
+        __syncthreads();
+      }
+      // the k-th smallest maximum, byte by byte from the top
+      if (t == 0) {
+        s.sel = 0ull;
+        s.rank = p.k - 1u;
+        s.dep_max = 0u;
+      }
+      for (int sh = 56; sh >= 0; sh -= 8) {
+        if (t < 256) s.hist[t] = 0u;
+        __syncthreads();
+        const unsigned long long sel = s.sel;
+        const unsigned long long high = sh == 56 ? 0ull : ~0ull << (sh + 8);
+#pragma unroll
+        for (uint32_t u = 0; u < kOrderPer; ++u) {
+          const uint32_t x = t + u * kOrderThreads;
+          if (x < n && (s.M[x] & high) == sel) atomicAdd(&s.hist[(s.M[x] >> sh) & 255u], 1u);
+        }
+        __syncthreads();
+        if (t < 32) {  // the bin that holds the rank
+          uint32_t v[8], sum = 0;
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            v[u] = s.hist[t * 8 + u];
+            sum += v[u];
+          }
+          uint32_t x = sum;
+#pragma unroll
+          for (int dd = 1; dd < 32; dd <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, dd);
+            if ((int)t >= dd) x += y;
+          }
+          const uint32_t rank = s.rank;
+          uint32_t acc = x - sum;
+          __syncwarp();
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            if (acc <= rank && rank < acc + v[u]) {  // one lane, one bin
+              s.sel = sel | ((unsigned long long)(t * 8 + u) << sh);
+              s.rank = rank - acc;
+            }
+            acc += v[u];
+          }
+        }
+        __syncthreads();
+      }
+      // blocks that share the k-th maximum lie on one path, the deepest (whose hash it is) first
+      const unsigned long long cut = s.sel;
+      const uint32_t rank = s.rank;
+#pragma unroll
+      for (uint32_t u = 0; u < kOrderPer; ++u) {
+        const uint32_t x = t + u * kOrderThreads;
+        if (x < n && s.M[x] == cut) atomicMax(&s.dep_max, (uint32_t)s.dep[x]);
+      }
+      __syncthreads();
+      const uint32_t dm = s.dep_max;
+#pragma unroll
+      for (uint32_t u = 0; u < kOrderPer; ++u) {
+        const uint32_t x = t + u * kOrderThreads;
+        if (x < n && (s.M[x] < cut || (s.M[x] == cut && s.dep[x] + rank >= dm))) gone |= 1u << u;
+      }
+    }
+    // evict: the slots first, then the surviving parents' counts, then the evicted blocks' own links
+#pragma unroll
+    for (uint32_t u = 0; u < kOrderPer; ++u) {
+      if (slot[u] == kLeafNoParent) continue;
+      const bool g = (gone >> u) & 1u;
+      if (g) slots[slot[u]] = psk::kEmpty;
+      meta.last_use[slot[u]] = g ? 0u : T;
+    }
+    for (uint32_t x = t; x < n_old; x += kOrderThreads) {
+      slots[old_slots[x]] = psk::kEmpty;
+      meta.last_use[old_slots[x]] = 0u;
+    }
+    __syncthreads();
+    auto drop = [&](uint32_t sl) {
+      const uint32_t ps = parent32(meta.parent[sl]);
+      if (ps != kLeafNoParent && __ldcg(slots + ps) != psk::kEmpty) atomicSub(meta.children + ps, 1u);
+    };
+#pragma unroll
+    for (uint32_t u = 0; u < kOrderPer; ++u)
+      if (slot[u] != kLeafNoParent && ((gone >> u) & 1u)) drop(slot[u]);
+    for (uint32_t x = t; x < n_old; x += kOrderThreads) drop(old_slots[x]);
+    __syncthreads();
+#pragma unroll
+    for (uint32_t u = 0; u < kOrderPer; ++u)
+      if (slot[u] != kLeafNoParent && ((gone >> u) & 1u)) {
+        meta.children[slot[u]] = 0u;
+        meta.parent[slot[u]] = psk::kNoParent;
+      }
+    for (uint32_t x = t; x < n_old; x += kOrderThreads) {
+      meta.children[old_slots[x]] = 0u;
+      meta.parent[old_slots[x]] = psk::kNoParent;
+    }
+    if (t == 0) {
+      const unsigned long long c = count[i] - p.todo;
+      count[i] = c;
+      if (c > cap[i]) atomicOr(more, kMoreFast);
+    }
+    __syncthreads();
+  }
+}
+
+// One block at a time (instances flagged slow), in rounds of two kernels:
 //   collect  all SMs scan the over-capacity instances' slots (coalesced) and append each leaf (a
 //            cached block with no cached child) to its instance's leaf buffer;
 //   evict    one thread block per over-capacity instance sorts its leaves by (last_use, hash), then
@@ -565,21 +1025,6 @@ constexpr uint64_t kEvictWaitNs = 1000000000ull;  // bound on the loader's idle 
 static_assert(kHeapMax < kDeltaSlots, "the count table never fills");
 constexpr int kCollectThreads = 256;
 constexpr uint32_t kCollectSlotsPerThread = 8;
-
-// A leaf candidate with its parent's slot (kLeafNoParent for none), so that evicting it needs no
-// dependent load before the parent's metadata can be read.  Five 32-bit words (the hash split).
-struct Leaf {
-  uint32_t last_use;
-  uint32_t slot;
-  uint32_t hash_lo, hash_hi;
-  uint32_t parent;
-};
-static_assert(sizeof(Leaf) == 20, "a leaf is five 32-bit words");
-constexpr uint32_t kLeafNoParent = 0xFFFFFFFFu;
-
-__device__ __forceinline__ uint32_t parent32(uint64_t p) {
-  return (p == psk::kNoParent || p == psk::kLinkPending) ? kLeafNoParent : (uint32_t)p;
-}
 
 __device__ __forceinline__ Leaf make_leaf(uint32_t last_use, uint32_t slot, uint64_t hash, uint64_t parent) {
   return Leaf{last_use, slot, (uint32_t)hash, (uint32_t)(hash >> 32), parent32(parent)};
@@ -728,9 +1173,9 @@ __device__ void evict_loader(const uint64_t* slots, const psk::LruMeta& meta, co
 __global__ void __launch_bounds__(kCollectThreads)
 leaf_collect_kernel(const uint64_t* __restrict__ slots, const psk::TableDesc* __restrict__ tdesc,
                     const unsigned long long* __restrict__ count, const uint64_t* __restrict__ cap, psk::LruMeta meta,
-                    Leaf* __restrict__ leafbuf, uint32_t* __restrict__ nleaf) {
+                    const uint32_t* __restrict__ slow, Leaf* __restrict__ leafbuf, uint32_t* __restrict__ nleaf) {
   const uint32_t i = blockIdx.y;
-  if (count[i] <= cap[i]) return;  // block-uniform
+  if (!slow[i] || count[i] <= cap[i]) return;  // block-uniform
   const psk::TableDesc d = tdesc[i];
   const uint64_t nslots = (uint64_t)d.nbkt * psk::kBucketSlots;
   const uint64_t stride = (uint64_t)gridDim.x * kCollectThreads;
@@ -746,7 +1191,8 @@ leaf_collect_kernel(const uint64_t* __restrict__ slots, const psk::TableDesc* __
 
 __global__ void __launch_bounds__(kEvictThreads)
 evict_kernel(uint64_t* slots, unsigned long long* count, const uint64_t* __restrict__ cap, psk::LruMeta meta,
-             const Leaf* __restrict__ leafbuf, const uint32_t* __restrict__ nleaf, uint32_t* more, uint32_t* err) {
+             const uint32_t* __restrict__ slow, const Leaf* __restrict__ leafbuf, const uint32_t* __restrict__ nleaf,
+             uint32_t* more, uint32_t* err) {
   extern __shared__ __align__(16) unsigned char ev_smem[];
   __shared__ EvictFlags flags;
   Leaf* leaves = reinterpret_cast<Leaf*>(ev_smem);
@@ -757,7 +1203,7 @@ evict_kernel(uint64_t* slots, unsigned long long* count, const uint64_t* __restr
   Leaf* heap = reinterpret_cast<Leaf*>(ev_smem + kOffHeap);
   const uint32_t i = blockIdx.x;
   const unsigned long long cnt = count[i];
-  if (cnt <= cap[i]) return;  // block-uniform
+  if (!slow[i] || cnt <= cap[i]) return;  // block-uniform
   // an earlier round gave up: no more rounds (read once, so that the whole block leaves together)
   if (__syncthreads_or(threadIdx.x == 0 && (*(volatile uint32_t*)err & psk::kErrTimeout) != 0u)) return;
   const uint32_t n = nleaf[i];
@@ -848,7 +1294,7 @@ evict_kernel(uint64_t* slots, unsigned long long* count, const uint64_t* __restr
       }
     }
     count[i] = cnt - evicted;
-    if (evicted > 0 && cnt - evicted > cap[i]) atomicOr(more, 1u);
+    if (evicted > 0 && cnt - evicted > cap[i]) atomicOr(more, kMoreSlow);
     psk::st_release_cta_shared_u32(&flags.exit, 1u);
   }
   __syncwarp();
@@ -944,28 +1390,56 @@ cudaError_t launch_advance(psk::StateSoA st, uint32_t I, const psk::ReqStore& rq
 }
 
 cudaError_t launch_evict(uint64_t* slots, const psk::TableDesc* tdesc, uint32_t I, unsigned long long* count,
-                         const uint64_t* cap, psk::LruMeta meta, void* leafbuf, uint32_t* nleaf, uint32_t* more,
-                         uint32_t* more_host, uint64_t max_instance_slots, uint32_t* err, cudaStream_t s) {
+                         const uint64_t* cap, psk::LruMeta meta, const EvictScratch& sc, uint32_t* more_host,
+                         uint64_t max_instance_slots, uint32_t max_use, uint32_t* err, int num_sms, cudaStream_t s) {
   const size_t smem = kEvictSmem;
   cudaError_t e = cudaFuncSetAttribute(evict_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(evict_order_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(OrderSmem));
   if (e != cudaSuccess) return e;
+  EvictPlan* plan = static_cast<EvictPlan*>(sc.plan);
+  const uint64_t chunks = (max_instance_slots + kScanChunk - 1) / kScanChunk;
+  const unsigned scan_grid = (unsigned)num_sms * 4u;
+  const unsigned inst_grid = I < (uint32_t)num_sms ? I : (unsigned)num_sms;
+  // histogram passes until a bin is one last_use value
+  int passes = 1;
+  for (uint64_t v = (uint64_t)max_use >> kHistBits; v; v >>= kHistBits) ++passes;
   const uint64_t per_block = (uint64_t)kCollectThreads * kCollectSlotsPerThread;
   const unsigned gx = (unsigned)((max_instance_slots + per_block - 1) / per_block);
-  for (int round = 0; round < 4096; ++round) {
-    if ((e = cudaMemsetAsync(nleaf, 0, (size_t)I * sizeof(uint32_t), s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(more, 0, sizeof(uint32_t), s)) != cudaSuccess) return e;
-    leaf_collect_kernel<<<dim3(gx ? gx : 1u, I), kCollectThreads, 0, s>>>(slots, tdesc, count, cap, meta,
-                                                                           static_cast<Leaf*>(leafbuf), nleaf);
+  if ((e = cudaMemsetAsync(sc.slow, 0, (size_t)I * sizeof(uint32_t), s)) != cudaSuccess) return e;
+  uint32_t todo = kMoreFast;
+  for (int round = 0; round < 4096 && todo; ++round) {
+    if ((e = cudaMemsetAsync(sc.more, 0, sizeof(uint32_t), s)) != cudaSuccess) return e;
+    if (todo & kMoreFast) {
+      evict_list_kernel<<<1, 1024, 0, s>>>(I, count, cap, sc.slow, max_use, plan, sc.list, sc.list + I);
+      for (int pass = 0; pass < passes; ++pass) {
+        evict_hist_kernel<<<scan_grid, kScanThreads, 0, s>>>(slots, tdesc, meta, plan, sc.list, sc.list + I, chunks,
+                                                            sc.hist, pass == 0);
+        evict_choose_kernel<<<inst_grid, 256, 0, s>>>(plan, sc.list, sc.list + I, sc.hist);
+      }
+      evict_gather_kernel<<<scan_grid, kScanThreads, 0, s>>>(slots, tdesc, meta, plan, sc.list, sc.list + I, chunks,
+                                                            sc.cand);
+      evict_order_kernel<<<inst_grid, kOrderThreads, sizeof(OrderSmem), s>>>(
+          slots, count, cap, meta, plan, sc.list, sc.list + I, sc.cand, sc.slow, sc.more, (uint32_t)kLeafMax, err);
+    }
+    if (todo & kMoreSlow) {
+      if ((e = cudaMemsetAsync(sc.nleaf, 0, (size_t)I * sizeof(uint32_t), s)) != cudaSuccess) return e;
+      leaf_collect_kernel<<<dim3(gx ? gx : 1u, I), kCollectThreads, 0, s>>>(
+          slots, tdesc, count, cap, meta, sc.slow, static_cast<Leaf*>(sc.leafbuf), sc.nleaf);
+      evict_kernel<<<I, kEvictThreads, smem, s>>>(slots, count, cap, meta, sc.slow, static_cast<const Leaf*>(sc.leafbuf),
+                                                  sc.nleaf, sc.more, err);
+    }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    evict_kernel<<<I, kEvictThreads, smem, s>>>(slots, count, cap, meta, static_cast<const Leaf*>(leafbuf), nleaf,
-                                                more, err);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = cudaMemcpyAsync(more_host, more, sizeof(uint32_t), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
+    if ((e = cudaMemcpyAsync(more_host, sc.more, sizeof(uint32_t), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
-    if (*more_host == 0u) break;
+    todo = *more_host;
   }
   return cudaSuccess;
 }
+
+size_t evict_plan_bytes(uint32_t I) { return (size_t)I * sizeof(EvictPlan); }
+size_t evict_hist_words(uint32_t I) { return (size_t)I * kHistBins; }
+size_t evict_cand_words(uint32_t I) { return (size_t)I * 2u * kClassMax; }
 
 size_t evict_leafbuf_bytes(uint32_t I) { return (size_t)I * kLeafMax * sizeof(Leaf); }
 
