@@ -350,8 +350,8 @@ ps_status run_probe_and_score(ps_ctx* c, const psk::WindowDev& wd, ps_scores* ou
   PS_TRY_CUDA(c, cudaMemsetAsync(c->d_stats, 0, kNumStats * sizeof(unsigned long long), c->stream));
   record(c, kEvProbe0);
   // window relations first: the probe derives the rows of requests that extend an earlier request
-  PS_TRY_CUDA(c, pskl::launch_relations(wd, c->model, c->d_lastslot, c->lastslot_n, c->d_rows, c->scratch, c->num_sms,
-                                        c->stream));
+  PS_TRY_CUDA(c, pskl::launch_relations(wd, c->model, c->d_lastslot, c->lastslot_n, c->d_rows, c->scratch, c->search,
+                                        c->num_sms, c->stream));
   record(c, kEvRelDone);
   PS_TRY_CUDA(c, pskl::launch_probe(c->d_slots, c->d_ovf, c->d_tdesc, c->I, wd, c->d_rows, c->scratch, hits, c->d_tpf,
                                     c->model, c->probe_grid, c->search, c->d_stats, c->ev[kEvProbeMid], c->stream));
@@ -862,15 +862,9 @@ ps_status ps_schedule_window(ps_ctx* c, const ps_window* w, ps_decisions* out, p
   s = run_probe_and_score(c, wd, opt_scores, &hit0);
   if (s != PS_OK) return s;
   record(c, kEvGreedy0);
-  if (c->search) {
-    PS_TRY_CUDA(c, pskl::launch_greedy_search(c->d_rows, wd, c->I, hit0, c->d_tpf, c->st, c->pend, c->model, c->d_delta,
-                                              c->delta_nslots, c->d_assign, c->d_dpath, c->d_hchosen, c->d_err,
-                                              c->gsync, c->stream));
-  } else {
-    PS_TRY_CUDA(c, pskl::launch_greedy(c->d_slots, c->d_ovf, c->d_tdesc, c->I, wd, hit0, c->st, c->pend, c->model,
-                                       c->d_delta, c->delta_nslots, c->d_assign, c->d_dpath, c->d_hchosen, c->d_err,
-                                       0, c->stream));
-  }
+  PS_TRY_CUDA(c, pskl::launch_greedy(c->d_rows, wd, c->I, hit0, c->d_tpf, c->st, c->pend, c->model, c->d_delta,
+                                     c->delta_nslots, c->d_assign, c->d_dpath, c->d_hchosen, c->d_err, c->gsync,
+                                     c->search, c->d_slots, c->d_ovf, c->d_tdesc, c->stream));
   record(c, kEvGreedy1);
   c->ev_used[2] = true;
   PS_TRY_CUDA(c, pskl::launch_delta_clear(c->d_delta, c->delta_nslots, c->stream));

@@ -1,336 +1,49 @@
 // Greedy in-window assignment (Algorithm 1 applied to the window's requests in arrival order).
 //
 // The paper's gateway decides each request online and updates the instance records along the
-// request path before the next decision (Section 4, Metadata service; Section 7).  Two kernels
-// replay that sequence for a whole window on the GPU:
-//   greedy_kernel       any cache (the probe's linear mode), described here;
-//   greedy_pipe_kernel  prefix-closed caches (the search mode), a pipelined cooperative launch of
-//                       deciding, insert, probe and summary blocks, described at its section below.
-// greedy_kernel is one persistent thread block whose threads each own up to IPT instances.  Per
-// request r:
-//   1. hit of r on instance i = hit0[r][i] (the probe kernel's result on the committed tables)
-//      extended through the window's delta table: an instance that has received blocks in this
-//      window is re-probed at position hit0, and if that block is now cached a warp finds the new
-//      first miss over delta and main (linear walk, or 32-ary search on prefix-closed caches: the
-//      delta only ever adds a chain's continuation to a cached prefix, so closure is kept).
-//      Instances untouched in the window need no probe.
-//   2. the whole row is re-evaluated from the current state (capacity guard, W, W_min, Eq. 8
-//      filter, TPOT/TTFT admission, D-C-Q key or LMetric fallback), reduced block-wide to the pick;
-//   3. the pick's state is updated (qr += 1, q += n, S += L) and its uncached blocks
-//      chain[h..nb) are inserted into the delta table for instance j.
-// The next request's row constants, hit row and the chain blocks at its hit positions are loaded
-// while the current request is decided, so a step starts with its inputs in registers.
-// Committed tables are never written here; the decisions and the updated state are a pending
-// window that ps_commit_window applies.  No step waits on another block: a single thread block with
-// __syncthreads barriers only.
+// request path before the next decision (Section 4, Metadata service; Section 7).  greedy_pipe_kernel
+// replays that sequence for a whole window on the GPU: a pipelined cooperative launch of one deciding
+// block, insert blocks and probe blocks.  Committed tables are never written here; the decisions and
+// the updated state are a pending window that ps_commit_window applies.
 #include "ps_internal.cuh"
 
 namespace {
 
-struct RowIn {
-  uint64_t o, nb;
-  uint32_t L;
-  float ttft_t, tpot_t;
-};
-
-__device__ __forceinline__ RowIn load_row(const psk::WindowDev& w, uint32_t r) {
-  RowIn x;
-  x.o = w.off[r];
-  x.nb = w.off[r + 1] - x.o;
-  x.L = w.L[r];
-  x.ttft_t = w.ttft_t[r];
-  x.tpot_t = w.tpot_t[r];
-  return x;
-}
-
-// Block-wide reductions without an extra barrier: after the per-warp partials are in shared
-// memory (and one __syncthreads), every warp reduces the (up to 32) partials with shuffles.
-__device__ __forceinline__ void cross_warp_min_any(const float* s_w, const int* s_a, int nw, float& wmin,
-                                                   bool& anyA) {
-  const int lane = threadIdx.x & 31;
-  const float v = lane < nw ? s_w[lane] : INFINITY;
-  const bool a = lane < nw ? (s_a[lane] != 0) : false;
-  wmin = psk::warp_fmin(v);
-  anyA = __any_sync(0xffffffffu, a);
-}
-
-// Per-warp (key, tie) partials -> the block's minimum, reduced by every warp.
-__device__ __forceinline__ void cross_warp_pick(const uint4* s_k, int nw, uint64_t* key, uint32_t* tie) {
-  const int lane = threadIdx.x & 31;
-  const uint4 pk = lane < nw ? s_k[lane] : make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0u);
-  uint32_t h;
-  psk::warp_pick_min(((uint64_t)pk.y << 32) | pk.x, pk.z, pk.w, key, tie, &h);
-}
-
-template <int IPT, bool SEARCH>
-__global__ void __launch_bounds__(1024, 1)
-greedy_kernel(const uint64_t* __restrict__ slots, const uint64_t* __restrict__ ovf,
-              const psk::TableDesc* __restrict__ tdesc, uint32_t I,
-              psk::WindowDev w, const uint32_t* __restrict__ hit0, psk::StateSoA committed,
-              psk::StateSoA pending, psk::DevModel m, psk::DeltaSlot* delta, uint64_t delta_nslots,
-              int32_t* __restrict__ assign, uint8_t* __restrict__ path, uint32_t* __restrict__ hit_chosen,
-              uint32_t* err) {
-  extern __shared__ unsigned long long smem_raw[];
-  int64_t* s_q = reinterpret_cast<int64_t*>(smem_raw);
-  int64_t* s_S = s_q + I;
-  int64_t* s_M = s_S + I;
-  int32_t* s_b = reinterpret_cast<int32_t*>(s_M + I);
-  int32_t* s_qr = s_b + I;
-  int32_t* s_Bmax = s_qr + I;
-  uint32_t* s_h = reinterpret_cast<uint32_t*>(s_Bmax + I);
-  uint32_t* s_walk = s_h + I;
-  uint32_t* s_end = s_walk + I;  // chain end of the last request assigned to the instance this window
-  psk::InstTerms* s_it = reinterpret_cast<psk::InstTerms*>(s_end + I);
-  uint8_t* s_touched = reinterpret_cast<uint8_t*>(s_it + I);
-  __shared__ float s_red_w[32];
-  __shared__ int s_red_a[32];
-  __shared__ uint4 s_red_k[32];
-  __shared__ uint32_t s_nwalk;
-
-  const int t = threadIdx.x;
-  const int NT = blockDim.x;
-  const int lane = t & 31;
-  const int warp = t >> 5;
-  const int NW = NT >> 5;
-
-  for (uint32_t i = t; i < I; i += NT) {
-    s_b[i] = committed.b[i];
-    s_qr[i] = committed.qr[i];
-    s_q[i] = committed.q[i];
-    s_S[i] = committed.S[i];
-    s_M[i] = committed.M[i];
-    s_Bmax[i] = committed.Bmax[i];
-    s_end[i] = 0;
-    s_touched[i] = 0;
-    s_it[i] = psk::inst_terms(m, s_b[i], s_qr[i], s_q[i], s_Bmax[i]);
-  }
-  if (t == 0) s_nwalk = 0;
-  // Inputs of the next request: row constants, hit row, chain block at each hit position.
-  RowIn nx{};
-  uint32_t hn[IPT];
-  uint64_t cn[IPT];
-  if (w.R > 0) nx = load_row(w, 0);
-#pragma unroll
-  for (int k = 0; k < IPT; ++k) {
-    const uint32_t i = t + k * NT;
-    hn[k] = (i < I && w.R > 0) ? __ldg(hit0 + i) : 0u;
-    cn[k] = (i < I && hn[k] < nx.nb) ? w.hash[nx.o + hn[k]] : 0ull;
-  }
-  __syncthreads();
-
-  for (uint32_t r = 0; r < w.R; ++r) {
-    const RowIn cur = nx;
-    const uint64_t o = cur.o;
-    const uint64_t nb = cur.nb;
-    const psk::RowConst rc = psk::row_const(m, cur.L, cur.ttft_t, cur.tpot_t);
-    uint32_t hc[IPT];
-#pragma unroll
-    for (int k = 0; k < IPT; ++k) {
-      const uint32_t i = t + k * NT;
-      hc[k] = hn[k];
-      if (i < I) {
-        if (s_touched[i] && hc[k] < nb && psk::delta_contains(delta, delta_nslots, i, cn[k])) {
-          const uint32_t at = atomicAdd(&s_nwalk, 1u);
-          s_walk[at] = i;
-        }
-        s_h[i] = hc[k];
-      }
-    }
-    // first half of the prefetch: row constants and hit row of request r + 1
-    const bool more = r + 1 < w.R;
-    if (more) {
-      nx = load_row(w, r + 1);
-#pragma unroll
-      for (int k = 0; k < IPT; ++k) {
-        const uint32_t i = t + k * NT;
-        if (i < I) hn[k] = __ldg(hit0 + (uint64_t)(r + 1) * I + i);
-      }
-    }
-    __syncthreads();  // (A) hits staged, walk list complete
-    const uint32_t nwalk = s_nwalk;
-    if (nwalk) {
-      for (uint32_t x = warp; x < nwalk; x += NW) {
-        const uint32_t i = s_walk[x];
-        const psk::TableDesc d = tdesc[i];
-        // Positions past hit0 are never in a prefix-closed main table (hit0 is its first miss), so
-        // the search only consults the delta; the linear walk checks both.
-        auto cached = [&](uint64_t k) {
-          const uint64_t key = w.hash[o + k];
-          return psk::delta_contains(delta, delta_nslots, i, key) ||
-                 (!SEARCH && psk::main_contains(slots, ovf, d, key));
-        };
-        // Likely answer: where the last request assigned to i in this window ended (the same
-        // session's previous step usually ends exactly there).
-        const uint64_t from = (uint64_t)s_h[i] + 1;
-        const uint64_t hnew = SEARCH ? psk::warp_first_miss_search_hint(from, nb, s_end[i], cached)
-                                     : psk::warp_first_miss_linear(from, nb, cached);
-        if (lane == 0) s_h[i] = (uint32_t)hnew;
-      }
-      __syncthreads();  // (B) extended hits visible
-#pragma unroll
-      for (int k = 0; k < IPT; ++k) {
-        const uint32_t i = t + k * NT;
-        if (i < I) hc[k] = s_h[i];
-      }
-    }
-    // Pass 1: capacity guard and recompute cost; W_min over A.
-    psk::PairEval ev[IPT];
-    float wmin = INFINITY;
-    bool anyA = false;
-#pragma unroll
-    for (int k = 0; k < IPT; ++k) {
-      const uint32_t i = t + k * NT;
-      if (i < I) {
-        ev[k] = psk::eval_pair_terms(m, rc, hc[k], s_it[i], s_q[i], s_S[i], s_M[i]);
-        if (ev[k].inA) {
-          wmin = fminf(wmin, ev[k].W);
-          anyA = true;
-        }
-      } else {
-        ev[k].inA = false;
-      }
-    }
-    wmin = psk::warp_fmin(wmin);
-    anyA = __any_sync(0xffffffffu, anyA);
-    if (lane == 0) {
-      s_red_w[warp] = wmin;
-      s_red_a[warp] = anyA ? 1 : 0;
-    }
-    __syncthreads();  // (C)
-    cross_warp_min_any(s_red_w, s_red_a, NW, wmin, anyA);
-    // second half of the prefetch: chain blocks of request r + 1 at its hit positions
-    if (more) {
-#pragma unroll
-      for (int k = 0; k < IPT; ++k) {
-        const uint32_t i = t + k * NT;
-        if (i < I && hn[k] < nx.nb) cn[k] = w.hash[nx.o + hn[k]];
-      }
-    }
-    // Pass 2: admission classes and the packed (class, value) key with its tie word.
-    uint64_t bkey = psk::kNoKey;
-    uint32_t btie = 0xFFFFFFFFu;
-#pragma unroll
-    for (int k = 0; k < IPT; ++k) {
-      const uint32_t i = t + k * NT;
-      if (i < I && ev[k].inA) {
-        const uint32_t cls = psk::pair_class(m, rc, ev[k], wmin);
-        if (cls <= 1u) {
-          uint64_t key;
-          uint32_t tie = i;
-          if (cls == 0u) {
-            key = psk::packed_key(0u, psk::value_in_t(m, psk::key0_bits(m, s_b[i], s_qr[i]), hc[k], ev[k].tpot,
-                                                      rc.tpot_target));
-            tie = psk::tie_in_t(m, i, s_qr[i]);
-          } else {
-            const int32_t Bp = s_b[i] + s_qr[i] + 1;
-            key = psk::packed_key(1u, psk::value_fallback(m, (uint64_t)(s_q[i] + ev[k].n), (uint32_t)Bp,
-                                                          psk::dcq_key0(s_b[i], s_qr[i]), hc[k]));
-          }
-          if (key < bkey || (key == bkey && tie < btie)) {
-            bkey = key;
-            btie = tie;
-          }
-        }
-      }
-    }
-    {
-      uint64_t wk;
-      uint32_t wt, wh;
-      psk::warp_pick_min(bkey, btie, 0u, &wk, &wt, &wh);
-      if (lane == 0) s_red_k[warp] = make_uint4((uint32_t)wk, (uint32_t)(wk >> 32), wt, 0u);
-    }
-    __syncthreads();  // (D)
-    uint64_t bk;
-    uint32_t bt;
-    cross_warp_pick(s_red_k, NW, &bk, &bt);
-    const bool pick = anyA && bk != psk::kNoKey;
-    const uint32_t j = bt & psk::kTieInstMask;
-    const uint32_t hj = pick ? s_h[j] : 0u;
-    if (t == 0) {
-      assign[r] = pick ? (int32_t)j : -1;
-      path[r] = pick ? (uint8_t)(bk >> 62) : (uint8_t)2;
-      hit_chosen[r] = hj;
-      if (pick) {
-        s_qr[j] += 1;
-        s_q[j] += (int64_t)rc.L - 16 * (int64_t)hj;
-        s_S[j] += (int64_t)rc.L;
-        s_end[j] = (uint32_t)nb;
-        s_touched[j] = 1;
-        s_it[j] = psk::inst_terms(m, s_b[j], s_qr[j], s_q[j], s_Bmax[j]);
-      }
-      s_nwalk = 0;
-    }
-    if (pick) {
-      for (uint64_t k = (uint64_t)hj + t; k < nb; k += NT)
-        if (!psk::delta_insert(delta, delta_nslots, j, w.hash[o + k])) atomicOr(err, psk::kErrDeltaFull);
-    }
-    __syncthreads();  // (E) state, delta and walk counter ready for the next request
-  }
-  for (uint32_t i = t; i < I; i += NT) {
-    pending.b[i] = s_b[i];
-    pending.qr[i] = s_qr[i];
-    pending.q[i] = s_q[i];
-    pending.S[i] = s_S[i];
-    pending.M[i] = s_M[i];
-    pending.Bmax[i] = s_Bmax[i];
-  }
-}
-
-size_t greedy_smem(uint32_t I) {
-  return (size_t)I * (3 * sizeof(int64_t) + 3 * sizeof(int32_t) + 3 * sizeof(uint32_t) + sizeof(psk::InstTerms) + 1) + 16;
-}
-
-template <int IPT, bool SEARCH>
-cudaError_t greedy_launch(const uint64_t* slots, const uint64_t* ovf, const psk::TableDesc* tdesc, uint32_t I,
-                          const psk::WindowDev& w, const uint32_t* hit0, psk::StateSoA committed,
-                          psk::StateSoA pending, const psk::DevModel& m, psk::DeltaSlot* delta,
-                          uint64_t delta_nslots, int32_t* assign, uint8_t* path, uint32_t* hit_chosen,
-                          uint32_t* err, uint32_t nt, cudaStream_t s) {
-  const size_t smem = greedy_smem(I);
-  cudaError_t e = cudaFuncSetAttribute(greedy_kernel<IPT, SEARCH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
-  if (e != cudaSuccess) return e;
-  greedy_kernel<IPT, SEARCH><<<1, nt, smem, s>>>(slots, ovf, tdesc, I, w, hit0, committed, pending, m, delta,
-                                                 delta_nslots, assign, path, hit_chosen, err);
-  return cudaGetLastError();
-}
-
-
 // ----------------------------------------------------------------------------------------------
-// Prefix-closed caches (the probe's search mode): a pipelined greedy pass over four kinds of
-// thread block in one cooperative launch.
+// The hit of a request is the first chain position not cached.  Chained block hashes make "block k
+// equal" stand for "blocks 0..k equal", and an earlier request of the window has its whole chain cached
+// on its instance, so with
+//     M(s, i) = max lcp(s, t) over the earlier requests t of the window that went to i
+// every position below M is cached on i while request s is decided, and from M on only the committed
+// table counts:
+//     hit(s, i) = hit0(s, i) if M <= hit0, else the first miss of main_i at or after M,
+// which on a prefix-closed cache (the probe's search mode) is M itself.  Requests up to s - kLag count
+// through the window's delta table, the later ones through their common prefixes with s (from the
+// relations pass).
 //
-// On a prefix-closed cache the hit of a request is the first chain position not cached, and the
-// union of prefix-closed sets has as first miss the largest of the sets' first misses.  The
-// cached set of instance i while request s is decided is main_i plus the chains of the window's
-// earlier requests assigned to i, so
-//     hit(s, i) = max( first miss of main_i + delta_i(<= s - kLag),
-//                      lcp(s, s - d) for each d = 1..kLag-1 such that request s - d went to i )
-// where delta_i(<= s - kLag) holds the blocks inserted for requests up to s - kLag and lcp(s, s - d) is
-// the common chain prefix (from the relations pass).
-//
-//   Deciding block (block 0).  A feeder warp stages each row's summary, row constants and probed
-//   hits in shared memory; the deciding warp decides the requests in arrival order from the
-//   summaries, correcting them for the last kSpecLag picks (the lag-d speculation below), updates
-//   the pick's state and publishes each decision as an insert job.  No table access is on its
-//   per-request path.
+//   Deciding block (block 0).  Decides the requests in arrival order and publishes each decision as a
+//   job (described at its section below).  No table access is on its per-request path, except where a
+//   cache is not prefix-closed (LIN) and a hit rises past hit0.
 //   Insert blocks.  Groups of kInsertGroup blocks take the jobs round-robin; a group's members split
-//   each job's chain blocks chain[h, nb) between them, insert them into delta_j and count the job done.
+//   each job's chain blocks between them, insert them into the delta table for the job's instance and
+//   count the job done.  On prefix-closed caches the blocks chain[h, nb) do; else the whole chain goes
+//   in, so that "block k of s is in the table for i" is exactly k < M and can be searched.
 //   Probe blocks.  Take the rows round-robin.  For row s they wait until the jobs <= s - kLag are
 //   done, replay those jobs (which instances have window inserts, where their last chain ended,
 //   which instances took s's ancestors), then per instance start from hit0, raise the position to
 //   the end of an ancestor's chain on the instance that took it (its chain is a prefix of s's, and
 //   its inserts are in), probe the delta table there when the instance has window inserts, hand the
-//   instances whose block is present to a warp search over the delta, and release the row's ready
-//   flag.  The main table is never probed here: positions past hit0 are absent from a
-//   prefix-closed main table.  Inserts of requests s - kLag + 1 .. s - 1 may land while a probe
-//   runs, in any order: any snapshot between delta(<= s - kLag) and delta(<= s - 1) gives a first
-//   miss between the two sets' first misses, and the max with the lcp terms is exact all the same.
-//   Summary blocks.  Take the rows round-robin; evaluate row s on every instance against the state
-//   before decision s - kSpecLag and publish its summary (below).
+//   instances whose block is present to a warp search over the delta (LIN: then a walk of the main
+//   table), and release the row's ready flag.  On prefix-closed caches the main table is never probed
+//   here: positions past hit0 are absent from it.  Inserts of requests s - kLag + 1 .. s - 1 may land
+//   while a probe runs, in any order: any snapshot between delta(<= s - kLag) and delta(<= s - 1)
+//   gives a position between the two sets' M, and the later requests' common prefixes make it exact.
 // Every cross-block wait is bounded (GreedySync::wait_ns, 1 s unless the caller set another limit);
-// on expiry the waiter records PS_ERR_TIMEOUT and stops waiting, so the launch always ends.  Each
-// role keeps the instance state it needs in its own shared memory.
+// on expiry the waiter records PS_ERR_TIMEOUT and stops waiting, so the launch always ends.
+//
+// Caches that are not prefix-closed took a kernel of their own before: one block that walked delta and
+// main 32 blocks a step on every instance whose hit rose, 50 us a decision (100 x 300: 15.2 ms of greedy
+// pass, 0.46 here).
 
 constexpr uint32_t kInsertBlocks = 64;  // insert blocks
 constexpr uint32_t kProbeBlocks = 64;   // probe blocks
@@ -396,6 +109,22 @@ constexpr uint32_t kInsertGroup = 4;
 constexpr int kInsertBatch = 4;
 static_assert(kInsertBlocks % kInsertGroup == 0, "whole insert groups");
 
+// The committed tables, for caches that are not prefix-closed.
+struct MainTables {
+  const uint64_t* slots;
+  const uint64_t* ovf;
+  const psk::TableDesc* tdesc;
+};
+
+// First position in [from, nb) of a chain that instance i's committed table does not hold (a warp).
+__device__ __noinline__ uint64_t main_first_miss(const MainTables& mt, uint32_t i, const uint64_t* chain, uint64_t from,
+                                                 uint64_t nb) {
+  const psk::TableDesc d = mt.tdesc[i];
+  return psk::warp_first_miss_linear(
+      from, nb, [&](uint64_t k) { return psk::main_contains(mt.slots, mt.ovf, d, __ldg(chain + k)); });
+}
+
+template <bool LIN>
 __device__ __forceinline__ void insert_tail(psk::DeltaSlot* delta, uint64_t nslots, uint32_t j,
                                             const uint64_t* __restrict__ chain, uint64_t first, uint64_t nb,
                                             uint64_t stride, uint32_t* err) {
@@ -420,6 +149,8 @@ __device__ __forceinline__ void insert_tail(psk::DeltaSlot* delta, uint64_t nslo
       if (key[q] == psk::kEmpty || key[q] == psk::kTomb) continue;
       if (old[q] == psk::kEmpty) {
         __stcg(&delta[slot[q]].tag, j + 1);
+      } else if (LIN && psk::delta_contains_from(delta, nslots, j, key[q], slot[q])) {
+        // another request of the window with this prefix brought the block to the instance before
       } else if (!psk::delta_insert_from(delta, nslots, j, key[q], psk::delta_next(slot[q], nslots))) {
         atomicOr(err, psk::kErrDeltaFull);
       }
@@ -427,6 +158,7 @@ __device__ __forceinline__ void insert_tail(psk::DeltaSlot* delta, uint64_t nslo
   }
 }
 
+template <bool LIN>
 __device__ void insert_blocks(const psk::RowPre* __restrict__ rows, const uint64_t* __restrict__ hash, uint32_t R,
                               psk::DeltaSlot* delta, uint64_t nslots, uint32_t* err, const psk::GreedySync& sync,
                               uint32_t ib, uint32_t ninsert) {
@@ -445,8 +177,8 @@ __device__ void insert_blocks(const psk::RowPre* __restrict__ rows, const uint64
     if (j != 0xFFFFFFFFu && job + psk::kLag < R) {
       const uint64_t off = __ldg(&rows[job].off);
       const uint32_t nb = __ldg(&rows[job].nb);
-      insert_tail(delta, nslots, j, hash + off, (uint64_t)hj + member * blockDim.x + t, nb,
-                  (uint64_t)kInsertGroup * blockDim.x, err);
+      insert_tail<LIN>(delta, nslots, j, hash + off, (LIN ? 0u : (uint64_t)hj) + member * blockDim.x + t, nb,
+                       (uint64_t)kInsertGroup * blockDim.x, err);
     }
     __syncthreads();
     if (t == 0) {
@@ -462,11 +194,12 @@ __device__ void insert_blocks(const psk::RowPre* __restrict__ rows, const uint64
 // row's ancestors), the hit0 row, the probe positions and the chain blocks there.  Only then does the
 // block wait until those jobs' inserts are done, so after the wait one delta lookup per instance
 // (and, rarely, a warp search) is left before the row is released.
-template <int IPT>
+template <int IPT, bool LIN>
 __device__ void probe_rows(const psk::RowPre* __restrict__ rows, const uint64_t* __restrict__ hash, uint32_t R,
                            uint32_t I, const uint32_t* __restrict__ hit0, const float* __restrict__ tpf0,
                            const psk::DevModel& m, const psk::DeltaSlot* delta, uint64_t nslots, uint32_t* err,
-                           const psk::GreedySync& sync, unsigned long long* smem_raw, uint32_t pb, uint32_t nprobe) {
+                           const psk::GreedySync& sync, unsigned long long* smem_raw, uint32_t pb, uint32_t nprobe,
+                           const MainTables& mt) {
   uint32_t* s_end = reinterpret_cast<uint32_t*>(smem_raw);  // chain end of the last job on i (0 = none)
   uint32_t* s_res = s_end + I;                               // search start / result per instance
   uint32_t* s_walk = s_res + I;                              // instances handed to a warp search
@@ -584,7 +317,7 @@ __device__ void probe_rows(const psk::RowPre* __restrict__ rows, const uint64_t*
 #pragma unroll
     for (int k = 0; k < IPT; ++k) {
       const uint32_t i = t + k * NT;
-      if (probe[k] && psk::delta_contains(delta, nslots, i, key[k])) {
+      if ((probe[k] && psk::delta_contains(delta, nslots, i, key[k])) || (LIN && i < I && pos[k] > h0[k])) {
         walk[k] = true;
         s_res[i] = pos[k];
         s_walk[atomicAdd(&s_nwalk, 1u)] = i;
@@ -596,7 +329,14 @@ __device__ void probe_rows(const psk::RowPre* __restrict__ rows, const uint64_t*
       for (uint32_t x = warp; x < nwalk; x += NW) {
         const uint32_t i = s_walk[x];
         auto cached = [&](uint64_t k) { return k < nb && psk::delta_contains(delta, nslots, i, __ldg(hash + off + k)); };
-        const uint64_t hnew = psk::warp_first_miss_search_hint((uint64_t)s_res[i] + 1, nb, s_end[i], cached);
+        uint64_t hnew;
+        if (!LIN) {
+          hnew = psk::warp_first_miss_search_hint((uint64_t)s_res[i] + 1, nb, s_end[i], cached);
+        } else {
+          const uint64_t from = s_res[i], lim = __ldg(&rows[s].limit);
+          hnew = from < lim ? psk::warp_first_miss_search_hint(from, lim, s_end[i], cached) : lim;
+          hnew = main_first_miss(mt, i, hash + off, hnew, nb);
+        }
         __syncwarp();
         if (lane == 0) s_res[i] = (uint32_t)hnew;
       }
@@ -761,11 +501,11 @@ __device__ __forceinline__ StepRow step_row(const psk::DevModel& m, const psk::R
 
 using psk::wait_smem_at_least;
 
-template <int IPT, bool GEN>
+template <int IPT, bool GEN, bool LIN>
 __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, uint32_t I, psk::StateSoA committed,
                             psk::StateSoA pending, const psk::DevModel& m, int32_t* assign, uint8_t* __restrict__ path,
                             uint32_t* __restrict__ hit_chosen, uint32_t* err, const psk::GreedySync& sync,
-                            unsigned long long* smem_raw) {
+                            unsigned long long* smem_raw, const uint64_t* __restrict__ hash, const MainTables& mt) {
   const uint32_t Ip = sync.ring_stride;
   const InstSmem a = inst_smem(smem_raw, Ip);
   uint32_t* s_hitr = reinterpret_cast<uint32_t*>(a.pad + Ip);  // [kFeedRing][Ip] hits
@@ -829,6 +569,12 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
     return src;
   };
   auto rank_of = [&](uint32_t x) { return (uint32_t)lane < ncw ? s_rank[x & 1u][lane] : 0xFFFFFFFFu; };
+
+  // LIN: what the last pick's hit on this row rises to (0: it does not), called by its owner's warp.
+  auto extend = [&](const psk::RowPre& row, uint32_t j, uint32_t hj) {
+    const uint32_t l = min(row.lcp[0], row.limit);
+    return l > hj ? (uint32_t)main_first_miss(mt, j, hash + row.off, l, row.nb) : 0u;
+  };
 
   if (warp == kFeederWarp) {
     // Rows are staged as soon as they are probed, several at once when they are ready together (so the
@@ -909,10 +655,19 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
         uint32_t* hp = s_hitr + slot * Ip + (up ? pk : 0);
         bool rose = false;
         if (up) {
-          const uint32_t l = row.lcp[lane + 1];
+          const uint32_t l = LIN ? min(row.lcp[lane + 1], row.limit) : row.lcp[lane + 1];
           rose = atomicMax(hp, l) < l;
         }
         __syncwarp();
+        if (LIN) {  // on from the common prefix in the committed table
+          for (unsigned rm = __ballot_sync(0xffffffffu, rose); rm; rm &= rm - 1u) {
+            const uint32_t i = (uint32_t)__shfl_sync(0xffffffffu, pk, __ffs(rm) - 1);
+            const uint64_t hx = main_first_miss(mt, i, hash + row.off, s_hitr[slot * Ip + i], row.nb);
+            __syncwarp();
+            if (lane == 0) s_hitr[slot * Ip + i] = (uint32_t)hx;
+            __syncwarp();
+          }
+        }
         if (rose) s_tpfr[slot * Ip + pk] = __float_as_uint(psk::t_pf32(m, row.L, *hp));
         __syncwarp();
       }
@@ -1059,6 +814,8 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
         if (who & (who - 1u)) src = warp_argmin(er, s_key[par][held ? lane : 0], eth.x);  // equal ranks
         const uint32_t j = __shfl_sync(0xffffffffu, eth.x, src) & psk::kTieInstMask;
         const uint32_t H = __shfl_sync(0xffffffffu, eth.y, src);
+        uint32_t lj = l0;
+        if (LIN && j / (32u * IPT) == warp) lj = extend(row, j, s_hitr[slot * Ip + j]);
         if (j / IPT == t) {
           // its state takes request s - 1 (qr + 1, q + L - 16 H, S + L), and its hit rises to the common
           // prefix of the two requests
@@ -1077,7 +834,7 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
           const float f = psk::ema_factor(m, (int32_t)y.z);
           const float tqv =
               __fadd_rn(__fmul_rn(m.a0, __int2float_rn((int32_t)(y.x & 0x3FFFFu))), __fmul_rn(m.a1, __int2float_rn(x.x)));
-          hj = l0 > hj ? l0 : hj;
+          hj = lj > hj ? lj : hj;
           float Wj;
           uint64_t keyj;
           uint32_t rankj, tiej;
@@ -1204,12 +961,15 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
         stopped = true;
         break;
       }
-      const uint32_t slot = s % kFeedRing;
+      const uint32_t slot = (s < R ? s : R - 1) % kFeedRing;
       uint32_t own = 0xFFFFFFFFu;  // this thread's index of the last pick, if it owns it
+      uint32_t lj = 0;             // what its hit on this row rises to
       if (s > 0) {
         const int src = decision(s - 1, rank_of(s - 1));
         const uint2 th = s_th[(s - 1) & 1u][src < 0 ? 0 : src];
         const uint32_t j = th.x & psk::kTieInstMask;
+        lj = s_row[slot].lcp[0];
+        if (LIN && src >= 0 && j / (32u * IPT) == warp) lj = extend(s_row[slot], j, s_hitr[slot * Ip + j]);
         if (src >= 0 && j / IPT == t) {
           own = j - i0;
           const int32_t b = a.b[j], qr = a.qr[j] + 1;
@@ -1248,12 +1008,11 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
         for (int k = 0; k < IPT; ++k) h[k] = tb[k] = 0u;
       }
       if (own != 0xFFFFFFFFu) {  // the last pick also took request s - 1: its common prefix with this row
-        const uint32_t l = row.lcp[0];
-        const uint32_t tl = __float_as_uint(psk::t_pf32(m, rc.L, l));
+        const uint32_t tl = __float_as_uint(psk::t_pf32(m, rc.L, lj));
 #pragma unroll
         for (int k = 0; k < IPT; ++k)
-          if ((uint32_t)k == own && l > h[k]) {
-            h[k] = l;
+          if ((uint32_t)k == own && lj > h[k]) {
+            h[k] = lj;
             tb[k] = tl;
           }
       }
@@ -1358,21 +1117,21 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
   }
 }
 
-template <int IPT, bool GEN>
+template <int IPT, bool GEN, bool LIN>
 __global__ void __launch_bounds__(kPipeThreads, 1)
 greedy_pipe_kernel(const psk::RowPre* __restrict__ rows, const uint64_t* __restrict__ hash, uint32_t R, uint32_t I,
                    const uint32_t* __restrict__ hit0, const float* __restrict__ tpf0, psk::StateSoA committed,
                    psk::StateSoA pending, psk::DevModel m, psk::DeltaSlot* delta, uint64_t nslots, int32_t* assign,
                    uint8_t* __restrict__ path, uint32_t* __restrict__ hit_chosen, uint32_t* err, psk::GreedySync sync,
-                   uint32_t ninsert) {
+                   uint32_t ninsert, MainTables mt) {
   extern __shared__ __align__(16) unsigned long long smem_raw[];
   if (blockIdx.x == 0) {
-    decide_rows<IPT, GEN>(rows, R, I, committed, pending, m, assign, path, hit_chosen, err, sync, smem_raw);
+    decide_rows<IPT, GEN, LIN>(rows, R, I, committed, pending, m, assign, path, hit_chosen, err, sync, smem_raw, hash, mt);
   } else if (blockIdx.x <= ninsert) {
-    insert_blocks(rows, hash, R, delta, nslots, err, sync, blockIdx.x - 1, ninsert);
+    insert_blocks<LIN>(rows, hash, R, delta, nslots, err, sync, blockIdx.x - 1, ninsert);
   } else {
-    probe_rows<IPT>(rows, hash, R, I, hit0, tpf0, m, delta, nslots, err, sync, smem_raw, blockIdx.x - 1 - ninsert,
-                    gridDim.x - 1 - ninsert);
+    probe_rows<IPT, LIN>(rows, hash, R, I, hit0, tpf0, m, delta, nslots, err, sync, smem_raw, blockIdx.x - 1 - ninsert,
+                         gridDim.x - 1 - ninsert, mt);
   }
 }
 
@@ -1388,10 +1147,12 @@ template <int IPT>
 cudaError_t greedy_pipe_launch(const psk::RowPre* rows, const psk::WindowDev& w, uint32_t I, const uint32_t* hit0,
                                const float* tpf0, psk::StateSoA committed, psk::StateSoA pending, const psk::DevModel& m,
                                psk::DeltaSlot* delta, uint64_t nslots, int32_t* assign, uint8_t* path,
-                               uint32_t* hit_chosen, uint32_t* err, const psk::GreedySync& sync, cudaStream_t s) {
+                               uint32_t* hit_chosen, uint32_t* err, const psk::GreedySync& sync, bool linear,
+                               MainTables mt, cudaStream_t s) {
   // not Algorithm 1's order (Table 4 / Table 3 variants), or Eq. 9's interference term
   const bool gen = m.sel != psk::kSelDCQ || m.fb_dcq || m.interference_mode != 0;
-  auto kern = gen ? greedy_pipe_kernel<IPT, true> : greedy_pipe_kernel<IPT, false>;
+  auto kern = linear ? greedy_pipe_kernel<IPT, true, true>
+                     : (gen ? greedy_pipe_kernel<IPT, true, false> : greedy_pipe_kernel<IPT, false, false>);
   const size_t smem = greedy_pipe_smem(I, sync.ring_stride);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -1405,7 +1166,7 @@ cudaError_t greedy_pipe_launch(const psk::RowPre* rows, const psk::WindowDev& w,
   const uint32_t nprobe = R < kProbeBlocks ? R : kProbeBlocks;
   void* args[] = {(void*)&rows, (void*)&hash, (void*)&R, (void*)&I, (void*)&hit0, (void*)&tpf0, (void*)&c, (void*)&p,
                   (void*)&mm, (void*)&delta, (void*)&nslots, (void*)&assign, (void*)&path, (void*)&hit_chosen,
-                  (void*)&err, (void*)&sy, (void*)&ninsert};
+                  (void*)&err, (void*)&sy, (void*)&ninsert, (void*)&mt};
   // all blocks must be resident at once: they wait on one another
   return cudaLaunchCooperativeKernel((const void*)kern, dim3(1 + ninsert + nprobe), dim3(kPipeThreads), args, smem, s);
 }
@@ -1414,30 +1175,12 @@ cudaError_t greedy_pipe_launch(const psk::RowPre* rows, const psk::WindowDev& w,
 
 namespace pskl {
 
-cudaError_t launch_greedy(const uint64_t* slots, const uint64_t* ovf, const psk::TableDesc* tdesc, uint32_t I,
-                          const psk::WindowDev& w, const uint32_t* hit0, psk::StateSoA committed,
-                          psk::StateSoA pending, const psk::DevModel& m, psk::DeltaSlot* delta,
-                          uint64_t delta_nslots, int32_t* assign, uint8_t* path, uint32_t* hit_chosen,
-                          uint32_t* err, int search, cudaStream_t s) {
-  uint32_t nt = (I + 31) / 32 * 32;
-  if (nt > 1024) nt = 1024;
-  const uint32_t ipt = (I + nt - 1) / nt;
-#define PS_GREEDY(IPT)                                                                                         \
-  return search ? greedy_launch<IPT, true>(slots, ovf, tdesc, I, w, hit0, committed, pending, m, delta,        \
-                                           delta_nslots, assign, path, hit_chosen, err, nt, s)                   \
-                : greedy_launch<IPT, false>(slots, ovf, tdesc, I, w, hit0, committed, pending, m, delta,       \
-                                            delta_nslots, assign, path, hit_chosen, err, nt, s)
-  if (ipt <= 1) PS_GREEDY(1);
-  if (ipt <= 2) PS_GREEDY(2);
-  if (ipt <= 4) PS_GREEDY(4);
-#undef PS_GREEDY
-  return cudaErrorInvalidValue;
-}
-
-cudaError_t launch_greedy_search(const psk::RowPre* rows, const psk::WindowDev& w, uint32_t I, const uint32_t* hit0,
+cudaError_t launch_greedy(const psk::RowPre* rows, const psk::WindowDev& w, uint32_t I, const uint32_t* hit0,
                                  const float* tpf0, psk::StateSoA committed, psk::StateSoA pending, const psk::DevModel& m,
                                  psk::DeltaSlot* delta, uint64_t delta_nslots, int32_t* assign, uint8_t* path,
-                                 uint32_t* hit_chosen, uint32_t* err, const psk::GreedySync& sync, cudaStream_t s) {
+                                 uint32_t* hit_chosen, uint32_t* err, const psk::GreedySync& sync, int search,
+                          const uint64_t* slots, const uint64_t* ovf, const psk::TableDesc* tdesc, cudaStream_t s) {
+  const MainTables mt{slots, ovf, tdesc};
   if (w.R == 0) return cudaSuccess;
   cudaError_t e = cudaMemsetAsync(sync.done, 0, (size_t)w.R * sizeof(uint32_t), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(sync.ready, 0, (size_t)w.R * sizeof(uint32_t), s);
@@ -1450,11 +1193,10 @@ cudaError_t launch_greedy_search(const psk::RowPre* rows, const psk::WindowDev& 
   const uint32_t ipt = (I + 32u * kComputeWarps - 1) / (32u * kComputeWarps);
 #define PS_GREEDY_P(IPT)                                                                                      \
   return greedy_pipe_launch<IPT>(rows, w, I, hit0, tpf0, committed, pending, m, delta, delta_nslots, assign, path, \
-                                 hit_chosen, err, sync, s)
+                                 hit_chosen, err, sync, search == 0, mt, s)
   if (ipt <= 1) PS_GREEDY_P(1);
   if (ipt <= 2) PS_GREEDY_P(2);
   if (ipt <= 4) PS_GREEDY_P(4);
-  if (ipt <= 8) PS_GREEDY_P(8);
 #undef PS_GREEDY_P
   return cudaErrorInvalidValue;
 }

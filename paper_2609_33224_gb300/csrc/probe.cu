@@ -4,18 +4,17 @@
 // chain length if every block is cached): the cached prefix of the request on that instance, the
 // quantity the paper's scheduler reads from its prefix tree (Section 7) to estimate KVC reuse.
 //
-// One thread block per request (grid-stride over requests).  The request's chain is staged in
-// shared memory once (coalesced 8-byte loads) and reused by every instance's probe; positions past
-// the staging capacity are read from global memory (L1/L2-resident: the same block re-reads them).
-//   linear mode (any cache): each warp walks one instance at a time, 32 consecutive chain positions
-//     per step, __ballot_sync collecting the misses and __ffs finding the first.
+//   linear mode (any cache): a work item is (row, group of instances), one warp per instance, 64
+//     consecutive chain positions per step (two lookups per lane in flight), __ballot_sync collecting
+//     the misses and __ffs finding the first.
 //   search mode (prefix-closed caches, where "block k cached" is monotone along the chain): the
 //     rows without an earlier prefix in the window come as a list from the relations pass; a work
 //     item is (row, chunk of 256 instances), one lane per instance.  A lane first looks up the
 //     row's hint position and the one before it together: the hint is the shortest common prefix
 //     with the previous requests of the window, which on most instances is exactly the cached
 //     prefix (typically a shared system prompt), so most pairs end after one round trip; the
-//     others binary-search the rest of their range.
+//     others binary-search the rest of their range.  Without relations (allocation-free scoring)
+//     one block takes a request, its chain staged in shared memory, and searches every instance.
 //
 // Rows whose chain starts with the whole chain of an earlier request of the window (its base, from
 // the relations pass) are derived in a second pass instead: the two chains agree block by block up
@@ -52,58 +51,78 @@ struct PairOut {
   }
 };
 
-template <int WARPS, bool SEARCH>
+template <int WARPS>
 __global__ void __launch_bounds__(WARPS * 32)
 probe_hits_kernel(const uint64_t* __restrict__ slots, const uint64_t* __restrict__ ovf,
                   const psk::TableDesc* __restrict__ tdesc,
                   uint32_t I, const uint64_t* __restrict__ off, const uint64_t* __restrict__ hash,
-                  uint32_t R, const psk::RowPre* __restrict__ rows, PairOut out,
-                  unsigned long long* __restrict__ stats) {
+                  uint32_t R, PairOut out) {
   extern __shared__ uint64_t s_chain[];
-  const int warp = threadIdx.x >> 5;
-  const int lane = threadIdx.x & 31;
-  uint64_t n_look = 0, n_rows = 0, n_staged = 0;  // this thread's share of the launch statistics
   for (uint32_t r = blockIdx.x; r < R; r += gridDim.x) {
-    if (rows && __ldg(&rows[r].base) >= 0) continue;  // derived in the second pass
     const uint64_t o = off[r];
     const uint64_t nb = off[r + 1] - o;
     const uint32_t Lr = out.tpf ? __ldg(out.L + r) : 0u;
     const uint64_t ns = nb < kStageBlocks ? nb : kStageBlocks;
-    if (threadIdx.x == 0) {
-      n_rows += 1;
-      n_staged += ns;
-    }
     for (uint64_t k = threadIdx.x; k < ns; k += WARPS * 32) s_chain[k] = __ldg(hash + o + k);
     __syncthreads();
     auto chain = [&](uint64_t k) { return k < ns ? s_chain[k] : __ldg(hash + o + k); };
-    if (SEARCH) {
-      for (uint32_t i = threadIdx.x; i < I; i += WARPS * 32) {
-        const psk::TableDesc d = tdesc[i];
-        uint64_t lo = 0, hi = nb;  // first miss in [lo, hi]
-        while (lo < hi) {
-          const uint64_t mid = (lo + hi) >> 1;
-          ++n_look;
-          if (psk::main_contains(slots, ovf, d, chain(mid))) lo = mid + 1; else hi = mid;
-        }
-        out.put(r, I, i, (uint32_t)lo, Lr);
+    for (uint32_t i = threadIdx.x; i < I; i += WARPS * 32) {
+      const psk::TableDesc d = tdesc[i];
+      uint64_t lo = 0, hi = nb;  // first miss in [lo, hi]
+      while (lo < hi) {
+        const uint64_t mid = (lo + hi) >> 1;
+        if (psk::main_contains(slots, ovf, d, chain(mid))) lo = mid + 1; else hi = mid;
       }
-    } else {
-      for (uint32_t i = warp; i < I; i += WARPS) {
-        const psk::TableDesc d = tdesc[i];
-        auto cached = [&](uint64_t k) {
-          ++n_look;
-          return psk::main_contains(slots, ovf, d, chain(k));
-        };
-        const uint64_t h = psk::warp_first_miss_linear(0, nb, cached);
-        if (lane == 0) out.put(r, I, i, (uint32_t)h, Lr);
-      }
+      out.put(r, I, i, (uint32_t)lo, Lr);
     }
     __syncthreads();
+  }
+}
+
+// Linear mode, the rows of the list (or all R rows): see the file comment.  A row's instances are spread
+// over the grid: with a block per row (its warps taking the instances in turn, 32 positions a step) 100
+// instances x 71 listed rows of about 290 cached blocks took 0.28 ms, 0.073 ms now.
+template <int WARPS>
+__global__ void __launch_bounds__(WARPS * 32)
+probe_linear_kernel(const uint64_t* __restrict__ slots, const uint64_t* __restrict__ ovf,
+                    const psk::TableDesc* __restrict__ tdesc, uint32_t I, const uint64_t* __restrict__ off,
+                    const uint64_t* __restrict__ hash, uint32_t R, psk::RowList list, PairOut out,
+                    unsigned long long* __restrict__ stats) {
+  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
+  const uint32_t ngroup = (I + WARPS - 1) / WARPS;
+  const uint64_t items = (uint64_t)(list.rows ? __ldg(list.count) : R) * ngroup;
+  uint64_t n_look = 0, n_rows = 0;
+  for (uint64_t item = blockIdx.x; item < items; item += gridDim.x) {
+    const uint32_t r = list.rows ? __ldg(list.rows + item / ngroup) : (uint32_t)(item / ngroup);
+    const uint32_t group = (uint32_t)(item % ngroup);
+    if (threadIdx.x == 0 && group == 0) n_rows += 1;
+    const uint32_t i = group * WARPS + warp;
+    if (i >= I) continue;  // warp-uniform
+    const uint64_t o = __ldg(off + r);
+    const uint64_t nb = __ldg(off + r + 1) - o;
+    const uint64_t* chain = hash + o;
+    const psk::TableDesc d = tdesc[i];
+    uint64_t h = nb;
+    for (uint64_t base = 0; base < nb; base += 64) {
+      const uint64_t ka = base + lane, kb = ka + 32;
+      const uint64_t key_a = ka < nb ? __ldg(chain + ka) : psk::kEmpty, key_b = kb < nb ? __ldg(chain + kb) : psk::kEmpty;
+      psk::Lookup la, lb;
+      psk::lookup_issue(slots, ovf, d, key_a, la);
+      psk::lookup_issue(slots, ovf, d, key_b, lb);
+      n_look += (ka < nb ? 1u : 0u) + (kb < nb ? 1u : 0u);
+      const bool pa = psk::lookup_finish(slots, ovf, d, key_a, la), pb = psk::lookup_finish(slots, ovf, d, key_b, lb);
+      const unsigned ma = __ballot_sync(0xffffffffu, ka < nb && !pa), mb = __ballot_sync(0xffffffffu, kb < nb && !pb);
+      if (ma | mb) {
+        h = base + (ma ? (uint64_t)(__ffs(ma) - 1) : 32u + (uint64_t)(__ffs(mb) - 1));
+        break;
+      }
+    }
+    if (lane == 0) out.put(r, I, i, (uint32_t)h, out.tpf ? __ldg(out.L + r) : 0u);
   }
   if (stats) {
     add_stat(stats + kStatRowsScratch, n_rows);
     add_stat(stats + kStatLookupsScratch, n_look);
-    add_stat(stats + kStatChainReads, n_staged);
+    add_stat(stats + kStatChainReads, n_look);
   }
 }
 
@@ -221,10 +240,9 @@ template <int WARPS>
 int max_grid(int num_sms) {
   int per_sm = 0, per_sm2 = 0;
   const int smem = (int)(kStageBlocks * sizeof(uint64_t));
-  cudaFuncSetAttribute(probe_hits_kernel<WARPS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  cudaFuncSetAttribute(probe_hits_kernel<WARPS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, probe_hits_kernel<WARPS, false>, WARPS * 32, smem);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm2, probe_hits_kernel<WARPS, true>, WARPS * 32, smem);
+  cudaFuncSetAttribute(probe_hits_kernel<WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, probe_hits_kernel<WARPS>, WARPS * 32, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm2, probe_linear_kernel<WARPS>, WARPS * 32, 0);
   if (per_sm2 < per_sm) per_sm = per_sm2;
   int per_sm3 = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm3, probe_search_kernel<WARPS>, WARPS * 32, 0);
@@ -255,9 +273,11 @@ cudaError_t launch_probe(const uint64_t* slots, const uint64_t* ovf, const psk::
     if (S && rows && list.rows)                                                                             \
       probe_search_kernel<W><<<grid, W * 32, 0, s>>>(slots, ovf, tdesc, I, w.off, w.hash, rows, list, out,   \
                                                      stats);                                                \
+    else if (S)                                                                                             \
+      probe_hits_kernel<W><<<g, W * 32, smem, s>>>(slots, ovf, tdesc, I, w.off, w.hash, w.R, out);          \
     else                                                                                                    \
-      probe_hits_kernel<W, S><<<g, W * 32, smem, s>>>(slots, ovf, tdesc, I, w.off, w.hash, w.R, rows, out,  \
-                                                     stats);                                                \
+      probe_linear_kernel<W><<<grid, W * 32, 0, s>>>(slots, ovf, tdesc, I, w.off, w.hash, w.R,              \
+                                                     rows ? list : psk::RowList{nullptr, nullptr}, out, stats); \
     cudaError_t e = cudaGetLastError();                                                                     \
     if (e != cudaSuccess || !rows) return e;                                                                \
     if (ev_mid) cudaEventRecord(ev_mid, s);                                                                 \

@@ -86,7 +86,9 @@ struct __align__(16) RowPre {
   uint32_t anc_nb[2]; // their chain lengths
   uint32_t lcp[kLcpBack];  // common chain prefix with requests r - 1 .. r - kLcpBack (blocks)
   uint32_t hint;      // the smallest of them (0 for the first request): where most instances' hits end
-  uint32_t pad[3];
+  uint32_t limit;     // no block from here on counts as cached: the chain's length, or (on caches that are not
+                      // prefix-closed) its first reserved hash
+  uint32_t pad[2];
 };
 constexpr int kRowWords = (int)(sizeof(RowPre) / 16);
 static_assert(sizeof(RowPre) % 16 == 0 && kRowWords <= 32, "RowPre is whole 16-byte words, staged by one warp");
@@ -107,7 +109,7 @@ struct GreedySync {
   uint32_t* done;            // [R] insert blocks done with the job (its blocks are all in at the group size)
   uint32_t* ready;           // [R] 1 once the row's probed hits are in the ring
   uint32_t* hitring;         // [kHitSlots][ring_stride] probed hits (row s in slot s % kHitSlots)
-  float* tpfring;            // [kHitSlots][ring_stride] T_pf at those hits (kNoTpfBits where it changed)
+  float* tpfring;            // [kHitSlots][ring_stride] T_pf at those hits
   uint32_t ring_stride;      // I rounded up to a multiple of 8
   uint64_t wait_ns;          // bound on any cross-block wait (ns); a waiter that gives up sets kErrTimeout
   unsigned long long* stats; // [kGreedyStats] counters of the pass (below)
@@ -392,27 +394,13 @@ __device__ __forceinline__ bool delta_contains(const DeltaSlot* delta, uint64_t 
   return delta_contains_from(delta, nslots, inst, key, delta_home(key, inst, nslots));
 }
 
-// Insert (inst, key) at the first empty slot from `slot` on (see delta_insert).
-__device__ __forceinline__ bool delta_insert_from(DeltaSlot* delta, uint64_t nslots, uint32_t inst, uint64_t key,
-                                                  uint64_t slot) {
-  for (uint64_t p = 0; p < nslots; ++p) {
-    if (atomicCAS(&delta[slot].hash, kEmpty, (unsigned long long)key) == kEmpty) {
-      __stcg(&delta[slot].tag, inst + 1);
-      return true;
-    }
-    slot = delta_next(slot, nslots);
-  }
-  return false;
-}
-
-// Insert (inst, key): the first empty slot from the key's home is claimed by compare-and-swap on
+// Insert (inst, key) at the first empty slot from `slot` on: the slot is claimed by compare-and-swap on
 // the hash, then the tag is stored (one round trip).  A lookup racing with the insert may see the
 // slot without its tag and report the pair absent, which only under-reports; it is visible to every
 // reader once the inserting block has released its done flag.  The table has twice as many slots as
 // a window has chain blocks, so it cannot fill; false reports a full table anyway.
-__device__ __forceinline__ bool delta_insert(DeltaSlot* delta, uint64_t nslots, uint32_t inst, uint64_t key) {
-  if (key == kEmpty || key == kTomb) return true;
-  uint64_t slot = delta_home(key, inst, nslots);
+__device__ __forceinline__ bool delta_insert_from(DeltaSlot* delta, uint64_t nslots, uint32_t inst, uint64_t key,
+                                                  uint64_t slot) {
   for (uint64_t p = 0; p < nslots; ++p) {
     if (atomicCAS(&delta[slot].hash, kEmpty, (unsigned long long)key) == kEmpty) {
       __stcg(&delta[slot].tag, inst + 1);
@@ -642,12 +630,6 @@ __device__ __forceinline__ RowConst row_const(const DevModel& m, uint32_t L, flo
   return rc;
 }
 
-struct PairEval {
-  float W, tpot, ttft;
-  int64_t n;   // uncached tokens
-  bool inA;    // capacity-eligible
-};
-
 __device__ __forceinline__ float ema_factor(const DevModel& m, int64_t B) {
   if (m.nseg == 1) return m.ema[0];
   int s = 0;
@@ -656,37 +638,8 @@ __device__ __forceinline__ float ema_factor(const DevModel& m, int64_t B) {
   return m.ema[s];
 }
 
-// RecomputeCost, capacity guard and the latency predictions of one (request, instance) pair.
-__device__ __forceinline__ PairEval eval_pair(const DevModel& m, const RowConst& rc, uint32_t h,
-                                              int32_t b, int32_t qr, int64_t q, int64_t S, int64_t M,
-                                              int32_t Bmax) {
-  PairEval e;
-  const int64_t c = 16 * (int64_t)h;
-  const int64_t n = (int64_t)rc.L - c;
-  const float tpf = t_pf(m, i64_to_f32(n), i64_to_f32(c));
-  e.n = n;
-  e.W = __fsub_rn(tpf, rc.t_cached);
-  const int64_t Bp = (int64_t)b + qr + 1;
-  const int64_t Sp = S + (int64_t)rc.L;
-  e.inA = (Bp <= (int64_t)Bmax) && (Sp <= M);
-  float dec = __fadd_rn(m.b0, __fmul_rn(m.b1, i64_to_f32(Bp)));
-  dec = __fadd_rn(dec, __fmul_rn(m.b2, i64_to_f32(Sp)));
-  dec = __fmul_rn(dec, ema_factor(m, Bp));
-  if (m.interference_mode == 0) {
-    e.tpot = __fadd_rn(dec, __fmul_rn(m.g_q, i64_to_f32(q + n)));
-  } else {
-    const float den = m.lout > 1.0f ? m.lout : 1.0f;
-    const float interf = ((int64_t)b + qr > 0) ? __fdiv_rn(tpf, den) : 0.0f;
-    e.tpot = __fadd_rn(dec, interf);
-  }
-  const float tq = __fadd_rn(__fmul_rn(m.a0, __int2float_rn(qr)), __fmul_rn(m.a1, i64_to_f32(q)));
-  e.ttft = __fadd_rn(tpf, tq);
-  return e;
-}
-
-// Terms of eval_pair that depend only on the instance state (b, qr, q, B_max): they change only
-// when the instance is picked, so the greedy keeps them per instance.  Same rounded operations as
-// eval_pair, so results are bit-identical.
+// Terms of a pair's evaluation that depend only on the instance state (b, qr, q, B_max): they change
+// only when the instance is picked, so kernels keep them per instance.
 struct InstTerms {
   float dec0;   // b0 + b1 * B, B = b + qr + 1
   float f;      // EMA factor of B's segment
@@ -742,32 +695,15 @@ __device__ __forceinline__ void pair_lat32(const DevModel& m, const RowConst& rc
   *ttft = __fadd_rn(tpf, tq);
 }
 
-// Marks a precomputed T_pf as not available (a NaN pattern T_pf never produces).
-constexpr uint32_t kNoTpfBits = 0xFFFFFFFFu;
-
-// The two halves of eval_pair with the instance terms precomputed (the greedy evaluates the
-// latencies only for pairs that pass the capacity guard and the recompute filter).  Together they
-// perform exactly eval_pair's rounded operations.
-//   pair_w:   T_pf at the hit (given unless tpf_in carries kNoTpfBits), W = T_pf(n, c) - T_pf(0, L),
-//             n, and the capacity guard (Algorithm 1 CapacityCandidates).
-//   pair_lat: TPOT (Eq. 5 / Eq. 9) and TTFT (Eq. 4) of the pair.
+// What the latencies of a (request, instance) pair need of its recompute cost: T_pf at the hit,
+// W = T_pf(n, c) - T_pf(0, L), the uncached tokens n and the capacity guard.
 struct PairW {
   float W, tpf;
   int64_t n;
   bool inA;
 };
 
-__device__ __forceinline__ PairW pair_w(const DevModel& m, const RowConst& rc, uint32_t h, float tpf_in,
-                                        const InstTerms& it, int64_t S, int64_t M) {
-  PairW x;
-  const int64_t c = 16 * (int64_t)h;
-  x.n = (int64_t)rc.L - c;
-  x.tpf = __float_as_uint(tpf_in) == kNoTpfBits ? t_pf(m, i64_to_f32(x.n), i64_to_f32(c)) : tpf_in;
-  x.W = __fsub_rn(x.tpf, rc.t_cached);
-  x.inA = it.okB && (S + (int64_t)rc.L <= M);
-  return x;
-}
-
+// TPOT (Eq. 5 / Eq. 9) and TTFT (Eq. 4) of a pair.
 __device__ __forceinline__ void pair_lat(const DevModel& m, const RowConst& rc, const PairW& x, const InstTerms& it,
                                          int64_t q, int64_t S, float* tpot, float* ttft) {
   const int64_t Sp = S + (int64_t)rc.L;
@@ -783,18 +719,6 @@ __device__ __forceinline__ void pair_lat(const DevModel& m, const RowConst& rc, 
   *ttft = __fadd_rn(x.tpf, it.tq);
 }
 
-// eval_pair with the instance terms precomputed, and T_pf given unless it carries kNoTpfBits.
-__device__ __forceinline__ PairEval eval_pair_tpf(const DevModel& m, const RowConst& rc, uint32_t h, float tpf_in,
-                                                  const InstTerms& it, int64_t q, int64_t S, int64_t M) {
-  const PairW x = pair_w(m, rc, h, tpf_in, it, S, M);
-  PairEval e;
-  e.n = x.n;
-  e.W = x.W;
-  e.inA = x.inA;
-  pair_lat(m, rc, x, it, q, S, &e.tpot, &e.ttft);
-  return e;
-}
-
 // Recompute filter (Eq. 8) of a capacity-eligible pair once W_min is known: W - W_min <= eta Z,
 // every pair of A when Z <= 0.
 __device__ __forceinline__ bool pair_in_c(const RowConst& rc, float W, float Wmin) {
@@ -808,19 +732,6 @@ __device__ __forceinline__ bool pair_admitted(const DevModel& m, const RowConst&
   bool ok = tpot < rc.tpot_target;
   if (m.ttft_filter) ok = ok && (ttft <= rc.ttft_budget);
   return ok;
-}
-
-__device__ __forceinline__ PairEval eval_pair_terms(const DevModel& m, const RowConst& rc, uint32_t h,
-                                                    const InstTerms& it, int64_t q, int64_t S, int64_t M) {
-  return eval_pair_tpf(m, rc, h, __uint_as_float(kNoTpfBits), it, q, S, M);
-}
-
-// Class of a capacity-eligible pair once W_min is known (Eq. 8, Alg. 1 TPOT filter + TTFT budget):
-// 0 in T, 1 in C \ T, 2 filtered by the recompute budget.
-__device__ __forceinline__ uint32_t pair_class(const DevModel& m, const RowConst& rc, const PairEval& e,
-                                               float Wmin) {
-  if (!pair_in_c(rc, e.W, Wmin)) return 2u;
-  return pair_admitted(m, rc, e.tpot, e.ttft) ? 0u : 1u;
 }
 
 // Order-preserving map of a non-NaN float to an unsigned integer (for integer warp reductions).
@@ -888,12 +799,6 @@ __device__ __forceinline__ uint64_t value_fallback(const DevModel& m, uint64_t q
   return qn * (uint64_t)Bp;
 }
 
-__device__ __forceinline__ float warp_fmin(float x) {
-#pragma unroll
-  for (int s = 16; s > 0; s >>= 1) x = fminf(x, __shfl_xor_sync(0xffffffffu, x, s));
-  return x;
-}
-
 // (class, value) of a pair of C as one 64-bit key, class in the top two bits: class-0 values are
 // below 2^62 and class-1 values below 2^59 ((q + n) < 2^41 times (b + qr + 1) < 2^18), so the
 // unsigned order of the packed key is the lexicographic order of (class, value).
@@ -951,11 +856,6 @@ int probe_max_grid(uint32_t I, int num_sms);
 cudaError_t launch_score(const uint32_t* hits, psk::StateSoA st, uint32_t I, const psk::WindowDev& w,
                          const psk::DevModel& m, float* tpot, float* ttft, uint8_t* cls, int32_t* best,
                          uint8_t* path, int num_sms, cudaStream_t s, const psk::ShardIO& sh = psk::ShardIO());
-cudaError_t launch_greedy(const uint64_t* slots, const uint64_t* ovf, const psk::TableDesc* tdesc, uint32_t I,
-                          const psk::WindowDev& w, const uint32_t* hit0, psk::StateSoA committed,
-                          psk::StateSoA pending, const psk::DevModel& m, psk::DeltaSlot* delta,
-                          uint64_t delta_nslots, int32_t* assign, uint8_t* path, uint32_t* hit_chosen,
-                          uint32_t* err, int search, cudaStream_t s);
 cudaError_t launch_delta_clear(psk::DeltaSlot* delta, uint64_t nslots, cudaStream_t s);
 // Rebuilds every chain of a window in the shared-prefix form (ps_window.parent) into hash (CSR at
 // full_off) from each request's own blocks (CSR at own_off) and its parent link.
@@ -963,11 +863,13 @@ cudaError_t launch_expand_chains(const uint64_t* full_off, const uint64_t* own_o
                                  const int32_t* parent, uint32_t R, uint64_t* hash, uint32_t* err, int num_sms,
                                  cudaStream_t s);
 cudaError_t launch_relations(const psk::WindowDev& w, const psk::DevModel& m, psk::LastSlot* tab, uint32_t tab_n,
-                             psk::RowPre* rows, psk::RowList list, int num_sms, cudaStream_t s);
-cudaError_t launch_greedy_search(const psk::RowPre* rows, const psk::WindowDev& w, uint32_t I, const uint32_t* hit0,
-                                 const float* tpf0, psk::StateSoA committed, psk::StateSoA pending, const psk::DevModel& m,
-                                 psk::DeltaSlot* delta, uint64_t delta_nslots, int32_t* assign, uint8_t* path,
-                                 uint32_t* hit_chosen, uint32_t* err, const psk::GreedySync& sync, cudaStream_t s);
+                             psk::RowPre* rows, psk::RowList list, int search, int num_sms, cudaStream_t s);
+// search 0: the caches need not be prefix-closed (rows' limits set, the committed tables probed too).
+cudaError_t launch_greedy(const psk::RowPre* rows, const psk::WindowDev& w, uint32_t I, const uint32_t* hit0,
+                          const float* tpf0, psk::StateSoA committed, psk::StateSoA pending, const psk::DevModel& m,
+                          psk::DeltaSlot* delta, uint64_t delta_nslots, int32_t* assign, uint8_t* path,
+                          uint32_t* hit_chosen, uint32_t* err, const psk::GreedySync& sync, int search,
+                          const uint64_t* slots, const uint64_t* ovf, const psk::TableDesc* tdesc, cudaStream_t s);
 cudaError_t launch_insert_chains(uint64_t* slots, uint64_t* ovf, const psk::TableDesc* tdesc, uint32_t I,
                                  unsigned long long* count, uint64_t nchains, const uint32_t* inst,
                                  const uint64_t* off, const uint64_t* hash, const uint64_t* parent,

@@ -61,6 +61,9 @@ __device__ __forceinline__ int32_t tab_resolve(const psk::LastSlot* tab, uint32_
   return -1;
 }
 
+// Equal blocks that can be cached: a reserved hash says nothing about the prefix it ends.
+__device__ __forceinline__ bool same_block(uint64_t x, uint64_t y) { return x == y && x + 1ull > 1ull; }
+
 constexpr int kScanPerLane = 8;  // parent-scan positions per lane and step (256 per warp step)
 static_assert(psk::kLcpBack == 32, "one lane per earlier request");
 
@@ -99,7 +102,7 @@ relations_kernel(psk::WindowDev w, psk::DevModel m, const psk::LastSlot* tab, ui
     // the first difference lies in [lo, hi] (hi: the end of the shorter chain, or a known difference)
     uint32_t lo = 0u, hi = has ? (uint32_t)(nb < nq ? nb : nq) : 0u;
     if (hi > 0u) {
-      if (a[hi - 1] == b[hi - 1]) lo = hi;
+      if (same_block(a[hi - 1], b[hi - 1])) lo = hi;
       else hi -= 1u;
     }
     for (;;) {
@@ -109,12 +112,12 @@ relations_kernel(psk::WindowDev w, psk::DevModel m, const psk::LastSlot* tab, ui
       const uint64_t* bs = w.hash + __shfl_sync(0xffffffffu, oq, src);
       const uint32_t ls = __shfl_sync(0xffffffffu, lo, src), hs = __shfl_sync(0xffffffffu, hi, src);
       const uint32_t x =
-          (uint32_t)psk::warp_search_range(ls, hs, [&](uint64_t k) { return a[k] == bs[k]; });
+          (uint32_t)psk::warp_search_range(ls, hs, [&](uint64_t k) { return same_block(a[k], bs[k]); });
       if (lane == src) {
         lo = hi = x;
       } else if (lo < hi && x >= lo && x <= hi) {  // this pair may well part at x too
-        const bool below = x == lo || a[x - 1] == b[x - 1];
-        const bool at = x >= hi || a[x] != b[x];
+        const bool below = x == lo || same_block(a[x - 1], b[x - 1]);
+        const bool at = x >= hi || !same_block(a[x], b[x]);
         if (!below) hi = x - 1u;
         else if (at) lo = hi = x;
         else lo = x + 1u;
@@ -178,6 +181,7 @@ relations_kernel(psk::WindowDev w, psk::DevModel m, const psk::LastSlot* tab, ui
       x.ttft_budget = rc.ttft_budget;
       x.tpot_target = rc.tpot_target;
       x.hint = r > 0u ? hint : 0u;
+      x.limit = (uint32_t)nb;
       x.par = par;
       x.par_nb = par_nb;
       x.base = -1;
@@ -185,6 +189,23 @@ relations_kernel(psk::WindowDev w, psk::DevModel m, const psk::LastSlot* tab, ui
     }
     __syncwarp();
     rows[r].lcp[lane] = lcp;
+  }
+}
+
+// First reserved hash of each chain (rows' limit), one warp per request.
+__global__ void __launch_bounds__(256)
+limit_kernel(psk::WindowDev w, psk::RowPre* rows) {
+  const uint32_t lane = threadIdx.x & 31u;
+  for (uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < w.R; r += (gridDim.x * blockDim.x) >> 5) {
+    const uint64_t o = w.off[r], nb = w.off[r + 1] - o;
+    for (uint64_t k0 = 0; k0 < nb; k0 += 32) {
+      const uint64_t key = k0 + lane < nb ? w.hash[o + k0 + lane] : 1ull;
+      const unsigned res = __ballot_sync(0xffffffffu, key == psk::kEmpty || key == psk::kTomb);
+      if (res) {
+        if (lane == 0) rows[r].limit = (uint32_t)k0 + (uint32_t)__ffs(res) - 1u;
+        break;
+      }
+    }
   }
 }
 
@@ -219,7 +240,7 @@ __global__ void base_kernel(uint32_t R, psk::RowPre* rows, psk::RowList list) {
 namespace pskl {
 
 cudaError_t launch_relations(const psk::WindowDev& w, const psk::DevModel& m, psk::LastSlot* tab, uint32_t tab_n,
-                             psk::RowPre* rows, psk::RowList list, int num_sms, cudaStream_t s) {
+                             psk::RowPre* rows, psk::RowList list, int search, int num_sms, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(list.count, 0, sizeof(uint32_t), s);
   if (e != cudaSuccess || w.R == 0) return e;
   e = cudaMemsetAsync(tab, 0, (size_t)tab_n * sizeof(psk::LastSlot), s);
@@ -232,6 +253,7 @@ cudaError_t launch_relations(const psk::WindowDev& w, const psk::DevModel& m, ps
   relations_kernel<<<g2, 256, 0, s>>>(w, m, tab, tab_n, rows);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
+  if (!search) limit_kernel<<<g2 < num_sms * 8 ? g2 : num_sms * 8, 256, 0, s>>>(w, rows);
   base_kernel<<<g1, 256, 0, s>>>(w.R, rows, list);
   return cudaGetLastError();
 }

@@ -78,3 +78,35 @@ def test_sums_beyond_32_bits(P, shift):
         ins.q[5::7] += 1 << 35
     for sel in (0, 5):
         _check(P, dict(wl.model, selector=sel), ins, wl.window)
+
+
+@pytest.mark.parametrize("sel,kv", [(0, 0), (5, 0), (0, 1 << 45)])
+def test_caches_with_holes(P, sel, kv):
+    """Caches that are not prefix-closed: hits that rise in the window go on through blocks the committed
+    table holds past a hole, and end at a reserved hash."""
+    wl = _workload(24, 150, seed=12)
+    ins, win = wl.instances, wl.window
+    rng = np.random.default_rng(2)
+    off = [0]
+    keep = rng.random(ins.chain_hash.size) > 0.02
+    for c in range(ins.chain_inst.size):
+        off.append(off[-1] + int(keep[int(ins.chain_off[c]):int(ins.chain_off[c + 1])].sum()))
+    ins.chain_hash, ins.chain_off = ins.chain_hash[keep], np.array(off, np.uint64)
+    # some blocks' hashes are the reserved 0, in every chain that holds them; the oracle, which reserves
+    # no value, sees a hash of its own in each of those places
+    zero = np.isin(win.chain_hash, rng.choice(win.chain_hash, 40))
+    own = dict(vars(win), chain_hash=win.chain_hash.copy())
+    own["chain_hash"][zero] = rng.integers(2, 2 ** 63, int(zero.sum()), dtype=np.int64).astype(np.uint64)
+    win.chain_hash[zero] = 0
+    owin = W.Window(**own)
+    if kv:
+        ins.M_KV[:] = kv
+    model = dict(wl.model, selector=sel)
+    orc = Oracle(ins.I, model).load(ins)
+    with P.Scheduler(ins.I, ins.cap_blocks, win.R, int(win.chain_off[-1]), model, table_load_factor=0.5,
+                     probe_mode=P.PS_PROBE_LINEAR) as s:
+        s.load_workload_instances(ins)
+        assert np.array_equal(s.score_window(win, want=("hits",))["hits"], orc.score_rows(owin)["hits"])
+        g, o = s.schedule_window(win), orc.schedule(owin)
+        for k in ("assign", "path", "hit_chosen"):
+            assert np.array_equal(g[k], o[k]), (k, np.nonzero(g[k] != o[k])[0][:5])
