@@ -493,13 +493,14 @@ ps_status ps_create(const ps_config* cfg, ps_ctx** out) {
     for (uint32_t i = 0; i < I; ++i)
       c->max_instance_slots = std::max<uint64_t>(c->max_instance_slots, (uint64_t)td[i].nbkt * psk::kBucketSlots);
     unsigned char* lb = nullptr;
-    unsigned char* plan = nullptr;
+    unsigned char *plan = nullptr, *blocks = nullptr;
     pskl::EvictScratch& ev = c->evict;
     ok = dalloc(c, &lb, pskl::evict_leafbuf_bytes(c->I)) == cudaSuccess && dalloc(c, &ev.nleaf, I) == cudaSuccess &&
          dalloc(c, &ev.more, 1) == cudaSuccess && dalloc(c, &plan, pskl::evict_plan_bytes(c->I)) == cudaSuccess &&
          dalloc(c, &ev.hist, pskl::evict_hist_words(c->I)) == cudaSuccess &&
-         dalloc(c, &ev.cand, pskl::evict_cand_words(c->I)) == cudaSuccess && dalloc(c, &ev.list, I + 1) == cudaSuccess &&
+         dalloc(c, &blocks, pskl::evict_blocks_bytes(c->I)) == cudaSuccess && dalloc(c, &ev.list, I + 1) == cudaSuccess &&
          dalloc(c, &ev.slow, I) == cudaSuccess;
+    ev.blocks = blocks;
     ev.leafbuf = lb;
     ev.plan = plan;
   }
@@ -545,7 +546,7 @@ ps_status ps_create(const ps_config* cfg, ps_ctx** out) {
   set = set && cudaMemcpyAsync(c->d_cap, c->cap.data(), I * sizeof(uint64_t), cudaMemcpyHostToDevice, c->stream) ==
                    cudaSuccess;
   if (c->lru)
-    set = set && cudaMemsetAsync(c->meta.last_use, 0, c->total_slots * 4, c->stream) == cudaSuccess &&
+    set = set && cudaMemsetAsync(c->meta.last_use, 0xFF, c->total_slots * 4, c->stream) == cudaSuccess &&
           cudaMemsetAsync(c->meta.children, 0, c->total_slots * 4, c->stream) == cudaSuccess &&
           cudaMemsetAsync(c->evict.hist, 0, pskl::evict_hist_words(c->I) * 4, c->stream) == cudaSuccess &&
           cudaMemsetAsync(c->meta.parent, 0xFF, c->total_slots * 8, c->stream) == cudaSuccess;  // kNoParent

@@ -270,6 +270,8 @@ __device__ __forceinline__ uint64_t main_find(const uint64_t* slots, const uint6
 // its number of cached children, and its parent's slot (kNoParent for a chain root or a parent that
 // was not cached when the block was inserted).  A slot is stable while its block is cached and a
 // parent outlives its children (eviction is leaf-first), so a cached block's parent slot stays valid.
+// An empty slot's last_use is kNoUse (a block may carry that stamp too: its slot holds a key).
+constexpr uint32_t kNoUse = 0xFFFFFFFFu;
 constexpr uint64_t kNoParent = ~0ull;
 constexpr uint64_t kLinkPending = ~1ull;  // inserted by a commit whose linking pass has not run yet
 struct LruMeta {
@@ -884,15 +886,15 @@ cudaError_t launch_commit(uint64_t* slots, uint64_t* ovf, const psk::TableDesc* 
 cudaError_t launch_advance(psk::StateSoA st, uint32_t I, const psk::ReqStore& rq, const psk::DevModel& m,
                            float window_ms, uint64_t prefill_tokens, uint32_t* err, cudaStream_t s);
 // Device scratch of the eviction: leafbuf holds evict_leafbuf_bytes(I) bytes, plan evict_plan_bytes(I),
-// hist evict_hist_words(I) words (zero between calls), cand evict_cand_words(I); nleaf, slow [I],
-// list [I + 1], more [1].
+// hist evict_hist_words(I) words (zero between calls), blocks evict_blocks_bytes(I) bytes; nleaf, slow
+// [I], list [I + 1], more [1].
 struct EvictScratch {
   void* leafbuf;
   uint32_t* nleaf;
   uint32_t* more;
   void* plan;
   uint32_t* hist;
-  uint32_t* cand;
+  void* blocks;
   uint32_t* list;
   uint32_t* slow;
 };
@@ -904,7 +906,7 @@ cudaError_t launch_evict(uint64_t* slots, const psk::TableDesc* tdesc, uint32_t 
                          uint64_t max_instance_slots, uint32_t max_use, uint32_t* err, int num_sms, cudaStream_t s);
 size_t evict_plan_bytes(uint32_t I);
 size_t evict_hist_words(uint32_t I);
-size_t evict_cand_words(uint32_t I);
+size_t evict_blocks_bytes(uint32_t I);
 size_t evict_leafbuf_bytes(uint32_t I);
 cudaError_t launch_check_parents(const uint64_t* slots, const uint64_t* ovf, const psk::TableDesc* tdesc, uint32_t I,
                                  uint64_t nchains, const uint32_t* inst, const uint64_t* parent,

@@ -195,7 +195,10 @@ insert_chains_kernel(uint64_t* slots, uint64_t* ovf, const psk::TableDesc* __res
             full = true;
           } else {
             stored = true;
-            if (meta.last_use) meta.last_use[slot] = last_use;
+            if (meta.last_use) {
+              meta.last_use[slot] = last_use;
+              meta.children[slot] = 0u;
+            }
           }
         } else if (slot != ~0ull && meta.last_use && meta.last_use[slot] < last_use) {
           meta.last_use[slot] = last_use;
@@ -559,26 +562,33 @@ __device__ __forceinline__ uint32_t parent32(uint64_t p) {
 // a block's subtree maximum has its own last_use.  So with T the last_use value at which the blocks
 // counted from the oldest reach the excess E, the evicted blocks are exactly: every block older than T,
 // and of the blocks stamped T the k missing ones with the smallest subtree maximum of the hash over
-// blocks stamped T.  Four kernels find and evict them, every step parallel:
+// blocks stamped T.  These kernels find and evict them, every step parallel:
 //   list      the instances over capacity;
 //   hist      per instance a histogram of last_use over its slots (and its number of leaves), in one
 //             pass for stamps below 2048 and one more per further 11 bits; choose picks T and k;
 //   gather    the slots stamped below T and those stamped T (up to kClassMax each; at most kClassMax
 //             evictions a round);
-//   order     one thread block per instance checks that the stamps do not increase downwards among
-//             these blocks and that none of them has a newer child; finds the subtree maxima of the
-//             class T by doubling over the parent links in shared memory (a block pushes its maximum
-//             to its ancestor 2^r links up in round r); selects the k smallest; evicts.
+//   detail    every gathered block's parent, children count and the parent's stamp, and the hashes of
+//             the class T, side by side (the metadata is scattered, a DRAM access each: this wants
+//             every warp of the chip), with the sums of the check that the stamps do not increase
+//             downwards among these blocks and that none of them has a newer child;
+//   index, jump  each class block's index in place of its (known) stamp, then its parent's index;
+//   order     one thread block per instance finds the subtree maxima of the class T by doubling over the
+//             parent links in shared memory (a block pushes its maximum to its ancestor 2^r links up in
+//             round r); selects the k smallest; evicts.
+// At most kEvictBatch instances a round.
 // An instance that fails the check, or has more blocks stamped T than shared memory holds, is evicted
-// one block at a time by the kernels after these.  Bound by the two scans of the tables (16 bytes a
-// slot).  1024 instances x 200K blocks, about 240 over capacity by up to 7.9K blocks: a streaming
-// window of 500 requests takes 2.08 ms; with one thread ordering each instance's evictions (1.2 us
-// each, 10 ms of the window) it took 11.8 ms.
+// one block at a time by the kernels after these.  Bound by the two scans (last_use twice and the
+// children counts once: 12 bytes a slot; an empty slot's stamp is kNoUse, so the keys are not read)
+// and the order kernel's chain of dependent steps.  1024 instances x 200K blocks, about 240 over
+// capacity by up to 7.9K blocks: hist 0.12 ms, gather 0.11, detail 0.09, index and jump 0.07, order 0.17
+// (0.43 ms where the order kernel read the metadata itself, a block an SM); the streaming window of 500
+// requests takes 1.74 ms, and took 11.8 ms with one thread ordering each instance's evictions (1.2 us each).
 constexpr uint32_t kClassMax = 16384;   // blocks of one last_use value ordered in shared memory
 constexpr uint32_t kHistBits = 11;
 constexpr uint32_t kHistBins = 1u << kHistBits;
 constexpr uint32_t kOrderThreads = 1024;
-constexpr uint32_t kOrderPer = kClassMax / kOrderThreads;  // blocks per thread
+constexpr uint32_t kOrderPer = kClassMax / kOrderThreads;  // class blocks per thread
 constexpr uint32_t kScanThreads = 512;
 constexpr uint64_t kScanChunk = 65536;  // slots a block scans before it merges its histogram
 constexpr uint32_t kNoJump = 0xFFFFu;
@@ -593,26 +603,49 @@ struct EvictPlan {
   uint32_t k;            // of them, blocks stamped T (T = lo once chosen)
   uint32_t n_old, n_cls; // gathered blocks
   uint32_t leaves;
+  uint32_t children, inside, bad;  // the check's sums: cached children of the gathered blocks, gathered
+                                   // blocks with a gathered parent; some child is newer than its parent
+  __device__ bool fits() const { return k != 0u && n_old <= kClassMax && n_cls <= kClassMax; }
+  __device__ bool in_order() const { return bad == 0u && children == inside; }
 };
+
+// The gathered blocks of the q-th listed instance: [0, kClassMax) stamped below T, [kClassMax, 2
+// kClassMax) stamped T (the class).
+constexpr uint32_t kEvictBatch = 256;
+struct EvictBlocks {
+  uint32_t* slot;   // [kEvictBatch][2 kClassMax]
+  uint32_t* par;    // the parent's slot
+  uint8_t* rel;     // the parent's stamp against T: kRel*
+  uint64_t* key;    // [kEvictBatch][kClassMax] the class's hashes
+  uint16_t* jump;   // [kEvictBatch][kClassMax] index of the parent in the class (kNoJump: none)
+};
+enum : uint8_t { kRelNone = 0, kRelOlder = 1, kRelClass = 2, kRelNewer = 3 };
+
 
 __global__ void __launch_bounds__(1024)
 evict_list_kernel(uint32_t I, const unsigned long long* __restrict__ count, const uint64_t* __restrict__ cap,
-                  const uint32_t* __restrict__ slow, uint32_t max_use, EvictPlan* plan, uint32_t* list, uint32_t* nlist) {
+                  const uint32_t* __restrict__ slow, uint32_t max_use, EvictPlan* plan, uint32_t* list, uint32_t* nlist,
+                  uint32_t* more) {
   __shared__ uint32_t s_n;
   if (threadIdx.x == 0) s_n = 0u;
   __syncthreads();
   for (uint32_t i = threadIdx.x; i < I; i += blockDim.x) {
     const unsigned long long c = count[i];
     if (c <= cap[i] || slow[i]) continue;
+    const uint32_t q = atomicAdd(&s_n, 1u);
+    if (q >= kEvictBatch) continue;
     const unsigned long long E = c - cap[i];
     EvictPlan p{};
     p.hi = max_use;
     p.todo = E < kClassMax ? (uint32_t)E : kClassMax;
     plan[i] = p;
-    list[atomicAdd(&s_n, 1u)] = i;
+    list[q] = i;
   }
   __syncthreads();
-  if (threadIdx.x == 0) *nlist = s_n;
+  if (threadIdx.x == 0) {
+    *nlist = s_n < kEvictBatch ? s_n : kEvictBatch;
+    if (s_n > kEvictBatch) atomicOr(more, kMoreFast);
+  }
 }
 
 // Bin width of an open range as a shift.
@@ -622,14 +655,14 @@ __device__ __forceinline__ uint32_t hist_shift(uint32_t lo, uint32_t hi) {
 }
 
 __global__ void __launch_bounds__(kScanThreads)
-evict_hist_kernel(const uint64_t* __restrict__ slots, const psk::TableDesc* __restrict__ tdesc, psk::LruMeta meta,
+evict_hist_kernel(const psk::TableDesc* __restrict__ tdesc, psk::LruMeta meta,
                   EvictPlan* plan, const uint32_t* __restrict__ list, const uint32_t* __restrict__ nlist,
                   uint64_t chunks, uint32_t* __restrict__ hist, bool first) {
   __shared__ uint32_t s_bin[kHistBins];
   __shared__ uint32_t s_leaves;
   const uint64_t items = (uint64_t)*nlist * chunks;
   for (uint64_t item = blockIdx.x; item < items; item += gridDim.x) {
-    const uint32_t i = list[item / chunks];
+    const uint32_t q = (uint32_t)(item / chunks), i = list[q];
     const psk::TableDesc d = tdesc[i];
     const uint64_t n = (uint64_t)d.nbkt * psk::kBucketSlots, x0 = (item % chunks) * kScanChunk;
     if (x0 >= n) continue;  // block-uniform
@@ -639,15 +672,17 @@ evict_hist_kernel(const uint64_t* __restrict__ slots, const psk::TableDesc* __re
     if (threadIdx.x == 0) s_leaves = 0u;
     __syncthreads();
     uint32_t leaves = 0;
-    // two slots a thread (tables are whole 8-slot buckets)
-    for (uint64_t x = x0 + 2u * threadIdx.x; x < x1; x += 2u * kScanThreads) {
-      const ulonglong2 key = __ldcs(reinterpret_cast<const ulonglong2*>(slots + d.base + x));
-      const uint2 lu = __ldcs(reinterpret_cast<const uint2*>(meta.last_use + d.base + x));
-      if (key.x != psk::kEmpty && lu.x >= lo && lu.x <= hi) atomicAdd(&s_bin[(lu.x - lo) >> sh], 1u);
-      if (key.y != psk::kEmpty && lu.y >= lo && lu.y <= hi) atomicAdd(&s_bin[(lu.y - lo) >> sh], 1u);
-      if (first) {
-        const uint2 ch = __ldcs(reinterpret_cast<const uint2*>(meta.children + d.base + x));
-        leaves += (key.x != psk::kEmpty && ch.x == 0u) + (key.y != psk::kEmpty && ch.y == 0u);
+    // four slots a thread (tables are whole 8-slot buckets); an empty slot's stamp says so
+    for (uint64_t x = x0 + 4u * threadIdx.x; x < x1; x += 4u * kScanThreads) {
+      const uint4 lu = __ldcs(reinterpret_cast<const uint4*>(meta.last_use + d.base + x));
+      uint4 ch = make_uint4(1u, 1u, 1u, 1u);
+      if (first) ch = __ldcs(reinterpret_cast<const uint4*>(meta.children + d.base + x));
+      const uint32_t l[4] = {lu.x, lu.y, lu.z, lu.w}, cc[4] = {ch.x, ch.y, ch.z, ch.w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (l[u] == psk::kNoUse) continue;
+        if (l[u] >= lo && l[u] <= hi) atomicAdd(&s_bin[(l[u] - lo) >> sh], 1u);
+        leaves += cc[u] == 0u;
       }
     }
     if (first) {
@@ -656,7 +691,7 @@ evict_hist_kernel(const uint64_t* __restrict__ slots, const psk::TableDesc* __re
     }
     __syncthreads();
     for (uint32_t b = threadIdx.x; b < kHistBins; b += kScanThreads)
-      if (s_bin[b]) atomicAdd(&hist[(uint64_t)i * kHistBins + b], s_bin[b]);
+      if (s_bin[b]) atomicAdd(&hist[(uint64_t)q * kHistBins + b], s_bin[b]);
     if (first && threadIdx.x == 0) atomicAdd(&plan[i].leaves, s_leaves);
     __syncthreads();
   }
@@ -677,7 +712,7 @@ evict_choose_kernel(EvictPlan* plan, const uint32_t* __restrict__ list, const ui
     uint32_t v[kPer], sum = 0;
 #pragma unroll
     for (uint32_t u = 0; u < kPer; ++u) {
-      uint32_t* b = &hist[(uint64_t)i * kHistBins + t * kPer + u];
+      uint32_t* b = &hist[(uint64_t)x * kHistBins + t * kPer + u];
       v[u] = *b;
       *b = 0u;
       sum += v[u];
@@ -709,9 +744,9 @@ evict_choose_kernel(EvictPlan* plan, const uint32_t* __restrict__ list, const ui
 
 // Gathers the slots stamped below T (first half of the instance's candidate buffer) and T (second half).
 __global__ void __launch_bounds__(kScanThreads)
-evict_gather_kernel(const uint64_t* __restrict__ slots, const psk::TableDesc* __restrict__ tdesc, psk::LruMeta meta,
+evict_gather_kernel(const psk::TableDesc* __restrict__ tdesc, psk::LruMeta meta,
                     EvictPlan* plan, const uint32_t* __restrict__ list, const uint32_t* __restrict__ nlist,
-                    uint64_t chunks, uint32_t* __restrict__ cand) {
+                    uint64_t chunks, EvictBlocks eb) {
   const uint64_t items = (uint64_t)*nlist * chunks;
   const uint32_t lane = threadIdx.x & 31u;
   for (uint64_t item = blockIdx.x; item < items; item += gridDim.x) {
@@ -720,24 +755,17 @@ evict_gather_kernel(const uint64_t* __restrict__ slots, const psk::TableDesc* __
     const uint64_t n = (uint64_t)d.nbkt * psk::kBucketSlots, x0 = (item % chunks) * kScanChunk;
     const uint64_t x1 = x0 + kScanChunk < n ? x0 + kScanChunk : n;
     const uint32_t T = plan[i].lo;
-    uint32_t* out = cand + (uint64_t)i * 2u * kClassMax;
+    uint32_t* out = eb.slot + (item / chunks) * 2u * kClassMax;
     for (uint64_t xb = x0; xb < x1; xb += 4u * kScanThreads) {  // (tables are whole 8-slot buckets)
       const uint64_t x = xb + 4u * threadIdx.x;
-      uint4 lu = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
-      const bool in = x < x1;
-      if (in) lu = __ldcs(reinterpret_cast<const uint4*>(meta.last_use + d.base + x));
+      uint4 lu = make_uint4(psk::kNoUse, psk::kNoUse, psk::kNoUse, psk::kNoUse);
+      if (x < x1) lu = __ldcs(reinterpret_cast<const uint4*>(meta.last_use + d.base + x));
       const uint32_t l[4] = {lu.x, lu.y, lu.z, lu.w};
       uint32_t oldm = 0u, clsm = 0u;
-      if (in && (l[0] <= T || l[1] <= T || l[2] <= T || l[3] <= T)) {
-        const ulonglong2 a = __ldcs(reinterpret_cast<const ulonglong2*>(slots + d.base + x));
-        const ulonglong2 b = __ldcs(reinterpret_cast<const ulonglong2*>(slots + d.base + x + 2));
-        const uint64_t key[4] = {a.x, a.y, b.x, b.y};
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (key[u] != psk::kEmpty) {
-            oldm |= (l[u] < T ? 1u : 0u) << u;
-            clsm |= (l[u] == T ? 1u : 0u) << u;
-          }
+      for (int u = 0; u < 4; ++u) {  // (T is never the mark of an empty slot)
+        oldm |= (l[u] < T ? 1u : 0u) << u;
+        clsm |= (l[u] == T ? 1u : 0u) << u;
       }
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
@@ -764,6 +792,69 @@ evict_gather_kernel(const uint64_t* __restrict__ slots, const psk::TableDesc* __
   }
 }
 
+constexpr uint32_t kDetailThreads = 512;
+
+__global__ void __launch_bounds__(kDetailThreads)
+evict_detail_kernel(const uint64_t* __restrict__ slots, psk::LruMeta meta, EvictPlan* plan,
+                    const uint32_t* __restrict__ list, const uint32_t* __restrict__ nlist, EvictBlocks eb) {
+  constexpr uint32_t kChunks = 2u * kClassMax / kDetailThreads;
+  const uint32_t items = *nlist * kChunks;
+  for (uint32_t item = blockIdx.x; item < items; item += gridDim.x) {
+    const uint32_t q = item / kChunks, x0 = (item % kChunks) * kDetailThreads;
+    const uint32_t i = list[q];
+    const EvictPlan p = plan[i];
+    const bool cls = x0 >= kClassMax;
+    const uint32_t n = cls ? p.n_cls : p.n_old, x = (cls ? x0 - kClassMax : x0) + threadIdx.x;
+    if (!p.fits() || (cls ? x0 - kClassMax : x0) >= n) continue;  // block-uniform
+    uint32_t ch = 0u, in = 0u;
+    bool bad = false;
+    if (x < n) {
+      const uint64_t at = (uint64_t)q * 2u * kClassMax + x0 + threadIdx.x;
+      const uint32_t sl = eb.slot[at];
+      ch = meta.children[sl];
+      const uint32_t ps = parent32(meta.parent[sl]);
+      const uint32_t lu = cls ? p.lo : meta.last_use[sl];
+      if (cls) eb.key[(uint64_t)q * kClassMax + x] = slots[sl];
+      uint8_t rel = kRelNone;
+      if (ps != kLeafNoParent) {
+        const uint32_t lp = meta.last_use[ps];
+        rel = lp < p.lo ? kRelOlder : (lp == p.lo ? kRelClass : kRelNewer);
+        in = lp <= p.lo;
+        bad = lp < lu;
+      }
+      eb.par[at] = ps;
+      eb.rel[at] = rel;
+    }
+    ch = __reduce_add_sync(0xffffffffu, ch);
+    in = __reduce_add_sync(0xffffffffu, in);
+    const bool anybad = __any_sync(0xffffffffu, bad);
+    if ((threadIdx.x & 31u) == 0u) {
+      if (ch) atomicAdd(&plan[i].children, ch);
+      if (in) atomicAdd(&plan[i].inside, in);
+      if (anybad) atomicOr(&plan[i].bad, 1u);
+    }
+  }
+}
+
+// JUMP false: a class block's index stands in for its (known) stamp; true: its parent's index is read.
+template <bool JUMP>
+__global__ void __launch_bounds__(kDetailThreads)
+evict_index_kernel(psk::LruMeta meta, const EvictPlan* __restrict__ plan, const uint32_t* __restrict__ list,
+                   const uint32_t* __restrict__ nlist, uint32_t max_leaves, EvictBlocks eb) {
+  constexpr uint32_t kChunks = kClassMax / kDetailThreads;
+  const uint32_t items = *nlist * kChunks;
+  for (uint32_t item = blockIdx.x; item < items; item += gridDim.x) {
+    const uint32_t q = item / kChunks, x = (item % kChunks) * kDetailThreads + threadIdx.x;
+    const EvictPlan& p = plan[list[q]];
+    if (!p.fits() || !p.in_order() || p.leaves > max_leaves || p.k >= p.n_cls || x >= p.n_cls) continue;
+    const uint64_t at = (uint64_t)q * 2u * kClassMax + kClassMax + x;
+    if (!JUMP) meta.last_use[eb.slot[at]] = x;
+    else
+      eb.jump[(uint64_t)q * kClassMax + x] =
+          (uint16_t)(eb.rel[at] == kRelClass ? meta.last_use[eb.par[at]] : kNoJump);
+  }
+}
+
 struct OrderSmem {
   unsigned long long M[kClassMax];  // subtree maximum of the hash over the class
   uint16_t jump[kClassMax];         // ancestor 2^r links up (kNoJump: past the class)
@@ -777,94 +868,48 @@ struct OrderSmem {
 __global__ void __launch_bounds__(kOrderThreads)
 evict_order_kernel(uint64_t* slots, unsigned long long* count, const uint64_t* __restrict__ cap, psk::LruMeta meta,
                    const EvictPlan* __restrict__ plan, const uint32_t* __restrict__ list,
-                   const uint32_t* __restrict__ nlist, const uint32_t* __restrict__ cand, uint32_t* slow, uint32_t* more,
+                   const uint32_t* __restrict__ nlist, EvictBlocks eb, uint32_t* slow, uint32_t* more,
                    uint32_t max_leaves, uint32_t* err) {
   extern __shared__ __align__(16) unsigned char order_raw[];
   OrderSmem& s = *reinterpret_cast<OrderSmem*>(order_raw);
-  __shared__ unsigned long long s_children, s_inside;
   const uint32_t t = threadIdx.x;
   for (uint32_t item = blockIdx.x; item < *nlist; item += gridDim.x) {
     const uint32_t i = list[item];
     const EvictPlan p = plan[i];
     const uint32_t T = p.lo, n = p.n_cls, n_old = p.n_old;
     if (p.leaves > max_leaves) {  // (the limit of the one-at-a-time kernels, kept for every instance)
-      if (t == 0) atomicOr(err, psk::kErrLeavesFull);
+      if (t == 0) {
+        atomicOr(err, psk::kErrLeavesFull);
+        slow[i] = 2u;  // not evicted in this call
+      }
       continue;
     }
-    if (n > kClassMax || n_old > kClassMax) {
+    if (!p.fits() || !p.in_order()) {
       if (t == 0) {
         slow[i] = 1u;
         atomicOr(more, kMoreSlow);
       }
       continue;
     }
-    const uint32_t* old_slots = cand + (uint64_t)i * 2u * kClassMax;
+    const uint32_t* old_slots = eb.slot + (uint64_t)item * 2u * kClassMax;
     const uint32_t* cls_slots = old_slots + kClassMax;
-    // check: every child of these blocks is one of them, and no child is newer than its parent
-    uint32_t slot[kOrderPer], par[kOrderPer];  // this thread's class blocks: slot, parent's slot if in the class
-    unsigned long long children = 0, inside = 0;
-    bool bad = false;
-#pragma unroll
-    for (uint32_t u = 0; u < kOrderPer; ++u) {
-      const uint32_t x = t + u * kOrderThreads;
-      slot[u] = par[u] = kLeafNoParent;
-      if (x < n) {
-        slot[u] = cls_slots[x];
-        children += meta.children[slot[u]];
-        const uint32_t ps = parent32(meta.parent[slot[u]]);
-        if (ps != kLeafNoParent) {
-          const uint32_t lp = meta.last_use[ps];
-          if (lp <= T) ++inside;
-          if (lp < T) bad = true;
-          if (lp == T) par[u] = ps;
-        }
-      }
-    }
-    for (uint32_t x = t; x < n_old; x += kOrderThreads) {
-      const uint32_t sl = old_slots[x];
-      children += meta.children[sl];
-      const uint32_t ps = parent32(meta.parent[sl]);
-      if (ps != kLeafNoParent) {
-        const uint32_t lp = meta.last_use[ps];
-        if (lp <= T) ++inside;
-        if (lp < meta.last_use[sl]) bad = true;
-      }
-    }
-    if (t == 0) {
-      s_children = 0ull;
-      s_inside = 0ull;
-    }
-    __syncthreads();
-    if (children) atomicAdd(&s_children, children);
-    if (inside) atomicAdd(&s_inside, inside);
-    bad = __syncthreads_or(bad ? 1 : 0) != 0;
-    if (bad || s_children != s_inside) {  // block-uniform
-      if (t == 0) {
-        slow[i] = 1u;
-        atomicOr(more, kMoreSlow);
-      }
-      __syncthreads();
-      continue;
-    }
-    uint32_t gone = 0u;  // bit u: this thread's class block u is evicted
-    if (p.k >= n) {
+    const uint32_t* old_par = eb.par + (uint64_t)item * 2u * kClassMax;
+    const uint32_t* cls_par = old_par + kClassMax;
+    const uint8_t* old_rel = eb.rel + (uint64_t)item * 2u * kClassMax;
+    const uint8_t* cls_rel = old_rel + kClassMax;
+    const bool whole = p.k >= n;
+    uint32_t gone = 0u;  // bit u: this thread's class block t + u kOrderThreads is evicted
+    if (whole) {
       gone = (1u << kOrderPer) - 1u;
     } else {
-      // A class block's index stands in for its (known) stamp while its children look it up.
 #pragma unroll
       for (uint32_t u = 0; u < kOrderPer; ++u) {
         const uint32_t x = t + u * kOrderThreads;
         if (x < n) {
-          meta.last_use[slot[u]] = x;
-          s.M[x] = slots[slot[u]];
+          s.M[x] = eb.key[(uint64_t)item * kClassMax + x];
+          s.jump[x] = eb.jump[(uint64_t)item * kClassMax + x];
           s.dep[x] = 1;
         }
-      }
-      __syncthreads();
-#pragma unroll
-      for (uint32_t u = 0; u < kOrderPer; ++u) {
-        const uint32_t x = t + u * kOrderThreads;
-        if (x < n) s.jump[x] = (uint16_t)(par[u] != kLeafNoParent ? __ldcg(meta.last_use + par[u]) : kNoJump);
       }
       __syncthreads();
       for (;;) {  // at most 14 rounds: a path holds at most kClassMax blocks
@@ -879,7 +924,8 @@ evict_order_kernel(uint64_t* slots, unsigned long long* count, const uint64_t* _
           if (x < n && s.jump[x] != kNoJump) {
             const uint32_t j = s.jump[x];
             any = true;
-            atomicMax(&s.M[j], s.M[x]);
+            const unsigned long long v = s.M[x];
+            if (s.M[j] < v) atomicMax(&s.M[j], v);
             nj[u] = s.jump[j];
             nd[u] = s.dep[j];
           }
@@ -909,7 +955,18 @@ evict_order_kernel(uint64_t* slots, unsigned long long* count, const uint64_t* _
 #pragma unroll
         for (uint32_t u = 0; u < kOrderPer; ++u) {
           const uint32_t x = t + u * kOrderThreads;
-          if (x < n && (s.M[x] & high) == sel) atomicAdd(&s.hist[(s.M[x] >> sh) & 255u], 1u);
+          // maxima crowd into few values of the upper bytes: a warp of one value adds once
+          const unsigned long long v = x < n ? s.M[x] : 0ull;
+          const bool in = x < n && (v & high) == sel;
+          const uint32_t digit = in ? (uint32_t)(v >> sh) & 255u : 256u;
+          const unsigned im = __ballot_sync(0xffffffffu, in);
+          if (im == 0u) continue;
+          const uint32_t d0 = __shfl_sync(0xffffffffu, digit, __ffs(im) - 1);
+          if (__all_sync(0xffffffffu, !in || digit == d0)) {
+            if ((t & 31u) == (uint32_t)__ffs(im) - 1u) atomicAdd(&s.hist[d0], (uint32_t)__popc(im));
+          } else if (in) {
+            atomicAdd(&s.hist[digit], 1u);
+          }
         }
         __syncthreads();
         if (t < 32) {  // the bin that holds the rank
@@ -955,38 +1012,31 @@ evict_order_kernel(uint64_t* slots, unsigned long long* count, const uint64_t* _
         if (x < n && (s.M[x] < cut || (s.M[x] == cut && s.dep[x] + rank >= dm))) gone |= 1u << u;
       }
     }
-    // evict: the slots first, then the surviving parents' counts, then the evicted blocks' own links
+    // evict: the slots first, then the counts of the parents that stay (an evicted slot keeps its links:
+    // whoever fills it sets its parent and children)
 #pragma unroll
     for (uint32_t u = 0; u < kOrderPer; ++u) {
-      if (slot[u] == kLeafNoParent) continue;
+      const uint32_t x = t + u * kOrderThreads;
+      if (x >= n) continue;
       const bool g = (gone >> u) & 1u;
-      if (g) slots[slot[u]] = psk::kEmpty;
-      meta.last_use[slot[u]] = g ? 0u : T;
+      if (g) slots[cls_slots[x]] = psk::kEmpty;
+      if (g || !whole) meta.last_use[cls_slots[x]] = g ? psk::kNoUse : T;
     }
     for (uint32_t x = t; x < n_old; x += kOrderThreads) {
       slots[old_slots[x]] = psk::kEmpty;
-      meta.last_use[old_slots[x]] = 0u;
+      meta.last_use[old_slots[x]] = psk::kNoUse;
     }
     __syncthreads();
-    auto drop = [&](uint32_t sl) {
-      const uint32_t ps = parent32(meta.parent[sl]);
-      if (ps != kLeafNoParent && __ldcg(slots + ps) != psk::kEmpty) atomicSub(meta.children + ps, 1u);
+    auto drop = [&](uint32_t ps, uint8_t rel) {
+      if (rel == kRelNewer || (rel == kRelClass && !whole && __ldcg(slots + ps) != psk::kEmpty))
+        atomicSub(meta.children + ps, 1u);
     };
 #pragma unroll
-    for (uint32_t u = 0; u < kOrderPer; ++u)
-      if (slot[u] != kLeafNoParent && ((gone >> u) & 1u)) drop(slot[u]);
-    for (uint32_t x = t; x < n_old; x += kOrderThreads) drop(old_slots[x]);
-    __syncthreads();
-#pragma unroll
-    for (uint32_t u = 0; u < kOrderPer; ++u)
-      if (slot[u] != kLeafNoParent && ((gone >> u) & 1u)) {
-        meta.children[slot[u]] = 0u;
-        meta.parent[slot[u]] = psk::kNoParent;
-      }
-    for (uint32_t x = t; x < n_old; x += kOrderThreads) {
-      meta.children[old_slots[x]] = 0u;
-      meta.parent[old_slots[x]] = psk::kNoParent;
+    for (uint32_t u = 0; u < kOrderPer; ++u) {
+      const uint32_t x = t + u * kOrderThreads;
+      if (x < n && ((gone >> u) & 1u)) drop(cls_par[x], cls_rel[x]);
     }
+    for (uint32_t x = t; x < n_old; x += kOrderThreads) drop(old_par[x], old_rel[x]);
     if (t == 0) {
       const unsigned long long c = count[i] - p.todo;
       count[i] = c;
@@ -1175,7 +1225,7 @@ leaf_collect_kernel(const uint64_t* __restrict__ slots, const psk::TableDesc* __
                     const unsigned long long* __restrict__ count, const uint64_t* __restrict__ cap, psk::LruMeta meta,
                     const uint32_t* __restrict__ slow, Leaf* __restrict__ leafbuf, uint32_t* __restrict__ nleaf) {
   const uint32_t i = blockIdx.y;
-  if (!slow[i] || count[i] <= cap[i]) return;  // block-uniform
+  if (slow[i] != 1u || count[i] <= cap[i]) return;  // block-uniform
   const psk::TableDesc d = tdesc[i];
   const uint64_t nslots = (uint64_t)d.nbkt * psk::kBucketSlots;
   const uint64_t stride = (uint64_t)gridDim.x * kCollectThreads;
@@ -1203,7 +1253,7 @@ evict_kernel(uint64_t* slots, unsigned long long* count, const uint64_t* __restr
   Leaf* heap = reinterpret_cast<Leaf*>(ev_smem + kOffHeap);
   const uint32_t i = blockIdx.x;
   const unsigned long long cnt = count[i];
-  if (!slow[i] || cnt <= cap[i]) return;  // block-uniform
+  if (slow[i] != 1u || cnt <= cap[i]) return;  // block-uniform
   // an earlier round gave up: no more rounds (read once, so that the whole block leaves together)
   if (__syncthreads_or(threadIdx.x == 0 && (*(volatile uint32_t*)err & psk::kErrTimeout) != 0u)) return;
   const uint32_t n = nleaf[i];
@@ -1279,7 +1329,7 @@ evict_kernel(uint64_t* slots, unsigned long long* count, const uint64_t* __restr
         }
       }
       slots[v.slot] = psk::kEmpty;
-      meta.last_use[v.slot] = 0;
+      meta.last_use[v.slot] = psk::kNoUse;
       meta.children[v.slot] = 0;
       meta.parent[v.slot] = psk::kNoParent;
       ++evicted;
@@ -1398,6 +1448,14 @@ cudaError_t launch_evict(uint64_t* slots, const psk::TableDesc* tdesc, uint32_t 
     e = cudaFuncSetAttribute(evict_order_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(OrderSmem));
   if (e != cudaSuccess) return e;
   EvictPlan* plan = static_cast<EvictPlan*>(sc.plan);
+  const uint64_t nb = I < kEvictBatch ? I : kEvictBatch;  // instances a round
+  uint32_t* const nlist = sc.list + nb;
+  EvictBlocks eb;
+  eb.key = static_cast<uint64_t*>(sc.blocks);
+  eb.slot = reinterpret_cast<uint32_t*>(eb.key + nb * kClassMax);
+  eb.par = eb.slot + nb * 2u * kClassMax;
+  eb.jump = reinterpret_cast<uint16_t*>(eb.par + nb * 2u * kClassMax);
+  eb.rel = reinterpret_cast<uint8_t*>(eb.jump + nb * kClassMax);
   const uint64_t chunks = (max_instance_slots + kScanChunk - 1) / kScanChunk;
   const unsigned scan_grid = (unsigned)num_sms * 4u;
   const unsigned inst_grid = I < (uint32_t)num_sms ? I : (unsigned)num_sms;
@@ -1411,16 +1469,17 @@ cudaError_t launch_evict(uint64_t* slots, const psk::TableDesc* tdesc, uint32_t 
   for (int round = 0; round < 4096 && todo; ++round) {
     if ((e = cudaMemsetAsync(sc.more, 0, sizeof(uint32_t), s)) != cudaSuccess) return e;
     if (todo & kMoreFast) {
-      evict_list_kernel<<<1, 1024, 0, s>>>(I, count, cap, sc.slow, max_use, plan, sc.list, sc.list + I);
+      evict_list_kernel<<<1, 1024, 0, s>>>(I, count, cap, sc.slow, max_use, plan, sc.list, nlist, sc.more);
       for (int pass = 0; pass < passes; ++pass) {
-        evict_hist_kernel<<<scan_grid, kScanThreads, 0, s>>>(slots, tdesc, meta, plan, sc.list, sc.list + I, chunks,
-                                                            sc.hist, pass == 0);
-        evict_choose_kernel<<<inst_grid, 256, 0, s>>>(plan, sc.list, sc.list + I, sc.hist);
+        evict_hist_kernel<<<scan_grid, kScanThreads, 0, s>>>(tdesc, meta, plan, sc.list, nlist, chunks, sc.hist, pass == 0);
+        evict_choose_kernel<<<inst_grid, 256, 0, s>>>(plan, sc.list, nlist, sc.hist);
       }
-      evict_gather_kernel<<<scan_grid, kScanThreads, 0, s>>>(slots, tdesc, meta, plan, sc.list, sc.list + I, chunks,
-                                                            sc.cand);
-      evict_order_kernel<<<inst_grid, kOrderThreads, sizeof(OrderSmem), s>>>(
-          slots, count, cap, meta, plan, sc.list, sc.list + I, sc.cand, sc.slow, sc.more, (uint32_t)kLeafMax, err);
+      evict_gather_kernel<<<scan_grid, kScanThreads, 0, s>>>(tdesc, meta, plan, sc.list, nlist, chunks, eb);
+      evict_detail_kernel<<<scan_grid, kDetailThreads, 0, s>>>(slots, meta, plan, sc.list, nlist, eb);
+      evict_index_kernel<false><<<scan_grid, kDetailThreads, 0, s>>>(meta, plan, sc.list, nlist, kLeafMax, eb);
+      evict_index_kernel<true><<<scan_grid, kDetailThreads, 0, s>>>(meta, plan, sc.list, nlist, kLeafMax, eb);
+      evict_order_kernel<<<inst_grid, kOrderThreads, sizeof(OrderSmem), s>>>(slots, count, cap, meta, plan, sc.list, nlist,
+                                                                            eb, sc.slow, sc.more, kLeafMax, err);
     }
     if (todo & kMoreSlow) {
       if ((e = cudaMemsetAsync(sc.nleaf, 0, (size_t)I * sizeof(uint32_t), s)) != cudaSuccess) return e;
@@ -1438,8 +1497,10 @@ cudaError_t launch_evict(uint64_t* slots, const psk::TableDesc* tdesc, uint32_t 
 }
 
 size_t evict_plan_bytes(uint32_t I) { return (size_t)I * sizeof(EvictPlan); }
-size_t evict_hist_words(uint32_t I) { return (size_t)I * kHistBins; }
-size_t evict_cand_words(uint32_t I) { return (size_t)I * 2u * kClassMax; }
+size_t evict_hist_words(uint32_t I) { return (size_t)(I < kEvictBatch ? I : kEvictBatch) * kHistBins; }
+size_t evict_blocks_bytes(uint32_t I) {  // per block: hash, two slots and parents, jump, two relations
+  return (size_t)(I < kEvictBatch ? I : kEvictBatch) * kClassMax * (8 + 2 * 4 + 2 * 4 + 2 + 2);
+}
 
 size_t evict_leafbuf_bytes(uint32_t I) { return (size_t)I * kLeafMax * sizeof(Leaf); }
 

@@ -106,3 +106,8 @@ def test_children_newer_than_their_parents(P):
     # the others stay in order
     later = [(i, _blocks(rng, 20), int(b[-1 if i == 0 else 0])) for i, b, _ in first if i < 2]
     _run(P, 4, [(first, 1), (later, 6), (_chains(rng, 4, 40, 30), 3)], 500)
+
+
+def test_more_instances_than_a_round(P):
+    rng = np.random.default_rng(6)
+    _run(P, 300, [(_chains(rng, 300, 1500, 8), k) for k in range(3)], 20)
