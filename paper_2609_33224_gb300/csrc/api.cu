@@ -344,7 +344,8 @@ cudaError_t deliver(ps_ctx* c, T* dst, const T* src, size_t n, int on_device) {
 
 void record(ps_ctx* c, int ev) { cudaEventRecord(c->ev[ev], c->stream); }
 
-ps_status run_probe_and_score(ps_ctx* c, const psk::WindowDev& wd, ps_scores* out, uint32_t** hits_used) {
+// want_tpf: the greedy pass follows and reads T_pf at every pair's hit.
+ps_status run_probe_and_score(ps_ctx* c, const psk::WindowDev& wd, ps_scores* out, uint32_t** hits_used, bool want_tpf) {
   const int dev_out = out ? out->outputs_on_device : 0;
   uint32_t* hits = (out && out->hits && dev_out) ? out->hits : c->d_hits;
   PS_TRY_CUDA(c, cudaMemsetAsync(c->d_stats, 0, kNumStats * sizeof(unsigned long long), c->stream));
@@ -353,7 +354,8 @@ ps_status run_probe_and_score(ps_ctx* c, const psk::WindowDev& wd, ps_scores* ou
   PS_TRY_CUDA(c, pskl::launch_relations(wd, c->model, c->d_lastslot, c->lastslot_n, c->d_rows, c->scratch, c->search,
                                         c->num_sms, c->stream));
   record(c, kEvRelDone);
-  PS_TRY_CUDA(c, pskl::launch_probe(c->d_slots, c->d_ovf, c->d_tdesc, c->I, wd, c->d_rows, c->scratch, hits, c->d_tpf,
+  PS_TRY_CUDA(c, pskl::launch_probe(c->d_slots, c->d_ovf, c->d_tdesc, c->I, wd, c->d_rows, c->scratch, hits,
+                                    want_tpf ? c->d_tpf : nullptr,
                                     c->model, c->probe_grid, c->search, c->d_stats, c->ev[kEvProbeMid], c->stream));
   record(c, kEvProbe1);
   c->ev_used[0] = true;
@@ -468,7 +470,7 @@ ps_status ps_create(const ps_config* cfg, ps_ctx** out) {
             dalloc(c, &c->gsync.stats, psk::kGreedyStats) == cudaSuccess &&
             dalloc(c, &c->gsync.hitring, (size_t)psk::kHitSlots * c->gsync.ring_stride) == cudaSuccess &&
             dalloc(c, &c->gsync.tpfring, (size_t)psk::kHitSlots * c->gsync.ring_stride) == cudaSuccess &&
-            dalloc(c, &c->d_rows, c->Rmax) == cudaSuccess && dalloc(c, &c->d_lastslot, c->lastslot_n) == cudaSuccess &&
+            dalloc(c, &c->d_rows, c->Rmax) == cudaSuccess && dalloc(c, &c->d_lastslot, c->lastslot_n + c->lastslot_n / 16) == cudaSuccess &&
             dalloc(c, &c->scratch.rows, c->Rmax) == cudaSuccess && dalloc(c, &c->scratch.count, 1) == cudaSuccess &&
             dalloc(c, &c->d_cprefix, 2 * ((size_t)c->Rmax + 1)) == cudaSuccess;
   for (psk::StateSoA* s : {&c->st, &c->pend}) {
@@ -759,7 +761,7 @@ ps_status ps_score_window(ps_ctx* c, const ps_window* w, ps_scores* out) {
   ps_status s = stage_window(c, w, &wd);
   if (s != PS_OK) return s;
   uint32_t* hits = nullptr;
-  s = run_probe_and_score(c, wd, out, &hits);
+  s = run_probe_and_score(c, wd, out, &hits, false);
   if (s != PS_OK) return s;
   return finish(c);
 }
@@ -774,7 +776,7 @@ ps_status ps_shard_wmin(ps_ctx* c, const ps_window* w, uint32_t* wmin_ord, int32
   if (s != PS_OK) return s;
   if (wd.R > 0 && !wmin_ord) return fail(c, PS_ERR_INVALID, "wmin_ord is NULL");
   uint32_t* hits = nullptr;
-  s = run_probe_and_score(c, wd, nullptr, &hits);  // the probe phase only: hits into the context's buffer
+  s = run_probe_and_score(c, wd, nullptr, &hits, false);  // the probe phase only: hits into the context's buffer
   if (s != PS_OK) return s;
   psk::ShardIO sh;
   sh.wmin_out = on_device ? wmin_ord : c->d_shard_wmin;
@@ -860,7 +862,7 @@ ps_status ps_schedule_window(ps_ctx* c, const ps_window* w, ps_decisions* out, p
   ps_status s = stage_window(c, w, &wd);
   if (s != PS_OK) return s;
   uint32_t* hit0 = nullptr;
-  s = run_probe_and_score(c, wd, opt_scores, &hit0);
+  s = run_probe_and_score(c, wd, opt_scores, &hit0, true);
   if (s != PS_OK) return s;
   record(c, kEvGreedy0);
   PS_TRY_CUDA(c, pskl::launch_greedy(c->d_rows, wd, c->I, hit0, c->d_tpf, c->st, c->pend, c->model, c->d_delta,
