@@ -7,6 +7,7 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include <algorithm>
@@ -24,6 +25,11 @@ enum Ev { kEvProbe0, kEvProbe1, kEvScore0, kEvScore1, kEvGreedy0, kEvGreedy1, kE
 constexpr int kNumPhases = 4;
 constexpr int kNumStats = 6;
 constexpr uint64_t kDefaultWaitNs = 1000000000ull;  // 1 s: bound on a cross-block wait of the greedy
+constexpr size_t kStateBytes = 36;                  // per instance: q, S, M_KV (8 each), b, qr, B_max (4 each)
+// Page-locked staging.  A small host window's arrays are packed there and copied in one piece, small
+// results land there and are handed on after the call's one synchronisation: a copy from or to ordinary
+// memory costs 8 to 10 us and waits, and a call would make up to seven of them.
+constexpr size_t kStageIn = 1u << 20, kStageOut = 1u << 18;
 
 struct DeviceGuard {
   int prev = -1;
@@ -56,8 +62,8 @@ struct ps_ctx {
   psk::TableDesc* d_tdesc = nullptr;
   unsigned long long* d_count = nullptr;
   psk::DeltaSlot* d_delta = nullptr;
-  uint64_t delta_nslots = 0;
-  psk::GreedySync gsync{nullptr, nullptr, nullptr, nullptr, nullptr, 0u, kDefaultWaitNs, nullptr};
+  uint64_t delta_nslots = 0;  // allocated; a window uses twice its own blocks
+  psk::GreedySync gsync{nullptr, nullptr, nullptr, nullptr, nullptr, 0u, kDefaultWaitNs, nullptr, 0};
   psk::RowPre* d_rows = nullptr;      // per-request constants and relations (search mode greedy)
   psk::LastSlot* d_lastslot = nullptr;
   psk::RowList scratch{nullptr, nullptr};  // rows the probe searches from scratch
@@ -83,9 +89,22 @@ struct ps_ctx {
   int32_t* d_assign = nullptr;
   uint8_t* d_dpath = nullptr;
   uint32_t* d_hchosen = nullptr;
-  uint32_t* d_err = nullptr;
-  uint32_t* h_err = nullptr;   // pinned: the device error word, read at the end of each call
-  uint32_t* h_more = nullptr;  // pinned: "another eviction round" flag
+  uint32_t* d_err = nullptr;     // [4]: the error word, -, a device window's number of blocks (u64)
+  unsigned char* h_pin = nullptr;  // one page-locked block for the four below
+  uint32_t* h_err = nullptr;     // [4] copy of d_err, read at the end of each call
+  uint32_t* h_more = nullptr;    // "another eviction round" flag
+  unsigned char* h_in = nullptr;   // [max(kStageIn, I * kStateBytes)]
+  unsigned char* h_out = nullptr;  // [kStageOut]
+  size_t h_out_used = 0;
+  struct Handover {
+    void* dst;
+    const void* src;
+    size_t bytes;
+  };
+  std::vector<Handover> handover;  // results to hand on from h_out once the stream is done
+  unsigned char* d_stage = nullptr;  // [kStageIn] a small host window's arrays
+  uint64_t win_blocks = 0;         // chain blocks of the window being staged
+  unsigned char *st_block = nullptr, *pend_block = nullptr, *gsync_block = nullptr, *zero_block = nullptr;
   cudaEvent_t ev[kNumEv] = {};
   bool ev_used[kNumPhases] = {};
   bool probe_split = false;            // kEvRelDone / kEvProbeMid recorded in the last probe phase
@@ -109,14 +128,18 @@ struct ps_ctx {
   psk::ReqStore rq{};
   uint64_t* d_cap = nullptr;
   uint32_t* d_outtok = nullptr;
-  std::vector<void*> allocs;
+  std::vector<std::pair<void**, size_t>> wanted;  // ps_create: blocks to lay out in the arena
+  void* arena = nullptr;                          // every device block of the context, one allocation
   std::string err;
 };
 
 namespace {
 
 ps_status fail(ps_ctx* c, ps_status s, const std::string& msg) {
-  if (c) c->err = msg;
+  if (c) {
+    c->err = msg;
+    c->handover.clear();  // a call that fails hands nothing on, then or later
+  }
   return s;
 }
 
@@ -127,15 +150,37 @@ ps_status fail(ps_ctx* c, ps_status s, const std::string& msg) {
       return fail((ctx), PS_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_));         \
   } while (0)
 
+// Registers a device block; alloc_arena lays all of them out in one allocation (an allocation each made
+// up most of a context's creation and destruction).
 template <class T>
-cudaError_t dalloc(ps_ctx* c, T** p, size_t count) {
-  void* v = nullptr;
-  const size_t bytes = count ? count * sizeof(T) : sizeof(T);
-  cudaError_t e = cudaMalloc(&v, bytes);
+void want(ps_ctx* c, T** p, size_t count) {
+  c->wanted.emplace_back(reinterpret_cast<void**>(p), (count ? count : 1) * sizeof(T));
+}
+
+cudaError_t alloc_arena(ps_ctx* c) {
+  constexpr size_t kAlign = 256;
+  size_t total = 0;
+  for (const auto& w : c->wanted) total += (w.second + kAlign - 1) / kAlign * kAlign;
+  cudaError_t e = cudaMalloc(&c->arena, total);
   if (e != cudaSuccess) return e;
-  c->allocs.push_back(v);
-  *p = static_cast<T*>(v);
+  unsigned char* at = static_cast<unsigned char*>(c->arena);
+  for (const auto& w : c->wanted) {
+    *w.first = at;
+    at += (w.second + kAlign - 1) / kAlign * kAlign;
+  }
+  c->wanted.clear();
   return cudaSuccess;
+}
+
+psk::StateSoA state_arrays(unsigned char* block, size_t I) {
+  psk::StateSoA s;
+  s.q = reinterpret_cast<int64_t*>(block);
+  s.S = s.q + I;
+  s.M = s.S + I;
+  s.b = reinterpret_cast<int32_t*>(s.M + I);
+  s.qr = s.b + I;
+  s.Bmax = s.qr + I;
+  return s;
 }
 
 bool finite_small(float x) { return std::isfinite(x) && std::fabs(x) <= 1e9f; }
@@ -199,10 +244,14 @@ ps_status device_errors(ps_ctx* c) {
   return fail(c, PS_ERR_CUDA, "unknown device error");
 }
 
-// Synchronise the stream, read the device error word, and reset it for the next call.
+// Synchronise the stream, hand staged results on, read the device error word, and reset it for the next
+// call.
 ps_status finish(ps_ctx* c) {
-  PS_TRY_CUDA(c, cudaMemcpyAsync(c->h_err, c->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, c->stream));
+  PS_TRY_CUDA(c, cudaMemcpyAsync(c->h_err, c->d_err, 4 * sizeof(uint32_t), cudaMemcpyDeviceToHost, c->stream));
   PS_TRY_CUDA(c, cudaStreamSynchronize(c->stream));
+  c->h_out_used = 0;
+  for (const ps_ctx::Handover& x : c->handover) std::memcpy(x.dst, x.src, x.bytes);
+  c->handover.clear();
   ps_status s = device_errors(c);
   if (*c->h_err) {
     PS_TRY_CUDA(c, cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), c->stream));
@@ -213,8 +262,10 @@ ps_status finish(ps_ctx* c) {
 }
 
 ps_status check_capacity(ps_ctx* c) {
-  std::vector<unsigned long long> cnt(c->I);
-  PS_TRY_CUDA(c, cudaMemcpy(cnt.data(), c->d_count, c->I * sizeof(unsigned long long), cudaMemcpyDeviceToHost));
+  const unsigned long long* cnt = reinterpret_cast<const unsigned long long*>(c->h_in);
+  PS_TRY_CUDA(c, cudaMemcpyAsync(c->h_in, c->d_count, c->I * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
+                                 c->stream));
+  PS_TRY_CUDA(c, cudaStreamSynchronize(c->stream));
   for (uint32_t i = 0; i < c->I; ++i)
     if (cnt[i] > c->cap[i])
       return fail(c, PS_ERR_CAPACITY, "instance " + std::to_string(i) + " holds " + std::to_string(cnt[i]) +
@@ -222,19 +273,44 @@ ps_status check_capacity(ps_ctx* c) {
   return PS_OK;
 }
 
-// Copies the request arrays shared by both window forms (L, targets, output lengths) to the device.
-ps_status stage_request_arrays(ps_ctx* c, const ps_window* w) {
-  if (!w->R) return PS_OK;
-  PS_TRY_CUDA(c, cudaMemcpyAsync(c->d_L, w->prompt_tokens, w->R * sizeof(uint32_t), cudaMemcpyHostToDevice, c->stream));
-  PS_TRY_CUDA(c, cudaMemcpyAsync(c->d_ttft, w->ttft_target, w->R * sizeof(float), cudaMemcpyHostToDevice, c->stream));
-  PS_TRY_CUDA(c, cudaMemcpyAsync(c->d_tpot, w->tpot_target, w->R * sizeof(float), cudaMemcpyHostToDevice, c->stream));
-  if (w->out_tokens) {
-    PS_TRY_CUDA(c, cudaMemcpyAsync(c->d_outtok, w->out_tokens, w->R * sizeof(uint32_t), cudaMemcpyHostToDevice,
-                                   c->stream));
-    c->pend_out = c->d_outtok;
+// Arrays of a host window on their way to the device: packed into the staging block and copied in one
+// piece when they fit (flush), else copied each to its own buffer.
+struct Stager {
+  ps_ctx* c;
+  bool packed;
+  size_t used = 0;
+  cudaError_t err = cudaSuccess;
+  Stager(ps_ctx* ctx, size_t bytes) : c(ctx), packed(bytes + 8 * 256 <= kStageIn) {}
+  template <class T>
+  const T* put(const T* src, size_t n, T* own) {
+    if (n == 0) return own;
+    if (!packed) {
+      const cudaError_t e = cudaMemcpyAsync(own, src, n * sizeof(T), cudaMemcpyHostToDevice, c->stream);
+      if (err == cudaSuccess) err = e;
+      return own;
+    }
+    std::memcpy(c->h_in + used, src, n * sizeof(T));
+    const T* at = reinterpret_cast<const T*>(c->d_stage + used);
+    used += (n * sizeof(T) + 255) / 256 * 256;
+    return at;
   }
-  return PS_OK;
+  cudaError_t flush() {
+    if (packed && used && err == cudaSuccess)
+      err = cudaMemcpyAsync(c->d_stage, c->h_in, used, cudaMemcpyHostToDevice, c->stream);
+    return err;
+  }
+};
+
+// The request arrays shared by both window forms (L, targets, output lengths).
+void stage_request_arrays(Stager& st, const ps_window* w, psk::WindowDev* out) {
+  ps_ctx* c = st.c;
+  out->L = st.put(w->prompt_tokens, w->R, c->d_L);
+  out->ttft_t = st.put(w->ttft_target, w->R, c->d_ttft);
+  out->tpot_t = st.put(w->tpot_target, w->R, c->d_tpot);
+  if (w->out_tokens && w->R) c->pend_out = st.put(w->out_tokens, w->R, c->d_outtok);
 }
+
+size_t request_bytes(const ps_window* w) { return (size_t)w->R * (w->out_tokens ? 16 : 12); }
 
 // Shared-prefix form (host inputs): validate the parent links and own-block counts, send each
 // request's own blocks, and rebuild the full chains on the device.
@@ -260,25 +336,18 @@ ps_status stage_window_tree(ps_ctx* c, const ps_window* w, psk::WindowDev* out) 
   const uint64_t nblk = full[R], nown = own[R];
   if (nblk > c->max_blocks) return fail(c, PS_ERR_INVALID, "window exceeds max_window_chain_blocks");
   if (nown > 0 && !w->chain_hash) return fail(c, PS_ERR_INVALID, "chain_hash is NULL");
-  PS_TRY_CUDA(c, cudaMemcpyAsync(c->d_off, full.data(), ((size_t)R + 1) * sizeof(uint64_t), cudaMemcpyHostToDevice,
-                                 c->stream));
-  if (R) {
-    PS_TRY_CUDA(c, cudaMemcpyAsync(c->d_own_off, own, ((size_t)R + 1) * sizeof(uint64_t), cudaMemcpyHostToDevice,
-                                   c->stream));
-    PS_TRY_CUDA(c, cudaMemcpyAsync(c->d_parent, w->parent, R * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream));
-  }
-  if (nown)
-    PS_TRY_CUDA(c, cudaMemcpyAsync(c->d_own_hash, w->chain_hash, nown * sizeof(uint64_t), cudaMemcpyHostToDevice,
-                                   c->stream));
-  ps_status s = stage_request_arrays(c, w);
-  if (s != PS_OK) return s;
-  PS_TRY_CUDA(c, pskl::launch_expand_chains(c->d_off, c->d_own_off, c->d_own_hash, c->d_parent, R, c->d_hash, c->d_err,
-                                            c->num_sms, c->stream));
-  out->off = c->d_off;
+  c->win_blocks = nblk;
+  Stager st(c, 2 * ((size_t)R + 1) * sizeof(uint64_t) + (size_t)R * sizeof(int32_t) + nown * sizeof(uint64_t) +
+                   request_bytes(w));
+  out->off = st.put(static_cast<const uint64_t*>(full.data()), (size_t)R + 1, c->d_off);
+  const uint64_t* d_own_off = st.put(own, R ? (size_t)R + 1 : 0, c->d_own_off);
+  const int32_t* d_parent = st.put(w->parent, R, c->d_parent);
+  const uint64_t* d_own = st.put(w->chain_hash, nown, c->d_own_hash);
+  stage_request_arrays(st, w, out);
+  PS_TRY_CUDA(c, st.flush());
+  PS_TRY_CUDA(c, pskl::launch_expand_chains(out->off, d_own_off, d_own, d_parent, R, c->d_hash, c->d_err, c->num_sms,
+                                            c->stream));
   out->hash = c->d_hash;
-  out->L = c->d_L;
-  out->ttft_t = c->d_ttft;
-  out->tpot_t = c->d_tpot;
   return PS_OK;
 }
 
@@ -292,6 +361,8 @@ ps_status stage_window(ps_ctx* c, const ps_window* w, psk::WindowDev* out) {
     return fail(c, PS_ERR_INVALID, "window array is NULL");
   out->R = w->R;
   c->pend_out = nullptr;
+  c->win_blocks = 0;
+  c->h_out_used = 0;
   if (w->inputs_on_device) {
     if (w->parent) return fail(c, PS_ERR_INVALID, "a window with parent links must be in host memory");
     c->pend_out = w->out_tokens;
@@ -301,11 +372,13 @@ ps_status stage_window(ps_ctx* c, const ps_window* w, psk::WindowDev* out) {
     out->ttft_t = w->ttft_target;
     out->tpot_t = w->tpot_target;
     if (w->R > 0) {
-      PS_TRY_CUDA(c, pskl::launch_validate_window(*out, c->max_blocks, c->d_err, c->stream));
+      PS_TRY_CUDA(c, pskl::launch_validate_window(*out, c->max_blocks, c->d_err,
+                                                  reinterpret_cast<unsigned long long*>(c->d_err + 2), c->stream));
       ps_status s = finish(c);
       if (s != PS_OK) return s;
       uint64_t nblk = 0;
-      PS_TRY_CUDA(c, cudaMemcpy(&nblk, w->chain_off + w->R, sizeof(uint64_t), cudaMemcpyDeviceToHost));
+      std::memcpy(&nblk, c->h_err + 2, sizeof(nblk));
+      c->win_blocks = nblk;
       if (nblk > 0 && !w->chain_hash) return fail(c, PS_ERR_INVALID, "chain_hash is NULL");
     }
     return PS_OK;
@@ -321,16 +394,12 @@ ps_status stage_window(ps_ctx* c, const ps_window* w, psk::WindowDev* out) {
   const uint64_t nblk = off[w->R];
   if (nblk > c->max_blocks) return fail(c, PS_ERR_INVALID, "window exceeds max_window_chain_blocks");
   if (nblk > 0 && !w->chain_hash) return fail(c, PS_ERR_INVALID, "chain_hash is NULL");
-  PS_TRY_CUDA(c, cudaMemcpyAsync(c->d_off, off, (w->R + 1) * sizeof(uint64_t), cudaMemcpyHostToDevice, c->stream));
-  if (nblk)
-    PS_TRY_CUDA(c, cudaMemcpyAsync(c->d_hash, w->chain_hash, nblk * sizeof(uint64_t), cudaMemcpyHostToDevice, c->stream));
-  ps_status s = stage_request_arrays(c, w);
-  if (s != PS_OK) return s;
-  out->off = c->d_off;
-  out->hash = c->d_hash;
-  out->L = c->d_L;
-  out->ttft_t = c->d_ttft;
-  out->tpot_t = c->d_tpot;
+  c->win_blocks = nblk;
+  Stager st(c, ((size_t)w->R + 1 + nblk) * sizeof(uint64_t) + request_bytes(w));
+  out->off = st.put(off, (size_t)w->R + 1, c->d_off);
+  out->hash = st.put(w->chain_hash, nblk, c->d_hash);
+  stage_request_arrays(st, w, out);
+  PS_TRY_CUDA(c, st.flush());
   return PS_OK;
 }
 
@@ -338,6 +407,13 @@ ps_status stage_window(ps_ctx* c, const ps_window* w, psk::WindowDev* out) {
 template <class T>
 cudaError_t deliver(ps_ctx* c, T* dst, const T* src, size_t n, int on_device) {
   if (!dst || n == 0 || dst == src) return cudaSuccess;
+  const size_t bytes = n * sizeof(T);
+  if (!on_device && c->h_out_used + bytes <= kStageOut) {  // handed on by finish()
+    unsigned char* at = c->h_out + c->h_out_used;
+    c->h_out_used += (bytes + 15) / 16 * 16;
+    c->handover.push_back({dst, at, bytes});
+    return cudaMemcpyAsync(at, src, bytes, cudaMemcpyDeviceToHost, c->stream);
+  }
   return cudaMemcpyAsync(dst, src, n * sizeof(T), on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
                          c->stream);
 }
@@ -348,7 +424,8 @@ void record(ps_ctx* c, int ev) { cudaEventRecord(c->ev[ev], c->stream); }
 ps_status run_probe_and_score(ps_ctx* c, const psk::WindowDev& wd, ps_scores* out, uint32_t** hits_used, bool want_tpf) {
   const int dev_out = out ? out->outputs_on_device : 0;
   uint32_t* hits = (out && out->hits && dev_out) ? out->hits : c->d_hits;
-  PS_TRY_CUDA(c, cudaMemsetAsync(c->d_stats, 0, kNumStats * sizeof(unsigned long long), c->stream));
+  // the probe's counters and the length of the list of searched rows
+  PS_TRY_CUDA(c, cudaMemsetAsync(c->zero_block, 0, (kNumStats + 1) * sizeof(unsigned long long), c->stream));
   record(c, kEvProbe0);
   // window relations first: the probe derives the rows of requests that extend an earlier request
   PS_TRY_CUDA(c, pskl::launch_relations(wd, c->model, c->d_lastslot, c->lastslot_n, c->d_rows, c->scratch, c->search,
@@ -462,70 +539,98 @@ ps_status ps_create(const ps_config* cfg, ps_ctx** out) {
   while (c->lastslot_n < 2 * c->Rmax) c->lastslot_n <<= 1;
   const size_t RI = (size_t)c->Rmax * c->I;
   const size_t I = c->I;
+  const size_t Rmax = c->Rmax;
   c->gsync.ring_stride = (c->I + 7u) / 8u * 8u;
-  bool ok = dalloc(c, &c->d_slots, c->total_slots) == cudaSuccess && dalloc(c, &c->d_ovf, c->total_ovf) == cudaSuccess &&
-            dalloc(c, &c->d_tdesc, I) == cudaSuccess && dalloc(c, &c->d_count, I) == cudaSuccess &&
-            dalloc(c, &c->d_delta, (size_t)dn) == cudaSuccess && dalloc(c, &c->gsync.jobs, c->Rmax) == cudaSuccess &&
-            dalloc(c, &c->gsync.done, c->Rmax) == cudaSuccess && dalloc(c, &c->gsync.ready, c->Rmax) == cudaSuccess &&
-            dalloc(c, &c->gsync.stats, psk::kGreedyStats) == cudaSuccess &&
-            dalloc(c, &c->gsync.hitring, (size_t)psk::kHitSlots * c->gsync.ring_stride) == cudaSuccess &&
-            dalloc(c, &c->gsync.tpfring, (size_t)psk::kHitSlots * c->gsync.ring_stride) == cudaSuccess &&
-            dalloc(c, &c->d_rows, c->Rmax) == cudaSuccess && dalloc(c, &c->d_lastslot, c->lastslot_n + c->lastslot_n / 16) == cudaSuccess &&
-            dalloc(c, &c->scratch.rows, c->Rmax) == cudaSuccess && dalloc(c, &c->scratch.count, 1) == cudaSuccess &&
-            dalloc(c, &c->d_cprefix, 2 * ((size_t)c->Rmax + 1)) == cudaSuccess;
-  for (psk::StateSoA* s : {&c->st, &c->pend}) {
-    ok = ok && dalloc(c, &s->b, I) == cudaSuccess && dalloc(c, &s->qr, I) == cudaSuccess &&
-         dalloc(c, &s->q, I) == cudaSuccess && dalloc(c, &s->S, I) == cudaSuccess &&
-         dalloc(c, &s->M, I) == cudaSuccess && dalloc(c, &s->Bmax, I) == cudaSuccess;
-  }
-  ok = ok && dalloc(c, &c->d_off, (size_t)c->Rmax + 1) == cudaSuccess &&
-       dalloc(c, &c->d_hash, c->max_blocks) == cudaSuccess &&
-       dalloc(c, &c->d_own_off, (size_t)c->Rmax + 1) == cudaSuccess &&
-       dalloc(c, &c->d_own_hash, c->max_blocks) == cudaSuccess && dalloc(c, &c->d_parent, c->Rmax) == cudaSuccess && dalloc(c, &c->d_L, c->Rmax) == cudaSuccess &&
-       dalloc(c, &c->d_ttft, c->Rmax) == cudaSuccess && dalloc(c, &c->d_tpot, c->Rmax) == cudaSuccess &&
-       dalloc(c, &c->d_hits, RI) == cudaSuccess && dalloc(c, &c->d_tpf, RI) == cudaSuccess && dalloc(c, &c->d_tpot_o, RI) == cudaSuccess &&
-       dalloc(c, &c->d_ttft_o, RI) == cudaSuccess && dalloc(c, &c->d_cls, RI) == cudaSuccess &&
-       dalloc(c, &c->d_best, c->Rmax) == cudaSuccess && dalloc(c, &c->d_path, c->Rmax) == cudaSuccess &&
-       dalloc(c, &c->d_assign, c->Rmax) == cudaSuccess && dalloc(c, &c->d_dpath, c->Rmax) == cudaSuccess &&
-       dalloc(c, &c->d_hchosen, c->Rmax) == cudaSuccess && dalloc(c, &c->d_err, 1) == cudaSuccess &&
-       dalloc(c, &c->d_stats, kNumStats) == cudaSuccess && dalloc(c, &c->d_shard_wmin, c->Rmax) == cudaSuccess &&
-       dalloc(c, &c->d_shard_key, c->Rmax) == cudaSuccess && dalloc(c, &c->d_shard_tie, c->Rmax) == cudaSuccess &&
-       dalloc(c, &c->d_cap, I) == cudaSuccess && dalloc(c, &c->d_outtok, c->Rmax) == cudaSuccess;
-  if (ok && c->lru) {
+  want(c, &c->d_slots, c->total_slots);
+  want(c, &c->d_ovf, c->total_ovf);
+  want(c, &c->d_tdesc, I);
+  want(c, &c->d_count, I);
+  want(c, &c->d_delta, (size_t)dn);
+  // one block, cleared before each greedy pass: counters, jobs, done and ready flags
+  const size_t gsync_bytes = psk::kGreedyStats * sizeof(unsigned long long) + Rmax * 16;
+  want(c, &c->gsync_block, gsync_bytes);
+  want(c, &c->gsync.hitring, (size_t)psk::kHitSlots * c->gsync.ring_stride);
+  want(c, &c->gsync.tpfring, (size_t)psk::kHitSlots * c->gsync.ring_stride);
+  want(c, &c->d_rows, Rmax);
+  want(c, &c->d_lastslot, c->lastslot_n + c->lastslot_n / 16);
+  want(c, &c->scratch.rows, Rmax);
+  want(c, &c->zero_block, (kNumStats + 1) * sizeof(unsigned long long));
+  want(c, &c->d_cprefix, 2 * (Rmax + 1));
+  want(c, &c->st_block, I * kStateBytes);
+  want(c, &c->pend_block, I * kStateBytes);
+  want(c, &c->d_stage, kStageIn);
+  want(c, &c->d_off, Rmax + 1);
+  want(c, &c->d_hash, c->max_blocks);
+  want(c, &c->d_own_off, Rmax + 1);
+  want(c, &c->d_own_hash, c->max_blocks);
+  want(c, &c->d_parent, Rmax);
+  want(c, &c->d_L, Rmax);
+  want(c, &c->d_ttft, Rmax);
+  want(c, &c->d_tpot, Rmax);
+  want(c, &c->d_hits, RI);
+  want(c, &c->d_tpf, RI);
+  want(c, &c->d_tpot_o, RI);
+  want(c, &c->d_ttft_o, RI);
+  want(c, &c->d_cls, RI);
+  want(c, &c->d_best, Rmax);
+  want(c, &c->d_path, Rmax);
+  want(c, &c->d_assign, Rmax);
+  want(c, &c->d_dpath, Rmax);
+  want(c, &c->d_hchosen, Rmax);
+  want(c, &c->d_err, 4);
+  want(c, &c->d_shard_wmin, Rmax);
+  want(c, &c->d_shard_key, Rmax);
+  want(c, &c->d_shard_tie, Rmax);
+  want(c, &c->d_cap, I);
+  want(c, &c->d_outtok, Rmax);
+  if (c->lru) {
     for (uint32_t i = 0; i < I; ++i)
       c->max_instance_slots = std::max<uint64_t>(c->max_instance_slots, (uint64_t)td[i].nbkt * psk::kBucketSlots);
-    unsigned char* lb = nullptr;
-    unsigned char *plan = nullptr, *blocks = nullptr;
     pskl::EvictScratch& ev = c->evict;
-    ok = dalloc(c, &lb, pskl::evict_leafbuf_bytes(c->I)) == cudaSuccess && dalloc(c, &ev.nleaf, I) == cudaSuccess &&
-         dalloc(c, &ev.more, 1) == cudaSuccess && dalloc(c, &plan, pskl::evict_plan_bytes(c->I)) == cudaSuccess &&
-         dalloc(c, &ev.hist, pskl::evict_hist_words(c->I)) == cudaSuccess &&
-         dalloc(c, &blocks, pskl::evict_blocks_bytes(c->I)) == cudaSuccess && dalloc(c, &ev.list, I + 1) == cudaSuccess &&
-         dalloc(c, &ev.slow, I) == cudaSuccess;
-    ev.blocks = blocks;
-    ev.leafbuf = lb;
-    ev.plan = plan;
+    want(c, reinterpret_cast<unsigned char**>(&ev.leafbuf), pskl::evict_leafbuf_bytes(c->I));
+    want(c, reinterpret_cast<unsigned char**>(&ev.plan), pskl::evict_plan_bytes(c->I));
+    want(c, reinterpret_cast<unsigned char**>(&ev.blocks), pskl::evict_blocks_bytes(c->I));
+    want(c, &ev.hist, pskl::evict_hist_words(c->I));
+    want(c, &ev.nleaf, I);
+    want(c, &ev.more, 1);
+    want(c, &ev.list, I + 1);
+    want(c, &ev.slow, I);
+    want(c, &c->meta.last_use, c->total_slots);
+    want(c, &c->meta.children, c->total_slots);
+    want(c, &c->meta.parent, c->total_slots);
   }
-  if (ok && c->lru)
-    ok = dalloc(c, &c->meta.last_use, c->total_slots) == cudaSuccess &&
-         dalloc(c, &c->meta.children, c->total_slots) == cudaSuccess &&
-         dalloc(c, &c->meta.parent, c->total_slots) == cudaSuccess;
-  if (ok && c->rq.M) {
+  if (c->rq.M) {
     const size_t IM = I * (size_t)c->rq.M;
-    ok = dalloc(c, &c->rq.q_head, I) == cudaSuccess && dalloc(c, &c->rq.q_len, I) == cudaSuccess &&
-         dalloc(c, &c->rq.q_L, IM) == cudaSuccess && dalloc(c, &c->rq.q_out, IM) == cudaSuccess &&
-         dalloc(c, &c->rq.q_rem, IM) == cudaSuccess && dalloc(c, &c->rq.d_len, I) == cudaSuccess &&
-         dalloc(c, &c->rq.d_L, IM) == cudaSuccess && dalloc(c, &c->rq.d_out, IM) == cudaSuccess &&
-         dalloc(c, &c->rq.d_rem, IM) == cudaSuccess;
+    want(c, &c->rq.q_head, I);
+    want(c, &c->rq.q_len, I);
+    want(c, &c->rq.q_L, IM);
+    want(c, &c->rq.q_out, IM);
+    want(c, &c->rq.q_rem, IM);
+    want(c, &c->rq.d_len, I);
+    want(c, &c->rq.d_L, IM);
+    want(c, &c->rq.d_out, IM);
+    want(c, &c->rq.d_rem, IM);
   }
-  if (!ok) {
+  if (alloc_arena(c) != cudaSuccess) {
     cudaGetLastError();
     return bail(PS_ERR_OOM);
   }
-  if (cudaMallocHost(&c->h_err, sizeof(uint32_t)) != cudaSuccess) return bail(PS_ERR_OOM);
-  *c->h_err = 0;
-  if (cudaMallocHost(&c->h_more, sizeof(uint32_t)) != cudaSuccess) return bail(PS_ERR_OOM);
-  *c->h_more = 0;
+  c->st = state_arrays(c->st_block, I);
+  c->pend = state_arrays(c->pend_block, I);
+  c->gsync.stats = reinterpret_cast<unsigned long long*>(c->gsync_block);
+  c->gsync.jobs = c->gsync.stats + psk::kGreedyStats;
+  c->gsync.done = reinterpret_cast<uint32_t*>(c->gsync.jobs + Rmax);
+  c->gsync.ready = c->gsync.done + Rmax;
+  c->gsync.clear_bytes = gsync_bytes;
+  c->d_stats = reinterpret_cast<unsigned long long*>(c->zero_block);
+  c->scratch.count = reinterpret_cast<uint32_t*>(c->d_stats + kNumStats);
+  const size_t in_bytes = (std::max(kStageIn, I * kStateBytes) + 255) / 256 * 256;
+  if (cudaMallocHost(&c->h_pin, 256 + in_bytes + kStageOut) != cudaSuccess) return bail(PS_ERR_OOM);
+  c->h_err = reinterpret_cast<uint32_t*>(c->h_pin);
+  c->h_more = c->h_err + 8;
+  c->h_in = c->h_pin + 256;
+  c->h_out = c->h_in + in_bytes;
+  std::memset(c->h_pin, 0, 256);
   for (int e = 0; e < kNumEv; ++e)
     if (cudaEventCreate(&c->ev[e]) != cudaSuccess) return bail(PS_ERR_CUDA);
   bool set = cudaMemsetAsync(c->d_slots, 0, c->total_slots * sizeof(uint64_t), c->stream) == cudaSuccess &&
@@ -535,16 +640,10 @@ ps_status ps_create(const ps_config* cfg, ps_ctx** out) {
              cudaMemsetAsync(c->d_count, 0, I * sizeof(unsigned long long), c->stream) == cudaSuccess &&
              cudaMemsetAsync(c->d_delta, 0, (size_t)dn * sizeof(psk::DeltaSlot), c->stream) ==
                  cudaSuccess &&
-             cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), c->stream) == cudaSuccess &&
-             cudaMemsetAsync(c->d_stats, 0, kNumStats * sizeof(unsigned long long), c->stream) == cudaSuccess;
-  for (psk::StateSoA* s : {&c->st, &c->pend}) {
-    set = set && cudaMemsetAsync(s->b, 0, I * 4, c->stream) == cudaSuccess &&
-          cudaMemsetAsync(s->qr, 0, I * 4, c->stream) == cudaSuccess &&
-          cudaMemsetAsync(s->q, 0, I * 8, c->stream) == cudaSuccess &&
-          cudaMemsetAsync(s->S, 0, I * 8, c->stream) == cudaSuccess &&
-          cudaMemsetAsync(s->M, 0, I * 8, c->stream) == cudaSuccess &&
-          cudaMemsetAsync(s->Bmax, 0, I * 4, c->stream) == cudaSuccess;
-  }
+             cudaMemsetAsync(c->d_err, 0, 4 * sizeof(uint32_t), c->stream) == cudaSuccess &&
+             cudaMemsetAsync(c->zero_block, 0, (kNumStats + 1) * sizeof(unsigned long long), c->stream) == cudaSuccess &&
+             cudaMemsetAsync(c->st_block, 0, I * kStateBytes, c->stream) == cudaSuccess &&
+             cudaMemsetAsync(c->pend_block, 0, I * kStateBytes, c->stream) == cudaSuccess;
   set = set && cudaMemcpyAsync(c->d_cap, c->cap.data(), I * sizeof(uint64_t), cudaMemcpyHostToDevice, c->stream) ==
                    cudaSuccess;
   if (c->lru)
@@ -568,9 +667,8 @@ void ps_destroy(ps_ctx* c) {
   {
     DeviceGuard g(c->device);
     if (c->stream) cudaStreamSynchronize(c->stream);
-    for (void* p : c->allocs) cudaFree(p);
-    if (c->h_err) cudaFreeHost(c->h_err);
-    if (c->h_more) cudaFreeHost(c->h_more);
+    if (c->arena) cudaFree(c->arena);
+    if (c->h_pin) cudaFreeHost(c->h_pin);
     for (cudaEvent_t e : c->ev)
       if (e) cudaEventDestroy(e);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
@@ -585,51 +683,39 @@ ps_status ps_load_instances(ps_ctx* c, const ps_instance_state* s, uint32_t n) {
   c->shard_pending = false;
   if (!s || n != c->I) return fail(c, PS_ERR_INVALID, "need exactly num_instances states");
   const uint32_t I = c->I;
-  std::vector<int32_t> b(I), qr(I), bm(I);
-  std::vector<int64_t> q(I), S(I), M(I);
+  const psk::StateSoA h = state_arrays(c->h_in, I);  // page-locked; no copy from it is in flight between calls
   for (uint32_t i = 0; i < I; ++i) {
     const ps_instance_state& x = s[i];
     if (x.b < 0 || x.b >= (1 << 17) || x.qr < 0 || x.qr >= (1 << 17) || x.q_tokens < 0 ||
         x.q_tokens >= (1ll << 40) || x.S_tokens < 0 || x.S_tokens >= (1ll << 50) || x.M_KV_tokens < 0 ||
         x.M_KV_tokens >= (1ll << 50) || x.B_max < 0)
       return fail(c, PS_ERR_INVALID, "instance " + std::to_string(i) + ": state out of range");
-    b[i] = x.b; qr[i] = x.qr; q[i] = x.q_tokens; S[i] = x.S_tokens; M[i] = x.M_KV_tokens; bm[i] = x.B_max;
+    h.b[i] = x.b; h.qr[i] = x.qr; h.q[i] = x.q_tokens; h.S[i] = x.S_tokens; h.M[i] = x.M_KV_tokens; h.Bmax[i] = x.B_max;
   }
   DeviceGuard g(c->device);
   c->pending = false;
-  PS_TRY_CUDA(c, cudaMemcpyAsync(c->st.b, b.data(), I * 4, cudaMemcpyHostToDevice, c->stream));
-  PS_TRY_CUDA(c, cudaMemcpyAsync(c->st.qr, qr.data(), I * 4, cudaMemcpyHostToDevice, c->stream));
-  PS_TRY_CUDA(c, cudaMemcpyAsync(c->st.q, q.data(), I * 8, cudaMemcpyHostToDevice, c->stream));
-  PS_TRY_CUDA(c, cudaMemcpyAsync(c->st.S, S.data(), I * 8, cudaMemcpyHostToDevice, c->stream));
-  PS_TRY_CUDA(c, cudaMemcpyAsync(c->st.M, M.data(), I * 8, cudaMemcpyHostToDevice, c->stream));
-  PS_TRY_CUDA(c, cudaMemcpyAsync(c->st.Bmax, bm.data(), I * 4, cudaMemcpyHostToDevice, c->stream));
+  PS_TRY_CUDA(c, cudaMemcpyAsync(c->st_block, c->h_in, I * kStateBytes, cudaMemcpyHostToDevice, c->stream));
   PS_TRY_CUDA(c, cudaStreamSynchronize(c->stream));
   return PS_OK;
 }
 
-static ps_status read_state(ps_ctx* c, const psk::StateSoA& st, ps_instance_state* out, uint32_t n) {
+static ps_status read_state(ps_ctx* c, const unsigned char* block, ps_instance_state* out, uint32_t n) {
   if (!out || n != c->I) return fail(c, PS_ERR_INVALID, "need exactly num_instances states");
   const uint32_t I = c->I;
-  std::vector<int32_t> b(I), qr(I), bm(I);
-  std::vector<int64_t> q(I), S(I), M(I);
   DeviceGuard g(c->device);
-  PS_TRY_CUDA(c, cudaMemcpyAsync(b.data(), st.b, I * 4, cudaMemcpyDeviceToHost, c->stream));
-  PS_TRY_CUDA(c, cudaMemcpyAsync(qr.data(), st.qr, I * 4, cudaMemcpyDeviceToHost, c->stream));
-  PS_TRY_CUDA(c, cudaMemcpyAsync(q.data(), st.q, I * 8, cudaMemcpyDeviceToHost, c->stream));
-  PS_TRY_CUDA(c, cudaMemcpyAsync(S.data(), st.S, I * 8, cudaMemcpyDeviceToHost, c->stream));
-  PS_TRY_CUDA(c, cudaMemcpyAsync(M.data(), st.M, I * 8, cudaMemcpyDeviceToHost, c->stream));
-  PS_TRY_CUDA(c, cudaMemcpyAsync(bm.data(), st.Bmax, I * 4, cudaMemcpyDeviceToHost, c->stream));
+  PS_TRY_CUDA(c, cudaMemcpyAsync(c->h_in, block, I * kStateBytes, cudaMemcpyDeviceToHost, c->stream));
   PS_TRY_CUDA(c, cudaStreamSynchronize(c->stream));
+  const psk::StateSoA h = state_arrays(c->h_in, I);
   for (uint32_t i = 0; i < I; ++i) {
-    out[i].b = b[i]; out[i].qr = qr[i]; out[i].q_tokens = q[i]; out[i].S_tokens = S[i];
-    out[i].M_KV_tokens = M[i]; out[i].B_max = bm[i];
+    out[i].b = h.b[i]; out[i].qr = h.qr[i]; out[i].q_tokens = h.q[i]; out[i].S_tokens = h.S[i];
+    out[i].M_KV_tokens = h.M[i]; out[i].B_max = h.Bmax[i];
   }
   return PS_OK;
 }
 
 ps_status ps_get_instances(ps_ctx* c, ps_instance_state* out, uint32_t n) {
   if (!c) return PS_ERR_INVALID;
-  return read_state(c, c->st, out, n);
+  return read_state(c, c->st_block, out, n);
 }
 
 ps_status ps_calibrate(ps_ctx* c, uint32_t n, const int32_t* batch, const int64_t* ctx_tokens,
@@ -674,7 +760,7 @@ ps_status ps_set_wait_limit(ps_ctx* c, uint64_t ns) {
 ps_status ps_get_pending_instances(ps_ctx* c, ps_instance_state* out, uint32_t n) {
   if (!c) return PS_ERR_INVALID;
   if (!c->pending) return fail(c, PS_ERR_STATE, "no pending window");
-  return read_state(c, c->pend, out, n);
+  return read_state(c, c->pend_block, out, n);
 }
 
 ps_status ps_insert_chains(ps_ctx* c, uint64_t nchains, const uint32_t* inst, const uint64_t* off,
@@ -746,8 +832,9 @@ ps_status ps_cached_blocks(ps_ctx* c, uint64_t* out, uint32_t n) {
   if (!c) return PS_ERR_INVALID;
   if (!out || n != c->I) return fail(c, PS_ERR_INVALID, "need num_instances entries");
   DeviceGuard g(c->device);
-  PS_TRY_CUDA(c, cudaMemcpyAsync(out, c->d_count, n * 8, cudaMemcpyDeviceToHost, c->stream));
+  PS_TRY_CUDA(c, cudaMemcpyAsync(c->h_in, c->d_count, n * 8, cudaMemcpyDeviceToHost, c->stream));
   PS_TRY_CUDA(c, cudaStreamSynchronize(c->stream));
+  std::memcpy(out, c->h_in, n * 8);
   return PS_OK;
 }
 
@@ -864,13 +951,14 @@ ps_status ps_schedule_window(ps_ctx* c, const ps_window* w, ps_decisions* out, p
   uint32_t* hit0 = nullptr;
   s = run_probe_and_score(c, wd, opt_scores, &hit0, true);
   if (s != PS_OK) return s;
+  const uint64_t nslots = std::min<uint64_t>(c->delta_nslots, std::max<uint64_t>(16, 2 * c->win_blocks));
   record(c, kEvGreedy0);
   PS_TRY_CUDA(c, pskl::launch_greedy(c->d_rows, wd, c->I, hit0, c->d_tpf, c->st, c->pend, c->model, c->d_delta,
-                                     c->delta_nslots, c->d_assign, c->d_dpath, c->d_hchosen, c->d_err, c->gsync,
+                                     nslots, c->d_assign, c->d_dpath, c->d_hchosen, c->d_err, c->gsync,
                                      c->search, c->d_slots, c->d_ovf, c->d_tdesc, c->stream));
   record(c, kEvGreedy1);
   c->ev_used[2] = true;
-  PS_TRY_CUDA(c, pskl::launch_delta_clear(c->d_delta, c->delta_nslots, c->stream));
+  PS_TRY_CUDA(c, pskl::launch_delta_clear(c->d_delta, nslots, c->stream));
   if (out) {
     PS_TRY_CUDA(c, deliver(c, out->assign, c->d_assign, wd.R, out->outputs_on_device));
     PS_TRY_CUDA(c, deliver(c, out->path, c->d_dpath, wd.R, out->outputs_on_device));
@@ -895,13 +983,7 @@ ps_status ps_commit_window(ps_ctx* c, uint32_t last_use) {
   PS_TRY_CUDA(c, pskl::launch_commit(c->d_slots, c->d_ovf, c->d_tdesc, c->I, c->d_count, c->pend_win, c->d_assign,
                                      c->d_hchosen, c->meta, last_use, c->rq, c->pend_out, c->d_cprefix, c->d_err,
                                      c->num_sms, c->stream));
-  const size_t I = c->I;
-  PS_TRY_CUDA(c, cudaMemcpyAsync(c->st.b, c->pend.b, I * 4, cudaMemcpyDeviceToDevice, c->stream));
-  PS_TRY_CUDA(c, cudaMemcpyAsync(c->st.qr, c->pend.qr, I * 4, cudaMemcpyDeviceToDevice, c->stream));
-  PS_TRY_CUDA(c, cudaMemcpyAsync(c->st.q, c->pend.q, I * 8, cudaMemcpyDeviceToDevice, c->stream));
-  PS_TRY_CUDA(c, cudaMemcpyAsync(c->st.S, c->pend.S, I * 8, cudaMemcpyDeviceToDevice, c->stream));
-  PS_TRY_CUDA(c, cudaMemcpyAsync(c->st.M, c->pend.M, I * 8, cudaMemcpyDeviceToDevice, c->stream));
-  PS_TRY_CUDA(c, cudaMemcpyAsync(c->st.Bmax, c->pend.Bmax, I * 4, cudaMemcpyDeviceToDevice, c->stream));
+  PS_TRY_CUDA(c, cudaMemcpyAsync(c->st_block, c->pend_block, c->I * kStateBytes, cudaMemcpyDeviceToDevice, c->stream));
   record(c, kEvCommit1);
   c->ev_used[3] = true;
   c->pending = false;

@@ -1182,10 +1182,7 @@ cudaError_t launch_greedy(const psk::RowPre* rows, const psk::WindowDev& w, uint
                           const uint64_t* slots, const uint64_t* ovf, const psk::TableDesc* tdesc, cudaStream_t s) {
   const MainTables mt{slots, ovf, tdesc};
   if (w.R == 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(sync.done, 0, (size_t)w.R * sizeof(uint32_t), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(sync.ready, 0, (size_t)w.R * sizeof(uint32_t), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(sync.jobs, 0, (size_t)w.R * sizeof(unsigned long long), s);
-  if (e == cudaSuccess && sync.stats) e = cudaMemsetAsync(sync.stats, 0, psk::kGreedyStats * sizeof(unsigned long long), s);
+  const cudaError_t e = cudaMemsetAsync(sync.stats, 0, sync.clear_bytes, s);
   if (e != cudaSuccess) return e;
   // IPT instances per compute thread of the deciding block (and at most that many per probe thread): as
   // few as its warps allow.  More per thread means fewer warps to combine but a longer step: greedy pass

@@ -133,7 +133,7 @@ ps_status ps_score_window_noalloc(const uint64_t* slots, const uint64_t* overflo
   // The error word keeps the previous call's value: clear it first.
   if (cudaMemsetAsync(err, 0, sizeof(uint32_t), s) != cudaSuccess) return PS_ERR_CUDA;
   const psk::WindowDev wd{w->chain_off, w->chain_hash, w->prompt_tokens, w->ttft_target, w->tpot_target, w->R};
-  if (pskl::launch_validate_window(wd, ~0ull, err, s) != cudaSuccess) return PS_ERR_CUDA;
+  if (pskl::launch_validate_window(wd, ~0ull, err, nullptr, s) != cudaSuccess) return PS_ERR_CUDA;
   const psk::TableDesc* td = reinterpret_cast<const psk::TableDesc*>(tables);
   check_tables_kernel<<<(num_instances + 255) / 256, 256, 0, s>>>(td, num_instances, err);
   if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;

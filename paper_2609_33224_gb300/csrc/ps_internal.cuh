@@ -112,7 +112,9 @@ struct GreedySync {
   float* tpfring;            // [kHitSlots][ring_stride] T_pf at those hits
   uint32_t ring_stride;      // I rounded up to a multiple of 8
   uint64_t wait_ns;          // bound on any cross-block wait (ns); a waiter that gives up sets kErrTimeout
-  unsigned long long* stats; // [kGreedyStats] counters of the pass (below)
+  unsigned long long* stats; // [kGreedyStats] counters of the pass (below); the first of clear_bytes bytes
+                             // that hold stats, jobs, done and ready and are cleared before each pass
+  size_t clear_bytes;
 };
 
 // Counters of one greedy pass (GreedySync::stats): decisions made, then SM clock cycles: the deciding
@@ -911,6 +913,7 @@ size_t evict_leafbuf_bytes(uint32_t I);
 cudaError_t launch_check_parents(const uint64_t* slots, const uint64_t* ovf, const psk::TableDesc* tdesc, uint32_t I,
                                  uint64_t nchains, const uint32_t* inst, const uint64_t* parent,
                                  uint32_t* err, int num_sms, cudaStream_t s);
+// err: the error word; nblk (may be null): receives the window's number of blocks.
 cudaError_t launch_validate_window(const psk::WindowDev& w, uint64_t max_blocks, uint32_t* err,
-                                   cudaStream_t s);
+                                   unsigned long long* nblk, cudaStream_t s);
 }  // namespace pskl

@@ -1365,7 +1365,8 @@ __global__ void check_parents_kernel(const uint64_t* slots, const uint64_t* ovf,
   }
 }
 
-__global__ void validate_window_kernel(psk::WindowDev w, uint64_t max_blocks, uint32_t* err) {
+__global__ void validate_window_kernel(psk::WindowDev w, uint64_t max_blocks, uint32_t* err, unsigned long long* nblk) {
+  if (nblk && blockIdx.x == 0 && threadIdx.x == 0) *nblk = w.off[w.R];
   for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < w.R; r += gridDim.x * blockDim.x) {
     const uint64_t a = w.off[r], b = w.off[r + 1];
     const uint32_t L = w.L[r];
@@ -1515,11 +1516,11 @@ cudaError_t launch_check_parents(const uint64_t* slots, const uint64_t* ovf, con
 }
 
 cudaError_t launch_validate_window(const psk::WindowDev& w, uint64_t max_blocks, uint32_t* err,
-                                   cudaStream_t s) {
+                                   unsigned long long* nblk, cudaStream_t s) {
   if (w.R == 0) return cudaSuccess;
   uint32_t blocks = (w.R + 255) / 256;
   if (blocks > 1024) blocks = 1024;
-  validate_window_kernel<<<blocks, 256, 0, s>>>(w, max_blocks, err);
+  validate_window_kernel<<<blocks, 256, 0, s>>>(w, max_blocks, err, nblk);
   return cudaGetLastError();
 }
 
