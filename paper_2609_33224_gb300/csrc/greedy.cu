@@ -518,7 +518,9 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
   __shared__ uint32_t s_begun;                             // steps [0, s_begun) have begun
   __shared__ uint32_t s_landed;                            // rows [0, s_landed) are staged
   __shared__ volatile int s_fail;                          // a bounded wait ran out (feeder and hit warp)
-  __shared__ volatile int s_stop;                          // set before a step's barrier: every warp leaves after it
+  // The step whose barrier is the last one, once a wait has run out (the hit warp sets it before it arrives
+  // there).  A step number, not a flag: a warp that looks late at step s must not leave for step s + 1.
+  __shared__ volatile uint32_t s_stop;
   const uint32_t t = threadIdx.x;
   const int lane = (int)(t & 31u);
   const uint32_t warp = t >> 5;
@@ -538,7 +540,7 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
     s_begun = 0u;
     s_landed = 0u;
     s_fail = 0;
-    s_stop = 0;
+    s_stop = 0xFFFFFFFFu;
   }
   narrow = __syncthreads_and(narrow ? 1 : 0) != 0;
   if (!narrow) {
@@ -634,11 +636,11 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
     for (uint32_t s = 0; s <= R; ++s) {
       // rows s and s + 1 must be staged when step s begins
       const long long c0 = clock64();
-      if (lane == 0 && !wait_smem_at_least(&s_landed, s + 2 < R ? s + 2 : R, &s_fail, err, sync.wait_ns)) s_stop = 1;
+      if (lane == 0 && !wait_smem_at_least(&s_landed, s + 2 < R ? s + 2 : R, &s_fail, err, sync.wait_ns)) s_stop = s;
       cyc_wait += (unsigned long long)(clock64() - c0);
       __syncwarp();
       bar_step();
-      if (s_stop) {
+      if (s_stop <= s) {
         if (lane == 0) s_fail = 1;  // the feeder stops too
         break;
       }
@@ -680,7 +682,7 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
     // Global stores stay in a warp of their own: a fence behind them would wait for their round trip.
     for (uint32_t s = 0; s <= R; ++s) {
       bar_step();
-      if (s_stop) break;
+      if (s_stop <= s) break;
       if (s == 0) continue;
       const int src = decision(s - 1, rank_of(s - 1));
       uint2 th = make_uint2(0xFFFFFFFFu, 0u);
@@ -796,7 +798,7 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
 #pragma unroll
         for (int k = 0; k < IPT; ++k) h[k] = tb[k] = 0u;
       }
-      if (s_stop) {
+      if (s_stop <= s) {
         stopped = true;
         break;
       }
@@ -957,7 +959,7 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
     uint32_t Lprev = 0;  // length of request s - 1
     for (uint32_t s = 0;; ++s) {
       bar_step();
-      if (s_stop) {
+      if (s_stop <= s) {
         stopped = true;
         break;
       }
