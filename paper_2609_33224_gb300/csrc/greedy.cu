@@ -388,9 +388,11 @@ __device__ __forceinline__ bool narrow_qs(int64_t q, int64_t S) {
 // decision, before -> now (before: row summaries computed by other blocks 8 decisions ahead and
 // corrected by one warp, with helper warps; 1.25 us of helper phase a step, and a pass over the row by
 // one warp, 20 to 30 us, where the summary did not cover the pick):
-//   64 instances 1.22 -> 0.55 us, 201: 1.43 -> 0.74, 256: 1.41 -> 0.62, 999: 3.3 -> 1.13, 1024: 1.60 -> 0.89.
-// 1024 instances are bound by issue slots (about 250 instructions a warp and step on 16 warps), small
-// pools by the chain.
+//   64 instances 1.22 -> 0.53 us, 201: 1.43 -> 0.67, 256: 1.41 -> 0.65, 999: 3.3 -> 0.86, 1024: 1.60 -> 0.83.
+// 1024 instances are bound by issue slots (about 230 instructions a warp and step on 16 warps, 55% of the
+// slots) beside the chain, small pools by the chain.  The pick's owner takes its place in the row by two
+// blocks, its W before the rest (1024 x 16384: 14.4 ms, 14.7 in one), and a warp's pick is handed on by
+// the lane that finds itself the only one, before the vote that says so (15.2 ms if after it).
 
 constexpr uint32_t kComputeWarps = 16;
 constexpr uint32_t kFeederWarp = kComputeWarps;
@@ -479,23 +481,21 @@ __device__ __forceinline__ int warp_argmin(uint32_t rank, uint64_t key, uint32_t
   return __ffs(who) - 1;
 }
 
-// What a step needs of a row's constants.  With the tests a model leaves out (TTFT filter, SLO
-// admission, recompute filter) the bound is +infinity, which every finite value passes.
+// What a step needs of a row's constants (RowPre's second word and a few more).
 struct StepRow {
   float t_cached, c_max, ttft_max, tpot_lim, tpot_target;
   uint32_t L;
 };
 
-__device__ __forceinline__ StepRow step_row(const psk::DevModel& m, const psk::RowPre& x) {
-  const uint4 w0 = reinterpret_cast<const uint4*>(&x)[0];  // off, nb, L
-  const float4 w1 = reinterpret_cast<const float4*>(&x)[1];  // t_cached, Z, etaZ, ttft_budget
+__device__ __forceinline__ StepRow step_row(const psk::RowPre& x) {
+  const float4 w1 = reinterpret_cast<const float4*>(&x)[1];
   StepRow r;
-  r.L = w0.w;
+  r.L = x.L;
   r.t_cached = w1.x;
-  r.c_max = w1.y > 0.0f ? w1.z : INFINITY;
+  r.c_max = w1.y;
+  r.tpot_lim = w1.z;
+  r.ttft_max = w1.w;
   r.tpot_target = x.tpot_target;
-  r.tpot_lim = m.slo_off ? INFINITY : x.tpot_target;
-  r.ttft_max = (m.slo_off || !m.ttft_filter) ? INFINITY : w1.w;
   return r;
 }
 
@@ -788,7 +788,7 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
       const uint2 eth = s_th[par][held ? lane : 0];
       const uint32_t slot = (s < R ? s : R - 1) % kFeedRing;
       const psk::RowPre& row = s_row[slot];
-      const StepRow rc = step_row(m, row);
+      const StepRow rc = step_row(row);
       const uint32_t l0 = row.lcp[0];
       uint32_t h[IPT], tb[IPT];
       if (loads) {
@@ -803,6 +803,8 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
         break;
       }
       const uint32_t mr = __reduce_min_sync(0xffffffffu, er);
+      uint32_t jt = __reduce_min_sync(0xffffffffu, er == mr ? eth.x : 0xFFFFFFFFu);
+      uint32_t H = __reduce_min_sync(0xffffffffu, er == mr ? eth.y : 0xFFFFFFFFu);
       const unsigned who = __ballot_sync(0xffffffffu, er == mr);
       float W[IPT];
       uint64_t key[IPT];
@@ -811,64 +813,76 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
       for (int k = 0; k < IPT; ++k)
         pair(rc, i0 + (uint32_t)k, h[k], __uint_as_float(tb[k]), room[k], q32[k], S32[k], Bp[k], dec0[k], fe[k], tq[k],
              kq[k], kdh[k], &W[k], &key[k], &rank[k], &tie[k]);
+      bool own = false;  // this thread owns the last pick
+      uint32_t j = 0, hj = 0;
+      int4 x = make_int4(0, 0, 0, 0);
+      float tpfj = 0.0f;
       if (mr != 0xFFFFFFFFu) {
-        int src = __ffs(who) - 1;
-        if (who & (who - 1u)) src = warp_argmin(er, s_key[par][held ? lane : 0], eth.x);  // equal ranks
-        const uint32_t j = __shfl_sync(0xffffffffu, eth.x, src) & psk::kTieInstMask;
-        const uint32_t H = __shfl_sync(0xffffffffu, eth.y, src);
+        if (who & (who - 1u)) {  // equal ranks
+          const int src = warp_argmin(er, s_key[par][held ? lane : 0], eth.x);
+          jt = __shfl_sync(0xffffffffu, eth.x, src);
+          H = __shfl_sync(0xffffffffu, eth.y, src);
+        }
+        j = jt & psk::kTieInstMask;
         uint32_t lj = l0;
         if (LIN && j / (32u * IPT) == warp) lj = extend(row, j, s_hitr[slot * Ip + j]);
         if (j / IPT == t) {
           // its state takes request s - 1 (qr + 1, q + L - 16 H, S + L), and its hit rises to the common
-          // prefix of the two requests
-          int4 x = a.qs[j];
-          uint4 y = a.kb[j];
-          uint32_t hj = s_hitr[slot * Ip + j];
-          x.x += (int32_t)Lprev - (int32_t)(H << 4);
-          x.y += (int32_t)Lprev;
+          // prefix of the two requests: first its W, then (the second block) the rest
+          own = true;
+          x = a.qs[j];
+          hj = s_hitr[slot * Ip + j];
           x.w -= 1;
           x.z = x.w < 0 ? -1 : x.z - (int32_t)Lprev;
-          y.x += 1u;
-          y.z += 1u;
-          a.qs[j] = x;
-          a.kb[j] = y;
-          const float d0 = __fadd_rn(m.b0, __fmul_rn(m.b1, __int2float_rn((int32_t)y.z)));
-          const float f = psk::ema_factor(m, (int32_t)y.z);
-          const float tqv =
-              __fadd_rn(__fmul_rn(m.a0, __int2float_rn((int32_t)(y.x & 0x3FFFFu))), __fmul_rn(m.a1, __int2float_rn(x.x)));
           hj = lj > hj ? lj : hj;
-          float Wj;
-          uint64_t keyj;
-          uint32_t rankj, tiej;
-          pair(rc, j, hj, psk::t_pf32(m, rc.L, hj), x.z, x.x, x.y, (int32_t)y.z, d0, f, tqv, y.x, y.y, &Wj, &keyj, &rankj,
-               &tiej);
+          tpfj = psk::t_pf32(m, rc.L, hj);
+          const float Wj = (int32_t)rc.L <= x.z ? __fsub_rn(tpfj, rc.t_cached) : INFINITY;
 #pragma unroll
           for (int k = 0; k < IPT; ++k)
-            if (i0 + (uint32_t)k == j) {
-              W[k] = Wj;
-              key[k] = keyj;
-              rank[k] = rankj;
-              tie[k] = tiej;
-              h[k] = hj;
-              q32[k] = x.x;
-              S32[k] = x.y;
-              room[k] = x.z;
-              Bp[k] = (int32_t)y.z;
-              kq[k] = y.x;
-              dec0[k] = d0;
-              fe[k] = f;
-              tq[k] = tqv;
-            }
+            if (i0 + (uint32_t)k == j) W[k] = Wj;
         }
       }
-      if (s == R) break;
-      Lprev = rc.L;
+      if (own) {
+        uint4 y = a.kb[j];
+        x.x += (int32_t)Lprev - (int32_t)(H << 4);
+        x.y += (int32_t)Lprev;
+        y.x += 1u;
+        y.z += 1u;
+        a.qs[j] = x;
+        a.kb[j] = y;
+        const float d0 = __fadd_rn(m.b0, __fmul_rn(m.b1, __int2float_rn((int32_t)y.z)));
+        const float f = psk::ema_factor(m, (int32_t)y.z);
+        const float tqv =
+            __fadd_rn(__fmul_rn(m.a0, __int2float_rn((int32_t)(y.x & 0x3FFFFu))), __fmul_rn(m.a1, __int2float_rn(x.x)));
+        float Wj;
+        uint64_t keyj;
+        uint32_t rankj, tiej;
+        pair(rc, j, hj, tpfj, x.z, x.x, x.y, (int32_t)y.z, d0, f, tqv, y.x, y.y, &Wj, &keyj, &rankj, &tiej);
+#pragma unroll
+        for (int k = 0; k < IPT; ++k)
+          if (i0 + (uint32_t)k == j) {
+            key[k] = keyj;
+            rank[k] = rankj;
+            tie[k] = tiej;
+            h[k] = hj;
+            q32[k] = x.x;
+            S32[k] = x.y;
+            room[k] = x.z;
+            Bp[k] = (int32_t)y.z;
+            kq[k] = y.x;
+            dec0[k] = d0;
+            fe[k] = f;
+            tq[k] = tqv;
+          }
+      }
       float wbest = W[0];
 #pragma unroll
       for (int k = 1; k < IPT; ++k) wbest = fminf(wbest, W[k]);
       uint32_t wmin_o = __reduce_min_sync(0xffffffffu, psk::f2ord(wbest));
+      if (ncw > 1u && lane == 0) s_w[warp] = wmin_o;
+      if (s == R) break;
+      Lprev = rc.L;
       if (ncw > 1u) {
-        if (lane == 0) s_w[warp] = wmin_o;
         bar_compute();
         wmin_o = __reduce_min_sync(0xffffffffu, s_w[lane & (kComputeWarps - 1)]);
       }
@@ -877,7 +891,7 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
       uint32_t rbest = 0xFFFFFFFFu;
 #pragma unroll
       for (int k = 0; k < IPT; ++k) {
-        const bool in = W[k] < INFINITY && __fsub_rn(W[k], wmin) <= rc.c_max;
+        const bool in = __fsub_rn(W[k], wmin) <= rc.c_max;
         rank[k] = in ? rank[k] : 0xFFFFFFFFu;
         rbest = min(rbest, rank[k]);
       }
@@ -893,7 +907,13 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
           bt = tie[k];
           bh = h[k];
         }
-      unsigned lanes = __ballot_sync(0xffffffffu, n_eq != 0u);
+      // the lane that holds it hands it on at once (with equal ranks several do, and the smallest again below)
+      if (n_eq != 0u) {
+        s_rank[s & 1u][warp] = mw;
+        s_th[s & 1u][warp] = make_uint2(bt, bh);
+        s_key[s & 1u][warp] = bk;
+      }
+      const unsigned lanes = __ballot_sync(0xffffffffu, n_eq != 0u);
       const unsigned many = IPT > 1 ? __ballot_sync(0xffffffffu, n_eq > 1u) : 0u;
       if (mw != 0xFFFFFFFFu && ((lanes & (lanes - 1u)) | many)) {
         // equal ranks: the smallest (key, tie) of the lane's, then of the warp's
@@ -905,12 +925,11 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
             bh = h[k];
           }
         const int win = warp_argmin(n_eq ? mw : 0xFFFFFFFFu, bk, bt);
-        lanes = 1u << win;
-      }
-      if (lane == __ffs(lanes) - 1) {
-        s_rank[s & 1u][warp] = mw;
-        s_th[s & 1u][warp] = make_uint2(bt, bh);
-        s_key[s & 1u][warp] = bk;
+        __syncwarp();
+        if (lane == win) {
+          s_th[s & 1u][warp] = make_uint2(bt, bh);
+          s_key[s & 1u][warp] = bk;
+        }
       }
       __syncwarp();
     }
@@ -999,7 +1018,7 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
       }
       if (s == R) break;
       const psk::RowPre& row = s_row[slot];
-      const StepRow rc = step_row(m, row);
+      const StepRow rc = step_row(row);
       Lprev = rc.L;
       uint32_t h[IPT], tb[IPT];
       if (loads) {
@@ -1075,7 +1094,7 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
       uint32_t bt[IPT], bh[IPT];
 #pragma unroll
       for (int k = 0; k < IPT; ++k) {
-        const bool in = W[k] < INFINITY && __fsub_rn(W[k], wmin) <= rc.c_max;
+        const bool in = __fsub_rn(W[k], wmin) <= rc.c_max;
         bk[k] = in ? key[k] : psk::kNoKey;
         bt[k] = tie[k];
         bh[k] = h[k];

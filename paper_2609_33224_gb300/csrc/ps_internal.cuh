@@ -75,9 +75,11 @@ struct __align__(16) RowPre {
   uint32_t nb;
   uint32_t L;
   float t_cached;     // T_pf(0, L)
-  float Z;            // T_pf(L, 0) - T_pf(0, L)
-  float etaZ;         // eta * Z
-  float ttft_budget;  // max(target, T_pf(L, 0))
+  // Bounds of the tests of a pair of A: W - W_min <= c_max (eta * Z; every finite value passes where Eq. 8
+  // filters nothing), TPOT < tpot_lim, TTFT <= ttft_max (+infinity where the model leaves the test out)
+  float c_max;
+  float tpot_lim;
+  float ttft_max;     // max(target, T_pf(L, 0))
   float tpot_target;
   int32_t par;        // deepest earlier request whose chain is a prefix of r's, -1 if none
   uint32_t par_nb;    // its chain length

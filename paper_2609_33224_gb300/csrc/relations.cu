@@ -196,9 +196,9 @@ relations_kernel(psk::WindowDev w, psk::DevModel m, const psk::LastSlot* tab, ui
       x.nb = (uint32_t)nb;
       x.L = rc.L;
       x.t_cached = rc.t_cached;
-      x.Z = rc.Z;
-      x.etaZ = rc.etaZ;
-      x.ttft_budget = rc.ttft_budget;
+      x.c_max = rc.Z > 0.0f ? rc.etaZ : 3.402823466e38f;
+      x.tpot_lim = m.slo_off ? INFINITY : rc.tpot_target;
+      x.ttft_max = (m.slo_off || !m.ttft_filter) ? INFINITY : rc.ttft_budget;
       x.tpot_target = rc.tpot_target;
       x.hint = r > 0u ? hint : 0u;
       x.limit = (uint32_t)nb;
