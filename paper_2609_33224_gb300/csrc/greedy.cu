@@ -388,8 +388,8 @@ __device__ __forceinline__ bool narrow_qs(int64_t q, int64_t S) {
 // decision, before -> now (before: row summaries computed by other blocks 8 decisions ahead and
 // corrected by one warp, with helper warps; 1.25 us of helper phase a step, and a pass over the row by
 // one warp, 20 to 30 us, where the summary did not cover the pick):
-//   64 instances 1.22 -> 0.53 us, 201: 1.43 -> 0.67, 256: 1.41 -> 0.65, 999: 3.3 -> 0.86, 1024: 1.60 -> 0.83.
-// 1024 instances are bound by issue slots (about 230 instructions a warp and step on 16 warps, 55% of the
+//   64 instances 1.22 -> 0.53 us, 201: 1.43 -> 0.67, 256: 1.41 -> 0.65, 999: 3.3 -> 0.85, 1024: 1.60 -> 0.82.
+// 1024 instances are bound by issue slots (about 215 instructions a warp and step on 16 warps, 55% of the
 // slots) beside the chain, small pools by the chain.  The pick's owner takes its place in the row by two
 // blocks, its W before the rest (1024 x 16384: 14.4 ms, 14.7 in one), and a warp's pick is handed on by
 // the lane that finds itself the only one, before the vote that says so (15.2 ms if after it).
@@ -464,6 +464,14 @@ __device__ __forceinline__ uint32_t key_rank(uint64_t key) {
   return key == psk::kNoKey ? 0xFFFFFFFFu : ((key >> 62) ? c1 : c0);
 }
 
+// Algorithm 1's packed key from its rank and two words, {key bits of qr, of b} in T and {q + n, B} in C \ T:
+// worked out only where ranks are equal.
+__device__ __forceinline__ uint64_t dcq_key(uint32_t rank, uint2 w, uint32_t h) {
+  if (rank == 0xFFFFFFFFu) return psk::kNoKey;
+  if (rank & 0x80000000u) return psk::packed_key(1u, (uint64_t)w.x * (uint64_t)w.y);
+  return (((uint64_t)w.y << 32) | w.x) | ((uint64_t)((1u << 26) - 1u - h) << 18);
+}
+
 // The lane holding the warp's smallest (key, tie), -1 if no lane has a key; rank = key_rank(key).
 __device__ __forceinline__ int warp_argmin(uint32_t rank, uint64_t key, uint32_t tie) {
   const uint32_t mr = __reduce_min_sync(0xffffffffu, rank);
@@ -513,7 +521,7 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
   __shared__ psk::RowPre s_row[kFeedRing];
   __shared__ uint32_t s_rank[2][kComputeWarps];            // a step's warp minima: their ranks (all ones: none) ...
   __shared__ uint2 s_th[2][kComputeWarps];                 // ... tie word and hit ...
-  __shared__ uint64_t s_key[2][kComputeWarps];             // ... and packed key
+  __shared__ uint2 s_key[2][kComputeWarps];                // ... and packed key, or dcq_key's words (`words`)
   __shared__ uint32_t s_w[kComputeWarps];                  // a step's warp minima of W over A (f2ord)
   __shared__ uint32_t s_begun;                             // steps [0, s_begun) have begun
   __shared__ uint32_t s_landed;                            // rows [0, s_landed) are staged
@@ -560,13 +568,18 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
   auto bar_compute = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(ncmp) : "memory"); };  // compute warps
   // Step x's pick from the warps' minima (after the next step's barrier), in every lane: the warp that
   // holds it, -1 if rejected.  r: this lane's entry of s_rank[x & 1] (all ones past the warps in use).
+  const bool words = !GEN && narrow;
+  auto key_at = [&](uint32_t x, uint32_t r, uint32_t l) {
+    const uint2 w = s_key[x & 1u][l];
+    return words ? dcq_key(r, w, s_th[x & 1u][l].y) : ((uint64_t)w.y << 32) | w.x;
+  };
   auto decision = [&](uint32_t x, uint32_t r) {
     const uint32_t mr = __reduce_min_sync(0xffffffffu, r);
     const unsigned who = __ballot_sync(0xffffffffu, r == mr);
     int src = __ffs(who) - 1;
     if (who & (who - 1u)) {  // equal ranks (or nobody has a pair)
       const uint32_t l = (uint32_t)lane < ncw ? lane : 0u;
-      src = warp_argmin(r, s_key[x & 1u][l], s_th[x & 1u][l].x);
+      src = warp_argmin(r, key_at(x, r, l), s_th[x & 1u][l].x);
     }
     return src;
   };
@@ -689,7 +702,7 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
       uint32_t cls = 2u;
       if (src >= 0) {
         th = s_th[(s - 1) & 1u][src];
-        cls = (uint32_t)(s_key[(s - 1) & 1u][src] >> 62);
+        cls = s_rank[(s - 1) & 1u][src] >> 31;
       }
       const uint32_t j = src < 0 ? 0xFFFFFFFFu : th.x & psk::kTieInstMask;
       if (lane == 0) psk::st_relaxed_u64(sync.jobs + s - 1, kJobValid | ((unsigned long long)th.y << 32) | j);
@@ -738,8 +751,8 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
         a.kb[i] = make_uint4(kq[k], kdh[k], (uint32_t)Bp[k], 0u);
       }
     }
-    // One pair on the given state: W (+infinity outside A), and the key, its rank and the tie word it
-    // has in C.
+    // One pair on the given state: W (+infinity outside A), and the key (GEN), its rank and the tie word
+    // it has in C.
     auto pair = [&](const StepRow& rc, uint32_t i, uint32_t h, float tpf, int32_t rm, int32_t q, int32_t S, int32_t B,
                     float d0, float f, float tqv, uint32_t kql, uint32_t kh, float* W, uint64_t* key, uint32_t* rank,
                     uint32_t* tie) {
@@ -763,10 +776,9 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
       if (!GEN) {  // Algorithm 1's order: D-C-Q in T, the LMetric product in C \ T
         // ranks: D and up to 13 bits of C; the product rounded towards zero (both factors exact in fp32,
         // else from the 64-bit product: the same rounding of the same value)
-        const uint64_t k0 = kd | ((uint64_t)((1u << 26) - 1u - h) << 18);
         const uint64_t v1 = qn * (uint64_t)(uint32_t)B;
         const float p1 = (uint32_t)qn < (1u << 24) ? __fmul_rz(qnf, __int2float_rn(B)) : __ull2float_rz(v1);
-        *key = adm ? k0 : psk::packed_key(1u, v1);
+        *key = 0ull;
         *rank = adm ? (kh << 1) | (8191u - min(h, 8191u)) : 0x80000000u | __float_as_uint(p1);
       } else {
         if (adm) {
@@ -819,7 +831,7 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
       float tpfj = 0.0f;
       if (mr != 0xFFFFFFFFu) {
         if (who & (who - 1u)) {  // equal ranks
-          const int src = warp_argmin(er, s_key[par][held ? lane : 0], eth.x);
+          const int src = warp_argmin(er, key_at(par, er, held ? lane : 0), eth.x);
           jt = __shfl_sync(0xffffffffu, eth.x, src);
           H = __shfl_sync(0xffffffffu, eth.y, src);
         }
@@ -887,44 +899,59 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
         wmin_o = __reduce_min_sync(0xffffffffu, s_w[lane & (kComputeWarps - 1)]);
       }
       const float wmin = psk::ord2f(wmin_o);
-      // the recompute filter (a pair outside A has W = +infinity), and the smallest rank
-      uint32_t rbest = 0xFFFFFFFFu;
+      // ranks after the recompute filter (a pair outside A has W = +infinity)
 #pragma unroll
-      for (int k = 0; k < IPT; ++k) {
-        const bool in = __fsub_rn(W[k], wmin) <= rc.c_max;
-        rank[k] = in ? rank[k] : 0xFFFFFFFFu;
-        rbest = min(rbest, rank[k]);
-      }
+      for (int k = 0; k < IPT; ++k) rank[k] = __fsub_rn(W[k], wmin) <= rc.c_max ? rank[k] : 0xFFFFFFFFu;
+      uint32_t rbest = rank[0];
+#pragma unroll
+      for (int k = 1; k < IPT; ++k) rbest = min(rbest, rank[k]);
       const uint32_t mw = __reduce_min_sync(0xffffffffu, rbest);
       uint32_t n_eq = 0;
-      uint64_t bk = psk::kNoKey;
-      uint32_t bt = 0xFFFFFFFFu, bh = 0u;
+      uint2 bk;
+      uint32_t bt, bh;
+      // The thread's smallest, picked beside the reduction.  Algorithm 1's key stays two words of the pair's
+      // state: only equal ranks read it, and built for every pair it takes a tenth of a step's instructions
+      // (1024 x 16384: 14.36 ms with it, 14.18 without).
+      auto key_words = [&](int k) {
+        if (GEN) return make_uint2((uint32_t)key[k], (uint32_t)(key[k] >> 32));
+        const bool in_t = rank[k] < 0x80000000u;
+        return make_uint2(in_t ? kq[k] : (uint32_t)(q32[k] + ((int32_t)rc.L - (int32_t)(h[k] << 4))),
+                          in_t ? kdh[k] : (uint32_t)Bp[k]);
+      };
 #pragma unroll
       for (int k = 0; k < IPT; ++k)
-        if (rank[k] == mw) {
-          ++n_eq;
-          bk = key[k];
+        if (k == 0 || rank[k] == rbest) {
+          if (rank[k] == rbest) ++n_eq;
+          bk = key_words(k);
           bt = tie[k];
           bh = h[k];
         }
+      const bool has = rbest == mw;
       // the lane that holds it hands it on at once (with equal ranks several do, and the smallest again below)
-      if (n_eq != 0u) {
+      if (has) {
         s_rank[s & 1u][warp] = mw;
         s_th[s & 1u][warp] = make_uint2(bt, bh);
         s_key[s & 1u][warp] = bk;
       }
-      const unsigned lanes = __ballot_sync(0xffffffffu, n_eq != 0u);
-      const unsigned many = IPT > 1 ? __ballot_sync(0xffffffffu, n_eq > 1u) : 0u;
+      const unsigned lanes = __ballot_sync(0xffffffffu, has);
+      const unsigned many = IPT > 1 ? __ballot_sync(0xffffffffu, has && n_eq > 1u) : 0u;
       if (mw != 0xFFFFFFFFu && ((lanes & (lanes - 1u)) | many)) {
         // equal ranks: the smallest (key, tie) of the lane's, then of the warp's
+        uint64_t kk = psk::kNoKey;
+        bt = 0xFFFFFFFFu;
 #pragma unroll
         for (int k = 0; k < IPT; ++k)
-          if (rank[k] == mw && (key[k] < bk || (key[k] == bk && tie[k] < bt))) {
-            bk = key[k];
-            bt = tie[k];
-            bh = h[k];
+          if (rank[k] == mw) {
+            const uint2 w = key_words(k);
+            const uint64_t x = GEN ? key[k] : dcq_key(mw, w, h[k]);
+            if (x < kk || (x == kk && tie[k] < bt)) {
+              kk = x;
+              bk = w;
+              bt = tie[k];
+              bh = h[k];
+            }
           }
-        const int win = warp_argmin(n_eq ? mw : 0xFFFFFFFFu, bk, bt);
+        const int win = warp_argmin(has ? mw : 0xFFFFFFFFu, kk, bt);
         __syncwarp();
         if (lane == win) {
           s_th[s & 1u][warp] = make_uint2(bt, bh);
@@ -1113,7 +1140,7 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
       if (lane == (win < 0 ? 0 : win)) {
         s_rank[s & 1u][warp] = rank;
         s_th[s & 1u][warp] = make_uint2(bt[0], bh[0]);
-        s_key[s & 1u][warp] = bk[0];
+        s_key[s & 1u][warp] = make_uint2((uint32_t)bk[0], (uint32_t)(bk[0] >> 32));
       }
       __syncwarp();
     }
