@@ -383,26 +383,29 @@ score_rows_kernel(const uint32_t* __restrict__ hits, psk::StateSoA st, uint32_t 
 // and the warps' picks go to shared slots, which one thread per row combines after the next pair's
 // barrier.  Shared reduction slots alternate between iterations, so one barrier per pair of rows
 // suffices.
+// Bound by instruction issue and latency with four warps a scheduler: 1024 x 16384 with every output
+// 75 us, 218 MB, 2.9 TB/s.  Three or four blocks an SM cost registers (80, 64: spills) and time (50 us more).
+// Blocks have a thread per four instances: 128 threads up to 512 instances (2 x 512 columns x 4096
+// requests scored in two reductions each: 300 us a window; 315 with 256 threads, half of them idle).
 constexpr uint32_t kBlkRowsAhead = 256;  // row constants computed per refill
-constexpr uint32_t kBlkThreads = 256;    // 4 instances a thread, up to 1024 instances
 
 struct BlkRow {
   float t_cached, Z, etaZ, ttft_budget, tpot_target;
   uint32_t L;
 };
 
-template <bool GEN, bool VEC, bool ALL>
-__global__ void __launch_bounds__(kBlkThreads, 2)
+template <int NT, bool GEN, bool VEC, bool ALL>
+__global__ void __launch_bounds__(NT, 512 / NT)
 score_block_kernel(const uint32_t* __restrict__ hits, psk::StateSoA st, uint32_t I, psk::WindowDev w, psk::DevModel m,
                    float* __restrict__ tpot_out, float* __restrict__ ttft_out, uint8_t* __restrict__ cls_out,
                    int32_t* __restrict__ best_out, uint8_t* __restrict__ path_out, psk::ShardIO sh) {
   __shared__ BlkRow s_rc[kBlkRowsAhead];
-  __shared__ __align__(16) uint32_t s_w[2][2][8];  // [parity][row of the pair][warp]
-  __shared__ unsigned long long s_k[2][2][8];
-  __shared__ uint32_t s_t[2][2][8];
+  constexpr int nw = NT / 32;
+  __shared__ __align__(16) uint32_t s_w[2][2][nw];  // [parity][row of the pair][warp]
+  __shared__ unsigned long long s_k[2][2][nw];
+  __shared__ uint32_t s_t[2][2][nw];
   const uint32_t t = threadIdx.x;
   const int lane = (int)(t & 31u), warp = (int)(t >> 5);
-  constexpr int nw = kBlkThreads / 32;  // the launch's block size
   const uint32_t i0 = 4u * t;
   constexpr bool all_pairs = ALL;  // some per-pair output is wanted (the launch checks)
   // instance terms (padding instances past I fail the capacity guard: room -1)
@@ -594,10 +597,10 @@ score_block_kernel(const uint32_t* __restrict__ hits, psk::StateSoA st, uint32_t
       const uint32_t rr = (r - r_lo) % kBlkRowsAhead;  // even, so row r + 1 is in the same batch
       if (rr == 0) {
         __syncthreads();  // every thread is done with the previous batch of row constants
-        const uint32_t x = r + t;
-        if (t < kBlkRowsAhead && x < r_hi) {
+        for (uint32_t y = t; y < kBlkRowsAhead && r + y < r_hi; y += NT) {
+          const uint32_t x = r + y;
           const psk::RowConst rc = psk::row_const(m, __ldg(w.L + x), __ldg(w.ttft_t + x), __ldg(w.tpot_t + x));
-          s_rc[t] = BlkRow{rc.t_cached, rc.Z, rc.etaZ, rc.ttft_budget, rc.tpot_target, rc.L};
+          s_rc[y] = BlkRow{rc.t_cached, rc.Z, rc.etaZ, rc.ttft_budget, rc.tpot_target, rc.L};
         }
         __syncthreads();
       }
@@ -632,11 +635,13 @@ score_block_kernel(const uint32_t* __restrict__ hits, psk::StateSoA st, uint32_t
         const int q = t == 0 ? 0 : 1;
         merge(prev_r + (uint32_t)q, q, q == 0 ? pw0 : pw1, par ^ 1u);
       }
-      {  // the eight warps' values of both rows, four 16-byte loads
-        const uint4* sw = reinterpret_cast<const uint4*>(&s_w[par][0][0]);
-        const uint4 a0 = sw[0], a1 = sw[1], b0 = sw[2], b1 = sw[3];
-        w0 = min(min(min(a0.x, a0.y), min(a0.z, a0.w)), min(min(a1.x, a1.y), min(a1.z, a1.w)));
-        w1 = min(min(min(b0.x, b0.y), min(b0.z, b0.w)), min(min(b1.x, b1.y), min(b1.z, b1.w)));
+      // the warps' values of both rows, by 16-byte loads
+      w0 = w1 = 0xFFFFFFFFu;
+#pragma unroll
+      for (int v = 0; v < nw / 4; ++v) {
+        const uint4 a = reinterpret_cast<const uint4*>(s_w[par][0])[v], b = reinterpret_cast<const uint4*>(s_w[par][1])[v];
+        w0 = min(w0, min(min(a.x, a.y), min(a.z, a.w)));
+        w1 = min(w1, min(min(b.x, b.y), min(b.z, b.w)));
       }
       if (sh.wmin_out) {  // column block, first reduction only
         if (t == 0) sh.wmin_out[r] = w0;
@@ -677,6 +682,7 @@ score_block_kernel(const uint32_t* __restrict__ hits, psk::StateSoA st, uint32_t
   else rows_loop(std::integral_constant<bool, false>());
 }
 
+template <int NT>
 cudaError_t score_block_launch(const uint32_t* hits, psk::StateSoA st, uint32_t I, const psk::WindowDev& w,
                                const psk::DevModel& m, float* tpot, float* ttft, uint8_t* cls, int32_t* best,
                                uint8_t* path, int num_sms, cudaStream_t s, const psk::ShardIO& sh) {
@@ -684,21 +690,20 @@ cudaError_t score_block_launch(const uint32_t* hits, psk::StateSoA st, uint32_t 
                    (reinterpret_cast<uintptr_t>(tpot) & 15u) == 0u && (reinterpret_cast<uintptr_t>(ttft) & 15u) == 0u &&
                    (reinterpret_cast<uintptr_t>(cls) & 3u) == 0u;
   const bool gen = m.sel != psk::kSelDCQ || m.fb_dcq;
-  const uint32_t threads = kBlkThreads;
   const bool all = tpot || ttft || cls;
-  decltype(&score_block_kernel<true, true, true>) kern;
+  decltype(&score_block_kernel<NT, true, true, true>) kern;
   if (all)
-    kern = vec ? (gen ? score_block_kernel<true, true, true> : score_block_kernel<false, true, true>)
-               : (gen ? score_block_kernel<true, false, true> : score_block_kernel<false, false, true>);
+    kern = vec ? (gen ? score_block_kernel<NT, true, true, true> : score_block_kernel<NT, false, true, true>)
+               : (gen ? score_block_kernel<NT, true, false, true> : score_block_kernel<NT, false, false, true>);
   else
-    kern = vec ? (gen ? score_block_kernel<true, true, false> : score_block_kernel<false, true, false>)
-               : (gen ? score_block_kernel<true, false, false> : score_block_kernel<false, false, false>);
+    kern = vec ? (gen ? score_block_kernel<NT, true, true, false> : score_block_kernel<NT, false, true, false>)
+               : (gen ? score_block_kernel<NT, true, false, false> : score_block_kernel<NT, false, false, false>);
   int per_sm = 0;  // one wave of resident blocks, each taking a contiguous range of rows
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, (int)threads, 0);
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, 0);
   if (e != cudaSuccess) return e;
   uint32_t grid = (uint32_t)num_sms * (uint32_t)(per_sm > 0 ? per_sm : 1);
   if (grid > w.R) grid = w.R;
-  kern<<<grid, threads, 0, s>>>(hits, st, I, w, m, tpot, ttft, cls, best, path, sh);
+  kern<<<grid, NT, 0, s>>>(hits, st, I, w, m, tpot, ttft, cls, best, path, sh);
   return cudaGetLastError();
 }
 
@@ -746,7 +751,8 @@ cudaError_t launch_score(const uint32_t* hits, psk::StateSoA st, uint32_t I, con
   if (w.R == 0) return cudaSuccess;
   if (I <= 128u) return score_launch<1>(hits, st, I, w, m, tpot, ttft, cls, best, path, num_sms, s, sh);
   if (I <= 256u) return score_launch<2>(hits, st, I, w, m, tpot, ttft, cls, best, path, num_sms, s, sh);
-  if (I <= 1024u) return score_block_launch(hits, st, I, w, m, tpot, ttft, cls, best, path, num_sms, s, sh);
+  if (I <= 512u) return score_block_launch<128>(hits, st, I, w, m, tpot, ttft, cls, best, path, num_sms, s, sh);
+  if (I <= 1024u) return score_block_launch<256>(hits, st, I, w, m, tpot, ttft, cls, best, path, num_sms, s, sh);
   return score_launch<4>(hits, st, I, w, m, tpot, ttft, cls, best, path, num_sms, s, sh);
 }
 
