@@ -734,7 +734,7 @@ evict_choose_kernel(EvictPlan* plan, const uint32_t* __restrict__ list, const ui
         plan[i].lo = lo;
         plan[i].hi = p.hi - lo < w ? p.hi : lo + w;
         plan[i].below = acc;
-        plan[i].k = p.todo - acc;
+        plan[i].k = sh == 0u && v[u] > kClassMax ? 0u : p.todo - acc;  // too many for the order kernel: not gathered
       }
       acc += v[u];
     }
@@ -751,6 +751,7 @@ evict_gather_kernel(const psk::TableDesc* __restrict__ tdesc, psk::LruMeta meta,
   const uint32_t lane = threadIdx.x & 31u;
   for (uint64_t item = blockIdx.x; item < items; item += gridDim.x) {
     const uint32_t i = list[item / chunks];
+    if (plan[i].k == 0u) continue;  // block-uniform
     const psk::TableDesc d = tdesc[i];
     const uint64_t n = (uint64_t)d.nbkt * psk::kBucketSlots, x0 = (item % chunks) * kScanChunk;
     const uint64_t x1 = x0 + kScanChunk < n ? x0 + kScanChunk : n;
@@ -1223,19 +1224,28 @@ __device__ void evict_loader(const uint64_t* slots, const psk::LruMeta& meta, co
 __global__ void __launch_bounds__(kCollectThreads)
 leaf_collect_kernel(const uint64_t* __restrict__ slots, const psk::TableDesc* __restrict__ tdesc,
                     const unsigned long long* __restrict__ count, const uint64_t* __restrict__ cap, psk::LruMeta meta,
-                    const uint32_t* __restrict__ slow, Leaf* __restrict__ leafbuf, uint32_t* __restrict__ nleaf) {
+                    const uint32_t* __restrict__ slow, uint32_t max_use, Leaf* __restrict__ leafbuf,
+                    uint32_t* __restrict__ nleaf) {
   const uint32_t i = blockIdx.y;
   if (slow[i] != 1u || count[i] <= cap[i]) return;  // block-uniform
   const psk::TableDesc d = tdesc[i];
   const uint64_t nslots = (uint64_t)d.nbkt * psk::kBucketSlots;
-  const uint64_t stride = (uint64_t)gridDim.x * kCollectThreads;
-  for (uint64_t x = (uint64_t)blockIdx.x * kCollectThreads + threadIdx.x; x < nslots; x += stride) {
-    const uint64_t s = d.base + x;
-    const uint64_t key = __ldcs(slots + s);
-    if (key == psk::kEmpty || key == psk::kTomb || meta.children[s] != 0u) continue;
-    const uint32_t at = atomicAdd(nleaf + i, 1u);
-    if (at < (uint32_t)kLeafMax)
-      leafbuf[(uint64_t)i * kLeafMax + at] = make_leaf(meta.last_use[s], (uint32_t)s, key, meta.parent[s]);
+  const uint64_t stride = 4u * (uint64_t)gridDim.x * kCollectThreads;
+  // four slots a thread (tables are whole 8-slot buckets); an empty slot's stamp says so unless blocks
+  // carry that stamp too, so only leaves' keys are read (8 bytes a slot instead of 12)
+  for (uint64_t x = 4u * ((uint64_t)blockIdx.x * kCollectThreads + threadIdx.x); x < nslots; x += stride) {
+    const uint4 lu = __ldcs(reinterpret_cast<const uint4*>(meta.last_use + d.base + x));
+    const uint4 ch = __ldcs(reinterpret_cast<const uint4*>(meta.children + d.base + x));
+    const uint32_t l[4] = {lu.x, lu.y, lu.z, lu.w}, cc[4] = {ch.x, ch.y, ch.z, ch.w};
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (cc[u] != 0u || (l[u] == psk::kNoUse && max_use != psk::kNoUse)) continue;
+      const uint64_t s = d.base + x + (uint64_t)u, key = slots[s];
+      if (key == psk::kEmpty || key == psk::kTomb) continue;
+      const uint32_t at = atomicAdd(nleaf + i, 1u);
+      if (at < (uint32_t)kLeafMax)
+        leafbuf[(uint64_t)i * kLeafMax + at] = make_leaf(l[u], (uint32_t)s, key, meta.parent[s]);
+    }
   }
 }
 
@@ -1467,6 +1477,7 @@ cudaError_t launch_evict(uint64_t* slots, const psk::TableDesc* tdesc, uint32_t 
   const unsigned gx = (unsigned)((max_instance_slots + per_block - 1) / per_block);
   if ((e = cudaMemsetAsync(sc.slow, 0, (size_t)I * sizeof(uint32_t), s)) != cudaSuccess) return e;
   uint32_t todo = kMoreFast;
+  // Instances left to the one-at-a-time kernels wait for the last batch, and then go together.
   for (int round = 0; round < 4096 && todo; ++round) {
     if ((e = cudaMemsetAsync(sc.more, 0, sizeof(uint32_t), s)) != cudaSuccess) return e;
     if (todo & kMoreFast) {
@@ -1482,17 +1493,17 @@ cudaError_t launch_evict(uint64_t* slots, const psk::TableDesc* tdesc, uint32_t 
       evict_order_kernel<<<inst_grid, kOrderThreads, sizeof(OrderSmem), s>>>(slots, count, cap, meta, plan, sc.list, nlist,
                                                                             eb, sc.slow, sc.more, kLeafMax, err);
     }
-    if (todo & kMoreSlow) {
+    if (todo == kMoreSlow) {
       if ((e = cudaMemsetAsync(sc.nleaf, 0, (size_t)I * sizeof(uint32_t), s)) != cudaSuccess) return e;
       leaf_collect_kernel<<<dim3(gx ? gx : 1u, I), kCollectThreads, 0, s>>>(
-          slots, tdesc, count, cap, meta, sc.slow, static_cast<Leaf*>(sc.leafbuf), sc.nleaf);
+          slots, tdesc, count, cap, meta, sc.slow, max_use, static_cast<Leaf*>(sc.leafbuf), sc.nleaf);
       evict_kernel<<<I, kEvictThreads, smem, s>>>(slots, count, cap, meta, sc.slow, static_cast<const Leaf*>(sc.leafbuf),
                                                   sc.nleaf, sc.more, err);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = cudaMemcpyAsync(more_host, sc.more, sizeof(uint32_t), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
-    todo = *more_host;
+    todo = *more_host | (todo & kMoreFast ? todo & kMoreSlow : 0u);
   }
   return cudaSuccess;
 }
