@@ -489,7 +489,7 @@ def main():
         # per decision: the request's hit and T_pf rows (8 B per instance) and its decision outputs
         greedy_bytes = int(R * (8 * I + 16))
         achieved = greedy_bytes / (km[dominant] / 1000) / 1e9
-        roof = {"bound": "hbm", "kernel": "greedy_pipe_kernel" if args.probe_mode == 1 else "greedy_kernel",
+        roof = {"bound": "hbm", "kernel": "greedy_pipe_kernel",
                 "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": (None if greedy_traffic is None or args.probe_mode != 1 else greedy_traffic * R),
                 "peak_source": peak_src, "algorithmic_bytes_per_launch": greedy_bytes,

@@ -17,7 +17,7 @@ namespace {
 //           a parent counts if it was cached before the block in the order above.
 // Bound by the dependent round trips of a tile (about 3 to L2 or memory), not by bandwidth: one warp
 // inserting block after block took 2.1 us a block.  Bringing up a context with 96 instances x 20000
-// blocks took 46.6 ms that way, 1.48 ms now.
+// blocks took 46.6 ms that way, 0.89 ms now.
 constexpr uint32_t kInsThreads = 512;
 constexpr uint32_t kInsQueue = 2 * kInsThreads;  // chains collected before their blocks are inserted
 constexpr uint32_t kInsSet = 2 * kInsThreads;    // hash set of a tile's new keys (a power of two)
@@ -583,7 +583,7 @@ __device__ __forceinline__ uint32_t parent32(uint64_t p) {
 // and the order kernel's chain of dependent steps.  1024 instances x 200K blocks, about 240 over
 // capacity by up to 7.9K blocks: hist 0.12 ms, gather 0.11, detail 0.09, index and jump 0.07, order 0.17
 // (0.43 ms where the order kernel read the metadata itself, a block an SM); the streaming window of 500
-// requests takes 1.74 ms, and took 11.8 ms with one thread ordering each instance's evictions (1.2 us each).
+// requests takes 1.59 ms, and took 11.8 ms with one thread ordering each instance's evictions (1.2 us each).
 constexpr uint32_t kClassMax = 16384;   // blocks of one last_use value ordered in shared memory
 constexpr uint32_t kHistBits = 11;
 constexpr uint32_t kHistBins = 1u << kHistBits;
