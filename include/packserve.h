@@ -313,7 +313,9 @@ PS_API ps_status ps_score_window(ps_ctx* ctx, const ps_window* w, ps_scores* out
 /* Greedy in-window assignment (Algorithm 1 per request in arrival order, each admitted request
  * updating its instance's state and caching its blocks there before the next decision).
  * The result is a pending window: the committed state and caches are unchanged until
- * ps_commit_window; the next ps_schedule_window or ps_load_instances discards it.
+ * ps_commit_window; the next ps_schedule_window, ps_load_instances or ps_load_requests discards it.
+ * Windows scored in between (ps_score_window, ps_shard_wmin) leave it as it is, whatever memory their
+ * arrays or its own are in.
  * opt_scores (may be NULL) receives the window's independent scores against the committed state
  * (hits = the hit lengths before the window; best/path as ps_score_window).
  * Errors: as ps_score_window, plus PS_ERR_TABLE_FULL if the delta table overflowed (cannot happen

@@ -43,6 +43,19 @@ struct DeviceGuard {
   }
 };
 
+// Device buffers that a host window's arrays are staged in: together in `stage` when they fit, else one by
+// one.  The context has two sets.  A pending window from host memory stays in the first until it is
+// committed or discarded (a commit reads it again); what is scored in between goes to the second.
+struct WindowBuffers {
+  unsigned char* stage = nullptr;  // [kStageIn]
+  uint64_t* off = nullptr;
+  uint64_t* hash = nullptr;
+  uint32_t* L = nullptr;
+  float* ttft = nullptr;
+  float* tpot = nullptr;
+  uint32_t* outtok = nullptr;
+};
+
 }  // namespace
 
 struct ps_ctx {
@@ -69,16 +82,12 @@ struct ps_ctx {
   psk::RowList scratch{nullptr, nullptr};  // rows the probe searches from scratch
   uint32_t lastslot_n = 0;
   psk::StateSoA st{}, pend{};
-  uint64_t* d_off = nullptr;
-  uint64_t* d_hash = nullptr;
+  WindowBuffers win_buf[2];
   // shared-prefix windows (ps_window.parent): each request's own blocks and parent link, staged
   uint64_t* d_own_off = nullptr;
-  uint64_t* d_own_hash = nullptr;
+  uint64_t* d_own_hash = nullptr;  // also the second set's chains: a pending window is past its expansion
   int32_t* d_parent = nullptr;
   std::vector<uint64_t> h_full_off;
-  uint32_t* d_L = nullptr;
-  float* d_ttft = nullptr;
-  float* d_tpot = nullptr;
   uint32_t* d_hits = nullptr;
   float* d_tpf = nullptr;  // T_pf at each pair's hit, from the probe, for the greedy pass
   float* d_tpot_o = nullptr;
@@ -102,14 +111,15 @@ struct ps_ctx {
     size_t bytes;
   };
   std::vector<Handover> handover;  // results to hand on from h_out once the stream is done
-  unsigned char* d_stage = nullptr;  // [kStageIn] a small host window's arrays
   uint64_t win_blocks = 0;         // chain blocks of the window being staged
+  const uint32_t* win_out = nullptr;  // its out_tokens on the device (nullptr: none given)
   unsigned char *st_block = nullptr, *pend_block = nullptr, *gsync_block = nullptr, *zero_block = nullptr;
   cudaEvent_t ev[kNumEv] = {};
   bool ev_used[kNumPhases] = {};
   bool probe_split = false;            // kEvRelDone / kEvProbeMid recorded in the last probe phase
   unsigned long long* d_stats = nullptr;  // probe launch counters (ps_last_probe_stats)
   bool pending = false;
+  bool pend_staged = false;  // the pending window lies in win_buf[0] (else in the caller's device buffers)
   psk::WindowDev pend_win{};
   // column-block scoring: the window of the last ps_shard_wmin, whose hits are in d_hits
   bool shard_pending = false;
@@ -127,7 +137,6 @@ struct ps_ctx {
   uint64_t max_instance_slots = 0;
   psk::ReqStore rq{};
   uint64_t* d_cap = nullptr;
-  uint32_t* d_outtok = nullptr;
   std::vector<std::pair<void**, size_t>> wanted;  // ps_create: blocks to lay out in the arena
   void* arena = nullptr;                          // every device block of the context, one allocation
   std::string err;
@@ -277,10 +286,14 @@ ps_status check_capacity(ps_ctx* c) {
 // piece when they fit (flush), else copied each to its own buffer.
 struct Stager {
   ps_ctx* c;
+  const bool beside;  // next to a pending window that is staged: into the second set
+  const WindowBuffers& buf;
   bool packed;
   size_t used = 0;
   cudaError_t err = cudaSuccess;
-  Stager(ps_ctx* ctx, size_t bytes) : c(ctx), packed(bytes + 8 * 256 <= kStageIn) {}
+  Stager(ps_ctx* ctx, size_t bytes)
+      : c(ctx), beside(ctx->pending && ctx->pend_staged), buf(ctx->win_buf[beside ? 1 : 0]),
+        packed(bytes + 8 * 256 <= kStageIn) {}
   template <class T>
   const T* put(const T* src, size_t n, T* own) {
     if (n == 0) return own;
@@ -290,24 +303,23 @@ struct Stager {
       return own;
     }
     std::memcpy(c->h_in + used, src, n * sizeof(T));
-    const T* at = reinterpret_cast<const T*>(c->d_stage + used);
+    const T* at = reinterpret_cast<const T*>(buf.stage + used);
     used += (n * sizeof(T) + 255) / 256 * 256;
     return at;
   }
   cudaError_t flush() {
     if (packed && used && err == cudaSuccess)
-      err = cudaMemcpyAsync(c->d_stage, c->h_in, used, cudaMemcpyHostToDevice, c->stream);
+      err = cudaMemcpyAsync(buf.stage, c->h_in, used, cudaMemcpyHostToDevice, c->stream);
     return err;
   }
 };
 
 // The request arrays shared by both window forms (L, targets, output lengths).
 void stage_request_arrays(Stager& st, const ps_window* w, psk::WindowDev* out) {
-  ps_ctx* c = st.c;
-  out->L = st.put(w->prompt_tokens, w->R, c->d_L);
-  out->ttft_t = st.put(w->ttft_target, w->R, c->d_ttft);
-  out->tpot_t = st.put(w->tpot_target, w->R, c->d_tpot);
-  if (w->out_tokens && w->R) c->pend_out = st.put(w->out_tokens, w->R, c->d_outtok);
+  out->L = st.put(w->prompt_tokens, w->R, st.buf.L);
+  out->ttft_t = st.put(w->ttft_target, w->R, st.buf.ttft);
+  out->tpot_t = st.put(w->tpot_target, w->R, st.buf.tpot);
+  if (w->out_tokens && w->R) st.c->win_out = st.put(w->out_tokens, w->R, st.buf.outtok);
 }
 
 size_t request_bytes(const ps_window* w) { return (size_t)w->R * (w->out_tokens ? 16 : 12); }
@@ -339,15 +351,23 @@ ps_status stage_window_tree(ps_ctx* c, const ps_window* w, psk::WindowDev* out) 
   c->win_blocks = nblk;
   Stager st(c, 2 * ((size_t)R + 1) * sizeof(uint64_t) + (size_t)R * sizeof(int32_t) + nown * sizeof(uint64_t) +
                    request_bytes(w));
-  out->off = st.put(static_cast<const uint64_t*>(full.data()), (size_t)R + 1, c->d_off);
+  out->off = st.put(static_cast<const uint64_t*>(full.data()), (size_t)R + 1, st.buf.off);
   const uint64_t* d_own_off = st.put(own, R ? (size_t)R + 1 : 0, c->d_own_off);
   const int32_t* d_parent = st.put(w->parent, R, c->d_parent);
-  const uint64_t* d_own = st.put(w->chain_hash, nown, c->d_own_hash);
+  // The second set's chains take d_own_hash, so the own blocks go through the delta table there: it is
+  // empty but for the greedy pass, holds four words a block, and is cleared again behind the expansion.
+  uint64_t* const own_buf = st.beside ? reinterpret_cast<uint64_t*>(c->d_delta) : c->d_own_hash;
+  const uint64_t* d_own = st.put(w->chain_hash, nown, own_buf);
   stage_request_arrays(st, w, out);
-  PS_TRY_CUDA(c, st.flush());
-  PS_TRY_CUDA(c, pskl::launch_expand_chains(out->off, d_own_off, d_own, d_parent, R, c->d_hash, c->d_err, c->num_sms,
-                                            c->stream));
-  out->hash = c->d_hash;
+  cudaError_t e = st.flush();
+  if (e == cudaSuccess)
+    e = pskl::launch_expand_chains(out->off, d_own_off, d_own, d_parent, R, st.buf.hash, c->d_err, c->num_sms, c->stream);
+  if (st.beside && !st.packed) {
+    const cudaError_t e2 = cudaMemsetAsync(c->d_delta, 0, nown * sizeof(uint64_t), c->stream);
+    if (e == cudaSuccess) e = e2;
+  }
+  PS_TRY_CUDA(c, e);
+  out->hash = st.buf.hash;
   return PS_OK;
 }
 
@@ -360,12 +380,12 @@ ps_status stage_window(ps_ctx* c, const ps_window* w, psk::WindowDev* out) {
   if (!w->chain_off || (w->R > 0 && (!w->prompt_tokens || !w->ttft_target || !w->tpot_target)))
     return fail(c, PS_ERR_INVALID, "window array is NULL");
   out->R = w->R;
-  c->pend_out = nullptr;
+  c->win_out = nullptr;
   c->win_blocks = 0;
   c->h_out_used = 0;
   if (w->inputs_on_device) {
     if (w->parent) return fail(c, PS_ERR_INVALID, "a window with parent links must be in host memory");
-    c->pend_out = w->out_tokens;
+    c->win_out = w->out_tokens;
     out->off = w->chain_off;
     out->hash = w->chain_hash;
     out->L = w->prompt_tokens;
@@ -396,8 +416,8 @@ ps_status stage_window(ps_ctx* c, const ps_window* w, psk::WindowDev* out) {
   if (nblk > 0 && !w->chain_hash) return fail(c, PS_ERR_INVALID, "chain_hash is NULL");
   c->win_blocks = nblk;
   Stager st(c, ((size_t)w->R + 1 + nblk) * sizeof(uint64_t) + request_bytes(w));
-  out->off = st.put(off, (size_t)w->R + 1, c->d_off);
-  out->hash = st.put(w->chain_hash, nblk, c->d_hash);
+  out->off = st.put(off, (size_t)w->R + 1, st.buf.off);
+  out->hash = st.put(w->chain_hash, nblk, st.buf.hash);
   stage_request_arrays(st, w, out);
   PS_TRY_CUDA(c, st.flush());
   return PS_OK;
@@ -558,15 +578,18 @@ ps_status ps_create(const ps_config* cfg, ps_ctx** out) {
   want(c, &c->d_cprefix, 2 * (Rmax + 1));
   want(c, &c->st_block, I * kStateBytes);
   want(c, &c->pend_block, I * kStateBytes);
-  want(c, &c->d_stage, kStageIn);
-  want(c, &c->d_off, Rmax + 1);
-  want(c, &c->d_hash, c->max_blocks);
+  for (WindowBuffers& b : c->win_buf) {
+    want(c, &b.stage, kStageIn);
+    want(c, &b.off, Rmax + 1);
+    want(c, &b.L, Rmax);
+    want(c, &b.ttft, Rmax);
+    want(c, &b.tpot, Rmax);
+    want(c, &b.outtok, Rmax);
+  }
+  want(c, &c->win_buf[0].hash, c->max_blocks);
   want(c, &c->d_own_off, Rmax + 1);
   want(c, &c->d_own_hash, c->max_blocks);
   want(c, &c->d_parent, Rmax);
-  want(c, &c->d_L, Rmax);
-  want(c, &c->d_ttft, Rmax);
-  want(c, &c->d_tpot, Rmax);
   want(c, &c->d_hits, RI);
   want(c, &c->d_tpf, RI);
   want(c, &c->d_tpot_o, RI);
@@ -582,7 +605,6 @@ ps_status ps_create(const ps_config* cfg, ps_ctx** out) {
   want(c, &c->d_shard_key, Rmax);
   want(c, &c->d_shard_tie, Rmax);
   want(c, &c->d_cap, I);
-  want(c, &c->d_outtok, Rmax);
   if (c->lru) {
     for (uint32_t i = 0; i < I; ++i)
       c->max_instance_slots = std::max<uint64_t>(c->max_instance_slots, (uint64_t)td[i].nbkt * psk::kBucketSlots);
@@ -615,6 +637,7 @@ ps_status ps_create(const ps_config* cfg, ps_ctx** out) {
     cudaGetLastError();
     return bail(PS_ERR_OOM);
   }
+  c->win_buf[1].hash = c->d_own_hash;
   c->st = state_arrays(c->st_block, I);
   c->pend = state_arrays(c->pend_block, I);
   c->gsync.stats = reinterpret_cast<unsigned long long*>(c->gsync_block);
@@ -967,7 +990,9 @@ ps_status ps_schedule_window(ps_ctx* c, const ps_window* w, ps_decisions* out, p
   s = finish(c);
   if (s != PS_OK) return s;
   c->pending = true;
+  c->pend_staged = w->inputs_on_device == 0;
   c->pend_win = wd;
+  c->pend_out = c->win_out;
   return PS_OK;
 }
 
