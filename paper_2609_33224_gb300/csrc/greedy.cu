@@ -200,7 +200,7 @@ __device__ void probe_rows(const psk::RowPre* __restrict__ rows, const uint64_t*
                            const psk::DevModel& m, const psk::DeltaSlot* delta, uint64_t nslots, uint32_t* err,
                            const psk::GreedySync& sync, unsigned long long* smem_raw, uint32_t pb, uint32_t nprobe,
                            const MainTables& mt) {
-  uint32_t* s_end = reinterpret_cast<uint32_t*>(smem_raw);  // chain end of the last job on i (0 = none)
+  uint32_t* s_end = reinterpret_cast<uint32_t*>(smem_raw);  // chain end of the last job with blocks on i (0 = none)
   uint32_t* s_res = s_end + I;                               // search start / result per instance
   uint32_t* s_walk = s_res + I;                              // instances handed to a warp search
   __shared__ uint32_t s_nwalk;
@@ -228,7 +228,7 @@ __device__ void probe_rows(const psk::RowPre* __restrict__ rows, const uint64_t*
     const int64_t need = (int64_t)s - psk::kLag + 1;  // jobs [0, need) count for this row
     if (warp == 0) {
       // Replay the published jobs [replayed, need), 32 at a time; for each instance the latest of
-      // them sets its chain end.
+      // them that has blocks sets its chain end.
       uint32_t f = s_replayed;
       bool abort = false;
       while ((int64_t)f < need && !abort) {
@@ -238,10 +238,10 @@ __device__ void probe_rows(const psk::RowPre* __restrict__ rows, const uint64_t*
         if (mine) jb = wait_job(sync.jobs + x, err, sync.wait_ns);
         abort = __any_sync(0xffffffffu, mine && jb == 0ull);
         if (abort) break;
-        const uint32_t j = mine ? job_pick(jb) : 0xFFFFFFFFu;
         const uint32_t nbx = mine ? __ldg(&rows[x].nb) : 0u;
+        const uint32_t j = nbx ? job_pick(jb) : 0xFFFFFFFFu;  // (a prompt without a block inserts nothing)
         const unsigned same = __match_any_sync(0xffffffffu, j);
-        if (mine && j < I && (31 - __clz(same)) == lane) s_end[j] = nbx;
+        if (j < I && (31 - __clz(same)) == lane) s_end[j] = nbx;
         const uint32_t n = (int64_t)f + 32 <= need ? 32u : (uint32_t)(need - (int64_t)f);
         f += n;
       }

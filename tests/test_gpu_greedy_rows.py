@@ -20,9 +20,10 @@ def P():
     return P
 
 
-def _check(P, model, ins, win):
+def _check(P, model, ins, win, mode=1):
     orc = Oracle(ins.I, model).load(ins)
-    with P.Scheduler(ins.I, ins.cap_blocks, win.R, int(win.chain_off[-1]), model, table_load_factor=0.5) as s:
+    with P.Scheduler(ins.I, ins.cap_blocks, win.R, int(win.chain_off[-1]), model, table_load_factor=0.5,
+                     probe_mode=mode) as s:
         s.load_workload_instances(ins)
         g = s.schedule_window(win)
         o = orc.schedule(win)
@@ -49,6 +50,57 @@ def test_instance_counts(P, I):
 def test_window_lengths(P, R):
     wl = _workload(12, R)
     _check(P, wl.model, wl.instances, wl.window)
+
+
+def _prompts(nb_of, chains, I):
+    """Window of one prompt per entry of nb_of (tokens; chains[k] its blocks' hashes), empty caches."""
+    off = np.zeros(len(chains) + 1, np.uint64)
+    off[1:] = np.cumsum([c.size for c in chains])
+    R = len(chains)
+    win = W.Window(chain_off=off, chain_hash=np.concatenate(chains).astype(np.uint64),
+                   prompt_tokens=np.array(nb_of, np.uint32), ttft_target=np.full(R, 1e7, np.float32),
+                   tpot_target=np.full(R, 1e4, np.float32), session=np.zeros(R, np.uint32), out_tokens=np.zeros(R, np.uint32))
+    z = np.zeros(I, np.int64)
+    ins = W.Instances(b=z.astype(np.int32), qr=z.astype(np.int32), q=z, S=z.copy(), M_KV=np.full(I, 10 ** 8, np.int64),
+                      B_max=np.full(I, 10 ** 5, np.int32), cap_blocks=np.full(I, 4096, np.uint64),
+                      chain_inst=np.zeros(0, np.uint32), chain_off=np.zeros(1, np.uint64),
+                      chain_hash=np.zeros(0, np.uint64), chain_parent=np.zeros(0, np.uint64))
+    return ins, win
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("shorts", [31, 32, 33, 45, 130])
+def test_prompts_without_a_block_hide_no_inserts(P, shorts, mode):
+    """A chain cached by the window's first request, prompts too short for a block on the same instance, then
+    requests that share half of that chain, from further back than the common prefixes reach."""
+    rng = np.random.default_rng(3)
+    new = lambda n: rng.integers(2, 2 ** 63, n, dtype=np.int64).astype(np.uint64)
+    base = new(10)
+    chains = [base] + [new(0)] * shorts + [np.concatenate([base[:5], new(3)]), base, new(4)]
+    ins, win = _prompts([160] + [8] * shorts + [128, 160, 64], chains, 1)
+    o = _check(P, dict(W.MODEL_DEFAULT), ins, win, mode)
+    assert o["hit_chosen"][shorts + 1:].tolist() == [5, 10, 0]
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("I,R,seed", [(3, 400, 1), (70, 900, 2)])
+def test_windows_of_mixed_prompt_lengths(P, I, R, seed, mode):
+    rng = np.random.default_rng(seed)
+    trunk = [rng.integers(2, 2 ** 63, 300, dtype=np.int64).astype(np.uint64) for _ in range(8)]
+    lens, chains = [], []
+    for _ in range(R):
+        if rng.random() < 0.4:
+            n, c = 0, np.zeros(0, np.uint64)
+        else:
+            t, cut = trunk[int(rng.integers(8))], int(rng.integers(1, 300))
+            c = t[:cut]
+            if rng.random() < 0.5:
+                c = np.concatenate([c, rng.integers(2, 2 ** 63, int(rng.integers(1, 20)), dtype=np.int64).astype(np.uint64)])
+            n = c.size
+        chains.append(c)
+        lens.append(16 * n + int(rng.integers(0, 16)))
+    ins, win = _prompts(lens, chains, I)
+    _check(P, dict(W.MODEL_DEFAULT), ins, win, mode)
 
 
 @pytest.mark.parametrize("selector", range(6))
