@@ -979,6 +979,8 @@ ps_status ps_schedule_window(ps_ctx* c, const ps_window* w, ps_decisions* out, p
   PS_TRY_CUDA(c, pskl::launch_greedy(c->d_rows, wd, c->I, hit0, c->d_tpf, c->st, c->pend, c->model, c->d_delta,
                                      nslots, c->d_assign, c->d_dpath, c->d_hchosen, c->d_err, c->gsync,
                                      c->search, c->d_slots, c->d_ovf, c->d_tdesc, c->stream));
+  if (wd.R == 0)  // nobody to decide: the greedy pass, which writes the pending state, does not run
+    PS_TRY_CUDA(c, cudaMemcpyAsync(c->pend_block, c->st_block, c->I * kStateBytes, cudaMemcpyDeviceToDevice, c->stream));
   record(c, kEvGreedy1);
   c->ev_used[2] = true;
   PS_TRY_CUDA(c, pskl::launch_delta_clear(c->d_delta, nslots, c->stream));

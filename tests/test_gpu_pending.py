@@ -84,3 +84,42 @@ def test_scoring_leaves_the_pending_window_alone(P, form_a, R_a, form_b, R_b, ca
         g, o = s.schedule_window(win_b), orc.schedule(B, window_id=2, streaming=True)
         for k in ("assign", "path", "hit_chosen"):
             assert np.array_equal(g[k], o[k]), k
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_empty_windows_leave_the_state_as_it_is(P, mode):
+    """A gateway whose interval holds no arrival: the pending state of an empty window is the committed one, on
+    a new context, after other windows and after the engines' progress."""
+    wl = W.generate(0, seed=22, num_instances=5, window_requests=40, num_sessions=12, cap_blocks=9000)
+    ins, A = wl.instances, wl.window
+    ins.M_KV[:] = 10 ** 8  # requests are admitted
+    empty = W.Window(**{k: (v[:1] if k == "chain_off" else v[:0]) for k, v in vars(A).items()})
+    orc = Oracle(ins.I, wl.model, track_lru=True).load(ins)
+    with P.Scheduler(ins.I, ins.cap_blocks, 64, int(A.chain_off[-1]) * 2, wl.model, probe_mode=mode, track_lru=True,
+                     max_active_requests=512) as s:
+        s.load_workload_instances(ins)
+
+        def nothing_arrives(win):
+            before = s.get_instances()
+            assert s.schedule_window(win)["assign"].size == 0
+            for state in (s.get_instances(pending=True), s.commit_window() or s.get_instances()):
+                for k, v in before.items():
+                    assert np.array_equal(state[k], v), k
+
+        nothing_arrives(empty)
+        orc.load_requests(wl.initial_requests())
+        s.load_requests(wl.initial_requests())
+        nothing_arrives(_Device(empty))
+        for w, win in enumerate((A, wl.next_window(40))):
+            g, o = s.schedule_window(win), orc.schedule(win, window_id=w + 1, streaming=True)
+            for k in ("assign", "path", "hit_chosen"):
+                assert np.array_equal(g[k], o[k]), k
+            assert (g["assign"] >= 0).any()
+            s.commit_window(last_use=w + 1)
+            nothing_arrives(empty)
+            s.advance_window(40.0, 20000, evict=False)
+            orc.advance(40.0, 20000, evict=False)
+            nothing_arrives(empty)
+            st, ost = s.get_instances(), orc.get_state()
+            for k in ("b", "qr", "q", "S"):
+                assert np.array_equal(st[k], ost[k]), k
