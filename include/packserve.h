@@ -316,6 +316,9 @@ PS_API ps_status ps_score_window(ps_ctx* ctx, const ps_window* w, ps_scores* out
  * ps_commit_window; the next ps_schedule_window, ps_load_instances or ps_load_requests discards it.
  * Windows scored in between (ps_score_window, ps_shard_wmin) leave it as it is, whatever memory their
  * arrays or its own are in.
+ * The greedy pass is one cooperative launch of up to 129 thread blocks, one to an SM, which must all be
+ * resident together: it starts once kernels of other streams leave it that many SMs, and takes fewer
+ * blocks (at least 6) on a device, or a stream, that has fewer.
  * opt_scores (may be NULL) receives the window's independent scores against the committed state
  * (hits = the hit lengths before the window; best/path as ps_score_window).
  * Errors: as ps_score_window, plus PS_ERR_TABLE_FULL if the delta table overflowed (cannot happen

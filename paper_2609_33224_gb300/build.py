@@ -42,6 +42,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(BUILD, exist_ok=True)
     nvcc = _nvcc()
     headers = [os.path.join(CSRC, "ps_internal.cuh"), os.path.join(CSRC, "calibrate.h"),
+               os.path.join(CSRC, "greedy_grid.h"),
                os.path.join(ROOT, "include", "packserve.h")]
     jobs = []
     for src in SOURCES:

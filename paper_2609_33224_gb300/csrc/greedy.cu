@@ -5,6 +5,7 @@
 // replays that sequence for a whole window on the GPU: a pipelined cooperative launch of one deciding
 // block, insert blocks and probe blocks.  Committed tables are never written here; the decisions and
 // the updated state are a pending window that ps_commit_window applies.
+#include "greedy_grid.h"
 #include "ps_internal.cuh"
 
 namespace {
@@ -45,8 +46,6 @@ namespace {
 // main 32 blocks a step on every instance whose hit rose, 50 us a decision (100 x 300: 15.2 ms of greedy
 // pass, 0.46 here).
 
-constexpr uint32_t kInsertBlocks = 64;  // insert blocks
-constexpr uint32_t kProbeBlocks = 64;   // probe blocks
 constexpr uint32_t kPipeThreads = 608;  // threads of every block of the launch
 constexpr uint32_t kFeedRing = 8;       // rows staged in the deciding block's shared memory
 constexpr unsigned long long kJobValid = 1ull << 63;  // a published job word (0 = not yet published)
@@ -105,9 +104,8 @@ __device__ __forceinline__ uint32_t job_hit(unsigned long long jb) { return (uin
 // inserts are in, so the job's blocks are all in when the count reaches kInsertGroup.  A thread
 // claims the home slots of kInsertBatch keys at once (the claims are independent) and follows the
 // rare occupied home slot on its own.
-constexpr uint32_t kInsertGroup = 4;
+using psgrid::kInsertGroup;
 constexpr int kInsertBatch = 4;
-static_assert(kInsertBlocks % kInsertGroup == 0, "whole insert groups");
 
 // The committed tables, for caches that are not prefix-closed.
 struct MainTables {
@@ -188,7 +186,7 @@ __device__ void insert_blocks(const psk::RowPre* __restrict__ rows, const uint64
   }
 }
 
-// Probe blocks: block p probes rows p, p + kProbeBlocks, ... in order (see the section comment).
+// Probe blocks: block p probes rows p, p + their number, ... in order (see the section comment).
 // Per row, everything that does not need the window's inserts comes first: replaying the published
 // jobs <= s - kLag (which instances have window inserts, their last chain end, the picks of the
 // row's ancestors), the hit0 row, the probe positions and the chain blocks there.  Only then does the
@@ -1196,7 +1194,7 @@ cudaError_t greedy_pipe_launch(const psk::RowPre* rows, const psk::WindowDev& w,
                                const float* tpf0, psk::StateSoA committed, psk::StateSoA pending, const psk::DevModel& m,
                                psk::DeltaSlot* delta, uint64_t nslots, int32_t* assign, uint8_t* path,
                                uint32_t* hit_chosen, uint32_t* err, const psk::GreedySync& sync, bool linear,
-                               MainTables mt, cudaStream_t s) {
+                               MainTables mt, int num_sms, cudaStream_t s) {
   // not Algorithm 1's order (Table 4 / Table 3 variants), or Eq. 9's interference term
   const bool gen = m.sel != psk::kSelDCQ || m.fb_dcq || m.interference_mode != 0;
   auto kern = linear ? greedy_pipe_kernel<IPT, true, true>
@@ -1209,14 +1207,19 @@ cudaError_t greedy_pipe_launch(const psk::RowPre* rows, const psk::WindowDev& w,
   psk::StateSoA c = committed, p = pending;
   psk::DevModel mm = m;
   psk::GreedySync sy = sync;
-  // A window of up to kLag requests has no row that reads the delta table, so nothing to insert.
-  uint32_t ninsert = R > (uint32_t)psk::kLag ? kInsertBlocks : 0u;
-  const uint32_t nprobe = R < kProbeBlocks ? R : kProbeBlocks;
+  uint32_t ninsert = 0;
   void* args[] = {(void*)&rows, (void*)&hash, (void*)&R, (void*)&I, (void*)&hit0, (void*)&tpf0, (void*)&c, (void*)&p,
                   (void*)&mm, (void*)&delta, (void*)&nslots, (void*)&assign, (void*)&path, (void*)&hit_chosen,
                   (void*)&err, (void*)&sy, (void*)&ninsert, (void*)&mt};
-  // all blocks must be resident at once: they wait on one another
-  return cudaLaunchCooperativeKernel((const void*)kern, dim3(1 + ninsert + nprobe), dim3(kPipeThreads), args, smem, s);
+  // All blocks must be resident at once, and one fits on an SM.  A stream may be limited to fewer SMs than the
+  // device reports: a launch that is too large for it is refused before it starts, and half as many tried.
+  for (uint32_t resident = (uint32_t)num_sms;; resident /= 2u) {
+    const psgrid::PipeGrid g = psgrid::pipe_grid(R, psk::kLag, resident);
+    ninsert = g.insert;
+    e = cudaLaunchCooperativeKernel((const void*)kern, dim3(g.blocks()), dim3(kPipeThreads), args, smem, s);
+    if (e != cudaErrorCooperativeLaunchTooLarge || g.blocks() <= psgrid::kMinBlocks) return e;
+    cudaGetLastError();
+  }
 }
 
 }  // namespace
@@ -1227,7 +1230,8 @@ cudaError_t launch_greedy(const psk::RowPre* rows, const psk::WindowDev& w, uint
                                  const float* tpf0, psk::StateSoA committed, psk::StateSoA pending, const psk::DevModel& m,
                                  psk::DeltaSlot* delta, uint64_t delta_nslots, int32_t* assign, uint8_t* path,
                                  uint32_t* hit_chosen, uint32_t* err, const psk::GreedySync& sync, int search,
-                          const uint64_t* slots, const uint64_t* ovf, const psk::TableDesc* tdesc, cudaStream_t s) {
+                                 const uint64_t* slots, const uint64_t* ovf, const psk::TableDesc* tdesc, int num_sms,
+                                 cudaStream_t s) {
   const MainTables mt{slots, ovf, tdesc};
   if (w.R == 0) return cudaSuccess;
   const cudaError_t e = cudaMemsetAsync(sync.stats, 0, sync.clear_bytes, s);
@@ -1238,7 +1242,7 @@ cudaError_t launch_greedy(const psk::RowPre* rows, const psk::WindowDev& w, uint
   const uint32_t ipt = (I + 32u * kComputeWarps - 1) / (32u * kComputeWarps);
 #define PS_GREEDY_P(IPT)                                                                                      \
   return greedy_pipe_launch<IPT>(rows, w, I, hit0, tpf0, committed, pending, m, delta, delta_nslots, assign, path, \
-                                 hit_chosen, err, sync, search == 0, mt, s)
+                                 hit_chosen, err, sync, search == 0, mt, num_sms, s)
   if (ipt <= 1) PS_GREEDY_P(1);
   if (ipt <= 2) PS_GREEDY_P(2);
   if (ipt <= 4) PS_GREEDY_P(4);

@@ -875,7 +875,8 @@ cudaError_t launch_greedy(const psk::RowPre* rows, const psk::WindowDev& w, uint
                           const float* tpf0, psk::StateSoA committed, psk::StateSoA pending, const psk::DevModel& m,
                           psk::DeltaSlot* delta, uint64_t delta_nslots, int32_t* assign, uint8_t* path,
                           uint32_t* hit_chosen, uint32_t* err, const psk::GreedySync& sync, int search,
-                          const uint64_t* slots, const uint64_t* ovf, const psk::TableDesc* tdesc, cudaStream_t s);
+                          const uint64_t* slots, const uint64_t* ovf, const psk::TableDesc* tdesc, int num_sms,
+                          cudaStream_t s);
 cudaError_t launch_insert_chains(uint64_t* slots, uint64_t* ovf, const psk::TableDesc* tdesc, uint32_t I,
                                  unsigned long long* count, uint64_t nchains, const uint32_t* inst,
                                  const uint64_t* off, const uint64_t* hash, const uint64_t* parent,
