@@ -253,15 +253,15 @@ ps_status device_errors(ps_ctx* c) {
   return fail(c, PS_ERR_CUDA, "unknown device error");
 }
 
-// Synchronise the stream, hand staged results on, read the device error word, and reset it for the next
-// call.
+// Synchronise the stream, read the device error word and reset it for the next call, and hand staged
+// results on if there was no error.
 ps_status finish(ps_ctx* c) {
   PS_TRY_CUDA(c, cudaMemcpyAsync(c->h_err, c->d_err, 4 * sizeof(uint32_t), cudaMemcpyDeviceToHost, c->stream));
   PS_TRY_CUDA(c, cudaStreamSynchronize(c->stream));
   c->h_out_used = 0;
-  for (const ps_ctx::Handover& x : c->handover) std::memcpy(x.dst, x.src, x.bytes);
-  c->handover.clear();
   ps_status s = device_errors(c);
+  for (const ps_ctx::Handover& x : c->handover) std::memcpy(x.dst, x.src, x.bytes);  // (none after an error)
+  c->handover.clear();
   if (*c->h_err) {
     PS_TRY_CUDA(c, cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), c->stream));
     PS_TRY_CUDA(c, cudaStreamSynchronize(c->stream));

@@ -65,6 +65,26 @@ def test_wait_limit_expires_then_the_context_recovers(P):
     assert g["assign"][0] >= 0 and g["hit_chosen"][0] == 0  # the long chain was admitted cold
 
 
+def test_a_timed_out_call_hands_no_results_on(P):
+    """Small results are staged and handed on once the call is known to have succeeded."""
+    import ctypes
+    I, R = 64, 40
+    win = _window(R, 65536)
+    assign, path, hit = np.full(R, 77, np.int32), np.full(R, 77, np.uint8), np.full(R, 77, np.uint32)
+    best = np.full(R, 77, np.int32)
+    with P.Scheduler(I, np.full(I, 1 << 17, np.uint64), R, int(win.chain_off[-1]), W.MODEL_DEFAULT) as s:
+        s.load_instances(0, 0, 0, 0, 1 << 24, 64)
+        s.set_wait_limit(1000)
+        w, d, sc = s.make_window(win), P.PsDecisions(), P.PsScores()
+        d.assign, d.path, d.hit_chosen, sc.best = assign.ctypes.data, path.ctypes.data, hit.ctypes.data, best.ctypes.data
+        call = lambda: P.lib().ps_schedule_window(s.handle, ctypes.byref(w), ctypes.byref(d), ctypes.byref(sc))
+        assert call() == P.PS_ERR_TIMEOUT
+        assert all((x == 77).all() for x in (assign, path, hit, best))
+        s.set_wait_limit(0)
+        assert call() == P.PS_OK
+        assert (path == 0).all() and (best == 0).all() and not (hit == 77).any() and not (assign == 77).any()
+
+
 def test_wait_limit_bounds(P):
     with P.Scheduler(2, [16, 16], 4, 64, W.MODEL_DEFAULT) as s:
         s.set_wait_limit(5 * 10 ** 9)
