@@ -144,8 +144,11 @@ struct ps_ctx {
 
 namespace {
 
+// A CUDA error ends a call with copies and kernels still queued.  They are waited for: they read the
+// page-locked staging, which the next call fills again, and the caller's own arrays.
 ps_status fail(ps_ctx* c, ps_status s, const std::string& msg) {
   if (c) {
+    if (s == PS_ERR_CUDA) cudaStreamSynchronize(c->stream);
     c->err = msg;
     c->handover.clear();  // a call that fails hands nothing on, then or later
   }
