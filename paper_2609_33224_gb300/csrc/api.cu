@@ -30,6 +30,7 @@ constexpr size_t kStateBytes = 36;                  // per instance: q, S, M_KV 
 // results land there and are handed on after the call's one synchronisation: a copy from or to ordinary
 // memory costs 8 to 10 us and waits, and a call would make up to seven of them.
 constexpr size_t kStageIn = 1u << 20, kStageOut = 1u << 18;
+constexpr int kMaxHandover = 9;  // staged results of a call: six score arrays and three of the decisions
 
 struct DeviceGuard {
   int prev = -1;
@@ -110,7 +111,8 @@ struct ps_ctx {
     const void* src;
     size_t bytes;
   };
-  std::vector<Handover> handover;  // results to hand on from h_out once the stream is done
+  Handover handover[kMaxHandover];  // results to hand on from h_out once the stream is done
+  int n_handover = 0;
   uint64_t win_blocks = 0;         // chain blocks of the window being staged
   const uint32_t* win_out = nullptr;  // its out_tokens on the device (nullptr: none given)
   unsigned char *st_block = nullptr, *pend_block = nullptr, *gsync_block = nullptr, *zero_block = nullptr;
@@ -150,7 +152,7 @@ ps_status fail(ps_ctx* c, ps_status s, const std::string& msg) {
   if (c) {
     if (s == PS_ERR_CUDA) cudaStreamSynchronize(c->stream);
     c->err = msg;
-    c->handover.clear();  // a call that fails hands nothing on, then or later
+    c->n_handover = 0;  // a call that fails hands nothing on, then or later
   }
   return s;
 }
@@ -263,8 +265,8 @@ ps_status finish(ps_ctx* c) {
   PS_TRY_CUDA(c, cudaStreamSynchronize(c->stream));
   c->h_out_used = 0;
   ps_status s = device_errors(c);
-  for (const ps_ctx::Handover& x : c->handover) std::memcpy(x.dst, x.src, x.bytes);  // (none after an error)
-  c->handover.clear();
+  for (int k = 0; k < c->n_handover; ++k) std::memcpy(c->handover[k].dst, c->handover[k].src, c->handover[k].bytes);
+  c->n_handover = 0;  // (none after an error)
   if (*c->h_err) {
     PS_TRY_CUDA(c, cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), c->stream));
     PS_TRY_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -431,10 +433,10 @@ template <class T>
 cudaError_t deliver(ps_ctx* c, T* dst, const T* src, size_t n, int on_device) {
   if (!dst || n == 0 || dst == src) return cudaSuccess;
   const size_t bytes = n * sizeof(T);
-  if (!on_device && c->h_out_used + bytes <= kStageOut) {  // handed on by finish()
+  if (!on_device && c->n_handover < kMaxHandover && c->h_out_used + bytes <= kStageOut) {  // handed on by finish()
     unsigned char* at = c->h_out + c->h_out_used;
     c->h_out_used += (bytes + 15) / 16 * 16;
-    c->handover.push_back({dst, at, bytes});
+    c->handover[c->n_handover++] = {dst, at, bytes};
     return cudaMemcpyAsync(at, src, bytes, cudaMemcpyDeviceToHost, c->stream);
   }
   return cudaMemcpyAsync(dst, src, n * sizeof(T), on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
