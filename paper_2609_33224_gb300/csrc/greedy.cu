@@ -1233,9 +1233,8 @@ cudaError_t launch_greedy(const psk::RowPre* rows, const psk::WindowDev& w, uint
                                  const uint64_t* slots, const uint64_t* ovf, const psk::TableDesc* tdesc, int num_sms,
                                  cudaStream_t s) {
   const MainTables mt{slots, ovf, tdesc};
-  if (w.R == 0) return cudaSuccess;
   const cudaError_t e = cudaMemsetAsync(sync.stats, 0, sync.clear_bytes, s);
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess || w.R == 0) return e;
   // IPT instances per compute thread of the deciding block (and at most that many per probe thread): as
   // few as its warps allow.  More per thread means fewer warps to combine but a longer step: greedy pass
   // with 1 / 2 / 4 a thread 0.32 / 0.33 / 0.44 ms at 256 x 512, with 2 / 4 / 8 14.6 / 17.0 / 25.2 at 1024 x 16384.

@@ -107,6 +107,7 @@ def test_empty_windows_leave_the_state_as_it_is(P, mode):
                     assert np.array_equal(state[k], v), k
 
         nothing_arrives(empty)
+        assert s.probe_stats()["greedy_fast"] == 0
         orc.load_requests(wl.initial_requests())
         s.load_requests(wl.initial_requests())
         nothing_arrives(_Device(empty))
@@ -115,8 +116,10 @@ def test_empty_windows_leave_the_state_as_it_is(P, mode):
             for k in ("assign", "path", "hit_chosen"):
                 assert np.array_equal(g[k], o[k]), k
             assert (g["assign"] >= 0).any()
+            assert s.probe_stats()["greedy_fast"] == (40 if mode else 0)
             s.commit_window(last_use=w + 1)
             nothing_arrives(empty)
+            assert s.probe_stats()["greedy_fast"] == 0  # decisions of the last call: none
             s.advance_window(40.0, 20000, evict=False)
             orc.advance(40.0, 20000, evict=False)
             nothing_arrives(empty)
