@@ -114,7 +114,7 @@ typedef struct {
  *   model                 the performance model above.
  *   probe_mode            how hit lengths are found (both give the same hits on the caches they
  *                         accept):
- *     PS_PROBE_LINEAR  (0) walk the chain 32 blocks per warp step until the first block that is
+ *     PS_PROBE_LINEAR  (0) walk the chain 64 blocks per warp step until the first block that is
  *                          not cached; exact for any cache contents.
  *     PS_PROBE_SEARCH  (1) the caches must be prefix-closed (every cached block's parent is
  *                          cached, as in the paper's Section 7 prefix tree).  Then "block k is
@@ -127,7 +127,8 @@ typedef struct {
  *                          PS_ERR_INVALID.
  *   track_lru             1: keep per-block (last_use, child count, parent) metadata so that
  *                         ps_advance_window can evict leaf-first LRU (the tables must then hold fewer
- *                         than 2^32 - 2 slots in total); 0: no eviction.
+ *                         than 2^32 - 2 slots in total; 16 bytes a slot, and per instance 80 KB of
+ *                         scratch, with 456 KB more for each of the first 256); 0: no eviction.
  *   max_active_requests   0: no request tracking.  > 0: each instance keeps up to this many queued
  *                         and this many decoding requests for ps_advance_window (streaming windows);
  *                         committed windows then need ps_window.out_tokens. */
@@ -226,8 +227,9 @@ typedef struct {
  * of Section 7 (Implementation: the scheduler's prefix tree of cached prefixes, here one hash table of
  * chained block hashes per instance) and the performance model of Section 5.  Allocates every table
  * and buffer up front (instance hash tables sized by cap_blocks / table_load_factor, a window-scoped
- * delta table of 2 * max_window_chain_blocks slots, window staging and score scratch).  Instances
- * start empty with zero state.  cfg is read during the call only.
+ * delta table of 2 * max_window_chain_blocks slots, window staging and score scratch) as one device
+ * allocation, and 1.3 MB of page-locked host memory.  Instances start empty with zero state.  cfg is
+ * read during the call only.
  * Errors: PS_ERR_INVALID (config), PS_ERR_CUDA, PS_ERR_OOM.  *out is NULL on failure. */
 PS_API ps_status ps_create(const ps_config* cfg, ps_ctx** out);
 

@@ -342,7 +342,9 @@ class Scheduler:
         self._check(lib().ps_set_wait_limit(self._h, int(ns)))
 
     def probe_stats(self) -> dict:
-        """Counters of the last probe phase (see ps_last_probe_stats)."""
+        """Counters of the last probe phase and greedy pass (see ps_last_probe_stats).  Some names are older
+        than what they hold: every decision counts as greedy_fast, cyc_feed_summary_wait is the feeder's
+        wait for probed rows, and greedy_full and the three cyc_summary_* are always 0."""
         v = np.zeros(16, np.uint64)
         self._check(lib().ps_last_probe_stats(self._h, v.ctypes.data, 16))
         names = ("rows_scratch", "rows_derived", "lookups_scratch", "lookups_derived", "chain_reads",

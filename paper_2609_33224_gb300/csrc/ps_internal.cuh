@@ -14,7 +14,8 @@
 //   delta table   window-scoped set of (instance, block) pairs cached by the window's own earlier
 //                 decisions: one 16-byte slot {hash, instance + 1} per pair, linear probing from the
 //                 pair's home slot, sized at twice the window's block bound so it can never fill.
-//                 Cleared after each window.
+//                 Cleared after each window, so empty outside the greedy pass (staging passes a
+//                 shared-prefix window's own blocks through it beside a pending window, and clears it).
 //   state         structure of arrays per instance (b, qr, q, S, M_KV, B_max).
 //   hits          u32 [R x I], request-major.
 #pragma once
@@ -51,10 +52,13 @@ struct TableDesc {
 };
 
 // One (block, instance) pair of the window's delta table: the block hash and instance id + 1 (0 while
-// the claiming thread has not yet written it).  Within one window each pair is inserted at most once:
-// a request inserts chain[h, nb) on its pick with h the exact first miss there, so none of those
-// blocks is cached on that instance yet (a block hash fixes its whole prefix, so an earlier insert of
-// the same block would have cached chain[0, that position] and moved the first miss past it).
+// the claiming thread has not yet written it).  On prefix-closed caches each pair is inserted at most
+// once in a window: a request inserts chain[h, nb) on its pick with h the exact first miss there, so none
+// of those blocks is cached on that instance yet (a block hash fixes its whole prefix, so an earlier
+// insert of the same block would have cached chain[0, that position] and moved the first miss past it).
+// On other caches (linear mode) every request inserts its whole chain; a pair found there is left alone,
+// and two requests inserted at the same time may store one twice, which a lookup does not notice.  Either
+// way a window stores no more pairs than it has chain blocks.
 struct DeltaSlot {
   unsigned long long hash;
   unsigned int tag;

@@ -584,6 +584,10 @@ __device__ __forceinline__ uint32_t parent32(uint64_t p) {
 // capacity by up to 7.9K blocks: hist 0.12 ms, gather 0.11, detail 0.09, index and jump 0.07, order 0.17
 // (0.43 ms where the order kernel read the metadata itself, a block an SM); the streaming window of 500
 // requests takes 1.59 ms, and took 11.8 ms with one thread ordering each instance's evictions (1.2 us each).
+// That is a cache filled by commits, or loaded with many stamps.  One loaded with a single stamp gains nothing
+// until its first blocks are gone: 200K blocks of one stamp an instance are more than kClassMax, so the scan
+// and the choice find that out (0.1 ms) and the kernels below do the work; advancing such a stream of
+// 1000-request windows takes 15.0 ms a window over the first 13 (15.0 with those kernels alone), 7.8 over 1000 (7.7).
 constexpr uint32_t kClassMax = 16384;   // blocks of one last_use value ordered in shared memory
 constexpr uint32_t kHistBits = 11;
 constexpr uint32_t kHistBins = 1u << kHistBits;

@@ -132,6 +132,19 @@ def test_sums_beyond_32_bits(P, shift):
         _check(P, dict(wl.model, selector=sel), ins, wl.window)
 
 
+@pytest.mark.parametrize("I", [1, 33, 512, 513, 1024, 1025, 2048])
+@pytest.mark.parametrize("sel", [0, 5])
+def test_instance_counts_in_linear_mode(P, I, sel):
+    """The linear kernels have an instance of their own per instances a thread (1, 2, 4); every cache here has
+    holes, and hits that rise in the window end at one or go on past it."""
+    wl = _workload(I, 80, seed=13)
+    ins = wl.instances
+    keep = np.random.default_rng(4).random(ins.chain_hash.size) > 0.03
+    n = np.concatenate([[0], np.cumsum(keep)])[ins.chain_off.astype(np.int64)]
+    ins.chain_hash, ins.chain_off = ins.chain_hash[keep], n.astype(np.uint64)
+    _check(P, dict(wl.model, selector=sel), ins, wl.window, mode=0)
+
+
 @pytest.mark.parametrize("sel,kv", [(0, 0), (5, 0), (0, 1 << 45)])
 def test_caches_with_holes(P, sel, kv):
     """Caches that are not prefix-closed: hits that rise in the window go on through blocks the committed

@@ -322,7 +322,7 @@ def test_config1_full_parity(P, tpot, mode):
 @pytest.mark.parametrize("mode", MODES)
 @pytest.mark.parametrize("seed,I,R", [(9, 2048, 48), (10, 1537, 33), (11, 2047, 5)])
 def test_random_ragged_windows_at_the_instance_limit(P, seed, I, R, mode):
-    """The largest context ps_create accepts (2048 instances; probe and summary threads then hold 8
+    """The largest context ps_create accepts (2048 instances; the greedy pass's threads then hold 4
     instances each), and ragged counts just below it."""
     ins, win = _random_case(seed, I, R)
     _check_window(P, dict(W.MODEL_DEFAULT), ins, win, mode=mode)
