@@ -287,7 +287,7 @@ ps_status check_capacity(ps_ctx* c) {
   return PS_OK;
 }
 
-// Arrays of a host window on their way to the device: packed into the staging block and copied in one
+// Arrays of a host window, or of chains to insert, on their way to the device: packed into the staging block and copied in one
 // piece when they fit (flush), else copied each to its own buffer.
 struct Stager {
   ps_ctx* c;
@@ -814,23 +814,27 @@ ps_status ps_insert_chains(ps_ctx* c, uint64_t nchains, const uint32_t* inst, co
     total = off[nchains];
     if (total && !hash) return fail(c, PS_ERR_INVALID, "hash is NULL");
     const size_t bytes = nchains * 4 + (nchains + 1) * 8 + nchains * 8 + total * 8 + 16;
-    PS_TRY_CUDA(c, cudaMalloc(&tmp, bytes));
-    uint64_t* t_off = static_cast<uint64_t*>(tmp);
-    uint64_t* t_parent = t_off + nchains + 1;
-    uint64_t* t_hash = t_parent + nchains;
-    uint32_t* t_inst = reinterpret_cast<uint32_t*>(t_hash + total);
-    cudaError_t e = cudaMemcpyAsync(t_off, off, (nchains + 1) * 8, cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(t_parent, parent, nchains * 8, cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess && total) e = cudaMemcpyAsync(t_hash, hash, total * 8, cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(t_inst, inst, nchains * 4, cudaMemcpyHostToDevice, c->stream);
+    // A small call goes through the staging block: with every block of the context in one allocation, the
+    // driver maps and unmaps a page for a buffer of the call's own (a chain of 10 blocks: 200 us that way).
+    Stager st(c, bytes);
+    uint64_t *t_off = nullptr, *t_parent = nullptr, *t_hash = nullptr;
+    uint32_t* t_inst = nullptr;
+    if (!st.packed) {
+      PS_TRY_CUDA(c, cudaMalloc(&tmp, bytes));
+      t_off = static_cast<uint64_t*>(tmp);
+      t_parent = t_off + nchains + 1;
+      t_hash = t_parent + nchains;
+      t_inst = reinterpret_cast<uint32_t*>(t_hash + total);
+    }
+    d_off = st.put(off, nchains + 1, t_off);
+    d_parent = st.put(parent, nchains, t_parent);
+    d_hash = st.put(hash, total, t_hash);
+    d_inst = st.put(inst, nchains, t_inst);
+    const cudaError_t e = st.flush();
     if (e != cudaSuccess) {
-      cudaFree(tmp);
+      if (tmp) cudaFree(tmp);
       return fail(c, PS_ERR_CUDA, std::string("copy chains: ") + cudaGetErrorString(e));
     }
-    d_off = t_off;
-    d_hash = t_hash;
-    d_inst = t_inst;
-    d_parent = t_parent;
   } else {
     PS_TRY_CUDA(c, cudaMemcpy(&total, off + nchains, 8, cudaMemcpyDeviceToHost));
   }

@@ -126,3 +126,29 @@ def test_empty_windows_leave_the_state_as_it_is(P, mode):
             st, ost = s.get_instances(), orc.get_state()
             for k in ("b", "qr", "q", "S"):
                 assert np.array_equal(st[k], ost[k]), k
+
+
+@pytest.mark.parametrize("form_a", ["host", "device"])
+@pytest.mark.parametrize("blocks", [3, 200000])  # a small call goes through the staging block
+def test_inserting_leaves_the_pending_window_alone(P, form_a, blocks):
+    wl = W.generate(0, seed=23, num_instances=6, window_requests=SMALL, num_sessions=10, cap_blocks=6000)
+    ins, A = wl.instances, wl.window
+    ins.M_KV[:] = 10 ** 8
+    ins.cap_blocks[:] = 300000
+    chain = np.random.default_rng(6).integers(2, 2 ** 63, blocks, dtype=np.int64).astype(np.uint64)
+    orc = Oracle(ins.I, wl.model, track_lru=True).load(ins)
+    o = orc.schedule(A, window_id=1)
+    orc.insert_chain(2, chain, last_use=1)
+    with P.Scheduler(ins.I, ins.cap_blocks, SMALL, int(A.chain_off[-1]), wl.model, track_lru=True) as s:
+        s.load_workload_instances(ins)
+        win = FORMS[form_a](A)
+        g = s.schedule_window(win)
+        s.insert_blocks(2, chain, last_use=1)
+        s.commit_window(last_use=1)
+        for k in ("assign", "path", "hit_chosen"):
+            assert np.array_equal(g[k], o[k]), k
+        assert [int(x) for x in s.cached_blocks()] == [orc.cached_blocks(i) for i in range(ins.I)]
+        assert np.array_equal(s.score_window(A, want=("hits",))["hits"], orc.score_rows(A)["hits"])
+        st, ost = s.get_instances(), orc.get_state()
+        for k in ("b", "qr", "q", "S"):
+            assert np.array_equal(st[k], ost[k]), k
