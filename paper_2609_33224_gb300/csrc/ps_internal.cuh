@@ -906,12 +906,13 @@ struct EvictScratch {
   void* blocks;
   uint32_t* list;
   uint32_t* slow;
+  bool class_first = true;  // the last call needed the class kernels: launch them first (host; a guess only)
 };
 // Leaf-first LRU eviction of every instance over capacity (rounds until none is; synchronises the
 // stream between rounds).  more_host one pinned word; max_instance_slots the largest table (slots) of
 // an instance; max_use the largest last_use stamp any block may have.
 cudaError_t launch_evict(uint64_t* slots, const psk::TableDesc* tdesc, uint32_t I, unsigned long long* count,
-                         const uint64_t* cap, psk::LruMeta meta, const EvictScratch& sc, uint32_t* more_host,
+                         const uint64_t* cap, psk::LruMeta meta, EvictScratch& sc, uint32_t* more_host,
                          uint64_t max_instance_slots, uint32_t max_use, uint32_t* err, int num_sms, cudaStream_t s);
 size_t evict_plan_bytes(uint32_t I);
 size_t evict_hist_words(uint32_t I);

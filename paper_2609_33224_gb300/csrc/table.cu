@@ -563,7 +563,8 @@ __device__ __forceinline__ uint32_t parent32(uint64_t p) {
 // counted from the oldest reach the excess E, the evicted blocks are exactly: every block older than T,
 // and of the blocks stamped T the k missing ones with the smallest subtree maximum of the hash over
 // blocks stamped T.  These kernels find and evict them, every step parallel:
-//   list      the instances over capacity;
+//   list      the instances over capacity (or, where every excess is small, flags them for the kernels after
+//             these);
 //   hist      per instance a histogram of last_use over its slots (and its number of leaves), in one
 //             pass for stamps below 2048 and one more per further 11 bits; choose picks T and k;
 //   gather    the slots stamped below T and those stamped T (up to kClassMax each; at most kClassMax
@@ -587,7 +588,8 @@ __device__ __forceinline__ uint32_t parent32(uint64_t p) {
 // That is a cache filled by commits, or loaded with many stamps.  One loaded with a single stamp gains nothing
 // until its first blocks are gone: 200K blocks of one stamp an instance are more than kClassMax, so the scan
 // and the choice find that out (0.1 ms) and the kernels below do the work; advancing such a stream of
-// 1000-request windows takes 15.0 ms a window over the first 13 (15.0 with those kernels alone), 7.8 over 1000 (7.7).
+// 1000-request windows takes 15.0 ms a window over the first 13 (15.0 with those kernels alone), 7.8 over 1000
+// (7.7); one of 4 instances over by 300 blocks, 0.65 ms (0.58).
 constexpr uint32_t kClassMax = 16384;   // blocks of one last_use value ordered in shared memory
 constexpr uint32_t kHistBits = 11;
 constexpr uint32_t kHistBins = 1u << kHistBits;
@@ -597,7 +599,14 @@ constexpr uint32_t kScanThreads = 512;
 constexpr uint64_t kScanChunk = 65536;  // slots a block scans before it merges its histogram
 constexpr uint32_t kNoJump = 0xFFFFu;
 static_assert(kClassMax < kNoJump, "16-bit block indices");
-constexpr uint32_t kMoreFast = 1u, kMoreSlow = 2u;  // bits of the "another round" word
+// Bits of the "another round" word: instances left for these kernels, for the one-at-a-time kernels; and
+// whether this call's list had any for these.
+constexpr uint32_t kMoreFast = 1u, kMoreSlow = 2u, kMoreListed = 4u;
+// Excess up to which every instance of a call goes block by block (and half the number of instances over
+// capacity more): that is 0.7 us a block on one thread, all instances side by side, against the launches and
+// steps of the class kernels.  A call's time, one by one / by classes: 2 of 8 instances over by 5 blocks
+// 55 / 101 us, by 64 about 97 / 101, by 200 193 / 91; 256 of 1024 over by 20 129 / 262, by 192 about 250 / 265.
+constexpr uint32_t kSmallExcess = 64u;
 
 // Per over-capacity instance: the last_use range still open, what was counted below it, and the choice.
 struct EvictPlan {
@@ -626,16 +635,35 @@ struct EvictBlocks {
 enum : uint8_t { kRelNone = 0, kRelOlder = 1, kRelClass = 2, kRelNewer = 3 };
 
 
+// Also starts the round word and, in a call's first round, the flags and the leaf counts.
 __global__ void __launch_bounds__(1024)
 evict_list_kernel(uint32_t I, const unsigned long long* __restrict__ count, const uint64_t* __restrict__ cap,
-                  const uint32_t* __restrict__ slow, uint32_t max_use, EvictPlan* plan, uint32_t* list, uint32_t* nlist,
-                  uint32_t* more) {
-  __shared__ uint32_t s_n;
-  if (threadIdx.x == 0) s_n = 0u;
+                  uint32_t* slow, uint32_t* nleaf, uint32_t max_use, EvictPlan* plan, uint32_t* list, uint32_t* nlist,
+                  uint32_t* more, bool first, bool class_runs) {
+  __shared__ uint32_t s_n, s_over;
+  __shared__ unsigned long long s_excess;
+  if (threadIdx.x == 0) {
+    s_n = 0u;
+    s_over = 0u;
+    s_excess = 0ull;
+  }
   __syncthreads();
+  for (uint32_t i = threadIdx.x; i < I; i += blockDim.x) {
+    if (first) slow[i] = nleaf[i] = 0u;
+    if (count[i] > cap[i] && !slow[i]) {
+      atomicAdd(&s_over, 1u);
+      atomicMax(&s_excess, count[i] - cap[i]);
+    }
+  }
+  __syncthreads();
+  const bool small = s_excess <= kSmallExcess + s_over / 2u;
   for (uint32_t i = threadIdx.x; i < I; i += blockDim.x) {
     const unsigned long long c = count[i];
     if (c <= cap[i] || slow[i]) continue;
+    if (small) {
+      slow[i] = 1u;
+      continue;
+    }
     const uint32_t q = atomicAdd(&s_n, 1u);
     if (q >= kEvictBatch) continue;
     const unsigned long long E = c - cap[i];
@@ -648,7 +676,8 @@ evict_list_kernel(uint32_t I, const unsigned long long* __restrict__ count, cons
   __syncthreads();
   if (threadIdx.x == 0) {
     *nlist = s_n < kEvictBatch ? s_n : kEvictBatch;
-    if (s_n > kEvictBatch) atomicOr(more, kMoreFast);
+    const bool left = class_runs ? s_n > kEvictBatch : s_n > 0u;
+    *more = (s_n ? kMoreListed : 0u) | (left ? kMoreFast : 0u) | (small && s_over && class_runs ? kMoreSlow : 0u);
   }
 }
 
@@ -1455,7 +1484,7 @@ cudaError_t launch_advance(psk::StateSoA st, uint32_t I, const psk::ReqStore& rq
 }
 
 cudaError_t launch_evict(uint64_t* slots, const psk::TableDesc* tdesc, uint32_t I, unsigned long long* count,
-                         const uint64_t* cap, psk::LruMeta meta, const EvictScratch& sc, uint32_t* more_host,
+                         const uint64_t* cap, psk::LruMeta meta, EvictScratch& sc, uint32_t* more_host,
                          uint64_t max_instance_slots, uint32_t max_use, uint32_t* err, int num_sms, cudaStream_t s) {
   const size_t smem = kEvictSmem;
   cudaError_t e = cudaFuncSetAttribute(evict_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1479,13 +1508,20 @@ cudaError_t launch_evict(uint64_t* slots, const psk::TableDesc* tdesc, uint32_t 
   for (uint64_t v = (uint64_t)max_use >> kHistBits; v; v >>= kHistBits) ++passes;
   const uint64_t per_block = (uint64_t)kCollectThreads * kCollectSlotsPerThread;
   const unsigned gx = (unsigned)((max_instance_slots + per_block - 1) / per_block);
-  if ((e = cudaMemsetAsync(sc.slow, 0, (size_t)I * sizeof(uint32_t), s)) != cudaSuccess) return e;
-  uint32_t todo = kMoreFast;
-  // Instances left to the one-at-a-time kernels wait for the last batch, and then go together.
+  // The first round launches the kernels that the call before turned out to need: the list says on the device
+  // which are needed now, and the others find nothing to do.  Instances left to the one-at-a-time kernels wait
+  // for the last batch, and then go together.
+  uint32_t todo = sc.class_first ? kMoreFast : kMoreSlow;
   for (int round = 0; round < 4096 && todo; ++round) {
-    if ((e = cudaMemsetAsync(sc.more, 0, sizeof(uint32_t), s)) != cudaSuccess) return e;
-    if (todo & kMoreFast) {
-      evict_list_kernel<<<1, 1024, 0, s>>>(I, count, cap, sc.slow, max_use, plan, sc.list, nlist, sc.more);
+    const bool class_runs = (todo & kMoreFast) != 0u;
+    if (class_runs || round == 0) {
+      evict_list_kernel<<<1, 1024, 0, s>>>(I, count, cap, sc.slow, sc.nleaf, max_use, plan, sc.list, nlist, sc.more,
+                                           round == 0, class_runs);
+    } else {
+      if ((e = cudaMemsetAsync(sc.more, 0, sizeof(uint32_t), s)) != cudaSuccess) return e;
+      if ((e = cudaMemsetAsync(sc.nleaf, 0, (size_t)I * sizeof(uint32_t), s)) != cudaSuccess) return e;
+    }
+    if (class_runs) {
       for (int pass = 0; pass < passes; ++pass) {
         evict_hist_kernel<<<scan_grid, kScanThreads, 0, s>>>(tdesc, meta, plan, sc.list, nlist, chunks, sc.hist, pass == 0);
         evict_choose_kernel<<<inst_grid, 256, 0, s>>>(plan, sc.list, nlist, sc.hist);
@@ -1497,8 +1533,7 @@ cudaError_t launch_evict(uint64_t* slots, const psk::TableDesc* tdesc, uint32_t 
       evict_order_kernel<<<inst_grid, kOrderThreads, sizeof(OrderSmem), s>>>(slots, count, cap, meta, plan, sc.list, nlist,
                                                                             eb, sc.slow, sc.more, kLeafMax, err);
     }
-    if (todo == kMoreSlow) {
-      if ((e = cudaMemsetAsync(sc.nleaf, 0, (size_t)I * sizeof(uint32_t), s)) != cudaSuccess) return e;
+    if (!class_runs) {
       leaf_collect_kernel<<<dim3(gx ? gx : 1u, I), kCollectThreads, 0, s>>>(
           slots, tdesc, count, cap, meta, sc.slow, max_use, static_cast<Leaf*>(sc.leafbuf), sc.nleaf);
       evict_kernel<<<I, kEvictThreads, smem, s>>>(slots, count, cap, meta, sc.slow, static_cast<const Leaf*>(sc.leafbuf),
@@ -1507,7 +1542,8 @@ cudaError_t launch_evict(uint64_t* slots, const psk::TableDesc* tdesc, uint32_t 
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = cudaMemcpyAsync(more_host, sc.more, sizeof(uint32_t), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
-    todo = *more_host | (todo & kMoreFast ? todo & kMoreSlow : 0u);
+    if (round == 0) sc.class_first = (*more_host & kMoreListed) != 0u;
+    todo = (*more_host & (kMoreFast | kMoreSlow)) | (class_runs ? todo & kMoreSlow : 0u);
   }
   return cudaSuccess;
 }

@@ -21,8 +21,9 @@ def P():
     return P
 
 
-def _run(P, I, calls, cap):
-    """calls: (chains [(inst, blocks, parent)], last_use); evicts after the last, compares the contents."""
+def _run(P, I, calls, cap, every_call=False):
+    """calls: (chains [(inst, blocks, parent)], last_use); evicts after the last (or after each), compares the
+    contents."""
     every = np.unique(np.concatenate([c[1] for ch, _ in calls for c in ch]))
     model = dict(W.MODEL_DEFAULT)
     st = dict(b=np.zeros(I, np.int32), qr=np.zeros(I, np.int32), q=np.zeros(I, np.int64), S=np.zeros(I, np.int64),
@@ -53,6 +54,11 @@ def _run(P, I, calls, cap):
             except P.PSError as e:
                 assert e.status == P.PS_ERR_CAPACITY, str(e)
             orc.insert_chains(*args, last_use=stamp)
+            if every_call:
+                s.advance_window(20.0, 1000, evict=True)
+                orc.advance(20.0, 1000)
+                assert s.cached_blocks().tolist() == [orc.cached_blocks(i) for i in range(I)]
+                assert np.array_equal(s.score_window(win, want=("hits",))["hits"], orc.score_rows(win)["hits"])
         for _ in range(2):  # the second advance finds nothing over capacity
             s.advance_window(20.0, 1000, evict=True)
             orc.advance(20.0, 1000)
@@ -111,3 +117,16 @@ def test_children_newer_than_their_parents(P):
 def test_more_instances_than_a_round(P):
     rng = np.random.default_rng(6)
     _run(P, 300, [(_chains(rng, 300, 1500, 8), k) for k in range(3)], 20)
+
+
+@pytest.mark.parametrize("I", [1, 5, 40])
+def test_small_and_large_excess_in_turn(P, I):
+    """Excesses on both sides of the one up to which blocks go one by one (64, and half the number of instances
+    over capacity more), in calls that follow one another in every order; some instances have none."""
+    rng = np.random.default_rng(I)
+    calls = [([(i, _blocks(rng, 300), 0) for i in range(I)], 0)]
+    sizes = [1, 64, 65, 0, 300, 200, 3, 80, 81, 82, 2, 64, 85, 299]
+    for k, n in enumerate(sizes):
+        over = [(i, _blocks(rng, n if i % 3 else max(1, n // 2)), 0) for i in range(I) if n and (i % 7 or I < 7)]
+        calls.append((over or [(0, _blocks(rng, 1), 0)], k + 1))
+    _run(P, I, calls, 300, every_call=True)
