@@ -462,12 +462,66 @@ __device__ __forceinline__ uint32_t key_rank(uint64_t key) {
   return key == psk::kNoKey ? 0xFFFFFFFFu : ((key >> 62) ? c1 : c0);
 }
 
-// Algorithm 1's packed key from its rank and two words, {key bits of qr, of b} in T and {q + n, B} in C \ T:
-// worked out only where ranks are equal.
-__device__ __forceinline__ uint64_t dcq_key(uint32_t rank, uint2 w, uint32_t h) {
+// The rank and the packed key of a pair from 32-bit words of its state, in every instance order (GEN; else
+// Algorithm 1's).  With a 64-bit key by the order for every pair and branches on the order, the other orders cost
+// 90 instructions a pair more: 1025 instances (four a thread) took 1.91 us a decision in the D order, 1.83 in
+// H-C-Q and 2.00 with Eq. 9; 1.50, 1.42 and 1.49 now (Algorithm 1's order: 1.11).  Ranks are made for every pair, keys only where ranks are equal, from two words of the pair:
+// {D-C-Q key bits of qr, of b} in T (H-C-Q: the headroom's bits) and under the D-C-Q fallback, {q + n, B}
+// under the product.
+// Where qr comes last in an order, the tie word of a pair in T starts with it, so that nearly always equal ranks
+// in T mean that the smallest tie word wins (exact).
+struct PairOrder {  // masks of the launch's order: a step has no branch on it
+  uint32_t d_mask, c_mask, q_mask;  // what a rank in T takes: b, cached blocks, queued requests ...
+  uint32_t head_mask, head_shift;   // ... or (H-C-Q) the headroom, and its bits that the rank leaves out
+  uint32_t fb_mask;                 // D-C-Q fallback
+  bool head_all;                    // head_mask is set
+  uint32_t tie_q;                   // the part of the tie word above the instance
+  uint32_t ex_mask, ex_any;         // a rank in T leaves only the tie word to compare if (rank & ex_mask) | ex_any
+  __device__ __forceinline__ bool exact(uint32_t rank) const {
+    return rank < 0x80000000u && ((rank & ex_mask) | ex_any) != 0u;
+  }
+};
+
+__device__ __forceinline__ PairOrder pair_order(const psk::DevModel& m) {
+  const bool dc = m.sel == psk::kSelDCQ || m.sel == psk::kSelDC, dq = m.sel == psk::kSelDQ, hcq = m.sel == psk::kSelHCQ;
+  PairOrder o;
+  o.d_mask = hcq ? 0u : ~0u;
+  o.c_mask = dc ? 8191u : 0u;
+  o.q_mask = m.sel == psk::kSelDQC ? 8191u : 0u;
+  o.head_mask = hcq ? 0x7FFFFFFFu : 0u;
+  o.head_all = hcq;
+  o.fb_mask = m.fb_dcq ? 0x7FFFFFFFu : 0u;
+  o.tie_q = m.sel == psk::kSelDCQ || dq || hcq ? 0x3FFFFu : 0u;
+  o.ex_mask = dc ? 8191u : 0u;  // 0 there: 8191 blocks or more, which the rank does not tell apart
+  o.ex_any = dq || m.sel == psk::kSelD ? 1u : 0u;
+  o.head_shift = m.slo_off ? 5u : 0u;  // an admitted pair's headroom is positive, unless everything is admitted
+  return o;
+}
+
+// In T: b, then up to 13 bits of h (more is better) or of qr; H-C-Q: the headroom (head: f2ord of it).
+template <bool GEN>
+__device__ __forceinline__ uint32_t rank_in_t(const PairOrder& o, uint32_t kq, uint32_t kdh, uint32_t h, uint32_t head) {
+  const uint32_t c = 8191u - min(h, 8191u);
+  if (!GEN) return (kdh << 1) | c;
+  return ((kdh << 1) & o.d_mask) | (c & o.c_mask) | ((kq >> 5) & o.q_mask) | ((head >> o.head_shift) & o.head_mask);
+}
+
+// In C \ T: the product rounded towards zero as fp32 (p), or the D-C-Q order's bits.
+template <bool GEN>
+__device__ __forceinline__ uint32_t rank_fallback(const PairOrder& o, uint32_t kdh, uint32_t h, float p) {
+  const uint32_t dc = (kdh << 1) | (8191u - min(h, 8191u));
+  return 0x80000000u | (GEN ? ((dc >> 1) & o.fb_mask) | (__float_as_uint(p) & ~o.fb_mask) : __float_as_uint(p));
+}
+
+template <bool GEN>
+__device__ __forceinline__ uint64_t pair_key(const psk::DevModel& m, uint32_t rank, uint2 w, uint32_t h) {
   if (rank == 0xFFFFFFFFu) return psk::kNoKey;
-  if (rank & 0x80000000u) return psk::packed_key(1u, (uint64_t)w.x * (uint64_t)w.y);
-  return (((uint64_t)w.y << 32) | w.x) | ((uint64_t)((1u << 26) - 1u - h) << 18);
+  const uint64_t kd = ((uint64_t)w.y << 32) | w.x;
+  const uint64_t C = (1u << 26) - 1u - h;
+  if (rank & 0x80000000u)
+    return psk::packed_key(1u, GEN && m.fb_dcq ? kd | (C << 18) : (uint64_t)w.x * (uint64_t)w.y);
+  if (!GEN) return kd | (C << 18);
+  return m.sel == psk::kSelHCQ ? ((uint64_t)w.x << 26) | C : psk::key0_from_dcq(m, kd) | psk::hit_bits(m, h);
 }
 
 // The lane holding the warp's smallest (key, tie), -1 if no lane has a key; rank = key_rank(key).
@@ -507,7 +561,7 @@ __device__ __forceinline__ StepRow step_row(const psk::RowPre& x) {
 
 using psk::wait_smem_at_least;
 
-template <int IPT, bool GEN, bool LIN>
+template <int IPT, bool GEN, bool EQ9, bool LIN>
 __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, uint32_t I, psk::StateSoA committed,
                             psk::StateSoA pending, const psk::DevModel& m, int32_t* assign, uint8_t* __restrict__ path,
                             uint32_t* __restrict__ hit_chosen, uint32_t* err, const psk::GreedySync& sync,
@@ -519,7 +573,7 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
   __shared__ psk::RowPre s_row[kFeedRing];
   __shared__ uint32_t s_rank[2][kComputeWarps];            // a step's warp minima: their ranks (all ones: none) ...
   __shared__ uint2 s_th[2][kComputeWarps];                 // ... tie word and hit ...
-  __shared__ uint2 s_key[2][kComputeWarps];                // ... and packed key, or dcq_key's words (`words`)
+  __shared__ uint2 s_key[2][kComputeWarps];                // ... and packed key, or pair_key's words (narrow)
   __shared__ uint32_t s_w[kComputeWarps];                  // a step's warp minima of W over A (f2ord)
   __shared__ uint32_t s_begun;                             // steps [0, s_begun) have begun
   __shared__ uint32_t s_landed;                            // rows [0, s_landed) are staged
@@ -566,18 +620,25 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
   auto bar_compute = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(ncmp) : "memory"); };  // compute warps
   // Step x's pick from the warps' minima (after the next step's barrier), in every lane: the warp that
   // holds it, -1 if rejected.  r: this lane's entry of s_rank[x & 1] (all ones past the warps in use).
-  const bool words = !GEN && narrow;
   auto key_at = [&](uint32_t x, uint32_t r, uint32_t l) {
     const uint2 w = s_key[x & 1u][l];
-    return words ? dcq_key(r, w, s_th[x & 1u][l].y) : ((uint64_t)w.y << 32) | w.x;
+    return narrow ? pair_key<GEN>(m, r, w, s_th[x & 1u][l].y) : ((uint64_t)w.y << 32) | w.x;
   };
+  const PairOrder order = pair_order(m);
+  auto exact = [&](uint32_t r) { return GEN && narrow && order.exact(r); };
   auto decision = [&](uint32_t x, uint32_t r) {
     const uint32_t mr = __reduce_min_sync(0xffffffffu, r);
     const unsigned who = __ballot_sync(0xffffffffu, r == mr);
     int src = __ffs(who) - 1;
     if (who & (who - 1u)) {  // equal ranks (or nobody has a pair)
       const uint32_t l = (uint32_t)lane < ncw ? lane : 0u;
-      src = warp_argmin(r, key_at(x, r, l), s_th[x & 1u][l].x);
+      const uint32_t tie = s_th[x & 1u][l].x;
+      if (exact(mr)) {
+        const uint32_t mt = __reduce_min_sync(0xffffffffu, r == mr ? tie : 0xFFFFFFFFu);
+        src = __ffs(__ballot_sync(0xffffffffu, r == mr && tie == mt)) - 1;
+      } else {
+        src = warp_argmin(r, key_at(x, r, l), tie);
+      }
     }
     return src;
   };
@@ -749,44 +810,28 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
         a.kb[i] = make_uint4(kq[k], kdh[k], (uint32_t)Bp[k], 0u);
       }
     }
-    // One pair on the given state: W (+infinity outside A), and the key (GEN), its rank and the tie word
-    // it has in C.
+    const float den = m.lout > 1.0f ? m.lout : 1.0f;
+    // One pair on the given state: W (+infinity outside A), and the rank and the tie word it has in C (and, under
+    // H-C-Q, its headroom's bits).  Without branches, so that a thread's pairs overlap.
     auto pair = [&](const StepRow& rc, uint32_t i, uint32_t h, float tpf, int32_t rm, int32_t q, int32_t S, int32_t B,
-                    float d0, float f, float tqv, uint32_t kql, uint32_t kh, float* W, uint64_t* key, uint32_t* rank,
+                    float d0, float f, float tqv, uint32_t kql, uint32_t kh, float* W, uint32_t* head, uint32_t* rank,
                     uint32_t* tie) {
       const int32_t n = (int32_t)rc.L - (int32_t)(h << 4);
       *W = (int32_t)rc.L <= rm ? __fsub_rn(tpf, rc.t_cached) : INFINITY;
       float dec = __fadd_rn(d0, __fmul_rn(m.b2, __int2float_rn(S + (int32_t)rc.L)));
       dec = __fmul_rn(dec, f);
       const float qnf = __int2float_rn(q + n);
-      float tpot;
-      if (!GEN || m.interference_mode == 0) {
-        tpot = __fadd_rn(dec, __fmul_rn(m.g_q, qnf));
-      } else {
-        const float den = m.lout > 1.0f ? m.lout : 1.0f;
-        tpot = __fadd_rn(dec, B > 1 ? __fdiv_rn(tpf, den) : 0.0f);
-      }
+      // queued prefill, or Eq. 9's interference
+      const float tpot = __fadd_rn(dec, EQ9 ? (B > 1 ? __fdiv_rn(tpf, den) : 0.0f) : __fmul_rn(m.g_q, qnf));
       const float ttft = __fadd_rn(tpf, tqv);
       const bool adm = (tpot < rc.tpot_lim) & (ttft <= rc.ttft_max);
-      const uint64_t kd = ((uint64_t)kh << 32) | kql;
-      const uint64_t qn = (uint64_t)(uint32_t)(q + n);
-      *tie = i;
-      if (!GEN) {  // Algorithm 1's order: D-C-Q in T, the LMetric product in C \ T
-        // ranks: D and up to 13 bits of C; the product rounded towards zero (both factors exact in fp32,
-        // else from the 64-bit product: the same rounding of the same value)
-        const uint64_t v1 = qn * (uint64_t)(uint32_t)B;
-        const float p1 = (uint32_t)qn < (1u << 24) ? __fmul_rz(qnf, __int2float_rn(B)) : __ull2float_rz(v1);
-        *key = 0ull;
-        *rank = adm ? (kh << 1) | (8191u - min(h, 8191u)) : 0x80000000u | __float_as_uint(p1);
-      } else {
-        if (adm) {
-          *key = psk::packed_key(0u, psk::value_in_t(m, psk::key0_from_dcq(m, kd), h, tpot, rc.tpot_target));
-          if (m.sel == psk::kSelHCQ) *tie |= (kql & 0x3FFFFu) << 12;
-        } else {
-          *key = psk::packed_key(1u, psk::value_fallback(m, qn, (uint32_t)B, kd, h));
-        }
-        *rank = key_rank(*key);
-      }
+      *tie = GEN ? i | (kql & (adm ? order.tie_q : 0u)) << 12 : i;
+      *head = GEN ? psk::f2ord(__fsub_rn(rc.tpot_target, tpot)) : 0u;
+      // The product rounded towards zero: both factors exact in fp32, else from the 64-bit product, the same
+      // rounding of the same value.
+      const uint32_t qn = (uint32_t)(q + n);
+      const float p1 = qn < (1u << 24) ? __fmul_rz(qnf, __int2float_rn(B)) : __ull2float_rz((uint64_t)qn * (uint32_t)B);
+      *rank = adm ? rank_in_t<GEN>(order, kql, kh, h, *head) : rank_fallback<GEN>(order, kh, h, p1);
     };
     uint32_t Lprev = 0;  // length of request s - 1
     for (uint32_t s = 0;; ++s) {
@@ -817,19 +862,19 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
       uint32_t H = __reduce_min_sync(0xffffffffu, er == mr ? eth.y : 0xFFFFFFFFu);
       const unsigned who = __ballot_sync(0xffffffffu, er == mr);
       float W[IPT];
-      uint64_t key[IPT];
-      uint32_t rank[IPT], tie[IPT];
+      uint32_t head[IPT], rank[IPT], tie[IPT];
 #pragma unroll
       for (int k = 0; k < IPT; ++k)
         pair(rc, i0 + (uint32_t)k, h[k], __uint_as_float(tb[k]), room[k], q32[k], S32[k], Bp[k], dec0[k], fe[k], tq[k],
-             kq[k], kdh[k], &W[k], &key[k], &rank[k], &tie[k]);
+             kq[k], kdh[k], &W[k], &head[k], &rank[k], &tie[k]);
       bool own = false;  // this thread owns the last pick
       uint32_t j = 0, hj = 0;
       int4 x = make_int4(0, 0, 0, 0);
       float tpfj = 0.0f;
       if (mr != 0xFFFFFFFFu) {
         if (who & (who - 1u)) {  // equal ranks
-          const int src = warp_argmin(er, key_at(par, er, held ? lane : 0), eth.x);
+          const int src = exact(mr) ? __ffs(__ballot_sync(0xffffffffu, er == mr && eth.x == jt)) - 1
+                                    : warp_argmin(er, key_at(par, er, held ? lane : 0), eth.x);
           jt = __shfl_sync(0xffffffffu, eth.x, src);
           H = __shfl_sync(0xffffffffu, eth.y, src);
         }
@@ -865,13 +910,12 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
         const float tqv =
             __fadd_rn(__fmul_rn(m.a0, __int2float_rn((int32_t)(y.x & 0x3FFFFu))), __fmul_rn(m.a1, __int2float_rn(x.x)));
         float Wj;
-        uint64_t keyj;
-        uint32_t rankj, tiej;
-        pair(rc, j, hj, tpfj, x.z, x.x, x.y, (int32_t)y.z, d0, f, tqv, y.x, y.y, &Wj, &keyj, &rankj, &tiej);
+        uint32_t headj, rankj, tiej;
+        pair(rc, j, hj, tpfj, x.z, x.x, x.y, (int32_t)y.z, d0, f, tqv, y.x, y.y, &Wj, &headj, &rankj, &tiej);
 #pragma unroll
         for (int k = 0; k < IPT; ++k)
           if (i0 + (uint32_t)k == j) {
-            key[k] = keyj;
+            head[k] = headj;
             rank[k] = rankj;
             tie[k] = tiej;
             h[k] = hj;
@@ -907,14 +951,15 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
       uint32_t n_eq = 0;
       uint2 bk;
       uint32_t bt, bh;
-      // The thread's smallest, picked beside the reduction.  Algorithm 1's key stays two words of the pair's
-      // state: only equal ranks read it, and built for every pair it takes a tenth of a step's instructions
-      // (1024 x 16384: 14.36 ms with it, 14.18 without).
+      // The thread's smallest, picked beside the reduction.  Its key stays two words of the pair's state: only
+      // equal ranks read it, and built for every pair it takes a tenth of a step's instructions (Algorithm 1's,
+      // 1024 x 16384: 14.36 ms with it, 14.18 without).
       auto key_words = [&](int k) {
-        if (GEN) return make_uint2((uint32_t)key[k], (uint32_t)(key[k] >> 32));
-        const bool in_t = rank[k] < 0x80000000u;
-        return make_uint2(in_t ? kq[k] : (uint32_t)(q32[k] + ((int32_t)rc.L - (int32_t)(h[k] << 4))),
-                          in_t ? kdh[k] : (uint32_t)Bp[k]);
+        const uint32_t qn = (uint32_t)(q32[k] + ((int32_t)rc.L - (int32_t)(h[k] << 4)));
+        if (!GEN) return rank[k] < 0x80000000u ? make_uint2(kq[k], kdh[k]) : make_uint2(qn, (uint32_t)Bp[k]);
+        const uint32_t fb = rank[k] < 0x80000000u ? ~0u : order.fb_mask;
+        const uint32_t x = order.head_all ? head[k] : kq[k];
+        return make_uint2(fb ? (rank[k] < 0x80000000u ? x : kq[k]) : qn, fb ? kdh[k] : (uint32_t)Bp[k]);
       };
 #pragma unroll
       for (int k = 0; k < IPT; ++k)
@@ -935,13 +980,14 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
       const unsigned many = IPT > 1 ? __ballot_sync(0xffffffffu, has && n_eq > 1u) : 0u;
       if (mw != 0xFFFFFFFFu && ((lanes & (lanes - 1u)) | many)) {
         // equal ranks: the smallest (key, tie) of the lane's, then of the warp's
+        const bool ex = exact(mw);  // the keys are equal too
         uint64_t kk = psk::kNoKey;
         bt = 0xFFFFFFFFu;
 #pragma unroll
         for (int k = 0; k < IPT; ++k)
           if (rank[k] == mw) {
             const uint2 w = key_words(k);
-            const uint64_t x = GEN ? key[k] : dcq_key(mw, w, h[k]);
+            const uint64_t x = ex ? 0ull : pair_key<GEN>(m, mw, w, h[k]);
             if (x < kk || (x == kk && tie[k] < bt)) {
               kk = x;
               bk = w;
@@ -949,9 +995,11 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
               bh = h[k];
             }
           }
-        const int win = warp_argmin(has ? mw : 0xFFFFFFFFu, kk, bt);
+        bool win;
+        if (ex) win = bt == __reduce_min_sync(0xffffffffu, bt) && has;
+        else win = lane == warp_argmin(has ? mw : 0xFFFFFFFFu, kk, bt);
         __syncwarp();
-        if (lane == win) {
+        if (win) {
           s_th[s & 1u][warp] = make_uint2(bt, bh);
           s_key[s & 1u][warp] = bk;
         }
@@ -1163,7 +1211,9 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
   }
 }
 
-template <int IPT, bool GEN, bool LIN>
+// GEN: not Algorithm 1's order (Table 4 / Table 3 variants); EQ9: Eq. 9's interference term; LIN: caches that are
+// not prefix-closed (built for every order).
+template <int IPT, bool GEN, bool EQ9, bool LIN>
 __global__ void __launch_bounds__(kPipeThreads, 1)
 greedy_pipe_kernel(const psk::RowPre* __restrict__ rows, const uint64_t* __restrict__ hash, uint32_t R, uint32_t I,
                    const uint32_t* __restrict__ hit0, const float* __restrict__ tpf0, psk::StateSoA committed,
@@ -1172,7 +1222,7 @@ greedy_pipe_kernel(const psk::RowPre* __restrict__ rows, const uint64_t* __restr
                    uint32_t ninsert, MainTables mt) {
   extern __shared__ __align__(16) unsigned long long smem_raw[];
   if (blockIdx.x == 0) {
-    decide_rows<IPT, GEN, LIN>(rows, R, I, committed, pending, m, assign, path, hit_chosen, err, sync, smem_raw, hash, mt);
+    decide_rows<IPT, GEN, EQ9, LIN>(rows, R, I, committed, pending, m, assign, path, hit_chosen, err, sync, smem_raw, hash, mt);
   } else if (blockIdx.x <= ninsert) {
     insert_blocks<LIN>(rows, hash, R, delta, nslots, err, sync, blockIdx.x - 1, ninsert);
   } else {
@@ -1195,10 +1245,11 @@ cudaError_t greedy_pipe_launch(const psk::RowPre* rows, const psk::WindowDev& w,
                                psk::DeltaSlot* delta, uint64_t nslots, int32_t* assign, uint8_t* path,
                                uint32_t* hit_chosen, uint32_t* err, const psk::GreedySync& sync, bool linear,
                                MainTables mt, int num_sms, cudaStream_t s) {
-  // not Algorithm 1's order (Table 4 / Table 3 variants), or Eq. 9's interference term
-  const bool gen = m.sel != psk::kSelDCQ || m.fb_dcq || m.interference_mode != 0;
-  auto kern = linear ? greedy_pipe_kernel<IPT, true, true>
-                     : (gen ? greedy_pipe_kernel<IPT, true, false> : greedy_pipe_kernel<IPT, false, false>);
+  const bool gen = m.sel != psk::kSelDCQ || m.fb_dcq, eq9 = m.interference_mode != 0;
+  decltype(&greedy_pipe_kernel<IPT, true, true, true>) kern;
+  if (linear) kern = eq9 ? greedy_pipe_kernel<IPT, true, true, true> : greedy_pipe_kernel<IPT, true, false, true>;
+  else if (gen) kern = eq9 ? greedy_pipe_kernel<IPT, true, true, false> : greedy_pipe_kernel<IPT, true, false, false>;
+  else kern = eq9 ? greedy_pipe_kernel<IPT, false, true, false> : greedy_pipe_kernel<IPT, false, false, false>;
   const size_t smem = greedy_pipe_smem(I, sync.ring_stride);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;

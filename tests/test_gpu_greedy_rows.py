@@ -132,6 +132,40 @@ def test_sums_beyond_32_bits(P, shift):
         _check(P, dict(wl.model, selector=sel), ins, wl.window)
 
 
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("ablation", ["F", "C", "CT"])
+@pytest.mark.parametrize("sel", range(6))
+def test_pairs_that_a_rank_does_not_tell_apart(P, sel, ablation, mode):
+    """A rank holds part of a key: here many pairs are equal in that part (hits and queues around the 8191 it
+    stops at, few values of b, b and h of 0 under the D-C-Q fallback, negative headrooms where everything is
+    admitted), so the rest of the key or the tie word decides."""
+    from oracle import ABLATIONS
+    rng = np.random.default_rng(sel)
+    I, R = 120, 40
+    trunk = rng.integers(2, 2 ** 63, 8300, dtype=np.int64).astype(np.uint64)
+    ins, win = _prompts([16 * 8300 + 3] * R, [trunk] * R, I)
+    ins.M_KV[:] = 2 ** 29
+    ins.cap_blocks[:] = 8400
+    ins.b[:] = rng.choice([0, 7], I)
+    ins.qr[:] = rng.choice([0, 3, 8190, 8191, 8192, 9000, 131000], I)
+    ins.B_max[:] = ins.b + ins.qr + 1  # each takes one request: every decision is the next in order
+    n = rng.choice([0, 1, 8189, 8190, 8191, 8192, 8250], I)
+    ins.chain_inst = np.arange(I, dtype=np.uint32)
+    ins.chain_off = np.concatenate([[0], np.cumsum(n)]).astype(np.uint64)
+    ins.chain_hash = np.concatenate([trunk[:k] for k in n])
+    ins.chain_parent = np.zeros(I, np.uint64)
+    win.tpot_target[::2] = 5.0  # missed: the fallback (or, with everything admitted, a negative headroom)
+    model = dict(W.MODEL_DEFAULT, eta=1e6, b1=0.0)
+    orc = Oracle(I, dict(model, selector=sel, **ABLATIONS[ablation])).load(ins)
+    with P.Scheduler(I, ins.cap_blocks, R, int(win.chain_off[-1]), dict(model, selector=sel, **P.ABLATIONS[ablation]),
+                     probe_mode=mode) as s:
+        s.load_workload_instances(ins)
+        g, o = s.schedule_window(win), orc.schedule(win)
+        for k in ("assign", "path", "hit_chosen"):
+            assert np.array_equal(g[k], o[k]), (k, np.nonzero(g[k] != o[k])[0][:5])
+    assert set(o["path"].tolist()) == ({0} if ablation == "C" else {0, 1})
+
+
 @pytest.mark.parametrize("I", [1, 33, 512, 513, 1024, 1025, 2048])
 @pytest.mark.parametrize("sel", [0, 5])
 def test_instance_counts_in_linear_mode(P, I, sel):
