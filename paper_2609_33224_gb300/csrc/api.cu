@@ -987,7 +987,7 @@ ps_status ps_schedule_window(ps_ctx* c, const ps_window* w, ps_decisions* out, p
   record(c, kEvGreedy0);
   PS_TRY_CUDA(c, pskl::launch_greedy(c->d_rows, wd, c->I, hit0, c->d_tpf, c->st, c->pend, c->model, c->d_delta,
                                      nslots, c->d_assign, c->d_dpath, c->d_hchosen, c->d_err, c->gsync,
-                                     c->search, c->d_slots, c->d_ovf, c->d_tdesc, c->num_sms, c->stream));
+                                     c->search, c->d_slots, c->d_ovf, c->d_tdesc, c->win_blocks, c->num_sms, c->stream));
   if (wd.R == 0)  // nobody to decide: the greedy pass, which writes the pending state, does not run
     PS_TRY_CUDA(c, cudaMemcpyAsync(c->pend_block, c->st_block, c->I * kStateBytes, cudaMemcpyDeviceToDevice, c->stream));
   record(c, kEvGreedy1);

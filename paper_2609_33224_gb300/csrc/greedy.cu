@@ -565,7 +565,8 @@ template <int IPT, bool GEN, bool EQ9, bool LIN>
 __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, uint32_t I, psk::StateSoA committed,
                             psk::StateSoA pending, const psk::DevModel& m, int32_t* assign, uint8_t* __restrict__ path,
                             uint32_t* __restrict__ hit_chosen, uint32_t* err, const psk::GreedySync& sync,
-                            unsigned long long* smem_raw, const uint64_t* __restrict__ hash, const MainTables& mt) {
+                            unsigned long long* smem_raw, const uint64_t* __restrict__ hash, const MainTables& mt,
+                            uint64_t tokens) {
   const uint32_t Ip = sync.ring_stride;
   const InstSmem a = inst_smem(smem_raw, Ip);
   uint32_t* s_hitr = reinterpret_cast<uint32_t*>(a.pad + Ip);  // [kFeedRing][Ip] hits
@@ -588,12 +589,13 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
   if (t < kComputeWarps) {
     s_w[t] = 0xFFFFFFFFu;
   }
-  // An instance only takes requests that fit its KV room, so S stays below max(S, M), and q gains at
-  // most what S gains: with these bounds 32 bits hold every q and S of the window.
+  // An instance only takes requests that fit its KV room, so S stays below max(S, M), it gains no more than the
+  // window's tokens, and q gains at most what S gains: with these bounds 32 bits hold every q and S of the
+  // window.  (A KV room above 2^31 - 1 counts as that much, still more than any prompt at the end.)
   bool narrow = true;
   for (uint32_t i = t; i < I; i += kPipeThreads) {
     const int64_t M = committed.M[i], S = committed.S[i], q = committed.q[i];
-    const int64_t gain = M > S ? M - S : 0;
+    const int64_t gain = M > S ? (M - S < (int64_t)tokens ? M - S : (int64_t)tokens) : 0;
     narrow = narrow && S + gain < (1ll << 30) && q + gain < (1ll << 30);
   }
   if (t == 0) {
@@ -1219,10 +1221,11 @@ greedy_pipe_kernel(const psk::RowPre* __restrict__ rows, const uint64_t* __restr
                    const uint32_t* __restrict__ hit0, const float* __restrict__ tpf0, psk::StateSoA committed,
                    psk::StateSoA pending, psk::DevModel m, psk::DeltaSlot* delta, uint64_t nslots, int32_t* assign,
                    uint8_t* __restrict__ path, uint32_t* __restrict__ hit_chosen, uint32_t* err, psk::GreedySync sync,
-                   uint32_t ninsert, MainTables mt) {
+                   uint32_t ninsert, MainTables mt, uint64_t tokens) {
   extern __shared__ __align__(16) unsigned long long smem_raw[];
   if (blockIdx.x == 0) {
-    decide_rows<IPT, GEN, EQ9, LIN>(rows, R, I, committed, pending, m, assign, path, hit_chosen, err, sync, smem_raw, hash, mt);
+    decide_rows<IPT, GEN, EQ9, LIN>(rows, R, I, committed, pending, m, assign, path, hit_chosen, err, sync, smem_raw, hash, mt,
+                                    tokens);
   } else if (blockIdx.x <= ninsert) {
     insert_blocks<LIN>(rows, hash, R, delta, nslots, err, sync, blockIdx.x - 1, ninsert);
   } else {
@@ -1244,7 +1247,7 @@ cudaError_t greedy_pipe_launch(const psk::RowPre* rows, const psk::WindowDev& w,
                                const float* tpf0, psk::StateSoA committed, psk::StateSoA pending, const psk::DevModel& m,
                                psk::DeltaSlot* delta, uint64_t nslots, int32_t* assign, uint8_t* path,
                                uint32_t* hit_chosen, uint32_t* err, const psk::GreedySync& sync, bool linear,
-                               MainTables mt, int num_sms, cudaStream_t s) {
+                               MainTables mt, uint64_t tokens, int num_sms, cudaStream_t s) {
   const bool gen = m.sel != psk::kSelDCQ || m.fb_dcq, eq9 = m.interference_mode != 0;
   decltype(&greedy_pipe_kernel<IPT, true, true, true>) kern;
   if (linear) kern = eq9 ? greedy_pipe_kernel<IPT, true, true, true> : greedy_pipe_kernel<IPT, true, false, true>;
@@ -1261,7 +1264,7 @@ cudaError_t greedy_pipe_launch(const psk::RowPre* rows, const psk::WindowDev& w,
   uint32_t ninsert = 0;
   void* args[] = {(void*)&rows, (void*)&hash, (void*)&R, (void*)&I, (void*)&hit0, (void*)&tpf0, (void*)&c, (void*)&p,
                   (void*)&mm, (void*)&delta, (void*)&nslots, (void*)&assign, (void*)&path, (void*)&hit_chosen,
-                  (void*)&err, (void*)&sy, (void*)&ninsert, (void*)&mt};
+                  (void*)&err, (void*)&sy, (void*)&ninsert, (void*)&mt, (void*)&tokens};
   // All blocks must be resident at once, and one fits on an SM.  A stream may be limited to fewer SMs than the
   // device reports: a launch that is too large for it is refused before it starts, and half as many tried.
   for (uint32_t resident = (uint32_t)num_sms;; resident /= 2u) {
@@ -1281,8 +1284,8 @@ cudaError_t launch_greedy(const psk::RowPre* rows, const psk::WindowDev& w, uint
                                  const float* tpf0, psk::StateSoA committed, psk::StateSoA pending, const psk::DevModel& m,
                                  psk::DeltaSlot* delta, uint64_t delta_nslots, int32_t* assign, uint8_t* path,
                                  uint32_t* hit_chosen, uint32_t* err, const psk::GreedySync& sync, int search,
-                                 const uint64_t* slots, const uint64_t* ovf, const psk::TableDesc* tdesc, int num_sms,
-                                 cudaStream_t s) {
+                                 const uint64_t* slots, const uint64_t* ovf, const psk::TableDesc* tdesc,
+                                 uint64_t win_blocks, int num_sms, cudaStream_t s) {
   const MainTables mt{slots, ovf, tdesc};
   const cudaError_t e = cudaMemsetAsync(sync.stats, 0, sync.clear_bytes, s);
   if (e != cudaSuccess || w.R == 0) return e;
@@ -1292,7 +1295,7 @@ cudaError_t launch_greedy(const psk::RowPre* rows, const psk::WindowDev& w, uint
   const uint32_t ipt = (I + 32u * kComputeWarps - 1) / (32u * kComputeWarps);
 #define PS_GREEDY_P(IPT)                                                                                      \
   return greedy_pipe_launch<IPT>(rows, w, I, hit0, tpf0, committed, pending, m, delta, delta_nslots, assign, path, \
-                                 hit_chosen, err, sync, search == 0, mt, num_sms, s)
+                                 hit_chosen, err, sync, search == 0, mt, 16u * (win_blocks + w.R), num_sms, s)
   if (ipt <= 1) PS_GREEDY_P(1);
   if (ipt <= 2) PS_GREEDY_P(2);
   if (ipt <= 4) PS_GREEDY_P(4);

@@ -875,12 +875,13 @@ cudaError_t launch_expand_chains(const uint64_t* full_off, const uint64_t* own_o
 cudaError_t launch_relations(const psk::WindowDev& w, const psk::DevModel& m, psk::LastSlot* tab, uint32_t tab_n,
                              psk::RowPre* rows, psk::RowList list, int search, int num_sms, cudaStream_t s);
 // search 0: the caches need not be prefix-closed (rows' limits set, the committed tables probed too).
+// win_blocks: the window's chain blocks.
 cudaError_t launch_greedy(const psk::RowPre* rows, const psk::WindowDev& w, uint32_t I, const uint32_t* hit0,
                           const float* tpf0, psk::StateSoA committed, psk::StateSoA pending, const psk::DevModel& m,
                           psk::DeltaSlot* delta, uint64_t delta_nslots, int32_t* assign, uint8_t* path,
                           uint32_t* hit_chosen, uint32_t* err, const psk::GreedySync& sync, int search,
-                          const uint64_t* slots, const uint64_t* ovf, const psk::TableDesc* tdesc, int num_sms,
-                          cudaStream_t s);
+                          const uint64_t* slots, const uint64_t* ovf, const psk::TableDesc* tdesc, uint64_t win_blocks,
+                          int num_sms, cudaStream_t s);
 cudaError_t launch_insert_chains(uint64_t* slots, uint64_t* ovf, const psk::TableDesc* tdesc, uint32_t I,
                                  unsigned long long* count, uint64_t nchains, const uint32_t* inst,
                                  const uint64_t* off, const uint64_t* hash, const uint64_t* parent,

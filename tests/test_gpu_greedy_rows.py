@@ -132,6 +132,23 @@ def test_sums_beyond_32_bits(P, shift):
         _check(P, dict(wl.model, selector=sel), ins, wl.window)
 
 
+@pytest.mark.parametrize("M", [2 ** 30, 2 ** 31 - 1, 2 ** 31 + 5, 2 ** 45, 2 ** 50 - 1])
+@pytest.mark.parametrize("below", [-16, -1, 0, 1, 400, 10 ** 6])
+def test_kv_room_beyond_32_bits(P, M, below):
+    """The window's tokens bound what an instance can gain, so rooms beyond 32 bits alone need no 64-bit sums;
+    held and queued tokens a few tokens on either side of where the sums would leave 2^30."""
+    wl = _workload(5, 60, seed=14)
+    ins = wl.instances
+    tokens = 16 * (int(wl.window.chain_off[-1]) + wl.window.R)
+    ins.M_KV[:] = M
+    ins.S[:4] = 2 ** 30 - tokens - below
+    ins.q[2:] = 2 ** 30 - tokens - below
+    ins.b[:], ins.qr[:] = 1, 0
+    wl.window.tpot_target[:] = 1e9  # every request is admitted somewhere
+    wl.window.ttft_target[:] = 1e9
+    _check(P, dict(wl.model, eta=1e6), ins, wl.window)
+
+
 @pytest.mark.parametrize("mode", [0, 1])
 @pytest.mark.parametrize("ablation", ["F", "C", "CT"])
 @pytest.mark.parametrize("sel", range(6))
