@@ -480,6 +480,16 @@ struct PairOrder {  // masks of the launch's order: a step has no branch on it
   __device__ __forceinline__ bool exact(uint32_t rank) const {
     return rank < 0x80000000u && ((rank & ex_mask) | ex_any) != 0u;
   }
+  // In T: b, then up to 13 bits of h (more is better) or of qr; H-C-Q: the headroom (head: f2ord of it).
+  __device__ __forceinline__ uint32_t in_t(uint32_t kq, uint32_t kdh, uint32_t h, uint32_t head) const {
+    return ((kdh << 1) & d_mask) | ((8191u - min(h, 8191u)) & c_mask) | ((kq >> 5) & q_mask) |
+           ((head >> head_shift) & head_mask);
+  }
+  // In C \ T: the product rounded towards zero as fp32 (p), or the D-C-Q order's bits.
+  __device__ __forceinline__ uint32_t fallback(uint32_t kdh, uint32_t h, float p) const {
+    const uint32_t dc = (kdh << 1) | (8191u - min(h, 8191u));
+    return 0x80000000u | ((dc >> 1) & fb_mask) | (__float_as_uint(p) & ~fb_mask);
+  }
 };
 
 __device__ __forceinline__ PairOrder pair_order(const psk::DevModel& m) {
@@ -496,21 +506,6 @@ __device__ __forceinline__ PairOrder pair_order(const psk::DevModel& m) {
   o.ex_any = dq || m.sel == psk::kSelD ? 1u : 0u;
   o.head_shift = m.slo_off ? 5u : 0u;  // an admitted pair's headroom is positive, unless everything is admitted
   return o;
-}
-
-// In T: b, then up to 13 bits of h (more is better) or of qr; H-C-Q: the headroom (head: f2ord of it).
-template <bool GEN>
-__device__ __forceinline__ uint32_t rank_in_t(const PairOrder& o, uint32_t kq, uint32_t kdh, uint32_t h, uint32_t head) {
-  const uint32_t c = 8191u - min(h, 8191u);
-  if (!GEN) return (kdh << 1) | c;
-  return ((kdh << 1) & o.d_mask) | (c & o.c_mask) | ((kq >> 5) & o.q_mask) | ((head >> o.head_shift) & o.head_mask);
-}
-
-// In C \ T: the product rounded towards zero as fp32 (p), or the D-C-Q order's bits.
-template <bool GEN>
-__device__ __forceinline__ uint32_t rank_fallback(const PairOrder& o, uint32_t kdh, uint32_t h, float p) {
-  const uint32_t dc = (kdh << 1) | (8191u - min(h, 8191u));
-  return 0x80000000u | (GEN ? ((dc >> 1) & o.fb_mask) | (__float_as_uint(p) & ~o.fb_mask) : __float_as_uint(p));
 }
 
 template <bool GEN>
@@ -827,13 +822,19 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
       const float tpot = __fadd_rn(dec, EQ9 ? (B > 1 ? __fdiv_rn(tpf, den) : 0.0f) : __fmul_rn(m.g_q, qnf));
       const float ttft = __fadd_rn(tpf, tqv);
       const bool adm = (tpot < rc.tpot_lim) & (ttft <= rc.ttft_max);
-      *tie = GEN ? i | (kql & (adm ? order.tie_q : 0u)) << 12 : i;
-      *head = GEN ? psk::f2ord(__fsub_rn(rc.tpot_target, tpot)) : 0u;
       // The product rounded towards zero: both factors exact in fp32, else from the 64-bit product, the same
       // rounding of the same value.
-      const uint32_t qn = (uint32_t)(q + n);
-      const float p1 = qn < (1u << 24) ? __fmul_rz(qnf, __int2float_rn(B)) : __ull2float_rz((uint64_t)qn * (uint32_t)B);
-      *rank = adm ? rank_in_t<GEN>(order, kql, kh, h, *head) : rank_fallback<GEN>(order, kh, h, p1);
+      const uint64_t qn = (uint64_t)(uint32_t)(q + n);
+      const uint64_t v1 = qn * (uint64_t)(uint32_t)B;
+      const float p1 = (uint32_t)qn < (1u << 24) ? __fmul_rz(qnf, __int2float_rn(B)) : __ull2float_rz(v1);
+      *tie = i;
+      if constexpr (GEN) {
+        *tie |= (kql & (adm ? order.tie_q : 0u)) << 12;
+        *head = psk::f2ord(__fsub_rn(rc.tpot_target, tpot));
+        *rank = adm ? order.in_t(kql, kh, h, *head) : order.fallback(kh, h, p1);
+      } else {  // Algorithm 1's order: D and up to 13 bits of C in T, the product in C \ T
+        *rank = adm ? (kh << 1) | (8191u - min(h, 8191u)) : 0x80000000u | __float_as_uint(p1);
+      }
     };
     uint32_t Lprev = 0;  // length of request s - 1
     for (uint32_t s = 0;; ++s) {
@@ -917,7 +918,7 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
 #pragma unroll
         for (int k = 0; k < IPT; ++k)
           if (i0 + (uint32_t)k == j) {
-            head[k] = headj;
+            if (GEN) head[k] = headj;
             rank[k] = rankj;
             tie[k] = tiej;
             h[k] = hj;
@@ -957,11 +958,16 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
       // equal ranks read it, and built for every pair it takes a tenth of a step's instructions (Algorithm 1's,
       // 1024 x 16384: 14.36 ms with it, 14.18 without).
       auto key_words = [&](int k) {
-        const uint32_t qn = (uint32_t)(q32[k] + ((int32_t)rc.L - (int32_t)(h[k] << 4)));
-        if (!GEN) return rank[k] < 0x80000000u ? make_uint2(kq[k], kdh[k]) : make_uint2(qn, (uint32_t)Bp[k]);
-        const uint32_t fb = rank[k] < 0x80000000u ? ~0u : order.fb_mask;
-        const uint32_t x = order.head_all ? head[k] : kq[k];
-        return make_uint2(fb ? (rank[k] < 0x80000000u ? x : kq[k]) : qn, fb ? kdh[k] : (uint32_t)Bp[k]);
+        const bool in_t = rank[k] < 0x80000000u;
+        if constexpr (GEN) {
+          const bool kd = in_t || order.fb_mask;
+          const uint32_t x = order.head_all && in_t ? head[k] : kq[k];
+          return make_uint2(kd ? x : (uint32_t)(q32[k] + ((int32_t)rc.L - (int32_t)(h[k] << 4))),
+                            kd ? kdh[k] : (uint32_t)Bp[k]);
+        } else {
+          return make_uint2(in_t ? kq[k] : (uint32_t)(q32[k] + ((int32_t)rc.L - (int32_t)(h[k] << 4))),
+                            in_t ? kdh[k] : (uint32_t)Bp[k]);
+        }
       };
 #pragma unroll
       for (int k = 0; k < IPT; ++k)
@@ -997,11 +1003,10 @@ __device__ void decide_rows(const psk::RowPre* __restrict__ rows, uint32_t R, ui
               bh = h[k];
             }
           }
-        bool win;
-        if (ex) win = bt == __reduce_min_sync(0xffffffffu, bt) && has;
-        else win = lane == warp_argmin(has ? mw : 0xFFFFFFFFu, kk, bt);
+        const int win = ex ? __ffs(__ballot_sync(0xffffffffu, bt == __reduce_min_sync(0xffffffffu, bt))) - 1
+                           : warp_argmin(has ? mw : 0xFFFFFFFFu, kk, bt);
         __syncwarp();
-        if (win) {
+        if (lane == win) {
           s_th[s & 1u][warp] = make_uint2(bt, bh);
           s_key[s & 1u][warp] = bk;
         }
