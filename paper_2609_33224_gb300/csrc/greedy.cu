@@ -465,7 +465,8 @@ __device__ __forceinline__ uint32_t key_rank(uint64_t key) {
 // The rank and the packed key of a pair from 32-bit words of its state, in every instance order (GEN; else
 // Algorithm 1's).  With a 64-bit key by the order for every pair and branches on the order, the other orders cost
 // 90 instructions a pair more: 1025 instances (four a thread) took 1.91 us a decision in the D order, 1.83 in
-// H-C-Q and 2.00 with Eq. 9; 1.50, 1.42 and 1.49 now (Algorithm 1's order: 1.11).  Ranks are made for every pair, keys only where ranks are equal, from two words of the pair:
+// H-C-Q and 2.00 with Eq. 9; 1.52, 1.43 and 1.49 now (Algorithm 1's order, whose kernels have their rank
+// written out: 1.11).  Ranks are made for every pair, keys only where ranks are equal, from two words of the pair:
 // {D-C-Q key bits of qr, of b} in T (H-C-Q: the headroom's bits) and under the D-C-Q fallback, {q + n, B}
 // under the product.
 // Where qr comes last in an order, the tie word of a pair in T starts with it, so that nearly always equal ranks
