@@ -290,8 +290,8 @@ ps_status check_capacity(ps_ctx* c) {
   return PS_OK;
 }
 
-// Arrays of a host window, or of chains to insert, on their way to the device: packed into the staging block and copied in one
-// piece when they fit (flush), else copied each to its own buffer.
+// Arrays of a host window, or of chains to insert, on their way to the device: packed into the staging
+// block and copied in one piece when they fit (flush), else copied each to its own buffer.
 struct Stager {
   ps_ctx* c;
   const bool beside;  // next to a pending window that is staged: into the second set
